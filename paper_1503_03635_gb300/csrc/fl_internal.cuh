@@ -372,9 +372,9 @@ struct Counters {
     unsigned long long mask_scanned; // hop census: of those, read by the mask merge
     unsigned long long delta_next;   // merge: sum of deg(u) * |D_h(u)| over changed u (delta ranks of the next hop's edge-merges)
     unsigned long long new_entries;  // merge: entries gained this hop (sum of |D_h(v)|)
-    unsigned long long key_or[2];    // keys: OR of the candidates' (hi, lo) key words
-    unsigned long long key_orn[2];   // keys: OR of their complements (a bit set in both varies)
-    unsigned long long key_ties;     // keys: adjacent equal hi words after sorting by hi
+    unsigned long long key_or;       // keys: OR of the candidates' radius words
+    unsigned long long key_orn;      // keys: OR of their complements (a bit set in both varies)
+    unsigned long long key_ties;     // keys: a run of equal radius prefixes too long to order in place
 };
 
 // ----------------------------------------------------------------- profiling
@@ -548,7 +548,7 @@ struct fl_solve {
     fl::DBuf kill;                 // uint8[n]: 1 + distance to a client claimed in the current round
     std::vector<int64_t> mis_log;  // rows of 6: the rounds of the last MIS (fl_mis_log)
     fl::DBuf X, stamp, mval, fr[2], frval, touched, ulist, ubuck, bcount;
-    fl::DBuf key_hi, key_lo, key_val, obj_tmp;  // key sort and objective scratch
+    fl::DBuf key_hi, key_lo, key_val, key_alt, obj_tmp;  // key sort and objective scratch
     fl::DBuf part_T;               // int32[n_parts]: largest ball radius of a part's undecided facilities
     fl::DBuf io;                   // per-vertex inputs/outputs in original order (relabelled graphs)
     fl::DBuf open;                 // uint8[n]
@@ -571,17 +571,25 @@ int scan_exclusive_i64(const int64_t* in, int64_t* out, int64_t n, cudaStream_t 
                        int cls = kProfSketchOther);
 int scan_exclusive_i32_to_i64(const int32_t* in, int64_t* out, int64_t n, cudaStream_t st, DBuf& tmp,
                               int cls = kProfSketchOther);
-// Stable LSD radix sort of (hi, lo) pairs with a payload, 4 bits per pass:
-// passes 0-15 take lo's digits, 16-31 hi's; [pass_begin, pass_end) (an even
-// count) may skip digits known to be equal.
-int sort_pairs_u128(uint64_t* hi, uint64_t* lo, uint32_t* val, int64_t n, cudaStream_t st, DBuf& tmp,
-                    int cls = kProfKeys, int pass_begin = 0, int pass_end = 32);
-// The same sort over the digits whose bit is set in `digits` (bit p: pass p
-// of the full sort, 0-15 lo's digits, 16-31 hi's), least significant first.
-// Leaving out digits that are equal in every key changes nothing: a pass
-// over such a digit is the identity.
-int sort_pairs_u128_digits(uint64_t* hi, uint64_t* lo, uint32_t* val, int64_t n, cudaStream_t st, DBuf& tmp,
-                           int cls, uint32_t digits);
+// Stable LSD radix sort of (key, payload) pairs (k_sort.cu).  The pairs are in
+// buffer `cur` before and after; shift[0..nd) are the low bits of the 8-bit
+// digits, least significant first.  A wait of the sort that runs out sets
+// kSortError in *err (never on a working device).
+constexpr int kSortDigits = 8;
+constexpr unsigned long long kSortError = 1ULL << 16;
+template <class K>
+struct SortPairs {
+    K* key[2];
+    uint32_t* val[2];
+    int cur = 0;
+};
+template <class K>
+int sort_pairs(SortPairs<K>& p, int64_t n, const int* shift, int nd, cudaStream_t st, DBuf& tmp, int cls,
+               unsigned long long* err);
+// 8-bit digits that cover the set bits of `varying` (bits > 0: only that many
+// from its highest one down); returns their number.  The keys agree below
+// shift[0] only if every varying bit is covered.
+int digit_windows(uint64_t varying, int bits, int* shift);
 
 int validate_csr(fl_graph* g);
 int build_work_lists(fl_graph* g);
@@ -594,7 +602,7 @@ int compute_ecc_bound(fl_graph* g);
 
 int check_costs(fl_solve* s);
 int compute_radii(fl_solve* s);
-int sort_candidates(fl_solve* s, int64_t* m_out);
+int sort_candidates(fl_solve* s, int64_t* m_out, const uint32_t** sorted);
 int open_facilities(fl_solve* s);
 // the greedy MIS and the assignment by weighted distance (k_wsolve.cu)
 int open_facilities_weighted(fl_solve* s);

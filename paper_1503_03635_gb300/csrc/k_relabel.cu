@@ -27,16 +27,14 @@ int grid_for(int64_t items, int per_block) {
 // order, kept by the stable sort).
 // *max_key_span: the largest degree (capped like the key), so that the sort
 // can leave out the key digits above it, equal in every key.
-__global__ void k_degree_keys(const int64_t* __restrict__ rowp, int64_t n, uint64_t* __restrict__ hi,
-                              uint64_t* __restrict__ lo, uint32_t* __restrict__ val,
-                              unsigned long long* __restrict__ max_deg) {
+__global__ void k_degree_keys(const int64_t* __restrict__ rowp, int64_t n, uint32_t* __restrict__ key,
+                              uint32_t* __restrict__ val, unsigned long long* __restrict__ max_deg) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     unsigned mx = 0;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
         const int64_t d = rowp[v + 1] - rowp[v];
         const uint64_t dc = (uint64_t)(d < 0x7fffffffLL ? d : 0x7fffffffLL);
-        hi[v] = 0x7fffffffULL - dc;
-        lo[v] = (uint64_t)v;
+        key[v] = 0x7fffffffu - (uint32_t)dc;
         val[v] = (uint32_t)v;
         mx = max(mx, (unsigned)dc);
     }
@@ -351,34 +349,37 @@ __global__ void k_ads_reorder(const int64_t* __restrict__ gofs, const int64_t* _
 int relabel_graph(fl_graph* g) {
     const int64_t n = g->n;
     cudaStream_t st = g->stream;
-    DBuf hi, lo, val, deg, rowp_new, cols_new;
+    DBuf key, val, deg, rowp_new, cols_new;
     int rc = FL_OK;
     do {
-        if ((rc = dalloc(hi, (size_t)n * 8)) || (rc = dalloc(lo, (size_t)n * 8)) || (rc = dalloc(val, (size_t)n * 4 + 64)) ||
+        if ((rc = dalloc(key, (size_t)n * 8)) || (rc = dalloc(val, (size_t)n * 8 + 64)) ||
             (rc = dalloc(deg, (size_t)n * 4 + 96)) || (rc = dalloc(rowp_new, (size_t)(n + 1) * 8)) ||
             (rc = dalloc(cols_new, (size_t)std::max<int64_t>(g->nnz, 1) * 4)) ||
             (rc = dalloc(g->rid, (size_t)n * 4)) || (rc = dalloc(g->inv, (size_t)n * 4)))
             break;
-        unsigned long long* max_deg = reinterpret_cast<unsigned long long*>(val.as<char>() + (((size_t)n * 4 + 15) & ~(size_t)15));
+        unsigned long long* max_deg = reinterpret_cast<unsigned long long*>(val.as<char>() + (((size_t)n * 8 + 15) & ~(size_t)15));
         cudaError_t e = cudaMemsetAsync(max_deg, 0, 8, st);
         if (e != cudaSuccess) { rc = status_of(e, "relabel", __FILE__, __LINE__); break; }
         FL_LAUNCH(kProfOther, k_degree_keys<<<grid_for(n, 256), 256, 0, st>>>(
-                                  g->rowp.as<int64_t>(), n, hi.as<uint64_t>(), lo.as<uint64_t>(), val.as<uint32_t>(),
-                                  max_deg));
+                                  g->rowp.as<int64_t>(), n, key.as<uint32_t>(), val.as<uint32_t>(), max_deg));
         unsigned long long hmax = 0;
         e = cudaMemcpyAsync(&hmax, max_deg, 8, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) { rc = status_of(e, "relabel", __FILE__, __LINE__); break; }
-        // keys lie in [2^31 - 1 - max, 2^31 - 1]: digits above the highest bit
+        // keys lie in [2^31 - 1 - max, 2^31 - 1]: the bits above the highest one
         // where the two ends differ are equal in every key
-        const uint64_t span = 0x7fffffffULL ^ (0x7fffffffULL - hmax);
-        uint32_t digits = 0;
-        for (int q = 0; q < 8 && (span >> (4 * q)) != 0; ++q) digits |= 1u << (16 + q);
-        if ((rc = sort_pairs_u128_digits(hi.as<uint64_t>(), lo.as<uint64_t>(), val.as<uint32_t>(), n, st, g->scratch,
-                                         kProfOther, digits)))
-            break;
+        uint64_t span = 0x7fffffffULL ^ (0x7fffffffULL - hmax);
+        for (int o = 1; o < 32; o <<= 1) span |= span >> o;
+        int shift[kSortDigits];
+        const int nd = digit_windows(span, 0, shift);
+        SortPairs<uint32_t> sp;
+        sp.key[0] = key.as<uint32_t>();
+        sp.key[1] = sp.key[0] + n;
+        sp.val[0] = val.as<uint32_t>();
+        sp.val[1] = sp.val[0] + n;
+        if ((rc = sort_pairs(sp, n, shift, nd, st, g->scratch, kProfOther, &g->ctr.as<Counters>()->error))) break;
         FL_LAUNCH(kProfOther, k_perm_maps<<<grid_for(n, 256), 256, 0, st>>>(
-                                  val.as<uint32_t>(), g->rowp.as<int64_t>(), n, g->rid.as<int32_t>(),
+                                  sp.val[sp.cur], g->rowp.as<int64_t>(), n, g->rid.as<int32_t>(),
                                   g->inv.as<int32_t>(), deg.as<int32_t>()));
         if ((rc = scan_exclusive_i32_to_i64(deg.as<int32_t>(), rowp_new.as<int64_t>(), n, st, g->scratch, kProfOther)))
             break;
@@ -421,13 +422,14 @@ int relabel_graph(fl_graph* g) {
                                           rp, cl, rid, inv, rpn, c_small, c_none, cn));
         }
         e = cudaGetLastError();
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) { rc = status_of(e, "relabel", __FILE__, __LINE__); break; }
+        if ((rc = read_counters(g))) break;
+        if (g->h_ctr->error & kSortError) { rc = FL_ETIMEOUT; set_error(rc, "vertex numbering: a sort's wait ran out"); break; }
         std::swap(g->rowp, rowp_new);
         std::swap(g->cols, cols_new);
         g->relabelled = true;
     } while (0);
-    dfree_after(st, {&hi, &lo, &val, &deg, &rowp_new, &cols_new});
+    dfree_after(st, {&key, &val, &deg, &rowp_new, &cols_new});
     return rc;
 }
 

@@ -536,14 +536,18 @@ int compute_radii_multi(const fl_graph* src, fl_graph* g, int64_t R, const doubl
 
 // ------------------------------------------------------------------ keys (r_f, pi_f)
 
+// Up to kRankMax candidates are ordered by counting (k_rank_keys), more by the
+// radix sort.  Measured (uniform and log-uniform costs): see k_rank_keys.
+constexpr int64_t kRankMax = 16384;
+
 __global__ void k_candidates(const double* __restrict__ r, int64_t n, uint64_t seed,
                              IdMap ids, uint64_t* __restrict__ hi,
                              uint64_t* __restrict__ lo, uint32_t* __restrict__ val, uint8_t* __restrict__ state,
                              Counters* ctr) {
-    // which key bits vary: OR of the words and of their complements, per
+    // which radius bits vary: OR of the words and of their complements, per
     // block in shared memory, then one global OR per block
-    __shared__ unsigned long long bits[4];
-    if (threadIdx.x < 4) bits[threadIdx.x] = 0;
+    __shared__ unsigned long long bits[2];
+    if (threadIdx.x < 2) bits[threadIdx.x] = 0;
     __syncthreads();
     __shared__ BlockAppend<8> sh;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -558,52 +562,123 @@ __global__ void k_candidates(const double* __restrict__ r, int64_t n, uint64_t s
         }
         long long at = block_append<8>(cand, &ctr->aux0, sh);
         const uint64_t h = cand ? (uint64_t)__double_as_longlong(rf) : 0;  // r >= 0: bit order = numeric order
-        const uint64_t l = cand ? facility_priority(seed, rank_id(ids, f)) : 0;
         if (at >= 0) {
             hi[at] = h;
-            lo[at] = l;
+            if (at < kRankMax) lo[at] = facility_priority(seed, rank_id(ids, f));
             val[at] = (uint32_t)f;
         }
         if (__ballot_sync(kFull, cand)) {
-            const uint64_t hn = cand ? ~h : 0, ln = cand ? ~l : 0;
-            uint64_t w[4] = {h, l, hn, ln};
+            uint64_t w[2] = {h, cand ? ~h : 0};
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
+            for (int q = 0; q < 2; ++q) {
                 const unsigned a = __reduce_or_sync(kFull, (unsigned)w[q]);
                 const unsigned b = __reduce_or_sync(kFull, (unsigned)(w[q] >> 32));
                 w[q] = ((uint64_t)b << 32) | a;
             }
             if (lane_id() == 0)
-                for (int q = 0; q < 4; ++q)
+                for (int q = 0; q < 2; ++q)
                     if (w[q] & ~bits[q]) atomicOr(&bits[q], (unsigned long long)w[q]);
         }
     }
     __syncthreads();
-    if (threadIdx.x < 4 && bits[threadIdx.x]) {
-        unsigned long long* dst = threadIdx.x < 2 ? &ctr->key_or[threadIdx.x] : &ctr->key_orn[threadIdx.x - 2];
-        atomicOr(dst, bits[threadIdx.x]);
+    if (threadIdx.x < 2 && bits[threadIdx.x]) atomicOr(threadIdx.x ? &ctr->key_orn : &ctr->key_or, bits[threadIdx.x]);
+}
+
+// Few candidates: each one's place in key order is the number of keys below
+// its own.  A block places 64 candidates, two per lane; its warps share the
+// scan of all keys, staged in shared memory 512 at a time (every lane reads
+// the same key: a broadcast).  Equal keys (parts of a batch with equal
+// part-local ids) keep their input order.  Quadratic, but one launch and no
+// pass over memory but the keys: bound by integer compares.
+constexpr int kRankTile = 512;
+
+__global__ void __launch_bounds__(256) k_rank_keys(const uint64_t* __restrict__ hi, const uint64_t* __restrict__ lo,
+                                                   const uint32_t* __restrict__ val, int m,
+                                                   uint32_t* __restrict__ sorted) {
+    __shared__ ulonglong2 key[kRankTile];
+    __shared__ int below[8][64];
+    const int lane = lane_id(), warp = threadIdx.x >> 5;
+    const int i0 = blockIdx.x * 64 + lane, i1 = i0 + 32;
+    const uint64_t h0 = i0 < m ? hi[i0] : 0, l0 = i0 < m ? lo[i0] : 0;
+    const uint64_t h1 = i1 < m ? hi[i1] : 0, l1 = i1 < m ? lo[i1] : 0;
+    int c0 = 0, c1 = 0;
+    for (int t = 0; t < m; t += kRankTile) {
+        const int cnt = min(kRankTile, m - t);
+        __syncthreads();
+        for (int j = threadIdx.x; j < cnt; j += 256) key[j] = make_ulonglong2(hi[t + j], lo[t + j]);
+        __syncthreads();
+        for (int j = warp; j < cnt; j += 8) {
+            const ulonglong2 k = key[j];
+            const int at = t + j;
+            c0 += (k.x < h0) | ((k.x == h0) & ((k.y < l0) | ((k.y == l0) & (at < i0))));
+            c1 += (k.x < h1) | ((k.x == h1) & ((k.y < l1) | ((k.y == l1) & (at < i1))));
+        }
+    }
+    below[warp][lane] = c0;
+    below[warp][lane + 32] = c1;
+    __syncthreads();
+    if (threadIdx.x < 64) {
+        const int i = blockIdx.x * 64 + threadIdx.x;
+        int rank = 0;
+        for (int w = 0; w < 8; ++w) rank += below[w][threadIdx.x];
+        if (i < m) sorted[rank] = val[i];
     }
 }
 
-// Any two adjacent equal hi words (radius ties) after sorting by hi.
-__global__ void k_key_ties(const uint64_t* __restrict__ hi, int64_t m, Counters* ctr) {
+__device__ __forceinline__ uint64_t priority_of(uint64_t seed, const IdMap& ids, uint32_t f) {
+    return facility_priority(seed, rank_id(ids, (int64_t)f));
+}
+
+// Keys sorted by the bits from `shift` up (and, with kByPrio, by the top half
+// of the priority below them): put each run that these bits leave equal in
+// the order of the whole key (r_f, pi_f), one thread per run.  A run longer
+// than `longest` is left alone and reported.
+template <bool kByPrio>
+__global__ void k_order_runs(uint64_t* key, uint32_t* val, int64_t m, int shift, int64_t longest, uint64_t seed,
+                             IdMap ids, Counters* ctr) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    bool tie = false;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i + 1 < m; i += stride)
-        tie |= hi[i] == hi[i + 1];
-    if (__any_sync(kFull, tie) && lane_id() == 0) atomicOr(&ctr->key_ties, 1ULL);
+    auto same = [&](int64_t i, int64_t j) {
+        if ((key[i] >> shift) != (key[j] >> shift)) return false;
+        return !kByPrio || (priority_of(seed, ids, val[i]) >> 32) == (priority_of(seed, ids, val[j]) >> 32);
+    };
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i + 1 < m; i += stride) {
+        if (!same(i, i + 1) || (i > 0 && same(i - 1, i))) continue;
+        int64_t end = i + 2;
+        while (end < m && end - i <= longest && same(i, end)) ++end;
+        if (end - i > longest) {
+            atomicOr(&ctr->key_ties, 1ULL);
+            continue;
+        }
+        for (int64_t a = i + 1; a < end; ++a) {
+            const uint64_t k = key[a];
+            const uint32_t v = val[a];
+            const uint64_t p = priority_of(seed, ids, v);
+            int64_t b = a;
+            for (; b > i; --b) {
+                const uint64_t kb = key[b - 1];
+                const uint32_t vb = val[b - 1];
+                if (kb < k || (kb == k && priority_of(seed, ids, vb) <= p)) break;
+                key[b] = kb;
+                val[b] = vb;
+            }
+            key[b] = k;
+            val[b] = v;
+        }
+    }
 }
 
-// Nibble digits (bit p: pass p of sort_pairs_u128_digits) of the key bits
-// that vary between candidates.
-static uint32_t varying_digits(const Counters& c) {
-    uint32_t d = 0;
-    for (int w = 0; w < 2; ++w) {
-        const uint64_t var = c.key_or[w] & c.key_orn[w];
-        for (int q = 0; q < 16; ++q)
-            if ((var >> (4 * q)) & 15u) d |= 1u << (q + (w == 0 ? 16 : 0));
-    }
-    return d;
+__global__ void k_prio_keys(const uint32_t* __restrict__ val, int64_t m, uint64_t seed, IdMap ids,
+                            uint32_t* __restrict__ key) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += stride)
+        key[i] = (uint32_t)(priority_of(seed, ids, val[i]) >> 32);
+}
+
+__global__ void k_radius_keys(const uint32_t* __restrict__ val, int64_t m, const double* __restrict__ r,
+                              uint64_t* __restrict__ key) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += stride)
+        key[i] = (uint64_t)__double_as_longlong(r[val[i]]);
 }
 
 __global__ void k_ordinals(const uint32_t* __restrict__ sorted_f, int64_t m, const double* __restrict__ r,
@@ -791,42 +866,85 @@ __global__ void k_open_list(const uint8_t* __restrict__ state, int64_t n, uint8_
     }
 }
 
-// Candidates (finite r_f) sorted by the key (r_f, pi_f): s->key_val holds
-// their ids in key order, s->state is 0 for a candidate and 3 otherwise.
-int sort_candidates(fl_solve* s, int64_t* m_out) {
+// Candidates (finite r_f) sorted by the key (r_f, pi_f): *sorted holds their
+// ids in key order, s->state is 0 for a candidate and 3 otherwise.
+//
+// Many candidates: radix sort by the leading bits of r_f that vary, as many
+// as tell most of them apart (log2 m + 16), then put the few short runs that
+// are left in order.  Costs that repeat give runs of equal radii of any
+// length: then the top half of pi_f is sorted first and r_f by all its varying
+// bits after it (each pass keeps the order of the one before), and again the
+// runs that are left are put in order.
+int sort_candidates(fl_solve* s, int64_t* m_out, const uint32_t** sorted) {
     fl_graph* g = s->g;
     const int64_t n = g->n;
     cudaStream_t st = g->stream;
     FL_TRY(dalloc(s->state, (size_t)n));
-    DBuf& hi = s->key_hi;
-    DBuf& lo = s->key_lo;
-    DBuf& val = s->key_val;
-    FL_TRY(dalloc(hi, (size_t)n * 8));
-    FL_TRY(dalloc(lo, (size_t)n * 8));
-    FL_TRY(dalloc(val, (size_t)n * 4));
+    FL_TRY(dalloc(s->key_hi, (size_t)n * 8));
+    FL_TRY(dalloc(s->key_lo, (size_t)n * 8));
+    FL_TRY(dalloc(s->key_val, (size_t)n * 4));
+    FL_TRY(dalloc(s->key_alt, (size_t)n * 12));
+    SortPairs<uint64_t> p;
+    p.key[0] = s->key_hi.as<uint64_t>();
+    p.key[1] = s->key_alt.as<uint64_t>();
+    p.val[0] = s->key_val.as<uint32_t>();
+    p.val[1] = reinterpret_cast<uint32_t*>(p.key[1] + n);
+    Counters* ctr = g->ctr.as<Counters>();
     FL_CUDA(cudaMemsetAsync(g->ctr.p, 0, sizeof(Counters), st));
-    FL_LAUNCH(kProfKeys, k_candidates<<<grid_for(n, 256), 256, 0, st>>>(s->radii.as<double>(), n, g->seed,
-                                                   idmap_of(g), hi.as<uint64_t>(),
-                                                   lo.as<uint64_t>(), val.as<uint32_t>(), s->state.as<uint8_t>(),
-                                                   g->ctr.as<Counters>()));
+    const IdMap ids = idmap_of(g);
+    FL_LAUNCH(kProfKeys, k_candidates<<<grid_for(n, 256), 256, 0, st>>>(s->radii.as<double>(), n, g->seed, ids,
+                                                   p.key[0], s->key_lo.as<uint64_t>(), p.val[0],
+                                                   s->state.as<uint8_t>(), ctr));
     FL_TRY(read_counters(g));
     const int64_t m = (int64_t)g->h_ctr->aux0;
     s->n_cand = m;
-    // Keys (r_f, pi_f): sort by r_f's varying digits; only when two radii are
-    // equal does the order need pi_f, and then the keys are sorted again by
-    // every varying digit (least significant first, so the result is the
-    // order of the whole 128-bit key).
-    const uint32_t digits = varying_digits(*g->h_ctr);
-    FL_TRY(sort_pairs_u128_digits(hi.as<uint64_t>(), lo.as<uint64_t>(), val.as<uint32_t>(), m, st, g->scratch,
-                                  kProfKeys, digits & 0xffff0000u));
-    if (m > 1) {
-        FL_LAUNCH(kProfKeys, k_key_ties<<<grid_for(m, 256), 256, 0, st>>>(hi.as<uint64_t>(), m, g->ctr.as<Counters>()));
-        FL_TRY(read_counters(g));
-        if (g->h_ctr->key_ties)
-            FL_TRY(sort_pairs_u128_digits(hi.as<uint64_t>(), lo.as<uint64_t>(), val.as<uint32_t>(), m, st, g->scratch,
-                                          kProfKeys, digits));
-    }
     *m_out = m;
+    *sorted = p.val[0];
+    if (m <= 1) return FL_OK;
+    if (m <= kRankMax) {
+        FL_LAUNCH(kProfKeys, k_rank_keys<<<(unsigned)((m + 63) / 64), 256, 0, st>>>(
+                                 p.key[0], s->key_lo.as<uint64_t>(), p.val[0], (int)m, p.val[1]));
+        FL_CUDA(cudaGetLastError());
+        *sorted = p.val[1];
+        return FL_OK;
+    }
+    const uint64_t varying = g->h_ctr->key_or & g->h_ctr->key_orn;
+    int shift[kSortDigits];
+    int lg = 0;
+    while ((1LL << lg) < m) ++lg;
+    bool ties = varying == 0;
+    if (!ties) {
+        const int nd = digit_windows(varying, lg + 16, shift);
+        FL_TRY(sort_pairs(p, m, shift, nd, st, g->scratch, kProfKeys, &ctr->error));
+        FL_LAUNCH(kProfKeys, k_order_runs<false><<<grid_for(m, 256), 256, 0, st>>>(p.key[p.cur], p.val[p.cur], m,
+                                                                                  shift[0], 16, g->seed, ids, ctr));
+        FL_CUDA(cudaGetLastError());
+        FL_TRY(read_counters(g));
+        if (g->h_ctr->error) FL_FAIL(FL_ETIMEOUT, "candidate keys: a sort's wait ran out");
+        ties = g->h_ctr->key_ties != 0;
+    }
+    if (ties) {
+        SortPairs<uint32_t> q;
+        q.key[0] = s->key_lo.as<uint32_t>();
+        q.key[1] = q.key[0] + n;
+        q.val[0] = p.val[p.cur];
+        q.val[1] = p.val[p.cur ^ 1];
+        FL_LAUNCH(kProfKeys, k_prio_keys<<<grid_for(m, 256), 256, 0, st>>>(q.val[0], m, g->seed, ids, q.key[0]));
+        FL_TRY(sort_pairs(q, m, shift, digit_windows(0xffffffffULL, 0, shift), st, g->scratch, kProfKeys,
+                          &ctr->error));
+        p.val[0] = q.val[q.cur];
+        p.val[1] = q.val[q.cur ^ 1];
+        p.cur = 0;
+        FL_LAUNCH(kProfKeys, k_radius_keys<<<grid_for(m, 256), 256, 0, st>>>(p.val[0], m, s->radii.as<double>(),
+                                                                             p.key[0]));
+        FL_TRY(sort_pairs(p, m, shift, digit_windows(varying, 0, shift), st, g->scratch, kProfKeys, &ctr->error));
+        FL_LAUNCH(kProfKeys, k_order_runs<true><<<grid_for(m, 256), 256, 0, st>>>(p.key[p.cur], p.val[p.cur], m, 0, m,
+                                                                                 g->seed, ids, ctr));
+        FL_CUDA(cudaGetLastError());
+        FL_TRY(read_counters(g));
+        if (g->h_ctr->error) FL_FAIL(FL_ETIMEOUT, "candidate keys: a sort's wait ran out");
+    }
+    *sorted = p.val[p.cur];
     return FL_OK;
 }
 
@@ -859,12 +977,12 @@ int open_facilities(fl_solve* s) {
     // solve-owned, grow-only scratch: a cudaFree per solve would synchronise
     // the whole device (and stall other solves running on other streams)
     int64_t m = 0;
-    FL_TRY(sort_candidates(s, &m));
-    DBuf& val = s->key_val;
+    const uint32_t* sorted = nullptr;
+    FL_TRY(sort_candidates(s, &m, &sorted));
     int32_t* ulist[2] = {s->ulist.as<int32_t>(), s->ulist.as<int32_t>() + n};
     FL_CUDA(cudaMemsetAsync(cnt, 0, 64, st));
     if (m > 0) {
-        FL_LAUNCH(kProfKeys, k_ordinals<<<grid_for(m, 256), 256, 0, st>>>(val.as<uint32_t>(), m, s->radii.as<double>(),
+        FL_LAUNCH(kProfKeys, k_ordinals<<<grid_for(m, 256), 256, 0, st>>>(sorted, m, s->radii.as<double>(),
                                                      g->ecc_ub.as<int32_t>(), s->ord.as<uint32_t>(),
                                                      s->fac_by_ord.as<int32_t>(), s->bcap.as<int32_t>(), ulist[0],
                                                      &cnt[4]));

@@ -1,4 +1,4 @@
-// k_util.cu -- errors, device buffers, scans, radix sort, CSR checks.
+// k_util.cu -- errors, device buffers, scans, CSR checks.
 #include <cstdio>
 #include <cstring>
 #include <map>
@@ -333,114 +333,6 @@ int scan_exclusive_i32_to_i64(const int32_t* in, int64_t* out, int64_t n, cudaSt
                               int cls) {
     FL_TRY(dalloc(tmp, scan_tmp_bytes(n)));
     return scan_rec<int32_t>(in, out, n, st, tmp.as<char>(), cls);
-}
-
-// ----------------------------------------------------------------- radix sort
-// Stable LSD radix sort of (hi, lo) 128-bit keys with a uint32 payload,
-// 4-bit digits (32 passes, lo word first).  Per pass: per-tile digit
-// histogram -> exclusive scan in digit-major order -> stable scatter, where
-// each thread owns 8 consecutive items and per-digit offsets come from a
-// block scan of 16 packed 16-bit counters (4 x uint64 words).
-
-constexpr int kSortThreads = 256;
-constexpr int kSortItems = 8;
-constexpr int kSortTile = kSortThreads * kSortItems;
-
-__global__ void k_digit_hist(const uint64_t* __restrict__ key, int64_t n, int shift, int nblocks,
-                             int32_t* __restrict__ hist) {
-    __shared__ int32_t h[16];
-    if (threadIdx.x < 16) h[threadIdx.x] = 0;
-    __syncthreads();
-    int64_t base = (int64_t)blockIdx.x * kSortTile + (int64_t)threadIdx.x * kSortItems;
-#pragma unroll
-    for (int i = 0; i < kSortItems; ++i)
-        if (base + i < n) atomicAdd(&h[(key[base + i] >> shift) & 15], 1);
-    __syncthreads();
-    if (threadIdx.x < 16) hist[(int64_t)threadIdx.x * nblocks + blockIdx.x] = h[threadIdx.x];
-}
-
-__global__ void k_digit_scatter(const uint64_t* __restrict__ key, const uint64_t* __restrict__ hi_in,
-                                const uint64_t* __restrict__ lo_in, const uint32_t* __restrict__ val_in,
-                                int64_t n, int shift, int nblocks, const int64_t* __restrict__ offs,
-                                uint64_t* __restrict__ hi_out, uint64_t* __restrict__ lo_out,
-                                uint32_t* __restrict__ val_out) {
-    __shared__ uint64_t wt[4][32];
-    __shared__ uint64_t tot[4];
-    int64_t base = (int64_t)blockIdx.x * kSortTile + (int64_t)threadIdx.x * kSortItems;
-    int dig[kSortItems];
-    uint64_t cnt[4] = {0, 0, 0, 0};
-#pragma unroll
-    for (int i = 0; i < kSortItems; ++i) {
-        dig[i] = (base + i < n) ? (int)((key[base + i] >> shift) & 15) : -1;
-        if (dig[i] >= 0) cnt[dig[i] >> 2] += 1ULL << (16 * (dig[i] & 3));
-    }
-    uint64_t ex[4];
-#pragma unroll
-    for (int w = 0; w < 4; ++w) ex[w] = block_excl_scan<uint64_t>(cnt[w], wt[w], &tot[w]);
-#pragma unroll
-    for (int i = 0; i < kSortItems; ++i) {
-        int d = dig[i];
-        if (d < 0) continue;
-        int w = d >> 2, sh = 16 * (d & 3);
-        int64_t local = (int64_t)((ex[w] >> sh) & 0xffff);
-        ex[w] += 1ULL << sh;
-        int64_t pos = offs[(int64_t)d * nblocks + blockIdx.x] + local;
-        hi_out[pos] = hi_in[base + i];
-        lo_out[pos] = lo_in[base + i];
-        val_out[pos] = val_in[base + i];
-    }
-}
-
-int sort_pairs_u128(uint64_t* hi, uint64_t* lo, uint32_t* val, int64_t n, cudaStream_t st, DBuf& tmp, int cls,
-                    int pass_begin, int pass_end) {
-    if (pass_begin < 0 || pass_end > 32 || pass_begin > pass_end || ((pass_end - pass_begin) & 1))
-        FL_FAIL(FL_EINVAL, "radix sort: bad pass range");
-    uint32_t digits = 0;
-    for (int p = pass_begin; p < pass_end; ++p) digits |= 1u << p;
-    return sort_pairs_u128_digits(hi, lo, val, n, st, tmp, cls, digits);
-}
-
-int sort_pairs_u128_digits(uint64_t* hi, uint64_t* lo, uint32_t* val, int64_t n, cudaStream_t st, DBuf& tmp,
-                           int cls, uint32_t digits) {
-    if (n <= 1 || digits == 0) return FL_OK;
-    int nblocks = (int)((n + kSortTile - 1) / kSortTile);
-    int64_t hn = 16LL * nblocks;
-    size_t need = (size_t)n * (8 + 8 + 4) + 256 * 8 + (size_t)hn * (4 + 8) + scan_tmp_bytes(hn);
-    FL_TRY(dalloc(tmp, need));
-    char* p = tmp.as<char>();
-    auto take = [&](size_t bytes) {
-        char* r = p;
-        p += (bytes + 255) & ~size_t(255);
-        return r;
-    };
-    uint64_t* hi2 = reinterpret_cast<uint64_t*>(take((size_t)n * 8));
-    uint64_t* lo2 = reinterpret_cast<uint64_t*>(take((size_t)n * 8));
-    uint32_t* val2 = reinterpret_cast<uint32_t*>(take((size_t)n * 4));
-    int32_t* hist = reinterpret_cast<int32_t*>(take((size_t)hn * 4));
-    int64_t* offs = reinterpret_cast<int64_t*>(take((size_t)hn * 8));
-    char* stmp = take(scan_tmp_bytes(hn));
-    uint64_t *ahi = hi, *alo = lo, *bhi = hi2, *blo = lo2;
-    uint32_t *aval = val, *bval = val2;
-    for (int pass = 0; pass < 32; ++pass) {
-        if (!((digits >> pass) & 1u)) continue;
-        const uint64_t* key = pass < 16 ? alo : ahi;
-        int shift = 4 * (pass & 15);
-        FL_LAUNCH(cls, k_digit_hist<<<nblocks, kSortThreads, 0, st>>>(key, n, shift, nblocks, hist));
-        FL_CUDA(cudaGetLastError());
-        FL_TRY(scan_rec<int32_t>(hist, offs, hn, st, stmp, cls));
-        FL_LAUNCH(cls, k_digit_scatter<<<nblocks, kSortThreads, 0, st>>>(key, ahi, alo, aval, n, shift, nblocks, offs,
-                                                          bhi, blo, bval));
-        FL_CUDA(cudaGetLastError());
-        std::swap(ahi, bhi);
-        std::swap(alo, blo);
-        std::swap(aval, bval);
-    }
-    if (__builtin_popcount(digits) & 1) {  // an odd number of passes: copy the result back
-        FL_CUDA(cudaMemcpyAsync(hi, ahi, (size_t)n * 8, cudaMemcpyDeviceToDevice, st));
-        FL_CUDA(cudaMemcpyAsync(lo, alo, (size_t)n * 8, cudaMemcpyDeviceToDevice, st));
-        FL_CUDA(cudaMemcpyAsync(val, aval, (size_t)n * 4, cudaMemcpyDeviceToDevice, st));
-    }
-    return FL_OK;
 }
 
 // ----------------------------------------------------------------- CSR checks

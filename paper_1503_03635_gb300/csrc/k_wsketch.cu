@@ -326,22 +326,29 @@ __global__ void k_wmaxlen(const int32_t* __restrict__ w, int64_t nnz, unsigned l
 // direction), the entry index as payload (a warp per source vertex u).
 __global__ void k_wrevkeys(const int64_t* __restrict__ rowp, const int32_t* __restrict__ cols,
                            const int32_t* __restrict__ wts, int64_t n, uint64_t* __restrict__ hi,
-                           uint64_t* __restrict__ lo, uint32_t* __restrict__ val) {
+                           uint32_t* __restrict__ lo, uint32_t* __restrict__ val) {
     const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t u = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < n; u += warps) {
         for (int64_t e = rowp[u] + lane_id(); e < rowp[u + 1]; e += 32) {
             const int64_t v = cols[e];
             const uint64_t a = (uint64_t)(u < v ? u : v), b = (uint64_t)(u < v ? v : u);
             hi[e] = (a << 32) | b;
-            lo[e] = ((uint64_t)(uint32_t)wts[e] << 1) | (u > v ? 1u : 0u);
+            lo[e] = ((uint32_t)wts[e] << 1) | (u > v ? 1u : 0u);
             val[e] = (uint32_t)e;
         }
     }
 }
 
+// out[i] = in[at[i]]
+template <class T>
+__global__ void k_wgather(const T* __restrict__ in, const uint32_t* __restrict__ at, int64_t m, T* __restrict__ out) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += stride) out[i] = in[at[i]];
+}
+
 // First index of the sorted keys at or above (h, l).
-__device__ __forceinline__ int64_t key_lower_bound(const uint64_t* __restrict__ hi, const uint64_t* __restrict__ lo,
-                                                   int64_t m, uint64_t h, uint64_t l) {
+__device__ __forceinline__ int64_t key_lower_bound(const uint64_t* __restrict__ hi, const uint32_t* __restrict__ lo,
+                                                   int64_t m, uint64_t h, uint32_t l) {
     int64_t a = 0, b = m;
     while (a < b) {
         const int64_t mid = (a + b) >> 1;
@@ -356,17 +363,18 @@ __device__ __forceinline__ int64_t key_lower_bound(const uint64_t* __restrict__ 
 // first half runs min -> max and second half max -> min; the i-th of each
 // half pair up (a self-loop pairs with itself).  A group whose halves differ
 // means a length that is not the same in both directions (bad = 1).
-__global__ void k_wpair(const uint64_t* __restrict__ hi, const uint64_t* __restrict__ lo,
+__global__ void k_wpair(const uint64_t* __restrict__ hi, const uint32_t* __restrict__ lo,
                         const uint32_t* __restrict__ val, int64_t m, uint32_t* __restrict__ rev,
                         unsigned long long* __restrict__ bad) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += stride) {
-        const uint64_t h = hi[i], l = lo[i];
+        const uint64_t h = hi[i];
+        const uint32_t l = lo[i];
         if ((h >> 32) == (h & 0xffffffffULL)) {
             rev[val[i]] = val[i];
             continue;
         }
-        const uint64_t l0 = l & ~1ULL;  // the group: keys (h, l0) and (h, l0 | 1)
+        const uint32_t l0 = l & ~1u;  // the group: keys (h, l0) and (h, l0 | 1)
         const int64_t g0 = key_lower_bound(hi, lo, m, h, l0);
         const int64_t g1 = key_lower_bound(hi, lo, m, h, l0 + 2);
         const int64_t half = (g1 - g0) >> 1;
@@ -396,34 +404,59 @@ int pair_reverse_edges(fl_graph* g) {
     DBuf hi, lo, val, flag;
     int rc = FL_OK;
     do {
-        if ((rc = dalloc(hi, (size_t)nnz * 8)) || (rc = dalloc(lo, (size_t)nnz * 8)) ||
-            (rc = dalloc(val, (size_t)nnz * 4)) || (rc = dalloc(flag, 16)))
+        if ((rc = dalloc(hi, (size_t)nnz * 16)) || (rc = dalloc(lo, (size_t)nnz * 8)) ||
+            (rc = dalloc(val, (size_t)nnz * 8)) || (rc = dalloc(flag, 16)))
             break;
         cudaError_t e = cudaMemsetAsync(flag.p, 0, 16, st);
         if (e != cudaSuccess) { rc = status_of(e, "edge pairing", __FILE__, __LINE__); break; }
+        SortPairs<uint64_t> sh;
+        SortPairs<uint32_t> sl;
+        for (int q = 0; q < 2; ++q) {
+            sh.key[q] = hi.as<uint64_t>() + q * nnz;
+            sl.key[q] = lo.as<uint32_t>() + q * nnz;
+            sh.val[q] = sl.val[q] = val.as<uint32_t>() + q * nnz;
+        }
+        unsigned long long* bad = flag.as<unsigned long long>();
+        const uint64_t* hi_of = sh.key[1];  // keys by entry
         FL_LAUNCH(kProfOther, k_wrevkeys<<<grid_for(n * 32, 256), 256, 0, st>>>(
                                   g->rowp.as<int64_t>(), g->cols.as<int32_t>(), g->wts.as<int32_t>(), n,
-                                  hi.as<uint64_t>(), lo.as<uint64_t>(), val.as<uint32_t>()));
-        // the digits that can vary: ids below n in both halves of hi, the
-        // length and the direction bit in lo
-        int nb = 1, wb = 1;
+                                  sh.key[1], sl.key[0], sl.val[0]));
+        // the bits that can vary: ids below n in both halves of hi, the
+        // length and the direction bit in lo; lo's digits first, then hi's
+        int nb = 1, wb = 1, shift[kSortDigits];
         while (nb < 31 && (1LL << nb) < n) ++nb;
         while (wb < 17 && (1 << wb) <= g->max_w) ++wb;
-        uint32_t digits = 0;
-        for (int d = 0; d * 4 < wb + 1; ++d) digits |= 1u << d;
-        for (int d = 0; d * 4 < nb; ++d) digits |= (1u << (16 + d)) | (1u << (24 + d));
-        if ((rc = sort_pairs_u128_digits(hi.as<uint64_t>(), lo.as<uint64_t>(), val.as<uint32_t>(), nnz, st,
-                                         g->scratch, kProfOther, digits)))
+        if ((rc = sort_pairs(sl, nnz, shift, digit_windows((2ULL << wb) - 1, 0, shift), st, g->scratch, kProfOther,
+                             bad)))
             break;
-        FL_LAUNCH(kProfOther, k_wpair<<<grid_for(nnz, 256), 256, 0, st>>>(
-                                  hi.as<uint64_t>(), lo.as<uint64_t>(), val.as<uint32_t>(), nnz,
-                                  g->wrev.as<uint32_t>(), flag.as<unsigned long long>()));
+        sh.cur = 0;
+        if (sl.cur == 1) {  // the payload goes with the first key buffer
+            std::swap(sh.val[0], sh.val[1]);
+        }
+        FL_LAUNCH(kProfOther, k_wgather<<<grid_for(nnz, 256), 256, 0, st>>>(hi_of, sh.val[0], nnz, sh.key[0]));
+        int nd = 0;
+        for (int half = 0; half < 2; ++half)
+            for (int b = 0; b < nb; b += 8) shift[nd++] = 32 * half + b;
+        if ((rc = sort_pairs(sh, nnz, shift, nd, st, g->scratch, kProfOther, bad))) break;
+        // lo in the sorted order, recomputed from the entries in a free buffer
+        const uint32_t* perm = sh.val[sh.cur];
+        uint32_t* lo_by_entry = sl.key[0];
+        uint32_t* lo_sorted = sl.key[1];
+        FL_LAUNCH(kProfOther, k_wrevkeys<<<grid_for(n * 32, 256), 256, 0, st>>>(
+                                  g->rowp.as<int64_t>(), g->cols.as<int32_t>(), g->wts.as<int32_t>(), n,
+                                  sh.key[sh.cur ^ 1], lo_by_entry, sh.val[sh.cur ^ 1]));
+        FL_LAUNCH(kProfOther, k_wgather<<<grid_for(nnz, 256), 256, 0, st>>>(lo_by_entry, perm, nnz, lo_sorted));
+        FL_LAUNCH(kProfOther, k_wpair<<<grid_for(nnz, 256), 256, 0, st>>>(sh.key[sh.cur], lo_sorted, perm, nnz,
+                                                                          g->wrev.as<uint32_t>(), bad));
         unsigned long long h = 0;
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaMemcpyAsync(&h, flag.p, 8, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) { rc = status_of(e, "edge pairing", __FILE__, __LINE__); break; }
-        if (h) {
+        if (h & kSortError) {
+            rc = FL_ETIMEOUT;
+            set_error(rc, "edge pairing: a sort's wait ran out");
+        } else if (h) {
             rc = FL_EINVAL;
             set_error(rc, "an edge's length must be the same in both directions");
         }

@@ -471,7 +471,8 @@ int open_facilities_weighted(fl_solve* s) {
     using clock = std::chrono::steady_clock;
     s->mis_log.clear();
     int64_t m = 0;
-    FL_TRY(sort_candidates(s, &m));
+    const uint32_t* sorted = nullptr;
+    FL_TRY(sort_candidates(s, &m, &sorted));
     FL_TRY(dalloc(s->ord, (size_t)n * 4));
     FL_TRY(dalloc(s->fac_by_ord, (size_t)std::max<int64_t>(m, 1) * 4));
     FL_TRY(dalloc(s->bcap, (size_t)n * 4));
@@ -491,7 +492,7 @@ int open_facilities_weighted(fl_solve* s) {
     FL_CUDA(cudaMemsetAsync(s->bcap.p, 0xff, (size_t)n * 4, st));
     FL_CUDA(cudaMemsetAsync(s->claimed.p, 0, (size_t)n, st));
     if (m > 0)
-        FL_LAUNCH(kProfKeys, k_wordinals<<<grid_for(m, 256), 256, 0, st>>>(s->key_val.as<uint32_t>(), m,
+        FL_LAUNCH(kProfKeys, k_wordinals<<<grid_for(m, 256), 256, 0, st>>>(sorted, m,
                                                                           s->radii.as<double>(), s->ord.as<uint32_t>(),
                                                                           fac_by_ord, bcap, bsort));
     FL_CUDA(cudaGetLastError());
