@@ -39,7 +39,7 @@ void destroy_graph(fl_graph* g) {
                     &g->ginfo, &g->gwt, &g->eid, &g->ecc_ub, &g->ctr, &g->scratch,
                     &g->relax_aux, &g->U, &g->DM[0], &g->DM[1], &g->PM, &g->seg_flag, &g->PH, &g->F[0], &g->F[1], &g->H[0],
                     &g->H[1], &g->W, &g->fbm, &g->URid, &g->vbase, &g->vpart, &g->rid,
-                    &g->inv, &g->xbits, &g->xaux, &g->xio};
+                    &g->inv, &g->xbits, &g->xaux, &g->xio, &g->items};
     for (DBuf* b : bufs) dfree_idle(*b);
     if (g->gbfs) {
         graph_bfs_release(g->gbfs);
@@ -59,7 +59,7 @@ void destroy_solve(fl_solve* s) {
                     &s->X, &s->stamp, &s->mval, &s->fr[0], &s->fr[1], &s->frval, &s->touched, &s->ulist,
                     &s->ubuck, &s->bcount, &s->open, &s->assign, &s->dist, &s->key_hi, &s->key_lo,
                     &s->key_val, &s->key_alt, &s->obj_tmp, &s->part_T, &s->io, &s->eps, &s->eps_tab, &s->eps_r,
-                    &s->eps_c};
+                    &s->eps_c, &s->rlist, &s->rctl, &s->reach, &s->kill};
     for (DBuf* b : bufs) dfree_idle(*b);
     delete s;
 }
@@ -185,7 +185,7 @@ int fl_graph_create(int64_t n, const int64_t* row_off, const int32_t* cols, int6
     g->stream = static_cast<cudaStream_t>(stream);
     int rc = FL_OK;
     do {
-        cudaError_t e = cudaMallocHost(reinterpret_cast<void**>(&g->h_ctr), sizeof(Counters));
+        cudaError_t e = cudaMallocHost(reinterpret_cast<void**>(&g->h_ctr), kPinnedBytes);
         if (e != cudaSuccess) { rc = status_of(e, "cudaMallocHost", __FILE__, __LINE__); break; }
         if ((rc = dalloc(g->ctr, sizeof(Counters)))) break;
         if ((rc = dalloc(g->rowp, (size_t)(n + 1) * 8))) break;
@@ -221,7 +221,7 @@ int fl_graph_create_weighted(int64_t n, const int64_t* row_off, const int32_t* c
     g->stream = static_cast<cudaStream_t>(stream);
     int rc = FL_OK;
     do {
-        cudaError_t e = cudaMallocHost(reinterpret_cast<void**>(&g->h_ctr), sizeof(Counters));
+        cudaError_t e = cudaMallocHost(reinterpret_cast<void**>(&g->h_ctr), kPinnedBytes);
         if (e != cudaSuccess) { rc = status_of(e, "cudaMallocHost", __FILE__, __LINE__); break; }
         if ((rc = dalloc(g->ctr, sizeof(Counters)))) break;
         if ((rc = dalloc(g->rowp, (size_t)(n + 1) * 8))) break;
@@ -672,7 +672,7 @@ int new_graph(int64_t n, int64_t nnz, cudaStream_t stream, fl_graph** out) {
     g->stream = stream;
     int rc = FL_OK;
     do {
-        cudaError_t e = cudaMallocHost(reinterpret_cast<void**>(&g->h_ctr), sizeof(Counters));
+        cudaError_t e = cudaMallocHost(reinterpret_cast<void**>(&g->h_ctr), kPinnedBytes);
         if (e != cudaSuccess) { rc = status_of(e, "cudaMallocHost", __FILE__, __LINE__); break; }
         if ((rc = dalloc(g->ctr, sizeof(Counters)))) break;
         if ((rc = dalloc(g->rowp, (size_t)(n + 1) * 8))) break;
@@ -862,6 +862,7 @@ int fl_batch_solve(fl_batch* b, int n_active, int k, uint64_t seed, const double
         view.n_mid = U->n_mid / R * n_active;
         view.n_hubs = U->n_hubs / R * n_active;
         view.n_seg = U->n_seg / R * n_active;
+        view.n_items = U->n_items / R * n_active;
     }
     s->g = &view;
     s->generation = view.generation;

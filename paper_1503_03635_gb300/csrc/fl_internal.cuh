@@ -125,6 +125,17 @@ constexpr int kHubDeg = 2048;
 constexpr int kSeg = 2048;
 // Non-hub vertices with at most kSmallDeg neighbours are pulled by one thread each.
 constexpr int kSmallDeg = 8;
+// Graphs of at most kResidentEdges CSR entries (and vertices) run their MIS and
+// BFS as resident kernels over work items of at most kItemEdges entries.  The
+// kernels read every row each round, the host-driven rounds only what the
+// frontier needs, so the line lies where the reads outgrow the launches.  MIS
+// with keys, resident against host-driven: Erdos-Renyi 0.08 M entries 0.57 /
+// 3.55 ms, 0.8 M 1.28 / 5.91, 10 M 1.90 / 4.10; R-MAT 1.8 M 0.46 / 1.18, 7.6 M
+// 1.05 / 1.40, 15.5 M 2.65 / 1.90.
+constexpr int64_t kResidentEdges = 10 << 20;
+constexpr int kItemEdges = 64;
+// Pinned host block of a graph: its Counters mirror, then scratch of a call.
+constexpr size_t kPinnedBytes = 16384;
 // Width of the small-rank universe of the sketch hops (the kUW smallest
 // ranks of a graph; a saturated sketch is a kUW-bit mask over them).
 constexpr int kUW = 1024;
@@ -463,6 +474,8 @@ struct fl_graph {
     fl::DBuf hub_seg;              // int64[n_hubs+1]: first segment of each hub
     fl::DBuf seg_hub;              // int32[n_seg]: hub of each segment
     int64_t n_low = 0, n_hubs = 0, n_seg = 0;
+    fl::DBuf items;                // int4[n_items]: work items of the resident kernels
+    int64_t n_items = 0;           // 0: the graph is too large for them
     fl::DBuf part;                 // uint64[n_seg*k]: partial bottom-k of each hub segment (scratch)
     // A graph that is a disjoint union of parts (batched instances): vertex v
     // of the part starting at vbase[v] has local id v - vbase[v], and ranks
@@ -546,6 +559,7 @@ struct fl_solve {
     fl::DBuf ord, fac_by_ord, bcap, state, claimed;  // MIS state
     fl::DBuf reach;                // uint8[n]: 1 + slack of a vertex in the current cover (gather pruning)
     fl::DBuf kill;                 // uint8[n]: 1 + distance to a client claimed in the current round
+    fl::DBuf rlist, rctl;          // resident kernels: item lists of the greedy rounds, control block and log
     std::vector<int64_t> mis_log;  // rows of 6: the rounds of the last MIS (fl_mis_log)
     fl::DBuf X, stamp, mval, fr[2], frval, touched, ulist, ubuck, bcount;
     fl::DBuf key_hi, key_lo, key_val, key_alt, obj_tmp;  // key sort and objective scratch
@@ -612,6 +626,10 @@ int msbfs(fl_graph* g, const int32_t* src_list, int64_t n_src, int32_t* label, i
 int msbfs_graph(fl_graph* g, const int32_t* src_list, int64_t n_src, int32_t* label, int32_t* dist, DBuf& X,
                 DBuf& stampb, int cls);
 void graph_bfs_release(GraphBfs* c);
+// resident kernels of small graphs (k_resident.cu); usable when g->n_items > 0
+int build_items(fl_graph* g);
+int mis_resident(fl_solve* s, int64_t m, bool* done);
+int msbfs_resident(fl_graph* g, const int32_t* src, int64_t n_src, int32_t* label, int32_t* dist, DBuf& ctl, int cls);
 
 // Per-vertex pruning of the rounds of a sweep (the MIS cover and gather
 // sweeps).  A round that first gives v a value below the limit records

@@ -1044,7 +1044,7 @@ int build_work_lists(fl_graph* g) {
         if (e) { rc = status_of(e, "work lists", __FILE__, __LINE__); break; }
     } while (0);
     dfree_after(st, {&low, &hub, &nseg, &low_pos, &hub_pos, &seg_pos, &small, &small_pos});
-    return rc;
+    return rc == FL_OK ? build_items(g) : rc;
 }
 
 // Census of a hop's work list (profiling): CSR entries of the listed

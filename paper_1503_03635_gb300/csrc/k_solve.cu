@@ -127,6 +127,11 @@ int msbfs(fl_graph* g, const int32_t* src_list, int64_t n_src, int32_t* label, i
           DBuf& stampb, DBuf* fr, DBuf& frval, int cls) {
     const int64_t n = g->n;
     cudaStream_t st = g->stream;
+    if (!g->lists_ready) {
+        FL_TRY(build_work_lists(g));
+        g->lists_ready = 1;
+    }
+    if (g->n_items > 0) return msbfs_resident(g, src_list, n_src, label, dist, frval, cls);
     FL_TRY(dalloc(X, (size_t)n * 16));
     FL_TRY(dalloc(stampb, (size_t)n * 4));
     FL_TRY(dalloc(fr[0], (size_t)n * 4));
@@ -957,19 +962,9 @@ int open_facilities(fl_solve* s) {
     FL_TRY(dalloc(s->fac_by_ord, (size_t)n * 4));
     FL_TRY(dalloc(s->bcap, (size_t)n * 4));
     FL_TRY(dalloc(s->state, (size_t)n));
-    FL_TRY(dalloc(s->claimed, (size_t)n));
-    FL_TRY(dalloc(s->X, (size_t)n * 16));          // two value buffers
-    FL_TRY(dalloc(s->stamp, (size_t)n * 4));
-    FL_TRY(dalloc(s->mval, (size_t)n * 4));
-    FL_TRY(dalloc(s->fr[0], (size_t)n * 4));
-    FL_TRY(dalloc(s->fr[1], (size_t)n * 4));
     FL_TRY(dalloc(s->frval, (size_t)n * 8 + 64));
-    FL_TRY(dalloc(s->touched, (size_t)n * 4));
     FL_TRY(dalloc(s->ulist, (size_t)n * 4 * 2));
-    FL_TRY(dalloc(s->ubuck, (size_t)n * 4));
     FL_TRY(dalloc(s->open, (size_t)n));
-    FL_TRY(dalloc(s->reach, (size_t)n));
-    FL_TRY(dalloc(s->kill, (size_t)n));
     s->mis_log.clear();
     unsigned long long* cnt = reinterpret_cast<unsigned long long*>(s->frval.as<char>() + (size_t)n * 8);
     // cnt[0], cnt[1]: frontier counts; cnt[2]: changed count (dense rounds);
@@ -988,6 +983,25 @@ int open_facilities(fl_solve* s) {
                                                      &cnt[4]));
     }
     FL_CUDA(cudaGetLastError());
+    if (!g->lists_ready) {
+        FL_TRY(build_work_lists(g));
+        g->lists_ready = 1;
+    }
+    if (g->n_items > 0) {
+        bool done = false;
+        FL_TRY(mis_resident(s, m, &done));
+        if (done) return FL_OK;
+    }
+    FL_TRY(dalloc(s->claimed, (size_t)n));
+    FL_TRY(dalloc(s->X, (size_t)n * 16));          // two value buffers
+    FL_TRY(dalloc(s->stamp, (size_t)n * 4));
+    FL_TRY(dalloc(s->mval, (size_t)n * 4));
+    FL_TRY(dalloc(s->fr[0], (size_t)n * 4));
+    FL_TRY(dalloc(s->fr[1], (size_t)n * 4));
+    FL_TRY(dalloc(s->touched, (size_t)n * 4));
+    FL_TRY(dalloc(s->ubuck, (size_t)n * 4));
+    FL_TRY(dalloc(s->reach, (size_t)n));
+    FL_TRY(dalloc(s->kill, (size_t)n));
     unsigned long long bmax = 0;
     FL_CUDA(cudaMemcpyAsync(&bmax, &cnt[4], 8, cudaMemcpyDeviceToHost, st));
     FL_CUDA(cudaMemsetAsync(s->claimed.p, 0, (size_t)n, st));
