@@ -899,13 +899,15 @@ int fl_batch_solve(fl_batch* b, int n_active, int k, uint64_t seed, const double
         const int32_t* ds = s->dist.as<int32_t>();
         if (P) {
             FL_TRY(dalloc(s->io, (size_t)b->U->n * 9));
+            // N open flags, then N distances from the next multiple of 4 bytes
             uint8_t* io = s->io.as<uint8_t>();
+            int32_t* dist_io = reinterpret_cast<int32_t*>(io + ((N + 3) & ~(int64_t)3));
             if (open_out) FL_TRY(permute_vertices<uint8_t>(P, op, io, n_active, false, st));
             if (assign_out) FL_TRY(permute_vertices<int32_t>(P, as, asg_d, n_active, false, st));
-            if (dist_out) FL_TRY(permute_vertices<int32_t>(P, ds, reinterpret_cast<int32_t*>(io + N), n_active, false, st));
+            if (dist_out) FL_TRY(permute_vertices<int32_t>(P, ds, dist_io, n_active, false, st));
             op = io;
             as = asg_d;
-            ds = reinterpret_cast<int32_t*>(io + N);
+            ds = dist_io;
         }
         FL_TRY(copy_out(open_out, op, (size_t)N, mem_kind, st));
         FL_TRY(copy_out(assign_out, as, (size_t)N * 4, mem_kind, st));
