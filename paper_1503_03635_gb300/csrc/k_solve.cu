@@ -400,73 +400,28 @@ __global__ void k_check_costs(const double* __restrict__ cost, int64_t n, Counte
     }
 }
 
-// Radius of facility f with opening cost c (Eq. 1 at eps -> 0), by the
-// warp: W_h = (#counted client entries of the hop-h group) x weight;
-// N_j = N_{j-1} + W_j; G_{j+1} = G_j + N_j; r = j + (c - G_j) / N_j at the
-// first j < L with G_{j+1} >= c, else L + (c - G_L) / N_L (L = last hop of
-// the ADS of f), +inf if N_L = 0.  Every operation is one IEEE-754 op in this
-// order (no contraction).  The loads are issued a row at a time: the group
-// words of up to 32 groups (one per lane), then the row's entry ids and their
-// client flags 32 at a time; per-group client counts come from ballots, and
-// the recurrence runs on registers.  Every lane returns the same value.
-__device__ double facility_radius(int64_t f, double c, int64_t io, const uint8_t* __restrict__ client,
-                                  const int64_t* __restrict__ gofs, const int64_t* __restrict__ eofs,
-                                  const uint32_t* __restrict__ ginfo, const double* __restrict__ gwt,
-                                  const int32_t* __restrict__ eid) {
-    const int lane = lane_id();
-    const int64_t g0 = gofs[f], ng = gofs[f + 1] - g0;
-    const int L = (int)(ginfo[g0 + ng - 1] & 0xffffu);
-    int64_t e = eofs[f];
-    double N = 0.0, G = 0.0;
-    int j = 0;
-    for (int64_t gc = 0; gc < ng; gc += 32) {
-        const int m = ng - gc < 32 ? (int)(ng - gc) : 32;
-        const uint32_t info = lane < m ? ginfo[g0 + gc + lane] : 0u;
-        const double wt = lane < m ? gwt[g0 + gc + lane] : 0.0;
-        const int cnt = (int)((info >> 16) & 0xffu);
-        const int counted = (int)(info >> 24);
-        const int incl = warp_incl_scan(cnt);
-        const int off = incl - cnt;  // first entry of group `lane` within this chunk
-        const int tot = __shfl_sync(kFull, incl, 31);
-        int clients = 0;             // lane g: counted client entries of group g
-        for (int p = 0; p < tot; p += 32) {
-            const int pos = p + lane;
-            const bool is_client = pos < tot && client[io + eid[e + pos]] != 0;
-            for (int gg = 0; gg < m; ++gg) {
-                const int s0 = __shfl_sync(kFull, off, gg);
-                const int cc = __shfl_sync(kFull, counted, gg);
-                const unsigned hit = __ballot_sync(kFull, is_client && pos >= s0 && pos < s0 + cc);
-                if (lane == gg) clients += __popc(hit);
-            }
-        }
-        for (int gg = 0; gg < m; ++gg) {
-            const int hop = (int)(__shfl_sync(kFull, info, gg) & 0xffffu);
-            const int cl = __shfl_sync(kFull, clients, gg);
-            const double w = __shfl_sync(kFull, wt, gg);
-            for (; j < hop; ++j) {  // hops without new entries: W_j = 0
-                if (j < L) {
-                    const double Gn = __dadd_rn(G, N);
-                    if (Gn >= c) return __dadd_rn((double)j, __ddiv_rn(__dsub_rn(c, G), N));
-                    G = Gn;
-                }
-            }
-            N = __dadd_rn(N, __dmul_rn((double)cl, w));
-            if (j < L) {
-                const double Gn = __dadd_rn(G, N);
-                if (Gn >= c) return __dadd_rn((double)j, __ddiv_rn(__dsub_rn(c, G), N));
-                G = Gn;
-            }
-            ++j;
-        }
-        e += tot;
-    }
-    return N > 0.0 ? __dadd_rn((double)L, __ddiv_rn(__dsub_rn(c, G), N)) : INFINITY;
-}
-
-// A warp per 32 consecutive vertices: one ballot finds the facilities (finite
-// cost), the others get +inf, and the warp computes each facility's radius in
-// turn.
+// Radius of facility f with opening cost c (Eq. 1 at eps -> 0): W_h =
+// (#counted client entries of the hop-h group) x weight; N_j = N_{j-1} + W_j;
+// G_{j+1} = G_j + N_j; r = j + (c - G_j) / N_j at the first j < L with
+// G_{j+1} >= c, else L + (c - G_L) / N_L (L = last hop of the ADS of f), +inf
+// if N_L = 0.  Every operation is one IEEE-754 op in this order (no
+// contraction).
 //
+// A warp takes 32 consecutive vertices.  It reads the entries of one facility
+// after the other, 32 ids per load and a window of kRadWindow entries of two
+// facilities in flight; each ballot of the client flags is one word of the
+// facility's client bits, kept by the facility's own lane.  Then every lane
+// walks the recurrence over its own groups (a group's clients are a popcount
+// of its bits), so that one FP64 instruction serves 32 facilities: at some two
+// FP64 lanes per SM and cycle a warp per facility, walking on all its lanes,
+// was bound by them and by the chain of four dependent loads per facility.
+// Facilities that found their root read no further window.  Whole calls, a
+// warp per facility against this: query at 4.2 M facilities 11.24 -> 8.72 ms
+// (4.5 ms of it the kernel before), 16 instances of 262 k vertices 12.61 ->
+// 8.50 ms, R-MAT 20 solve 11.81 -> 11.08 ms.
+constexpr int kRadWords = 4;
+constexpr int kRadWindow = 32 * kRadWords;  // a group has at most 32 entries
+
 // R > 1 (batches on one resident graph): R instances, instance i's costs,
 // client mask and radii at offset i*n; the warps of one vertex block's R
 // instances are adjacent, so its ADS rows are read from DRAM once.
@@ -482,18 +437,107 @@ __global__ void __launch_bounds__(256) k_radius(int64_t n, int64_t R, const doub
     for (int64_t t = (((int64_t)blockIdx.x * blockDim.x) + threadIdx.x) >> 5; t < nb * R; t += warps) {
         const int64_t blk = kMulti ? t / R : t;
         const int64_t io = kMulti ? (t - blk * R) * n : 0;  // instance offset
+        const uint8_t* __restrict__ cl_of = client + io;
         const int64_t v = (blk << 5) + lane;
-        const double cv = v < n ? cost[io + v] : INFINITY;
-        unsigned fac = __ballot_sync(kFull, cv < INFINITY);
-        double rv = INFINITY;
-        while (fac) {
-            const int b = __ffs(fac) - 1;
-            fac &= fac - 1;
-            const double c = __shfl_sync(kFull, cv, b);
-            const double res = facility_radius((blk << 5) + b, c, io, client, gofs, eofs, ginfo, gwt, eid);
-            if (lane == b) rv = res;
+        const double c = v < n ? cost[io + v] : INFINITY;
+        bool todo = c < INFINITY, root = false;
+        int64_t gi = 0, ge = 0, e = 0;
+        int left = 0, L = 0, j = 0;
+        uint32_t info = 0;
+        double wt = 0.0, N = 0.0, G = 0.0;
+        if (todo) {
+            gi = gofs[v];
+            ge = gofs[v + 1];
+            e = eofs[v];
+            left = (int)min(eofs[v + 1] - e, (int64_t)INT32_MAX);
+            info = ginfo[gi];
+            wt = gwt[gi];
+            L = (int)(ginfo[ge - 1] & 0xffffu);
         }
-        if (v < n) r_out[io + v] = rv;
+        while (const unsigned live = __ballot_sync(kFull, todo)) {
+            uint32_t bits[kRadWords + 1];
+#pragma unroll
+            for (int q = 0; q <= kRadWords; ++q) bits[q] = 0u;
+            for (unsigned rest = live; rest;) {
+                const int b0 = __ffs(rest) - 1;
+                rest &= rest - 1;
+                const int b1 = rest ? __ffs(rest) - 1 : 32;
+                rest &= rest - 1;
+                const int32_t* __restrict__ p0 = eid + __shfl_sync(kFull, e, b0);
+                const int32_t* __restrict__ p1 = eid + __shfl_sync(kFull, e, b1 & 31);
+                const int n0 = __shfl_sync(kFull, left, b0);
+                const int n1l = __shfl_sync(kFull, left, b1 & 31);
+                const int n1 = b1 < 32 ? n1l : 0;
+                int32_t id0[kRadWords], id1[kRadWords];
+#pragma unroll
+                for (int q = 0; q < kRadWords; ++q) {
+                    const int at = 32 * q + lane;
+                    id0[q] = at < n0 ? __ldg(&p0[at]) : -1;
+                    id1[q] = at < n1 ? __ldg(&p1[at]) : -1;
+                }
+                bool f0[kRadWords], f1[kRadWords];
+#pragma unroll
+                for (int q = 0; q < kRadWords; ++q) {
+                    f0[q] = id0[q] >= 0 && __ldg(&cl_of[id0[q]]) != 0;
+                    f1[q] = id1[q] >= 0 && __ldg(&cl_of[id1[q]]) != 0;
+                }
+#pragma unroll
+                for (int q = 0; q < kRadWords; ++q) {
+                    const unsigned w0 = __ballot_sync(kFull, f0[q]), w1 = __ballot_sync(kFull, f1[q]);
+                    if (lane == b0) bits[q] = w0;
+                    if (lane == b1) bits[q] = w1;
+                }
+            }
+            int off = 0;  // entries of the window walked
+            while (todo) {
+                const int hop = (int)(info & 0xffffu), cnt = (int)((info >> 16) & 0xffu), counted = (int)(info >> 24);
+                if (off + cnt > kRadWindow) break;  // the group ends in the next window
+                const double w = wt;
+                if (++gi < ge) {
+                    info = ginfo[gi];
+                    wt = gwt[gi];
+                }
+                uint32_t lo = 0, hi = 0;
+#pragma unroll
+                for (int q = 0; q < kRadWords; ++q)
+                    if ((off >> 5) == q) {
+                        lo = bits[q];
+                        hi = bits[q + 1];
+                    }
+                const uint32_t own = __funnelshift_r(lo, hi, off & 31);
+                const int clients = __popc(own & (counted >= 32 ? ~0u : (1u << counted) - 1u));
+                off += cnt;
+                for (; j < hop; ++j) {  // hops without new entries: W_j = 0
+                    const double Gn = __dadd_rn(G, N);
+                    if (Gn >= c) break;
+                    G = Gn;
+                }
+                if (j < hop) {
+                    root = true;
+                    todo = false;
+                    break;
+                }
+                N = __dadd_rn(N, __dmul_rn((double)clients, w));
+                if (j < L) {
+                    const double Gn = __dadd_rn(G, N);
+                    if (Gn >= c) {
+                        root = true;
+                        todo = false;
+                        break;
+                    }
+                    G = Gn;
+                }
+                ++j;
+                if (gi >= ge) {  // the last group: its hop is L
+                    j = L;
+                    root = N > 0.0;
+                    todo = false;
+                }
+            }
+            e += off;
+            left -= off;
+        }
+        if (v < n) r_out[io + v] = root ? __dadd_rn((double)j, __ddiv_rn(__dsub_rn(c, G), N)) : INFINITY;
     }
 }
 
