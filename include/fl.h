@@ -462,13 +462,12 @@ int fl_hop_model(const fl_graph* g, int64_t cap, int64_t* n_hops, int64_t* edge_
  *                           smallest-id nearest open facility and its hop
  *                           distance, -1 where none is reachable.
  *   stream                  cudaStream_t for all work; returns after it ends.
- * Scratch (about 28 MB) is one fixed device array of the library, held by
+ * Scratch (about 17 MB) is one fixed device array of the library, held by
  * every GPU that loads it until the process exits.  The first call on a
  * device looks up that array's device address (cudaGetSymbolAddress); make
  * that first call before any stream capture on the device.  Every call
- * synchronises `stream` several times: after validating the CSR and once per
- * BFS level, to read the next frontier's size into host memory, so no call
- * can be captured into a CUDA graph.  All calls
+ * synchronises `stream` at its end, to read whether the CSR was valid, so no
+ * call can be captured into a CUDA graph.  All calls
  * share the array and each clears what must start at zero; calls that
  * overlap on the GPU race.
  */

@@ -365,6 +365,63 @@ __device__ __forceinline__ uint64_t grp_compact(const Grp<G>& g, uint64_t x, uns
     return g.l < total ? y : fill;
 }
 
+// ----------------------------------------------------------------- resident kernels
+// A cooperative launch of blocks of kResThreads threads, at most one per SM,
+// that separates its passes by grid barriers.
+
+constexpr int kResThreads = 1024;
+constexpr int kResWarps = kResThreads / 32;
+constexpr unsigned kWaitLimit = 1u << 25;   // barrier polls; past the limit the kernel returns
+
+struct GridBar {
+    unsigned long long pass[8];       // per pass (mod 8): counts of its threads << 32 | blocks arrived
+    unsigned err;                     // bit 0: a barrier wait ran out (other bits: the kernel's own)
+    unsigned pad;
+};
+
+__device__ __forceinline__ unsigned long long ld_acquire(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// End of a pass: a grid barrier that adds up the threads' counts on the way
+// (one word per pass holds both, so the last poll also brings the total).
+// *total is the same on every thread; false when the wait ran out.  The word
+// of two passes ahead is cleared here.
+__device__ __forceinline__ bool end_pass(GridBar* c, unsigned& pass, unsigned mine, unsigned* total) {
+    __shared__ unsigned s_sum[kResWarps];
+    __shared__ unsigned long long s_word;
+    mine = __reduce_add_sync(kFull, mine);
+    if (lane_id() == 0) s_sum[threadIdx.x >> 5] = mine;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const unsigned x = __reduce_add_sync(kFull, s_sum[threadIdx.x]);
+        if (threadIdx.x == 0) {
+            if (blockIdx.x == 0) c->pass[(pass + 2) & 7] = 0;
+            unsigned long long* word = &c->pass[pass & 7];
+            __threadfence();
+            atomicAdd(word, ((unsigned long long)x << 32) | 1ULL);
+            unsigned long long w = 0;
+            unsigned polls = 0;
+            while ((unsigned)(w = ld_acquire(word)) < gridDim.x) {
+                if (++polls > kWaitLimit) {
+                    atomicOr(&c->err, 1u);
+                    w = ~0ULL;
+                    break;
+                }
+            }
+            __threadfence();
+            s_word = w;
+        }
+    }
+    __syncthreads();
+    const unsigned long long w = s_word;
+    *total = (unsigned)(w >> 32);
+    ++pass;
+    return w != ~0ULL;
+}
+
 // ----------------------------------------------------------------- device counters
 
 // Small block of device counters read back by the host between launches.

@@ -30,68 +30,21 @@ namespace fl {
 
 namespace {
 
-constexpr int kThreads = 1024;
-constexpr int kWarps = kThreads / 32;
 constexpr uint32_t kNone = 0xffffffffu;
 constexpr uint64_t kDone = ~0ULL;           // fk of a vertex that is no undecided facility
-constexpr unsigned kWaitLimit = 1u << 25;   // barrier polls
 constexpr int kMaxBall = 1023;              // larger ball radii take the host-driven rounds
 constexpr int kRoundsPerLaunch = 32;        // greedy rounds (bounds the log)
 constexpr int kFastRows = 128;              // log rows copied with the control block
 
 // Control block of a launch (device).
 struct Ctl {
-    unsigned long long pass[8];       // per pass (mod 8): counts of its threads << 32 | blocks arrived
-    unsigned err;                     // 1: a barrier wait ran out; 2: a ball without clients; 4: the level cap
+    GridBar bar;                      // its err: 1: a barrier wait ran out; 2: a ball without clients; 4: the level cap
     unsigned deep;                    // 1: a ball radius above kMaxBall (nothing was done)
     unsigned n_list[2];               // items of the current / next greedy round
     unsigned tmax[2];                 // largest ball radius of the undecided, by round parity
     unsigned hist[2][kMaxBall + 1];   // undecided facilities by ball radius, by round parity
     long long rounds, n_u, n_open, log_n;
 };
-
-__device__ __forceinline__ unsigned long long ld_acquire(const unsigned long long* p) {
-    unsigned long long v;
-    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-
-// End of a pass: a grid barrier that adds up the threads' counts on the way
-// (one word per pass holds both, so the last poll also brings the total).
-// *total is the same on every thread; false when the wait ran out.  The word
-// of two passes ahead is cleared here.
-__device__ __forceinline__ bool end_pass(Ctl* c, unsigned& pass, unsigned mine, unsigned* total) {
-    __shared__ unsigned s_sum[kWarps];
-    __shared__ unsigned long long s_word;
-    mine = __reduce_add_sync(kFull, mine);
-    if (lane_id() == 0) s_sum[threadIdx.x >> 5] = mine;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        const unsigned x = __reduce_add_sync(kFull, s_sum[threadIdx.x]);
-        if (threadIdx.x == 0) {
-            if (blockIdx.x == 0) c->pass[(pass + 2) & 7] = 0;
-            unsigned long long* word = &c->pass[pass & 7];
-            __threadfence();
-            atomicAdd(word, ((unsigned long long)x << 32) | 1ULL);
-            unsigned long long w = 0;
-            unsigned polls = 0;
-            while ((unsigned)(w = ld_acquire(word)) < gridDim.x) {
-                if (++polls > kWaitLimit) {
-                    atomicOr(&c->err, 1u);
-                    w = ~0ULL;
-                    break;
-                }
-            }
-            __threadfence();
-            s_word = w;
-        }
-    }
-    __syncthreads();
-    const unsigned long long w = s_word;
-    *total = (unsigned)(w >> 32);
-    ++pass;
-    return w != ~0ULL;
-}
 
 struct ItemGraph {
     const int32_t* __restrict__ cols;
@@ -168,19 +121,19 @@ __device__ __forceinline__ void log_row(const MisArgs& a, long long rd, int kind
     a.c->log_n = at + 1;
 }
 
-__global__ void __launch_bounds__(kThreads, 1) k_mis_resident(MisArgs a) {
+__global__ void __launch_bounds__(kResThreads, 1) k_mis_resident(MisArgs a) {
     __shared__ unsigned s_hist[kMaxBall + 1];
     __shared__ unsigned s_t;
     Ctl* c = a.c;
     const int lane = lane_id();
-    const int64_t warp0 = ((int64_t)blockIdx.x * kThreads + threadIdx.x) >> 5;
-    const int64_t warps = (int64_t)gridDim.x * kWarps;
+    const int64_t warp0 = ((int64_t)blockIdx.x * kResThreads + threadIdx.x) >> 5;
+    const int64_t warps = (int64_t)gridDim.x * kResWarps;
     const bool scribe = blockIdx.x == 0 && threadIdx.x == 0;
     unsigned pass = 0, total = 0;
 
     // Undecided facilities by ball radius: block counts, then the grid's.
     auto hist_begin = [&]() {
-        for (int i = threadIdx.x; i <= kMaxBall; i += kThreads) s_hist[i] = 0;
+        for (int i = threadIdx.x; i <= kMaxBall; i += kResThreads) s_hist[i] = 0;
         if (threadIdx.x == 0) s_t = 0;
         __syncthreads();
     };
@@ -193,7 +146,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mis_resident(MisArgs a) {
     };
     auto hist_end = [&](int parity) {
         __syncthreads();
-        for (int i = threadIdx.x; i < (int)s_t; i += kThreads)
+        for (int i = threadIdx.x; i < (int)s_t; i += kResThreads)
             if (s_hist[i]) atomicAdd(&c->hist[parity][i], s_hist[i]);
         if (threadIdx.x == 0 && s_t) atomicMax(&c->tmax[parity], s_t - 1);
     };
@@ -222,7 +175,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mis_resident(MisArgs a) {
             a.X[0][v] = a.X[1][v] = kNone;
         }
         hist_end(1);
-        if (!end_pass(c, pass, deep, &total)) return;
+        if (!end_pass(&c->bar, pass, deep, &total)) return;
         if (total) {
             if (scribe) c->deep = 1;
             return;
@@ -280,7 +233,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mis_resident(MisArgs a) {
                     }
                 }
             }
-            if (!end_pass(c, pass, changed, &total)) return;
+            if (!end_pass(&c->bar, pass, changed, &total)) return;
             if (scribe && front) log_row(a, rounds, 0, t, front, 1, now_ns() - t0);
             x ^= 1;
         }
@@ -289,7 +242,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mis_resident(MisArgs a) {
         // cover reached: the list of this round's other sweeps and of the next round
         unsigned seeds = 0;
         if (blockIdx.x == 0) {  // the other parity's buckets: filled after the next barriers
-            for (int i = threadIdx.x; i <= kMaxBall; i += kThreads) c->hist[par ^ 1][i] = 0;
+            for (int i = threadIdx.x; i <= kMaxBall; i += kResThreads) c->hist[par ^ 1][i] = 0;
             if (threadIdx.x == 0) c->tmax[par ^ 1] = 0;
         }
         for (int64_t b = warp0 * 32; b < n_list; b += warps * 32) {
@@ -320,7 +273,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mis_resident(MisArgs a) {
                 if (keep) next[at + __popc(mk & ((1u << lane) - 1u))] = p;
             }
         }
-        if (!end_pass(c, pass, seeds, &total)) return;
+        if (!end_pass(&c->bar, pass, seeds, &total)) return;
         const int64_t n_next = (int64_t)__ldcg(&c->n_list[cl ^ 1]);
         // ---- gather: after b rounds a facility of ball radius b holds the
         // smallest seed of its ball; it decides in the pass that follows (those
@@ -331,7 +284,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mis_resident(MisArgs a) {
                 a.fk[v] = kDone;
                 return true;
             }
-            if (y == kNone) atomicOr(&c->err, 2u);
+            if (y == kNone) atomicOr(&c->bar.err, 2u);
             return false;
         };
         int y = 0;
@@ -359,7 +312,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mis_resident(MisArgs a) {
                     }
                 }
             }
-            if (!end_pass(c, pass, changed, &total)) return;
+            if (!end_pass(&c->bar, pass, changed, &total)) return;
             if (scribe && front) log_row(a, rounds, 1, b, front, 1, now_ns() - t0);
             y ^= 1;
         }
@@ -379,7 +332,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mis_resident(MisArgs a) {
                 ++fresh;
             }
         }
-        if (!end_pass(c, pass, fresh, &total)) return;
+        if (!end_pass(&c->bar, pass, fresh, &total)) return;
         // ---- kill: vertices within b of a newly claimed client after b rounds
         for (int b = 1; b <= T && total; ++b) {
             const unsigned long long t0 = now_ns();
@@ -396,7 +349,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mis_resident(MisArgs a) {
                     ++marked;
                 }
             }
-            if (!end_pass(c, pass, marked, &total)) return;
+            if (!end_pass(&c->bar, pass, marked, &total)) return;
             if (scribe) log_row(a, rounds, 4, b, total, 1, now_ns() - t0);
         }
         // ---- the facilities of radius T decide; an undecided facility with a
@@ -421,12 +374,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_mis_resident(MisArgs a) {
             hist_add((unsigned)(f >> 32));
         }
         hist_end(par ^ 1);
-        if (!end_pass(c, pass, left, &total)) return;
+        if (!end_pass(&c->bar, pass, left, &total)) return;
         if (scribe) log_row(a, rounds, 3, T, n_u, n_u - (long long)total, now_ns() - t_round);
         n_u = (long long)total;
         whole = false;
         cl ^= 1;
-        if (__ldcg(&c->err)) return;
+        if (__ldcg(&c->bar.err)) return;
     }
     if (n_u == 0) {  // the open set and its list
         unsigned opened = 0;
@@ -466,25 +419,25 @@ struct BfsArgs {
 // Level-synchronous BFS: level L gives every vertex without a distance the
 // smallest label among its neighbours at distance L - 1.  In place: a
 // distance written in this level is L and does not pass for L - 1.
-__global__ void __launch_bounds__(kThreads, 1) k_bfs_resident(BfsArgs a) {
+__global__ void __launch_bounds__(kResThreads, 1) k_bfs_resident(BfsArgs a) {
     const int lane = lane_id();
-    const int64_t tid = (int64_t)blockIdx.x * kThreads + threadIdx.x, threads = (int64_t)gridDim.x * kThreads;
+    const int64_t tid = (int64_t)blockIdx.x * kResThreads + threadIdx.x, threads = (int64_t)gridDim.x * kResThreads;
     unsigned pass = 0, total = 0;
     for (int64_t v = tid; v < a.g.n; v += threads) {
         a.label[v] = kNone;
         a.dist[v] = -1;
     }
-    if (!end_pass(a.c, pass, 0, &total)) return;
+    if (!end_pass(&a.c->bar, pass, 0, &total)) return;
     for (int64_t i = tid; i < a.n_src; i += threads) {
         const int32_t s = a.src[i];
         a.label[s] = (uint32_t)(a.label_of ? a.label_of[s] : s);
         a.dist[s] = 0;
     }
-    if (!end_pass(a.c, pass, 0, &total)) return;
+    if (!end_pass(&a.c->bar, pass, 0, &total)) return;
     total = a.n_src > 0;
     for (int64_t L = 1; total; ++L) {
         if (L > a.cap) {
-            if (tid == 0) a.c->err = 4;
+            if (tid == 0) a.c->bar.err = 4;
             return;
         }
         unsigned reached = 0;
@@ -502,7 +455,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_bfs_resident(BfsArgs a) {
                 ++reached;
             }
         }
-        if (!end_pass(a.c, pass, reached, &total)) return;
+        if (!end_pass(&a.c->bar, pass, reached, &total)) return;
     }
 }
 
@@ -532,7 +485,7 @@ int resident_blocks(int64_t n_items, int* out) {
     int dev = 0, sms = 0;
     FL_CUDA(cudaGetDevice(&dev));
     FL_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int64_t want = (n_items * 8 + kThreads - 1) / kThreads;
+    const int64_t want = (n_items * 8 + kResThreads - 1) / kResThreads;
     *out = (int)std::max<int64_t>(1, std::min<int64_t>(sms, want));
     return FL_OK;
 }
@@ -628,14 +581,14 @@ int mis_resident(fl_solve* s, int64_t m, bool* done) {
         void* args[] = {&a};
         cudaError_t le = cudaSuccess;
         FL_LAUNCH(kProfMis, le = cudaLaunchCooperativeKernel((const void*)k_mis_resident, dim3(blocks),
-                                                             dim3(kThreads), args, 0, st));
+                                                             dim3(kResThreads), args, 0, st));
         FL_CUDA(le);
         FL_CUDA(cudaMemcpyAsync(h, s->rctl.p, h_b, cudaMemcpyDeviceToHost, st));
         FL_CUDA(cudaStreamSynchronize(st));
         const Ctl* c = reinterpret_cast<const Ctl*>(h);
         if (c->deep) return FL_OK;
-        if (c->err & 1u) FL_FAIL(FL_ETIMEOUT, "greedy MIS: a barrier wait ran out");
-        if (c->err) FL_FAIL(FL_ECUDA, "greedy MIS: inconsistent gather state");
+        if (c->bar.err & 1u) FL_FAIL(FL_ETIMEOUT, "greedy MIS: a barrier wait ran out");
+        if (c->bar.err) FL_FAIL(FL_ECUDA, "greedy MIS: inconsistent gather state");
         const size_t at = s->mis_log.size(), rows = (size_t)c->log_n;
         s->mis_log.resize(at + rows * 6);
         if (rows <= (size_t)kFastRows) {
@@ -652,7 +605,7 @@ int mis_resident(fl_solve* s, int64_t m, bool* done) {
         if (c->rounds > m) FL_FAIL(FL_ETIMEOUT, "greedy MIS did not converge");
         // barrier and pass counters start again; the round state stays
         a.resume = 1;
-        FL_CUDA(cudaMemsetAsync(a.c->pass, 0, sizeof(a.c->pass), st));
+        FL_CUDA(cudaMemsetAsync(a.c->bar.pass, 0, sizeof(a.c->bar.pass), st));
         FL_CUDA(cudaMemsetAsync(&a.c->log_n, 0, 8, st));
     }
     *done = true;
@@ -679,11 +632,11 @@ int msbfs_resident(fl_graph* g, const int32_t* src, int64_t n_src, int32_t* labe
     FL_CUDA(cudaMemsetAsync(ctl.p, 0, sizeof(Ctl), st));
     void* args[] = {&a};
     cudaError_t le = cudaSuccess;
-    FL_LAUNCH(cls, le = cudaLaunchCooperativeKernel((const void*)k_bfs_resident, dim3(blocks), dim3(kThreads), args,
+    FL_LAUNCH(cls, le = cudaLaunchCooperativeKernel((const void*)k_bfs_resident, dim3(blocks), dim3(kResThreads), args,
                                                     0, st));
     FL_CUDA(le);
     unsigned* h = reinterpret_cast<unsigned*>(g->h_ctr + 1);
-    FL_CUDA(cudaMemcpyAsync(h, &a.c->err, 4, cudaMemcpyDeviceToHost, st));
+    FL_CUDA(cudaMemcpyAsync(h, &a.c->bar.err, 4, cudaMemcpyDeviceToHost, st));
     FL_CUDA(cudaStreamSynchronize(st));
     const unsigned err = *h;
     if (err & 4u) FL_FAIL(FL_ETIMEOUT, "BFS reached its level cap");

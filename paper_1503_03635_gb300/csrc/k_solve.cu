@@ -21,64 +21,6 @@ static int grid_for(int64_t items, int per_block) {
 }
 
 // ------------------------------------------------------------------ frontier propagation
-// A frontier is a list of vertices with a device-side count.  One round:
-// snapshot (copy each frontier vertex's value, so a round moves values exactly
-// one hop), then push: for every edge (v, u), X[u] = min(X[u], val(v) + add);
-// u joins the next frontier the first time it decreases in the round.
-
-__global__ void k_snapshot(const int32_t* __restrict__ fr, const unsigned long long* __restrict__ n_fr,
-                           const unsigned long long* __restrict__ X, unsigned long long* __restrict__ frval,
-                           unsigned long long* __restrict__ reset_next,
-                           uint32_t* __restrict__ tstamp, uint32_t tval, int32_t* __restrict__ touched,
-                           unsigned long long* __restrict__ n_touched) {
-    const int64_t n = (int64_t)*n_fr;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *reset_next = 0;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += stride) {
-        int64_t i = base + lane_id();
-        bool fresh = false;
-        int32_t v = 0;
-        if (i < n) {
-            v = fr[i];
-            frval[i] = X[v];
-            if (tstamp) fresh = atomicExch(&tstamp[v], tval) != tval;
-        }
-        if (tstamp) {
-            long long at = warp_append(fresh, n_touched);
-            if (at >= 0) touched[at] = v;
-        }
-    }
-}
-
-__global__ void __launch_bounds__(256) k_push(const int32_t* __restrict__ fr, const unsigned long long* __restrict__ frval,
-                                              const unsigned long long* __restrict__ n_fr,
-                                              const int64_t* __restrict__ rowp, const int32_t* __restrict__ cols,
-                                              unsigned long long add, unsigned long long* __restrict__ X,
-                                              uint32_t* __restrict__ stamp, uint32_t sv, int32_t* __restrict__ fr_next,
-                                              unsigned long long* __restrict__ n_next) {
-    const int lane = lane_id();
-    const int64_t n = (int64_t)*n_fr;
-    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t w = (((int64_t)blockIdx.x * blockDim.x) + threadIdx.x) >> 5; w < n; w += warps) {
-        const int32_t v = fr[w];
-        const unsigned long long val = frval[w] + add;
-        const int64_t beg = rowp[v], end = rowp[v + 1];
-        for (int64_t cb = beg; cb < end; cb += 32) {
-            int64_t e = cb + lane;
-            bool fresh = false;
-            int32_t u = 0;
-            if (e < end) {
-                u = cols[e];
-                if (val < X[u]) {
-                    unsigned long long old = atomicMin(&X[u], val);
-                    if (val < old) fresh = atomicExch(&stamp[u], sv) != sv;
-                }
-            }
-            long long at = warp_append(fresh, n_next);
-            if (at >= 0) fr_next[at] = u;
-        }
-    }
-}
 
 // Seeds: X[s] = min(X[s], val(s)); s joins the frontier when it decreases.
 // With `reach`, a seed that held no value below `limit` records reach_val.
@@ -417,8 +359,8 @@ __global__ void k_check_costs(const double* __restrict__ cost, int64_t n, Counte
 // was bound by them and by the chain of four dependent loads per facility.
 // Facilities that found their root read no further window.  Whole calls, a
 // warp per facility against this: query at 4.2 M facilities 11.24 -> 8.72 ms
-// (4.5 ms of it the kernel before), 16 instances of 262 k vertices 12.61 ->
-// 8.50 ms, R-MAT 20 solve 11.81 -> 11.08 ms.
+// (the kernel 4.52 -> 0.57), 16 instances of 262 k vertices 12.61 -> 8.50 ms
+// (5.05 -> 0.59), R-MAT 20 solve 11.81 -> 11.08 ms.
 constexpr int kRadWords = 4;
 constexpr int kRadWindow = 32 * kRadWords;  // a group has at most 32 entries
 
