@@ -15,16 +15,27 @@
 // of the coming levels, and a second ring of bitmaps over the CSR entries
 // marks which entries (v, u) of an active v deliver at that level (u posts
 // to the entry of v's row paired with its own entry (u, v), so v reads only
-// the neighbours that gained).  An active v merges into its bottom-k sketch the
-// entries of each such neighbour u at distance L - w(u, v); the ranks that enter
-// form v's group at distance L, with the HIP weight and counted prefix of
-// the unweighted build (the sketch after the level, ties at one distance in
-// ascending rank).  A vertex's entries are kept in distance order in a
-// fixed-capacity row, so each edge keeps a cursor into its neighbour's row
-// that only moves forward.  Entries appended at level L have distance L and
-// are never read in the same level (every length is >= 1): a level reads the
-// row counts as they were when it started and writes the new counts to a
-// second array, which a commit pass over the active vertices copies back.
+// the neighbours that gained).  u posts to v only if one of the ranks it
+// gained is below v's k-th rank and not in v's sketch: k-th ranks only fall
+// and a rank that leaves a sketch never returns, so the others could not
+// enter v's sketch at level L either.  (Most are already there: every
+// neighbour of v that holds a rank would offer it again.)  An active v merges
+// into its bottom-k sketch the entries of each posting neighbour u at distance
+// L - w(u, v), found by bisection in u's row, which is in distance order; the
+// ranks that enter form v's group at distance L, with the HIP weight and
+// counted prefix of the unweighted build (the sketch after the level, ties at
+// one distance in ascending rank).  Entries appended at level L have distance
+// L and are never read in the same level (every length is >= 1): a level reads
+// the row counts as they were when it started and writes the new counts to a
+// second array, which the next level's first pass copies back.
+//
+// The whole loop is one resident kernel, two grid barriers per level (collect
+// the active vertices; merge and post), in place of three launches and a look
+// at the ring by the host.  A warp per active vertex; rows above kWLong
+// entries are posted by the whole block, so that no level waits for one warp
+// on a hub.  Bound by the latency of the dependent loads of a post (column,
+// k-th rank, sketch).  R-MAT, 65 k vertices, lengths up to 100, k = 16, 313
+// levels: 115 ms of level kernels and some 15 ms of gaps before, 36 ms now.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -69,9 +80,7 @@ struct WArgs {
     int32_t* ecnt;           // n: entries at the start of the level (read)
     int32_t* ecnt_n;         // n: entries after the level (written by the active vertices)
     int32_t* gcnt;           // n: groups
-    int32_t* cursor;         // nnz
     WGroup* glog;            // group log
-    unsigned long long* glog_n;
     unsigned long long glog_cap;
     uint32_t* ring;          // R bitmaps of `words` words
     int64_t words;
@@ -79,212 +88,321 @@ struct WArgs {
     const uint32_t* rev;     // nnz: the entry (v, u) paired with each entry (u, v)
     uint32_t* marks;         // R bitmaps of `mwords` words over the CSR entries
     int64_t mwords;
-    unsigned long long* pend;  // R activation counts
-    unsigned long long* err;   // 1: a row overflowed; 2: a distance above 65535; 4: the group log overflowed
+    unsigned* pend;          // R: nonzero when the slot has activations
+    int32_t* act[2];         // active vertices of the even / odd steps (n each)
+    int64_t n;
+    struct WCtl* c;
 };
 
-__device__ __forceinline__ void activate(const WArgs& a, int32_t u, int64_t level) {
-    const int slot = (int)(level % a.R);
-    const uint32_t bit = 1u << (u & 31);
-    const uint32_t old = atomicOr(&a.ring[(int64_t)slot * a.words + (u >> 5)], bit);
-    if (!(old & bit)) atomicAdd(&a.pend[slot], 1ULL);
+// Control block of the build (device, zero at its start).
+struct WCtl {
+    GridBar bar;
+    unsigned long long n_act[2];  // active vertices of the even / odd steps
+    unsigned long long glog_n;    // groups logged
+    unsigned long long err;       // 1: a row overflowed; 2: a distance above 65535; 4: the group log overflowed
+    long long last;               // the largest level that added groups
+    long long levels;             // levels run
+};
+
+constexpr int kWLong = 512;   // longer rows are posted by the whole block
+constexpr int kWQueue = 32;   // of them, queued per block and level
+
+__device__ __forceinline__ WEnt load_ent(const WEnt* p) {
+    const int2 x = __ldcg(reinterpret_cast<const int2*>(p));
+    return WEnt{x.x, x.y};
 }
 
-// The source of CSR entry e = (u, v) gained entries that reach v at `level`:
-// mark v's paired entry (v, u) and activate v.
-__device__ __forceinline__ void post(const WArgs& a, int64_t e, int64_t level) {
-    const int slot = (int)(level % a.R);
-    const uint32_t re = a.rev[e];
-    atomicOr(&a.marks[(int64_t)slot * a.mwords + (re >> 5)], 1u << (re & 31));
-    activate(a, a.cols[e], level);
+// Is rank x in the ascending sketch row of k ranks (kEmpty padded)?  The row
+// may be rewritten meanwhile: every value read is of the old or the new sketch.
+__device__ __forceinline__ bool in_sketch(const uint64_t* row, int k, uint64_t x) {
+    int lo = 0, hi = k;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        const uint64_t y = __ldcg(&row[mid]);
+        if (y == x) return true;
+        if (y < x) lo = mid + 1;
+        else hi = mid;
+    }
+    return false;
 }
 
-// Level 0: every vertex's own rank; its neighbours become active at the
-// lengths of its edges.
-__global__ void k_winit(WArgs a, int64_t n) {
-    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int lane = lane_id();
-    for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < n; v += warps) {
-        if (lane < a.k) a.S[v * a.k + lane] = lane == 0 ? vertex_rank(a.seed, v) : kEmpty;
-        if (lane == 0) {
-            a.Scnt[v] = 1;
-            a.ent[v * a.cap] = WEnt{(int32_t)v, 0};
-            a.ecnt[v] = 1;
-            a.gcnt[v] = 1;
-            WGroup gr;
-            gr.wt = 1.0;  // a ball of one vertex (k >= 2)
-            gr.v = (int32_t)v;
-            gr.gidx = 0;
-            gr.dist = 0;
-            gr.cnt = 1;
-            gr.counted = 1;
-            gr.first = 0;
-            a.glog[v] = gr;
+// The ranks gained by v at level L (lane j < dcnt: the j-th, ascending) go to
+// the entries e0 + first, + step, ... of its row (all 32 lanes call).
+__device__ __forceinline__ void post_row(const WArgs& a, int64_t e0, int64_t e1, int first, int step, uint64_t gained,
+                                         int dcnt, int64_t L) {
+    for (int64_t b = e0 + first; b < e1; b += step) {
+        const int64_t e = b + lane_id();
+        bool open = e < e1, want = false;
+        int32_t u = 0;
+        int64_t lv = 0;
+        uint64_t kth = 0;
+        if (open) {
+            u = __ldg(&a.cols[e]);
+            lv = L + __ldg(&a.wts[e]);
+            kth = __ldcg(&a.S[(int64_t)u * a.k + a.k - 1]);
+            if (lv > 65535) {
+                atomicOr(&a.c->err, 2ULL);
+                open = false;
+            }
         }
-        for (int64_t e = a.rowp[v] + lane; e < a.rowp[v + 1]; e += 32) {
-            a.cursor[e] = 0;
-            post(a, e, a.wts[e]);
+        for (int j = 0; j < dcnt && __any_sync(kFull, open); ++j) {
+            const uint64_t x = __shfl_sync(kFull, gained, j);
+            if (!open) continue;
+            if (x >= kth) open = false;
+            else if (!in_sketch(a.S + (int64_t)u * a.k, a.k, x)) {
+                want = true;
+                open = false;
+            }
+        }
+        if (want) {
+            const int slot = (int)((uint32_t)lv % (uint32_t)a.R);
+            const uint32_t re = __ldg(&a.rev[e]);
+            atomicOr(&a.marks[(int64_t)slot * a.mwords + (re >> 5)], 1u << (re & 31));
+            uint32_t* word = &a.ring[(int64_t)slot * a.words + (u >> 5)];
+            const uint32_t bit = 1u << (u & 31);
+            if (!(__ldcg(word) & bit) && !(atomicOr(word, bit) & bit)) a.pend[slot] = 1u;
         }
     }
 }
 
-// Active vertices of a level from its ring slot (the slot is cleared).
-__global__ void k_wcollect(uint32_t* __restrict__ bm, int64_t words, int64_t n, int32_t* __restrict__ out,
-                           unsigned long long* __restrict__ n_out) {
-    __shared__ BlockAppend<8> sh;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t bb = (int64_t)blockIdx.x * blockDim.x; bb < words * 32; bb += stride) {
-        const int64_t v = bb + threadIdx.x;
-        const int64_t w = v >> 5;
-        const uint32_t word = w < words ? bm[w] : 0u;
-        const bool in = v < n && ((word >> (v & 31)) & 1u);
-        const long long at = block_append<8>(in, n_out, sh);
-        if (at >= 0) out[at] = (int32_t)v;
-        __syncwarp();
-        if ((threadIdx.x & 31) == 0 && w < words && word) bm[w] = 0u;
-    }
-}
+__global__ void __launch_bounds__(kResThreads, 1) k_wbuild(WArgs a) {
+    __shared__ uint64_t s_gained[kWQueue][32];
+    __shared__ int32_t s_v[kWQueue];
+    __shared__ int s_cnt[kWQueue];
+    __shared__ unsigned s_queued, s_next;
+    WCtl* c = a.c;
+    const int lane = lane_id(), k = a.k;
+    const int64_t tid = (int64_t)blockIdx.x * kResThreads + threadIdx.x, threads = (int64_t)gridDim.x * kResThreads;
+    // item i to warp i / gridDim of block i mod gridDim: neighbours in a list go to different blocks
+    const int64_t item0 = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x, warps = threads >> 5;
+    unsigned pass = 0, total = 0;
+    if (threadIdx.x == 0) s_queued = 0;
 
-// One level: a warp per active vertex (see the file comment).
-__global__ void __launch_bounds__(256) k_wlevel(WArgs a, const int32_t* __restrict__ act,
-                                                const unsigned long long* __restrict__ n_act_d, int32_t L) {
-    __shared__ int32_t s_stage[8][1024];      // per warp: the delivering entries of 32 mark words
-    const int64_t n_act = (int64_t)*n_act_d;  // the vertices the collect pass listed
-    const int lane = lane_id();
-    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n_act; i += warps) {
-        const int32_t v = act[i];
-        const int cnt_old = a.Scnt[v];
-        const uint64_t s_old = lane < cnt_old ? a.S[(int64_t)v * a.k + lane] : kEmpty;
-        uint64_t s = s_old;
-        int cnt = cnt_old;
-        uint64_t kth = cnt == a.k ? __shfl_sync(kFull, s, a.k - 1) : kEmpty;
-        const int64_t e0 = a.rowp[v], e1 = a.rowp[v + 1];
-        const uint32_t* mk = a.marks + (int64_t)(L % a.R) * a.mwords;
-        int32_t* stage = s_stage[threadIdx.x >> 5];
-        const int64_t w1 = (e1 + 31) >> 5;
-        for (int64_t wb = e0 >> 5; wb < w1; wb += 32) {
-            // 32 words of marks at once: their set bits inside [e0, e1) are the
-            // delivering entries, staged in row order (a hub's row holds
-            // thousands of entries, a few of which deliver at a level)
-            const int64_t wi = wb + lane;
-            uint32_t bits = 0;
-            if (wi < w1) {
-                bits = mk[wi];
-                const int64_t first = wi << 5;
-                if (first < e0) bits &= ~0u << (int)(e0 - first);
-                if (e1 - first < 32) bits &= (1u << (int)(e1 - first)) - 1u;
+    // v gained ranks at level L: post them, or leave a long row to the block
+    auto post = [&](int32_t v, int64_t e0, int64_t e1, uint64_t gained, int dcnt, int64_t L) {
+        if (e1 - e0 > kWLong) {
+            unsigned at = 0;
+            if (lane == 0) at = atomicAdd(&s_queued, 1u);
+            at = __shfl_sync(kFull, at, 0);
+            if (at < kWQueue) {
+                s_gained[at][lane] = gained;
+                if (lane == 0) {
+                    s_v[at] = v;
+                    s_cnt[at] = dcnt;
+                }
+                return;
             }
-            const int mine = __popc(bits);
-            int pre = mine;
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(kFull, pre, o);
-                if (lane >= o) pre += y;
+        }
+        post_row(a, e0, e1, 0, 32, gained, dcnt, L);
+    };
+    auto post_queued = [&](int64_t L) {
+        __syncthreads();
+        const int queued = (int)min(s_queued, (unsigned)kWQueue);
+        for (int q = 0; q < queued; ++q) {
+            const int32_t v = s_v[q];
+            post_row(a, __ldg(&a.rowp[v]), __ldg(&a.rowp[v + 1]), (int)(threadIdx.x & ~31u), kResThreads,
+                     s_gained[q][lane], s_cnt[q], L);
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) s_queued = 0;
+    };
+
+    // level 0: every vertex's own rank
+    for (int64_t i = tid; i < a.n * k; i += threads) a.S[i] = i % k == 0 ? vertex_rank(a.seed, i / k) : kEmpty;
+    for (int64_t v = tid; v < a.n; v += threads) {
+        a.ent[v * a.cap] = WEnt{(int32_t)v, 0};
+        a.Scnt[v] = 1;
+        a.ecnt[v] = 1;
+        a.gcnt[v] = 1;
+        WGroup gr;
+        gr.wt = 1.0;  // a ball of one vertex (k >= 2)
+        gr.v = (int32_t)v;
+        gr.gidx = 0;
+        gr.dist = 0;
+        gr.cnt = 1;
+        gr.counted = 1;
+        gr.first = 0;
+        a.glog[v] = gr;
+    }
+    if (tid == 0) c->glog_n = (unsigned long long)a.n;
+    if (!end_pass(&c->bar, pass, 0, &total)) return;
+    for (int64_t v = item0; v < a.n; v += warps)
+        post((int32_t)v, __ldg(&a.rowp[v]), __ldg(&a.rowp[v + 1]), lane == 0 ? vertex_rank(a.seed, v) : kEmpty, 1, 0);
+    post_queued(0);
+    if (!end_pass(&c->bar, pass, 0, &total)) return;
+
+    int64_t L = 0, n_prev = 0;
+    for (unsigned step = 0;; ++step) {
+        // the next level with activations
+        if (threadIdx.x == 0) s_next = ~0u;
+        __syncthreads();
+        for (int d = 1 + threadIdx.x; d <= a.R; d += kResThreads)
+            if (__ldcg(&a.pend[(uint32_t)(L + d) % (uint32_t)a.R])) {
+                atomicMin(&s_next, (unsigned)d);
+                break;
             }
-            const int total = __shfl_sync(kFull, pre, 31);
-            if (total == 0) continue;
-            pre -= mine;
-            for (uint32_t b = bits; b; b &= b - 1u) stage[pre++] = (int32_t)((wi << 5) + (__ffs(b) - 1) - e0);
-            __syncwarp();
-            for (int cb = 0; cb < total; cb += 32) {
-                const int j = cb + lane;
-                int32_t u = 0, c0 = 0, c1 = 0;
-                if (j < total) {
-                    const int64_t e = e0 + stage[j];
-                    u = a.cols[e];
-                    const int32_t x = L - a.wts[e];
-                    if (x >= 0) {
-                        const int32_t have = min(a.ecnt[u], a.cap);
-                        const WEnt* row = a.ent + (int64_t)u * a.cap;
-                        int32_t c = min(a.cursor[e], have);
-                        while (c < have && row[c].dist < x) ++c;
-                        c0 = c;
-                        while (c < have && row[c].dist == x) ++c;
-                        c1 = c;
-                        a.cursor[e] = c;  // later levels ask for larger distances
+        __syncthreads();
+        const int par = (int)(step & 1);
+        // the level before: its new row counts become current
+        for (int64_t i = tid; i < n_prev; i += threads) {
+            const int32_t v = __ldcg(&a.act[par ^ 1][i]);
+            a.ecnt[v] = __ldcg(&a.ecnt_n[v]);
+        }
+        if (s_next == ~0u) break;
+        L += s_next;
+        const int slot = (int)((uint32_t)L % (uint32_t)a.R);
+        unsigned mine = 0;
+        uint32_t* bm = a.ring + (int64_t)slot * a.words;
+        for (int64_t w = tid >> 5; w < a.words; w += warps) {
+            const uint32_t word = __ldcg(&bm[w]);
+            if (!word) continue;
+            const bool in = (word >> lane) & 1u;
+            const long long at = warp_append(in, &c->n_act[par]);
+            if (in) a.act[par][at] = (int32_t)(w * 32 + lane);
+            mine += in;
+            if (lane == 0) bm[w] = 0u;
+        }
+        if (!end_pass(&c->bar, pass, mine, &total)) return;
+        n_prev = (int64_t)total;
+        if (tid == 0) {
+            c->n_act[par ^ 1] = 0;
+            a.pend[slot] = 0;  // no post of this level targets its own slot
+            ++c->levels;
+        }
+        for (int64_t i = item0; i < n_prev; i += warps) {
+            const int32_t v = __ldcg(&a.act[par][i]);
+            const uint64_t s_old = lane < k ? __ldcg(&a.S[(int64_t)v * k + lane]) : kEmpty;
+            const int64_t e0 = __ldg(&a.rowp[v]), e1 = __ldg(&a.rowp[v + 1]);
+            uint64_t s = s_old;
+            int cnt = __popc(__ballot_sync(kFull, s_old != kEmpty));
+            uint64_t kth = __shfl_sync(kFull, s, k - 1);  // kEmpty while the sketch is not full
+            uint32_t* mk = a.marks + (int64_t)slot * a.mwords;
+            const int64_t w1 = (e1 + 31) >> 5;
+            for (int64_t wb = e0 >> 5; wb < w1; wb += 32) {
+                // 32 words of marks at once: their set bits inside [e0, e1) are the delivering entries
+                const int64_t wi = wb + lane;
+                uint32_t bits = 0;
+                if (wi < w1) {
+                    bits = __ldcg(&mk[wi]);
+                    const int64_t first = wi << 5;
+                    uint32_t mask = ~0u;
+                    if (first < e0) mask &= ~0u << (int)(e0 - first);
+                    if (e1 - first < 32) mask &= (1u << (int)(e1 - first)) - 1u;
+                    bits &= mask;
+                    if (bits) {  // read: the slot serves level L + R next
+                        if (mask == ~0u) mk[wi] = 0u;
+                        else atomicAnd(&mk[wi], ~bits);
                     }
                 }
-                // each lane offers its entry's candidates one per round
-                while (__any_sync(kFull, c0 < c1)) {
-                    uint64_t r = kEmpty;
-                    if (c0 < c1) {
-                        r = vertex_rank(a.seed, a.ent[(int64_t)u * a.cap + c0].id);
-                        ++c0;
-                        if (r >= kth) r = kEmpty;  // cannot enter a full sketch
+                const int mine_n = __popc(bits);
+                const int incl = warp_incl_scan(mine_n);
+                const int n_del = __shfl_sync(kFull, incl, 31);
+                for (int cb = 0; cb < n_del; cb += 32) {
+                    const int j = cb + lane;
+                    // the word that holds the j-th set bit: the words whose bits all come before it
+                    int wl = 0;
+#pragma unroll
+                    for (int st = 16; st > 0; st >>= 1)
+                        if (__shfl_sync(kFull, incl, wl + st - 1) <= j) wl += st;
+                    const uint32_t word = __shfl_sync(kFull, bits, wl);
+                    const int before = __shfl_sync(kFull, incl - mine_n, wl);
+                    const WEnt* row = nullptr;
+                    int32_t at = 0, have = 0, x = 0;
+                    if (j < n_del) {
+                        const int64_t e = ((wb + wl) << 5) + nth_set_bit(word, j - before);
+                        const int32_t u = __ldg(&a.cols[e]);
+                        x = (int32_t)(L - __ldg(&a.wts[e]));
+                        have = min(__ldcg(&a.ecnt[u]), a.cap);
+                        row = a.ent + (int64_t)u * a.cap;
+                        int lo = 0, hi = have;
+                        while (lo < hi) {
+                            const int mid = (lo + hi) >> 1;
+                            if (load_ent(&row[mid]).dist < x) lo = mid + 1;
+                            else hi = mid;
+                        }
+                        at = lo;
                     }
-                    if (warp_member(s, r)) r = kEmpty;  // already held
-                    r = warp_sort(r);
-                    const uint64_t prev = __shfl_up_sync(kFull, r, 1);
-                    const bool keep = r != kEmpty && (lane == 0 || prev != r);
-                    r = warp_compact(r, __ballot_sync(kFull, keep), kEmpty);
-                    if (__ballot_sync(kFull, r != kEmpty) == 0) continue;
-                    s = warp_merge_low(s, r);
-                    if (lane >= a.k) s = kEmpty;
-                    cnt = __popc(__ballot_sync(kFull, s != kEmpty));
-                    kth = cnt == a.k ? __shfl_sync(kFull, s, a.k - 1) : kEmpty;
+                    // each lane offers its entry's candidates one per round
+                    for (;;) {
+                        uint64_t r = kEmpty;
+                        if (at < have) {
+                            const WEnt en = load_ent(&row[at]);
+                            ++at;
+                            if (en.dist == x) r = vertex_rank(a.seed, en.id);
+                            else at = have;
+                        }
+                        if (!__any_sync(kFull, r != kEmpty)) break;
+                        unsigned m = __ballot_sync(kFull, r < kth);
+                        if (__popc(m) <= 4) {
+                            for (; m; m &= m - 1) {
+                                const uint64_t y = __shfl_sync(kFull, r, __ffs(m) - 1);
+                                if (y >= kth || __ballot_sync(kFull, s == y)) continue;
+                                const int p = __popc(__ballot_sync(kFull, s < y));
+                                const uint64_t up = __shfl_up_sync(kFull, s, 1);
+                                s = lane > p ? up : (lane == p ? y : s);
+                                if (lane >= k) s = kEmpty;
+                                if (cnt < k) ++cnt;
+                                kth = __shfl_sync(kFull, s, k - 1);
+                            }
+                            continue;
+                        }
+                        if (r >= kth) r = kEmpty;
+                        if (warp_member(s, r)) r = kEmpty;  // already held
+                        r = warp_sort(r);
+                        const uint64_t prev = __shfl_up_sync(kFull, r, 1);
+                        const bool keep = r != kEmpty && (lane == 0 || prev != r);
+                        r = warp_compact(r, __ballot_sync(kFull, keep), kEmpty);
+                        s = warp_merge_low(s, r);
+                        if (lane >= k) s = kEmpty;
+                        cnt = __popc(__ballot_sync(kFull, s != kEmpty));
+                        kth = __shfl_sync(kFull, s, k - 1);
+                    }
                 }
             }
-            __syncwarp();
-        }
-        // the entries gained at distance L: in the new sketch, not in the old
-        // (every lane takes part in the membership shuffles)
-        const bool held = warp_member(s_old, s);
-        const bool fresh = s != kEmpty && !held;
-        const unsigned fm = __ballot_sync(kFull, fresh);
-        const int32_t base = a.ecnt[v];
-        if (!fm) {
-            if (lane == 0) a.ecnt_n[v] = base;
-            continue;
-        }
-        const int dcnt = __popc(fm);
-        if (base + dcnt > a.cap) {
+            // the entries gained at distance L: in the new sketch, not in the old
+            // (every lane takes part in the membership shuffles)
+            const bool held = warp_member(s_old, s);
+            const bool fresh = s != kEmpty && !held;
+            const unsigned fm = __ballot_sync(kFull, fresh);
+            const int32_t base = __ldcg(&a.ecnt[v]);
+            const int dcnt = __popc(fm);
+            if (!fm || base + dcnt > a.cap) {
+                if (lane == 0) {
+                    a.ecnt_n[v] = base;
+                    if (fm) atomicOr(&c->err, 1ULL);
+                }
+                continue;
+            }
+            const int counted = __popc(fm & (cnt < k ? kFull : ((1u << (k - 1)) - 1u)));
+            if (fresh) {
+                const int at = base + __popc(fm & ((1u << lane) - 1u));
+                a.ent[(int64_t)v * a.cap + at] = WEnt{(int32_t)rank_vertex(a.seed, s), (int32_t)L};
+            }
+            if (lane < k) a.S[(int64_t)v * k + lane] = s;
             if (lane == 0) {
-                a.ecnt_n[v] = base;
-                atomicOr(a.err, 1ULL);
+                a.ecnt_n[v] = base + dcnt;
+                a.Scnt[v] = (uint8_t)cnt;
+                c->last = L;
+                const unsigned long long gi = atomicAdd(&c->glog_n, 1ULL);
+                if (gi < a.glog_cap) {
+                    WGroup gr;
+                    gr.wt = hip_weight(cnt, k, kth);
+                    gr.v = v;
+                    gr.gidx = __ldcg(&a.gcnt[v]);
+                    gr.dist = (int32_t)L;
+                    gr.cnt = dcnt;
+                    gr.counted = counted;
+                    gr.first = base;
+                    a.glog[gi] = gr;
+                    a.gcnt[v] = gr.gidx + 1;
+                } else {
+                    atomicOr(&c->err, 4ULL);
+                }
             }
-            continue;
+            post(v, e0, e1, warp_compact(s, fm, kEmpty), dcnt, L);
         }
-        const int counted = __popc(fm & (cnt < a.k ? kFull : ((1u << (a.k - 1)) - 1u)));
-        const double wt = hip_weight(cnt, a.k, __shfl_sync(kFull, s, a.k - 1));
-        if (fresh) {
-            const int at = base + __popc(fm & ((1u << lane) - 1u));
-            a.ent[(int64_t)v * a.cap + at] = WEnt{(int32_t)rank_vertex(a.seed, s), L};
-        }
-        if (lane < a.k) a.S[(int64_t)v * a.k + lane] = s;
-        if (lane == 0) {
-            a.ecnt_n[v] = base + dcnt;
-            a.Scnt[v] = (uint8_t)cnt;
-            const unsigned long long gi = atomicAdd(a.glog_n, 1ULL);
-            if (gi < a.glog_cap) {
-                WGroup gr;
-                gr.wt = wt;
-                gr.v = v;
-                gr.gidx = a.gcnt[v]++;
-                gr.dist = L;
-                gr.cnt = dcnt;
-                gr.counted = counted;
-                gr.first = base;
-                a.glog[gi] = gr;
-            } else {
-                atomicOr(a.err, 4ULL);
-            }
-        }
-        for (int64_t e = e0 + lane; e < e1; e += 32) {
-            const int64_t lv = (int64_t)L + a.wts[e];
-            if (lv > 65535) atomicOr(a.err, 2ULL);
-            else post(a, e, lv);
-        }
-    }
-}
-
-// End of a level: the active vertices' new row counts become current.
-__global__ void k_wcommit(const int32_t* __restrict__ act, const unsigned long long* __restrict__ n_act_d,
-                          const int32_t* __restrict__ ecnt_n, int32_t* __restrict__ ecnt) {
-    const int64_t n_act = (int64_t)*n_act_d;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_act; i += stride) {
-        const int32_t v = act[i];
-        ecnt[v] = ecnt_n[v];
+        post_queued(L);
+        if (!end_pass(&c->bar, pass, 0, &total)) return;
     }
 }
 
@@ -493,17 +611,17 @@ int build_sketches_weighted(fl_graph* g, int k, uint64_t seed) {
     const double expect = (double)k * (1.0 + std::log(std::max(1.0, (double)n / k)));
     int64_t cap = std::min<int64_t>(n, (int64_t)(2.0 * expect) + 64);
     const int64_t mwords = (nnz + 31) / 32;
-    DBuf ent, ecnt, ecnt_n, gcnt, cursor, glog, ring, pend, act, cnt, marks;
+    DBuf ent, ecnt, ecnt_n, gcnt, glog, ring, pend, act, cnt, marks;
     int rc = FL_OK;
     for (;;) {
         const unsigned long long glog_cap = (unsigned long long)n * (unsigned long long)cap;
         if ((rc = dalloc(g->S, (size_t)n * k * 8)) || (rc = dalloc(g->Scnt, (size_t)n)) ||
             (rc = dalloc(ent, (size_t)n * cap * sizeof(WEnt))) || (rc = dalloc(ecnt, (size_t)n * 4)) ||
             (rc = dalloc(ecnt_n, (size_t)n * 4)) ||
-            (rc = dalloc(gcnt, (size_t)n * 4)) || (rc = dalloc(cursor, (size_t)std::max<int64_t>(nnz, 1) * 4)) ||
+            (rc = dalloc(gcnt, (size_t)n * 4)) ||
             (rc = dalloc(glog, (size_t)glog_cap * sizeof(WGroup))) ||
-            (rc = dalloc(ring, (size_t)R * words * 4 + 16)) || (rc = dalloc(pend, (size_t)R * 8)) ||
-            (rc = dalloc(act, (size_t)n * 4)) || (rc = dalloc(cnt, 64)) ||
+            (rc = dalloc(ring, (size_t)R * words * 4 + 16)) || (rc = dalloc(pend, (size_t)R * 4)) ||
+            (rc = dalloc(act, (size_t)n * 8)) || (rc = dalloc(cnt, sizeof(WCtl))) ||
             (rc = dalloc(marks, (size_t)R * mwords * 4 + 16)))
             break;
         WArgs a;
@@ -519,75 +637,46 @@ int build_sketches_weighted(fl_graph* g, int k, uint64_t seed) {
         a.ecnt = ecnt.as<int32_t>();
         a.ecnt_n = ecnt_n.as<int32_t>();
         a.gcnt = gcnt.as<int32_t>();
-        a.cursor = cursor.as<int32_t>();
         a.glog = glog.as<WGroup>();
-        unsigned long long* c = cnt.as<unsigned long long>();  // [0] log size, [1] errors, [2] active
-        a.glog_n = c;
         a.glog_cap = glog_cap;
-        a.err = c + 1;
         a.ring = ring.as<uint32_t>();
         a.words = words;
         a.R = R;
-        a.pend = pend.as<unsigned long long>();
+        a.pend = pend.as<unsigned>();
+        a.act[0] = act.as<int32_t>();
+        a.act[1] = a.act[0] + n;
+        a.n = n;
+        a.c = cnt.as<WCtl>();
         a.rev = g->wrev.as<uint32_t>();
         a.marks = marks.as<uint32_t>();
         a.mwords = mwords;
         cudaError_t e = cudaMemsetAsync(ring.p, 0, (size_t)R * words * 4, st);
         if (e == cudaSuccess) e = cudaMemsetAsync(marks.p, 0, (size_t)R * mwords * 4, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(pend.p, 0, (size_t)R * 8, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(cnt.p, 0, 64, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(pend.p, 0, (size_t)R * 4, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(cnt.p, 0, sizeof(WCtl), st);
         if (e != cudaSuccess) { rc = status_of(e, "weighted build", __FILE__, __LINE__); break; }
-        const unsigned long long nlog0 = (unsigned long long)n;  // level 0 takes log slots 0..n-1
-        e = cudaMemcpyAsync(c, &nlog0, 8, cudaMemcpyHostToDevice, st);
-        if (e != cudaSuccess) { rc = status_of(e, "weighted build", __FILE__, __LINE__); break; }
-        FL_LAUNCH(kProfSketchMerge, k_winit<<<grid_for(n, 8), 256, 0, st>>>(a, n));
-        std::vector<unsigned long long> hp((size_t)R);
-        int64_t L = 0, last = 0, levels = 0;
-        unsigned long long logged = nlog0, now = 0;
-        for (;;) {
-            e = cudaMemcpyAsync(hp.data(), pend.p, (size_t)R * 8, cudaMemcpyDeviceToHost, st);
-            if (e == cudaSuccess) e = cudaMemcpyAsync(&now, c, 8, cudaMemcpyDeviceToHost, st);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-            if (e != cudaSuccess) { rc = status_of(e, "weighted build", __FILE__, __LINE__); break; }
-            if (now > logged) {  // the level just run added groups: the largest distance so far
-                last = L;
-                logged = now;
-            }
-            int64_t next = -1;  // the next level with activations
-            for (int d = 1; d <= R; ++d)
-                if (hp[(size_t)((L + d) % R)]) { next = L + d; break; }
-            if (next < 0) break;
-            L = next;
-            if (L > 65535) { rc = FL_EINVAL; set_error(rc, "a distance above 65535"); break; }
-            const int slot = (int)(L % R);
-            e = cudaMemsetAsync(&c[2], 0, 8, st);
-            if (e == cudaSuccess) e = cudaMemsetAsync(&a.pend[slot], 0, 8, st);
-            if (e != cudaSuccess) { rc = status_of(e, "weighted build", __FILE__, __LINE__); break; }
-            FL_LAUNCH(kProfSketchExpand, k_wcollect<<<grid_for(words * 32, 256), 256, 0, st>>>(
-                                             a.ring + (int64_t)slot * words, words, n, act.as<int32_t>(), &c[2]));
-            const int64_t n_act = (int64_t)hp[(size_t)slot];  // sizes the grids; the kernels read the list's count
-            FL_LAUNCH(kProfSketchMerge, k_wlevel<<<grid_for(n_act, 8), 256, 0, st>>>(a, act.as<int32_t>(), &c[2],
-                                                                                       (int32_t)L));
-            FL_LAUNCH(kProfSketchMerge, k_wcommit<<<grid_for(n_act, 256), 256, 0, st>>>(
-                                            act.as<int32_t>(), &c[2], a.ecnt_n, a.ecnt));
-            // the level's entry marks are read: the slot serves level L + R next
-            e = cudaMemsetAsync(a.marks + (int64_t)slot * mwords, 0, (size_t)mwords * 4, st);
-            if (e != cudaSuccess) { rc = status_of(e, "weighted build", __FILE__, __LINE__); break; }
-            ++levels;
+        int dev = 0, sms = 0;
+        e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess) {
+            const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(sms, (n + 31) / 32));
+            void* args[] = {&a};
+            FL_LAUNCH(kProfSketchMerge, e = cudaLaunchCooperativeKernel((const void*)k_wbuild, dim3(blocks),
+                                                                        dim3(kResThreads), args, 0, st));
         }
-        if (rc != FL_OK) break;
-        unsigned long long hc[2] = {0, 0};
-        e = cudaMemcpyAsync(hc, c, 16, cudaMemcpyDeviceToHost, st);
+        WCtl hc{};
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&hc, cnt.p, sizeof(WCtl), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) { rc = status_of(e, "weighted build", __FILE__, __LINE__); break; }
-        if (hc[1] & 2ULL) { rc = FL_EINVAL; set_error(rc, "a distance above 65535"); break; }
-        if ((hc[1] & 5ULL) && cap < n) {  // a row overflowed: twice the capacity
+        if (hc.bar.err) { rc = FL_ETIMEOUT; set_error(rc, "weighted build: a barrier wait ran out"); break; }
+        if (hc.err & 2ULL) { rc = FL_EINVAL; set_error(rc, "a distance above 65535"); break; }
+        if ((hc.err & 5ULL) && cap < n) {  // a row overflowed: twice the capacity
             cap = std::min<int64_t>(n, cap * 2);
             continue;
         }
-        if (hc[1]) { rc = FL_ECUDA; set_error(rc, "weighted build: inconsistent row capacity"); break; }
+        if (hc.err) { rc = FL_ECUDA; set_error(rc, "weighted build: inconsistent row capacity"); break; }
         // vertex-major ADS
-        const int64_t m = (int64_t)hc[0];
+        const int64_t m = (int64_t)hc.glog_n;
         if ((rc = dalloc(g->gofs, (size_t)(n + 1) * 8)) || (rc = dalloc(g->eofs, (size_t)(n + 1) * 8))) break;
         if ((rc = scan_exclusive_i32_to_i64(gcnt.as<int32_t>(), g->gofs.as<int64_t>(), n, st, g->scratch)) ||
             (rc = scan_exclusive_i32_to_i64(ecnt.as<int32_t>(), g->eofs.as<int64_t>(), n, st, g->scratch)))
@@ -621,12 +710,12 @@ int build_sketches_weighted(fl_graph* g, int k, uint64_t seed) {
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) { rc = status_of(e, "weighted build", __FILE__, __LINE__); break; }
-        g->hops = last;
+        g->hops = hc.last;
         g->edge_merges = 0;
-        g->wlevels = levels;
+        g->wlevels = hc.levels;
         break;
     }
-    dfree_after(st, {&ent, &ecnt, &ecnt_n, &gcnt, &cursor, &glog, &ring, &pend, &act, &cnt, &marks});
+    dfree_after(st, {&ent, &ecnt, &ecnt_n, &gcnt, &glog, &ring, &pend, &act, &cnt, &marks});
     return rc;
 }
 
