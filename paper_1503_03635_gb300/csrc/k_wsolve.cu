@@ -17,9 +17,13 @@
 // vertex u at time t reaches neighbour v at time t + w(u, v).  A ring of
 // R = (largest length + 1) slots holds the arrivals of the coming times: slot
 // t mod R keeps, per vertex, the smallest value arriving at time t, and the
-// list of vertices that have one.  Step t drains its slot into the labels
-// (a vertex whose label drops joins the step's frontier) and the frontier
-// pushes its labels along its edges into later slots.
+// list of vertices that have one.  Step t drains its slot into the labels and
+// a vertex whose label drops pushes it along its edges into later slots.
+// A sweep is one resident kernel with one grid barrier per time that has
+// arrivals; times without are passed over.  With three launches per time step
+// a sweep was bound by them and by the largest hub, pushed by one warp: the 24
+// sweeps (2819 times) of an R-MAT graph with 65 k vertices and lengths up to
+// 100 took 45 ms, 13.9 ms now; bound by the barriers and dependent loads.
 //   cover:  facility f enters at time H - B_f with its key ordinal (H = the
 //           largest B_f), so every wave ends at H and the label of v at H is
 //           the smallest key whose ball holds v;
@@ -44,8 +48,6 @@ namespace fl {
 namespace {
 
 constexpr uint32_t kNone = 0xffffffffu;
-constexpr int kChunk = 16;  // time steps between two looks at the ring's counts
-
 int grid_for(int64_t items, int per_block, int cap = 152 * 4) {
     int64_t b = (items + per_block - 1) / per_block;
     if (b < 1) b = 1;
@@ -61,10 +63,7 @@ struct WSweep {
     int R;
     uint32_t* pend;             // R*n: smallest value arriving at each vertex at the slot's time (kNone: none)
     int32_t* plist;             // R*n: vertices with an arrival, per slot
-    unsigned long long* pcnt;   // R
-    int32_t* fr[2];             // frontier of the even / odd steps (2n each)
-    unsigned long long* fcnt;   // 2
-    unsigned long long* err;    // bit 1: a decision saw an impossible value
+    unsigned long long* pcnt;   // 2R: list lengths, of time t at t mod 2R
     uint32_t* lab;              // current label (kNone: none)
     const int32_t* dl;          // deadline: the label at this time is kept in dlab (or NULL)
     uint32_t* dlab;             // smallest arrival up to the deadline
@@ -77,8 +76,8 @@ struct WSweep {
 
 // One arrival of x at v at time t; true when v joins the step's frontier.
 __device__ __forceinline__ bool arrive(const WSweep& a, int32_t v, uint32_t x, int64_t t) {
-    if (a.dl && t <= (int64_t)a.dl[v] && x < a.dlab[v]) a.dlab[v] = x;
-    const uint32_t old = a.lab[v];
+    if (a.dl && t <= (int64_t)__ldg(&a.dl[v]) && x < __ldcg(&a.dlab[v])) a.dlab[v] = x;
+    const uint32_t old = __ldcg(&a.lab[v]);
     if (a.first) {
         if (old != kNone) return false;
         a.dist[v] = (int32_t)t;
@@ -108,127 +107,188 @@ __device__ int64_t warp_lower_bound(const int32_t* __restrict__ bs, int64_t m, i
     return lo;
 }
 
-// Appends the lanes' vertices with `want` to list (all 32 lanes call it).
-__device__ __forceinline__ void warp_append(bool want, int32_t v, int32_t* list, unsigned long long* cnt) {
-    const unsigned mask = __ballot_sync(kFull, want);
-    if (!mask) return;
-    const int leader = __ffs(mask) - 1;
-    unsigned long long base = 0;
-    if (lane_id() == leader) base = atomicAdd(cnt, (unsigned long long)__popc(mask));
-    base = __shfl_sync(kFull, base, leader);
-    if (want) list[base + __popc(mask & ((1u << lane_id()) - 1u))] = v;
+// Control block of a sweep (device, zero at its start).
+struct WSweepCtl {
+    GridBar bar;
+    long long t_end, steps;  // last time that had arrivals, times run
+};
+
+// The cover's entering facilities (m = 0 for sweeps whose sources all enter
+// at time 0): candidates in key order have non-decreasing B_f (bsort[i] = B of
+// the i-th), a candidate's value is its ordinal.  Or the sources of time 0:
+// every vertex with mask[v] (all when NULL) enters with val[v] (its id when
+// val is NULL), unless that is kNone.
+struct WEntry {
+    const int32_t* fac_by_ord;
+    const int32_t* bsort;
+    const uint8_t* state;
+    int64_t m;
+    bool seeds;
+    const uint32_t* val;
+    const uint8_t* mask;
+};
+
+constexpr int kPLong = 512;   // longer rows are pushed by the whole block
+constexpr int kPQueue = 128;  // of them, queued per block and step
+
+// x arrives at v at time t: into the ring.
+__device__ __forceinline__ void send(const WSweep& a, int32_t v, uint32_t x, uint32_t t) {
+    const int64_t slot = (int64_t)(t % (uint32_t)a.R) * a.n;
+    if (atomicMin(&a.pend[slot + v], x) == kNone)
+        a.plist[slot + (int64_t)atomicAdd(&a.pcnt[t % (2u * (uint32_t)a.R)], 1ULL)] = v;
 }
 
-// Step t, part 1: the arrivals of slot t mod R.
-__global__ void k_wdrain(WSweep a, int64_t t) {
-    const int s = (int)(t % a.R);
-    const int p = (int)(t & 1);
-    if (blockIdx.x == 0 && threadIdx.x == 0) a.fcnt[p ^ 1] = 0;  // the next step's frontier
-    const int64_t cnt = (int64_t)a.pcnt[s];
-    uint32_t* pend = a.pend + (int64_t)s * a.n;
-    const int32_t* list = a.plist + (int64_t)s * a.n;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < cnt; base += stride) {
-        const int64_t i = base + lane_id();
-        bool join = false;
-        int32_t v = 0;
-        if (i < cnt) {
-            v = list[i];
-            const uint32_t x = pend[v];
-            pend[v] = kNone;
-            join = arrive(a, v, x, t);
+// v's label x goes out along the entries e0 + first, + step, ... of its row.
+// An arrival that cannot lower u's label is not sent: u's label already holds
+// a value at most x from an arrival at or before t, and that arrival was also
+// kept by u's deadline whenever this one would be.  (A label that drops in
+// this same step does so by an arrival at t.)
+__device__ __forceinline__ void push_row(const WSweep& a, int64_t e0, int64_t e1, int first, int step, uint32_t x,
+                                         int64_t t, int64_t H) {
+    for (int64_t e = e0 + first + lane_id(); e < e1; e += step) {
+        const int32_t u = __ldg(&a.cols[e]);
+        const uint32_t lu = __ldcg(&a.lab[u]);
+        if (a.first ? lu != kNone : lu <= x) continue;
+        const int64_t t2 = t + __ldg(&a.wts[e]);
+        if (a.fts) {  // u relays nothing useful after its slack H - (first cover arrival)
+            const int32_t fu = __ldg(&a.fts[u]);
+            if (fu < 0 || t2 > H - (int64_t)fu) continue;
         }
-        warp_append(join, v, a.fr[p], &a.fcnt[p]);
-    }
-}
-
-// Step t, part 2 (cover): the undecided facilities with B_f = H - t enter.
-// Candidates in key order have non-decreasing B_f (bsort[i] = B of the i-th),
-// so they are one range of fac_by_ord, found by search; a candidate's value
-// is its ordinal.
-__global__ void k_winject(WSweep a, const int32_t* __restrict__ fac_by_ord, const int32_t* __restrict__ bsort,
-                          const uint8_t* __restrict__ state, int64_t m, int64_t H, int64_t t) {
-    __shared__ int64_t range[2];
-    if (threadIdx.x < 64) {  // warp 0: first B >= H - t; warp 1: first B > H - t
-        const int64_t at = warp_lower_bound(bsort, m, H - t + (int64_t)(threadIdx.x >> 5));
-        if (lane_id() == 0) range[threadIdx.x >> 5] = at;
-    }
-    __syncthreads();
-    const int p = (int)(t & 1);
-    const int64_t end = range[1];
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = range[0] + (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < end;
-         base += stride) {
-        const int64_t i = base + lane_id();
-        bool join = false;
-        int32_t f = 0;
-        if (i < end) {
-            f = fac_by_ord[i];
-            if (state[f] == 0) join = arrive(a, f, (uint32_t)i, t);
+        if (t2 > H) {
+            if (a.first) a.past[u] = 1;
+            continue;
         }
-        warp_append(join, f, a.fr[p], &a.fcnt[p]);
+        send(a, u, x, (uint32_t)t2);
     }
 }
 
-// Time 0 of a sweep: every vertex with mask[v] (all when NULL) enters with
-// val[v] (its id when val is NULL), unless that is kNone.
-__global__ void k_wseed(WSweep a, const uint32_t* __restrict__ val, const uint8_t* __restrict__ mask) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < a.n; base += stride) {
-        const int64_t v = base + lane_id();
-        bool join = false;
-        if (v < a.n && (!mask || mask[v])) {
-            const uint32_t x = val ? val[v] : (uint32_t)v;
-            if (x != kNone) join = arrive(a, (int32_t)v, x, 0);
-        }
-        warp_append(join, (int32_t)v, a.fr[0], &a.fcnt[0]);
-    }
-}
-
-// Step t, part 3: the frontier's labels go out along its edges (a warp per
-// frontier vertex).  An arrival that cannot lower v's label is not sent: v's
-// label already holds a value at most x from an arrival at or before t, and
-// that arrival was also kept by v's deadline whenever this one would be.
-__global__ void __launch_bounds__(256) k_wpush(WSweep a, int64_t t, int64_t H) {
-    const int s = (int)(t % a.R);
-    if (blockIdx.x == 0 && threadIdx.x == 0) a.pcnt[s] = 0;  // drained; no push of this step targets it
-    const int p = (int)(t & 1);
-    const int64_t cnt = (int64_t)a.fcnt[p];
+// One sweep over times 0..H.
+//
+// A facility that enters at time te is sent to itself as an arrival of te as
+// soon as te is less than R away.  The list length of time t is read by every
+// block in step t and cleared in the next one, t': t' <= t + R - 1, so no
+// send of step t' (to times up to t' + R - 1) uses the same of the 2R counters.
+__global__ void __launch_bounds__(kResThreads, 1) k_wsweep(WSweep a, WEntry in, int64_t H, WSweepCtl* c) {
+    __shared__ int32_t s_v[kPQueue];
+    __shared__ uint32_t s_x[kPQueue];
+    __shared__ unsigned s_queued, s_next;
+    __shared__ long long s_first;
     const int lane = lane_id();
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < cnt; i += warps) {
-        const int32_t u = a.fr[p][i];
-        const uint32_t x = a.lab[u];
-        const int64_t e1 = a.rowp[u + 1];
-        for (int64_t e = a.rowp[u] + lane; e < e1; e += 32) {
-            const int32_t v = a.cols[e];
-            const uint32_t lv = a.lab[v];
-            if (a.first ? lv != kNone : lv <= x) continue;
-            const int64_t t2 = t + a.wts[e];
-            if (a.fts) {  // v relays nothing useful after its slack H - (first cover arrival)
-                const int32_t fv = a.fts[v];
-                if (fv < 0 || t2 > H - (int64_t)fv) continue;
+    const int64_t tid = (int64_t)blockIdx.x * kResThreads + threadIdx.x, threads = (int64_t)gridDim.x * kResThreads;
+    // chunk i to warp i / gridDim of block i mod gridDim: neighbours in a list go to different blocks
+    const int64_t item0 = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x, warps = threads >> 5;
+    unsigned pass = 0, total = 0;
+    if (threadIdx.x == 0) s_queued = 0;
+
+    // the facilities with entry times below t + R that have not entered:
+    // candidates [first, left); left = first
+    int64_t left = in.m;
+    auto enter = [&](int64_t t) {
+        if (left == 0) return;
+        if (threadIdx.x < 32) {
+            const int64_t at = warp_lower_bound(in.bsort, left, H - t - a.R + 1);
+            if (lane == 0) s_first = at;
+        }
+        __syncthreads();
+        const int64_t first = s_first;
+        __syncthreads();
+        for (int64_t i = first + tid; i < left; i += threads) {
+            const int32_t f = __ldg(&in.fac_by_ord[i]);
+            if (__ldg(&in.state[f]) == 0) send(a, f, (uint32_t)i, (uint32_t)(H - (int64_t)__ldg(&in.bsort[i])));
+        }
+        left = first;
+    };
+    // the first time from t + from on, below t + R, that has arrivals (-1: none)
+    auto next_time = [&](int64_t t, int from) -> int64_t {
+        if (threadIdx.x == 0) s_next = ~0u;
+        __syncthreads();
+        for (int d = from + (int)threadIdx.x; d < a.R; d += kResThreads)
+            if (__ldcg(&a.pcnt[(uint32_t)(t + d) % (2u * (uint32_t)a.R)])) {
+                atomicMin(&s_next, (unsigned)d);
+                break;
             }
-            if (t2 > H) {
-                if (a.first) a.past[v] = 1;
-                continue;
+        __syncthreads();
+        const unsigned d = s_next;
+        __syncthreads();
+        return d == ~0u ? -1 : t + (int64_t)d;
+    };
+
+    if (in.seeds)
+        for (int64_t v = tid; v < a.n; v += threads)
+            if (!in.mask || in.mask[v]) {
+                const uint32_t x = in.val ? in.val[v] : (uint32_t)v;
+                if (x != kNone) send(a, (int32_t)v, x, 0u);
             }
-            const int64_t s2 = t2 % a.R;
-            const uint32_t old = atomicMin(&a.pend[s2 * a.n + v], x);
-            if (old == kNone) {
-                const unsigned long long at = atomicAdd(&a.pcnt[s2], 1ULL);
-                a.plist[s2 * a.n + (int64_t)at] = v;
+    enter(0);
+    if (!end_pass(&c->bar, pass, 0, &total)) return;
+    int64_t t = next_time(0, 0), prev = -1, steps = 0;
+    for (;;) {
+        if (t < 0) {  // nothing in flight: the next entry, or the end
+            if (left == 0) break;
+            const int64_t te = H - (int64_t)__ldg(&in.bsort[left - 1]);
+            if (tid == 0 && prev >= 0) a.pcnt[(uint32_t)prev % (2u * (uint32_t)a.R)] = 0;
+            prev = -1;
+            if (!end_pass(&c->bar, pass, 0, &total)) return;
+            enter(te);
+            if (!end_pass(&c->bar, pass, 0, &total)) return;
+            t = next_time(te, 0);
+            continue;
+        }
+        const int64_t slot = (int64_t)((uint32_t)t % (uint32_t)a.R) * a.n;
+        const int64_t cnt = (int64_t)__ldcg(&a.pcnt[(uint32_t)t % (2u * (uint32_t)a.R)]);
+        if (tid == 0 && prev >= 0) a.pcnt[(uint32_t)prev % (2u * (uint32_t)a.R)] = 0;
+        // chunks of a few arrivals per warp, one lane each to drain them
+        const int64_t per = min((int64_t)32, (cnt + warps - 1) / warps);
+        for (int64_t i0 = item0 * per; i0 < cnt; i0 += warps * per) {
+            const int64_t i = i0 + lane;
+            bool join = false;
+            int32_t v = 0;
+            uint32_t x = kNone;
+            if (lane < per && i < cnt) {
+                v = __ldcg(&a.plist[slot + i]);
+                x = __ldcg(&a.pend[slot + v]);
+                a.pend[slot + v] = kNone;
+                join = arrive(a, v, x, t);
+            }
+            for (unsigned m = __ballot_sync(kFull, join); m; m &= m - 1) {
+                const int l = __ffs(m) - 1;
+                const int32_t u = __shfl_sync(kFull, v, l);
+                const uint32_t y = __shfl_sync(kFull, x, l);
+                const int64_t e0 = __ldg(&a.rowp[u]), e1 = __ldg(&a.rowp[u + 1]);
+                if (e1 - e0 > kPLong) {
+                    unsigned at = 0;
+                    if (lane == 0) at = atomicAdd(&s_queued, 1u);
+                    at = __shfl_sync(kFull, at, 0);
+                    if (at < kPQueue) {
+                        if (lane == 0) {
+                            s_v[at] = u;
+                            s_x[at] = y;
+                        }
+                        continue;
+                    }
+                }
+                push_row(a, e0, e1, 0, 32, y, t, H);
             }
         }
+        __syncthreads();
+        const int queued = (int)min(s_queued, (unsigned)kPQueue);
+        for (int q = 0; q < queued; ++q) {
+            const int32_t u = s_v[q];
+            push_row(a, __ldg(&a.rowp[u]), __ldg(&a.rowp[u + 1]), (int)(threadIdx.x & ~31u), kResThreads, s_x[q], t, H);
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) s_queued = 0;
+        enter(t);
+        ++steps;
+        if (!end_pass(&c->bar, pass, 0, &total)) return;
+        prev = t;
+        t = next_time(t, 1);
     }
-}
-
-// The earliest time >= t at which a candidate enters the cover (H - B_f for
-// the largest B_f <= H - t, decided or not), or ~0 when none does (one warp).
-__global__ void k_wnext(const int32_t* __restrict__ bsort, int64_t m, int64_t H, int64_t t,
-                        unsigned long long* __restrict__ out) {
-    const int64_t lo = warp_lower_bound(bsort, m, H - t + 1);
-    if (lane_id() == 0) *out = lo == 0 ? ~0ULL : (unsigned long long)(H - (int64_t)bsort[lo - 1]);
+    if (tid == 0) {
+        if (prev >= 0) a.pcnt[(uint32_t)prev % (2u * (uint32_t)a.R)] = 0;
+        c->t_end = prev < 0 ? 0 : prev;
+        c->steps = steps;
+    }
 }
 
 // Ordinals and ball radii of the sorted candidates: ord[f] = position in key
@@ -354,24 +414,23 @@ __global__ void k_wbeyond(int64_t n, const uint8_t* __restrict__ past, const uin
         if (past[v] && lab[v] == kNone) atomicOr(err, 2ULL);
 }
 
-// Device state of the sweeps of one call: the ring, the frontiers, counters.
+// Device state of the sweeps of one call: the ring and counters.
 struct WRing {
-    DBuf pend, plist, fr, cnt;
+    DBuf pend, plist, cnt, ctl;
     int R = 0;
     int64_t n = 0;
-    unsigned long long* c = nullptr;  // [0, R): slot counts; R, R+1: frontier counts; R+2: errors;
-                                      // R+3: next entry time; R+4..R+6: undecided count, max B, min B;
-                                      // R+7: joined; R+8: claimed; R+9: open
+    unsigned long long* c = nullptr;  // [0, 2R): list lengths; then kErr ... kOpen
+    enum { kErr = 0, kUndecided = 1, kMaxB = 2, kMinB = 3, kJoined = 4, kClaimed = 5, kOpen = 6, kWords = 8 };
     int alloc(fl_graph* g) {
         R = g->max_w + 1;
         n = g->n;
         FL_TRY(dalloc(pend, (size_t)R * n * 4));
         FL_TRY(dalloc(plist, (size_t)R * n * 4));
-        FL_TRY(dalloc(fr, (size_t)n * 16));
-        FL_TRY(dalloc(cnt, (size_t)(R + 16) * 8));
-        c = cnt.as<unsigned long long>();
+        FL_TRY(dalloc(cnt, (size_t)(2 * R + kWords) * 8));
+        FL_TRY(dalloc(ctl, sizeof(WSweepCtl)));
+        c = cnt.as<unsigned long long>() + 2 * R;
         FL_CUDA(cudaMemsetAsync(pend.p, 0xff, (size_t)R * n * 4, g->stream));
-        FL_CUDA(cudaMemsetAsync(cnt.p, 0, (size_t)(R + 16) * 8, g->stream));
+        FL_CUDA(cudaMemsetAsync(cnt.p, 0, (size_t)(2 * R + kWords) * 8, g->stream));
         return FL_OK;
     }
     WSweep sweep(const fl_graph* g) const {
@@ -383,11 +442,7 @@ struct WRing {
         a.R = R;
         a.pend = pend.as<uint32_t>();
         a.plist = plist.as<int32_t>();
-        a.pcnt = c;
-        a.fr[0] = fr.as<int32_t>();
-        a.fr[1] = fr.as<int32_t>() + 2 * n;
-        a.fcnt = c + R;
-        a.err = c + R + 2;
+        a.pcnt = cnt.as<unsigned long long>();
         a.lab = nullptr;
         a.dl = nullptr;
         a.dlab = nullptr;
@@ -398,67 +453,30 @@ struct WRing {
         a.first = 0;
         return a;
     }
-    // Before a sweep's sources enter: both frontiers empty (the slots are
-    // empty after every sweep).
-    int begin(cudaStream_t st) const {
-        cudaError_t e = cudaMemsetAsync(c + R, 0, 16, st);
-        return e == cudaSuccess ? FL_OK : status_of(e, "weighted sweep", __FILE__, __LINE__);
-    }
-    void release(cudaStream_t st) { dfree_after(st, {&pend, &plist, &fr, &cnt}); }
+    void release(cudaStream_t st) { dfree_after(st, {&pend, &plist, &cnt, &ctl}); }
 };
 
-// The cover's entering facilities (NULL for sweeps whose sources all enter
-// at time 0 through k_wseed).
-struct Entry {
-    const int32_t* fac_by_ord;
-    const int32_t* bsort;
-    const uint8_t* state;
-    int64_t m;
-    int64_t t_last;  // no facility enters after this time
-};
-
-// Runs steps 0..H of a sweep whose time-0 sources have entered.  Between
-// chunks of steps the host reads the ring's counts: when nothing is pending
-// it jumps to the next entry time, or stops.  *t_end = the last step run,
-// *steps = the steps run.
-int run_sweep(fl_graph* g, WRing& ring, const WSweep& a, int64_t H, const Entry* entry, int cls, int64_t* t_end,
-              int64_t* steps) {
+// Runs one sweep (the ring is empty before and after).  *t_end = the last
+// time that had arrivals, *steps = the times run.
+int run_sweep(fl_graph* g, WRing& ring, WSweep a, int64_t H, WEntry in, int cls, int64_t* t_end, int64_t* steps) {
     cudaStream_t st = g->stream;
-    const int R = ring.R;
-    const int gd = grid_for(a.n, 256);
-    const int gp = grid_for(a.n * 32, 256);
-    const int gi = entry ? grid_for(entry->m, 256, 152) : 1;
-    std::vector<unsigned long long> hc((size_t)R + 4);
-    int64_t t = 0, ran = 0, last = 0;
-    for (;;) {
-        for (int j = 0; j < kChunk && t <= H; ++j, ++t) {
-            FL_LAUNCH(cls, k_wdrain<<<gd, 256, 0, st>>>(a, t));
-            if (entry && t <= entry->t_last)
-                FL_LAUNCH(cls, k_winject<<<gi, 256, 0, st>>>(a, entry->fac_by_ord, entry->bsort, entry->state,
-                                                              entry->m, H, t));
-            FL_LAUNCH(cls, k_wpush<<<gp, 256, 0, st>>>(a, t, H));
-            last = t;
-            ++ran;
-        }
-        FL_CUDA(cudaGetLastError());
-        if (t > H) break;
-        if (entry && t <= entry->t_last)
-            FL_LAUNCH(cls, k_wnext<<<1, 32, 0, st>>>(entry->bsort, entry->m, H, t, ring.c + R + 3));
-        FL_CUDA(cudaMemcpyAsync(hc.data(), ring.c, (size_t)(R + 4) * 8, cudaMemcpyDeviceToHost, st));
-        FL_CUDA(cudaStreamSynchronize(st));
-        unsigned long long pending = 0;
-        for (int s2 = 0; s2 < R; ++s2) pending += hc[(size_t)s2];
-        if (pending) continue;
-        // nothing in flight: the next entry, or the end
-        if (!entry || t > entry->t_last || hc[(size_t)R + 3] == ~0ULL) break;
-        const int64_t next = (int64_t)hc[(size_t)R + 3];
-        if (next > t) {
-            FL_CUDA(cudaMemsetAsync(ring.c + R, 0, 16, st));  // both frontiers are empty
-            t = next;
-        }
-    }
-    *t_end = last;
-    *steps = ran;
+    int dev = 0, sms = 0;
+    FL_CUDA(cudaGetDevice(&dev));
+    FL_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(sms, (a.n + 31) / 32));
+    WSweepCtl* c = ring.ctl.as<WSweepCtl>();
+    FL_CUDA(cudaMemsetAsync(c, 0, sizeof(WSweepCtl), st));
+    void* args[] = {&a, &in, &H, &c};
+    cudaError_t le = cudaSuccess;
+    FL_LAUNCH(cls, le = cudaLaunchCooperativeKernel((const void*)k_wsweep, dim3(blocks), dim3(kResThreads), args, 0,
+                                                    st));
+    FL_CUDA(le);
+    WSweepCtl h{};
+    FL_CUDA(cudaMemcpyAsync(&h, c, sizeof(WSweepCtl), cudaMemcpyDeviceToHost, st));
+    FL_CUDA(cudaStreamSynchronize(st));
+    if (h.bar.err) FL_FAIL(FL_ETIMEOUT, "weighted sweep: a barrier wait ran out");
+    *t_end = h.t_end;
+    *steps = h.steps;
     return FL_OK;
 }
 
@@ -498,27 +516,26 @@ int open_facilities_weighted(fl_solve* s) {
     FL_CUDA(cudaGetLastError());
     WRing ring;
     int rc = ring.alloc(g);
-    const int R = ring.R;
     unsigned long long* c = ring.c;
     int64_t rounds = 0;
     while (rc == FL_OK) {
         const auto round_t0 = clock::now();
-        unsigned long long h[6] = {0, 0, 0, 0, 0, 0};
-        cudaError_t e = cudaMemsetAsync(c + R + 4, 0, 16, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(c + R + 6, 0xff, 8, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(c + R + 7, 0, 16, st);
+        unsigned long long h[4] = {0, 0, 0, 0};
+        cudaError_t e = cudaMemsetAsync(c + WRing::kUndecided, 0, 16, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(c + WRing::kMinB, 0xff, 8, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(c + WRing::kJoined, 0, 16, st);
         if (e != cudaSuccess) { rc = status_of(e, "weighted MIS", __FILE__, __LINE__); break; }
         if (m > 0)
-            FL_LAUNCH(kProfMis, k_wundecided<<<grid_for(m, 256), 256, 0, st>>>(fac_by_ord, bcap, state, m, c + R + 4));
-        e = cudaMemcpyAsync(h, c + R + 2, 48, cudaMemcpyDeviceToHost, st);
+            FL_LAUNCH(kProfMis, k_wundecided<<<grid_for(m, 256), 256, 0, st>>>(fac_by_ord, bcap, state, m,
+                                                                               c + WRing::kUndecided));
+        e = cudaMemcpyAsync(h, c, 32, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) { rc = status_of(e, "weighted MIS", __FILE__, __LINE__); break; }
         if (h[0]) { rc = FL_ECUDA; set_error(rc, "weighted MIS: a ball's smallest label is above its own key"); break; }
-        const int64_t nu = (int64_t)h[2];
+        const int64_t nu = (int64_t)h[WRing::kUndecided];
         if (nu == 0) break;
         if (++rounds > m + 1) { rc = FL_ETIMEOUT; set_error(rc, "weighted MIS did not converge"); break; }
-        const int64_t H = (int64_t)h[3];
-        Entry entry{fac_by_ord, bsort, state, m, H - (int64_t)h[4]};
+        const int64_t H = (int64_t)h[WRing::kMaxB];
         auto timed = [&](int kind, int64_t t_end, int64_t steps, clock::time_point t0) {
             const double us = std::chrono::duration<double, std::micro>(clock::now() - t0).count();
             s->mis_log.insert(s->mis_log.end(), {rounds, (int64_t)kind, t_end, steps, 0, (int64_t)us});
@@ -532,7 +549,10 @@ int open_facilities_weighted(fl_solve* s) {
         e = cudaMemsetAsync(cover, 0xff, (size_t)n * 4, st);
         if (e == cudaSuccess) e = cudaMemsetAsync(ft, 0xff, (size_t)n * 4, st);
         if (e != cudaSuccess) { rc = status_of(e, "weighted MIS", __FILE__, __LINE__); break; }
-        if ((rc = ring.begin(st)) || (rc = run_sweep(g, ring, a, H, &entry, kProfMis, &t_end, &steps))) break;
+        // candidates of a larger B_f than any undecided one have been decided
+        if ((rc = run_sweep(g, ring, a, H, WEntry{fac_by_ord, bsort, state, m, false, nullptr, nullptr}, kProfMis,
+                            &t_end, &steps)))
+            break;
         timed(0, t_end, steps, t0);
         // gather
         t0 = clock::now();
@@ -543,17 +563,17 @@ int open_facilities_weighted(fl_solve* s) {
         a.fts = ft;
         e = cudaMemsetAsync(lab, 0xff, (size_t)n * 8, st);  // lab and dlab
         if (e != cudaSuccess) { rc = status_of(e, "weighted MIS", __FILE__, __LINE__); break; }
-        if ((rc = ring.begin(st))) break;
-        FL_LAUNCH(kProfMis, k_wseed<<<grid_for(n, 256), 256, 0, st>>>(a, cover, s->client.as<uint8_t>()));
-        if ((rc = run_sweep(g, ring, a, H, nullptr, kProfMis, &t_end, &steps))) break;
+        if ((rc = run_sweep(g, ring, a, H, WEntry{nullptr, nullptr, nullptr, 0, true, cover, s->client.as<uint8_t>()},
+                            kProfMis, &t_end, &steps)))
+            break;
         timed(1, t_end, steps, t0);
         if (m > 0)
-            FL_LAUNCH(kProfMis, k_wdecide<<<grid_for(m, 256), 256, 0, st>>>(fac_by_ord, m, dlab, state, c + R + 7,
-                                                                            c + R + 2));
+            FL_LAUNCH(kProfMis, k_wdecide<<<grid_for(m, 256), 256, 0, st>>>(fac_by_ord, m, dlab, state,
+                                                                            c + WRing::kJoined, c));
         FL_LAUNCH(kProfMis, k_wclaim<<<grid_for(n, 256), 256, 0, st>>>(n, s->client.as<uint8_t>(), cover, fac_by_ord,
                                                                        state, s->claimed.as<uint8_t>(),
-                                                                       s->kill.as<uint8_t>(), c + R + 8));
-        e = cudaMemcpyAsync(h, c + R + 7, 16, cudaMemcpyDeviceToHost, st);
+                                                                       s->kill.as<uint8_t>(), c + WRing::kClaimed));
+        e = cudaMemcpyAsync(h, c + WRing::kJoined, 16, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) { rc = status_of(e, "weighted MIS", __FILE__, __LINE__); break; }
         const int64_t joined = (int64_t)h[0], claimed = (int64_t)h[1];
@@ -563,9 +583,10 @@ int open_facilities_weighted(fl_solve* s) {
             t0 = clock::now();
             e = cudaMemsetAsync(lab, 0xff, (size_t)n * 8, st);
             if (e != cudaSuccess) { rc = status_of(e, "weighted MIS", __FILE__, __LINE__); break; }
-            if ((rc = ring.begin(st))) break;
-            FL_LAUNCH(kProfMis, k_wseed<<<grid_for(n, 256), 256, 0, st>>>(a, nullptr, s->kill.as<uint8_t>()));
-            if ((rc = run_sweep(g, ring, a, H, nullptr, kProfMis, &t_end, &steps))) break;
+            if ((rc = run_sweep(g, ring, a, H,
+                                WEntry{nullptr, nullptr, nullptr, 0, true, nullptr, s->kill.as<uint8_t>()}, kProfMis,
+                                &t_end, &steps)))
+                break;
             timed(4, t_end, steps, t0);
             FL_LAUNCH(kProfMis, k_wkill<<<grid_for(m, 256), 256, 0, st>>>(fac_by_ord, m, dlab, state));
         }
@@ -575,12 +596,12 @@ int open_facilities_weighted(fl_solve* s) {
     }
     if (rc == FL_OK) {
         unsigned long long no = 0;
-        cudaError_t e = cudaMemsetAsync(c + R + 9, 0, 8, st);
+        cudaError_t e = cudaMemsetAsync(c + WRing::kOpen, 0, 8, st);
         if (e == cudaSuccess) {
-            FL_LAUNCH(kProfMis, k_wopen<<<grid_for(n, 256), 256, 0, st>>>(state, n, s->open.as<uint8_t>(), c + R + 9));
+            FL_LAUNCH(kProfMis, k_wopen<<<grid_for(n, 256), 256, 0, st>>>(state, n, s->open.as<uint8_t>(), c + WRing::kOpen));
             e = cudaGetLastError();
         }
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&no, c + R + 9, 8, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&no, c + WRing::kOpen, 8, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) rc = status_of(e, "weighted MIS", __FILE__, __LINE__);
         s->n_open = (int64_t)no;
@@ -609,16 +630,14 @@ int assign_weighted(fl_solve* s) {
         a.past = s->kill.as<uint8_t>();
         a.first = 1;
         int64_t t_end = 0, steps = 0;
-        rc = ring.begin(st);
-        if (rc == FL_OK) {
-            FL_LAUNCH(kProfBfs, k_wseed<<<grid_for(n, 256), 256, 0, st>>>(a, nullptr, s->open.as<uint8_t>()));
-            rc = run_sweep(g, ring, a, 2147483647LL, nullptr, kProfBfs, &t_end, &steps);
-        }
+        rc = run_sweep(g, ring, a, 2147483647LL,
+                       WEntry{nullptr, nullptr, nullptr, 0, true, nullptr, s->open.as<uint8_t>()}, kProfBfs, &t_end,
+                       &steps);
         unsigned long long err = 0;
         if (rc == FL_OK) {
             FL_LAUNCH(kProfBfs, k_wbeyond<<<grid_for(n, 256), 256, 0, st>>>(n, s->kill.as<uint8_t>(), a.lab,
-                                                                           ring.c + ring.R + 2));
-            cudaError_t e = cudaMemcpyAsync(&err, ring.c + ring.R + 2, 8, cudaMemcpyDeviceToHost, st);
+                                                                           ring.c));
+            cudaError_t e = cudaMemcpyAsync(&err, ring.c, 8, cudaMemcpyDeviceToHost, st);
             if (e == cudaSuccess) e = cudaStreamSynchronize(st);
             if (e != cudaSuccess) rc = status_of(e, "weighted assignment", __FILE__, __LINE__);
         }
