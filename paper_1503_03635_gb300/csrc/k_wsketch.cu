@@ -21,7 +21,7 @@
 // enter v's sketch at level L either.  (Most are already there: every
 // neighbour of v that holds a rank would offer it again.)  An active v merges
 // into its bottom-k sketch the entries of each posting neighbour u at distance
-// L - w(u, v), found by bisection in u's row, which is in distance order; the
+// L - w(u, v), found by an 8-way search in u's row, which is in distance order; the
 // ranks that enter form v's group at distance L, with the HIP weight and
 // counted prefix of the unweighted build (the sketch after the level, ties at
 // one distance in ascending rank).  Entries appended at level L have distance
@@ -35,7 +35,8 @@
 // entries are posted by the whole block, so that no level waits for one warp
 // on a hub.  Bound by the latency of the dependent loads of a post (column,
 // k-th rank, sketch).  R-MAT, 65 k vertices, lengths up to 100, k = 16, 313
-// levels: 115 ms of level kernels and some 15 ms of gaps before, 36 ms now.
+// levels: 115 ms of level kernels and some 15 ms of gaps before, 29 ms now (36
+// with bisections in place of the 8-way search and the 8-wide sketch test).
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -112,18 +113,50 @@ __device__ __forceinline__ WEnt load_ent(const WEnt* p) {
     return WEnt{x.x, x.y};
 }
 
-// Is rank x in the ascending sketch row of k ranks (kEmpty padded)?  The row
-// may be rewritten meanwhile: every value read is of the old or the new sketch.
-__device__ __forceinline__ bool in_sketch(const uint64_t* row, int k, uint64_t x) {
-    int lo = 0, hi = k;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        const uint64_t y = __ldcg(&row[mid]);
-        if (y == x) return true;
-        if (y < x) lo = mid + 1;
-        else hi = mid;
+// Which of the gained ranks (lane j < dcnt of the warp: the j-th) are in the
+// sketch row of k ranks, as a mask per lane (all 32 lanes call; a lane without
+// a row passes NULL), and the row's k-th rank.  Eight ranks are loaded at a
+// time, so that a row costs one or two L2 latencies instead of the five of a
+// bisection.  The row may be rewritten meanwhile: every value read is of the
+// old or the new sketch.
+__device__ __forceinline__ unsigned held_ranks(const uint64_t* row, int k, uint64_t gained, int dcnt, uint64_t* kth) {
+    unsigned held = 0;
+    uint64_t last = kEmpty;
+    for (int c = 0; c < k; c += 8) {
+        uint64_t y[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) y[q] = row && c + q < k ? __ldcg(&row[c + q]) : kEmpty;
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            if (c + q == k - 1) last = y[q];
+        for (int j = 0; j < dcnt; ++j) {
+            const uint64_t x = __shfl_sync(kFull, gained, j);
+            bool hit = false;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) hit |= y[q] == x;
+            if (hit) held |= 1u << j;
+        }
     }
-    return false;
+    *kth = last;
+    return held;
+}
+
+// First entry of the row's `have` entries (in distance order) at distance x or
+// more: eight parts per round, their bounds loaded together.
+__device__ __forceinline__ int first_at(const WEnt* row, int have, int32_t x) {
+    int lo = 0, hi = have;
+    while (lo < hi) {
+        const int part = (hi - lo + 7) >> 3;
+        int below = 0;  // probes lo + part - 1, lo + 2 part - 1, ... below x (a prefix)
+#pragma unroll
+        for (int q = 1; q <= 7; ++q) {
+            const int at = lo + q * part - 1;
+            below += at < hi && load_ent(&row[at]).dist < x;
+        }
+        if (below < 7) hi = min(hi, lo + (below + 1) * part - 1);
+        lo += below * part;
+    }
+    return lo;
 }
 
 // The ranks gained by v at level L (lane j < dcnt: the j-th, ascending) go to
@@ -132,29 +165,23 @@ __device__ __forceinline__ void post_row(const WArgs& a, int64_t e0, int64_t e1,
                                          int dcnt, int64_t L) {
     for (int64_t b = e0 + first; b < e1; b += step) {
         const int64_t e = b + lane_id();
-        bool open = e < e1, want = false;
+        const uint64_t* row = nullptr;
         int32_t u = 0;
         int64_t lv = 0;
-        uint64_t kth = 0;
-        if (open) {
+        if (e < e1) {
             u = __ldg(&a.cols[e]);
             lv = L + __ldg(&a.wts[e]);
-            kth = __ldcg(&a.S[(int64_t)u * a.k + a.k - 1]);
-            if (lv > 65535) {
-                atomicOr(&a.c->err, 2ULL);
-                open = false;
-            }
+            if (lv > 65535) atomicOr(&a.c->err, 2ULL);
+            else row = a.S + (int64_t)u * a.k;
         }
-        for (int j = 0; j < dcnt && __any_sync(kFull, open); ++j) {
+        uint64_t kth;
+        const unsigned held = held_ranks(row, a.k, gained, dcnt, &kth);
+        bool want = false;
+        for (int j = 0; j < dcnt; ++j) {
             const uint64_t x = __shfl_sync(kFull, gained, j);
-            if (!open) continue;
-            if (x >= kth) open = false;
-            else if (!in_sketch(a.S + (int64_t)u * a.k, a.k, x)) {
-                want = true;
-                open = false;
-            }
+            want |= x < kth && !((held >> j) & 1u);
         }
-        if (want) {
+        if (want && row) {
             const int slot = (int)((uint32_t)lv % (uint32_t)a.R);
             const uint32_t re = __ldg(&a.rev[e]);
             atomicOr(&a.marks[(int64_t)slot * a.mwords + (re >> 5)], 1u << (re & 31));
@@ -314,13 +341,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_wbuild(WArgs a) {
                         x = (int32_t)(L - __ldg(&a.wts[e]));
                         have = min(__ldcg(&a.ecnt[u]), a.cap);
                         row = a.ent + (int64_t)u * a.cap;
-                        int lo = 0, hi = have;
-                        while (lo < hi) {
-                            const int mid = (lo + hi) >> 1;
-                            if (load_ent(&row[mid]).dist < x) lo = mid + 1;
-                            else hi = mid;
-                        }
-                        at = lo;
+                        at = first_at(row, have, x);
                     }
                     // each lane offers its entry's candidates one per round
                     for (;;) {
