@@ -37,8 +37,8 @@ void destroy_graph(fl_graph* g) {
                     &g->S, &g->Scnt, &g->D[0], &g->D[1], &g->Dcnt[0], &g->Dcnt[1], &g->frontier[0],
                     &g->frontier[1], &g->stamp, &g->vg, &g->ve, &g->stg_ent, &g->stg_grp, &g->gofs, &g->eofs,
                     &g->ginfo, &g->gwt, &g->eid, &g->ecc_ub, &g->ctr, &g->scratch,
-                    &g->relax_aux, &g->U, &g->DM[0], &g->DM[1], &g->PM, &g->seg_flag, &g->PH, &g->F[0], &g->F[1], &g->H[0],
-                    &g->H[1], &g->W, &g->fbm, &g->URid, &g->vbase, &g->vpart, &g->rid,
+                    &g->relax_aux, &g->ord, &g->ord_rid, &g->DM[0], &g->DM[1], &g->PM, &g->seg_flag, &g->PH, &g->F[0], &g->F[1], &g->H[0],
+                    &g->H[1], &g->W, &g->fbm, &g->vbase, &g->vpart, &g->rid,
                     &g->inv, &g->xbits, &g->xaux, &g->xio, &g->items};
     for (DBuf* b : bufs) dfree_idle(*b);
     if (g->gbfs) {
@@ -305,8 +305,7 @@ int fl_hop_model(const fl_graph* g, int64_t cap, int64_t* n_hops, int64_t* edge_
     return FL_OK;
 }
 
-__global__ void k_export_sketch(const uint64_t* __restrict__ S, const uint8_t* __restrict__ Scnt, int64_t n,
-                                int32_t* __restrict__ cnt) {
+__global__ void k_export_sketch(const uint8_t* __restrict__ Scnt, int64_t n, int32_t* __restrict__ cnt) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) cnt[v] = Scnt[v];
 }
@@ -328,10 +327,10 @@ int fl_export_sketches(fl_graph* g, uint64_t* S, int32_t* cnt, int mem_kind) {
     if (bad_kind(mem_kind)) FL_FAIL(FL_EINVAL, "bad mem_kind");
     ProfScope ps(g);
     cudaStream_t st = g->stream;
-    if (S && g->relabelled) {
+    if (S && !g->wts.p) {  // ordinals of an unweighted build
         DBuf tmp;
         FL_TRY(dalloc(tmp, (size_t)g->n * g->k * 8));
-        int rc = sketch_rows_original(g, tmp.as<uint64_t>());
+        int rc = sketch_ranks_original(g, tmp.as<uint64_t>());
         if (!rc) rc = copy_out(S, tmp.p, (size_t)g->n * g->k * 8, mem_kind, st);
         cudaError_t e = cudaStreamSynchronize(st);
         dfree(tmp);
@@ -343,8 +342,8 @@ int fl_export_sketches(fl_graph* g, uint64_t* S, int32_t* cnt, int mem_kind) {
     if (cnt) {
         DBuf tmp;
         FL_TRY(dalloc(tmp, (size_t)g->n * 8));
-        FL_LAUNCH(kProfOther, k_export_sketch<<<152 * 4, 256, 0, st>>>(g->S.as<uint64_t>(), g->Scnt.as<uint8_t>(), g->n,
-                                                 tmp.as<int32_t>()));
+        FL_LAUNCH(kProfOther, k_export_sketch<<<152 * 4, 256, 0, st>>>(g->Scnt.as<uint8_t>(), g->n,
+                                                                              tmp.as<int32_t>()));
         int32_t* src = tmp.as<int32_t>();
         int rc = FL_OK;
         if (g->relabelled) {
@@ -736,6 +735,7 @@ int fl_batch_create_union(int n_graphs, const int64_t* n_of, const int64_t* nnz_
     if (rc == FL_OK) {
         fl_graph* U = b->U;
         U->n_parts = n_graphs;
+        for (int i = 0; i < n_graphs; ++i) U->max_part = std::max(U->max_part, n_of[i]);
         set_current_prof(&U->prof, st);
         for (int i = 0; i < n_graphs && rc == FL_OK; ++i) {
             // each graph's offsets must run from 0 to its nnz

@@ -136,8 +136,8 @@ constexpr int64_t kResidentEdges = 10 << 20;
 constexpr int kItemEdges = 64;
 // Pinned host block of a graph: its Counters mirror, then scratch of a call.
 constexpr size_t kPinnedBytes = 16384;
-// Width of the small-rank universe of the sketch hops (the kUW smallest
-// ranks of a graph; a saturated sketch is a kUW-bit mask over them).
+// Width of the masks of the sketch hops (a sketch that holds only ordinals
+// below kUW is a kUW-bit mask).
 constexpr int kUW = 1024;
 constexpr int kUSlices = kUW / 256;  // a mask is read and merged in 256-bit slices
 constexpr int kUWords = kUW / 64;
@@ -282,87 +282,6 @@ __device__ __forceinline__ long long block_append(bool pred, unsigned long long*
     }
     __syncthreads();
     return pred ? (long long)(sh.off[warp] + __popc(m & ((1u << lane) - 1u))) : -1LL;
-}
-
-// ----------------------------------------------------------------- group primitives
-// A group is G consecutive lanes of a warp (G = 16 or 32) that works on one
-// vertex; a G-lane list holds up to G uint64 values, one per lane, ascending,
-// padded with kEmpty.  All sync intrinsics use the group's own lane mask, so
-// the two half-warp groups of a warp may diverge.
-
-template <int G>
-struct Grp {
-    unsigned mask;
-    int l;      // lane within the group
-    int shift;  // position of the group's bits in a warp ballot
-    __device__ __forceinline__ Grp() {
-        const int lane = lane_id();
-        l = lane & (G - 1);
-        shift = (G == 32) ? 0 : (lane & 16);
-        mask = (G == 32) ? kFull : (0xffffu << shift);
-    }
-    __device__ __forceinline__ unsigned ballot(bool p) const {
-        unsigned b = __ballot_sync(mask, p);
-        return (G == 32) ? b : ((b >> shift) & 0xffffu);
-    }
-    template <class T>
-    __device__ __forceinline__ T shfl(T x, int src) const { return __shfl_sync(mask, x, src, G); }
-    template <class T>
-    __device__ __forceinline__ T shfl_xor(T x, int m) const { return __shfl_xor_sync(mask, x, m, G); }
-    template <class T>
-    __device__ __forceinline__ T shfl_up(T x, int d) const { return __shfl_up_sync(mask, x, d, G); }
-};
-
-// Bitonic sort of a G-lane list (ascending).
-template <int G>
-__device__ __forceinline__ uint64_t grp_sort(const Grp<G>& g, uint64_t x) {
-#pragma unroll
-    for (int k = 2; k <= G; k <<= 1) {
-#pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            uint64_t y = g.shfl_xor(x, j);
-            bool up = (g.l & k) == 0 || k == G;
-            bool low = (g.l & j) == 0;
-            x = (low == up) ? umin64(x, y) : umax64(x, y);
-        }
-    }
-    return x;
-}
-
-// The G smallest of two ascending G-lane lists, ascending.
-template <int G>
-__device__ __forceinline__ uint64_t grp_merge_low(const Grp<G>& g, uint64_t a, uint64_t b) {
-    uint64_t c = umin64(a, g.shfl(b, G - 1 - g.l));
-#pragma unroll
-    for (int j = G / 2; j > 0; j >>= 1) {
-        uint64_t y = g.shfl_xor(c, j);
-        c = (g.l & j) ? umax64(c, y) : umin64(c, y);
-    }
-    return c;
-}
-
-// Is x an entry of the ascending G-lane list L?  (every lane of the group calls)
-template <int G>
-__device__ __forceinline__ bool grp_member(const Grp<G>& g, uint64_t L, uint64_t x) {
-    int pos = 0;
-#pragma unroll
-    for (int s = G / 2; s > 0; s >>= 1) {
-        uint64_t y = g.shfl(L, pos + s - 1);
-        if (y < x) pos += s;
-    }
-    uint64_t last = g.shfl(L, G - 1);
-    if (pos == G - 1 && last < x) pos = G;
-    uint64_t y = g.shfl(L, pos & (G - 1));
-    return pos < G && y == x;
-}
-
-// Gather the lanes in `keep` (group-relative bits) to lanes 0.., order kept.
-template <int G>
-__device__ __forceinline__ uint64_t grp_compact(const Grp<G>& g, uint64_t x, unsigned keep, uint64_t fill) {
-    int total = __popc(keep);
-    int src = g.l < total ? nth_set_bit(keep, g.l) : 0;
-    uint64_t y = g.shfl(x, src);
-    return g.l < total ? y : fill;
 }
 
 // ----------------------------------------------------------------- resident kernels
@@ -533,7 +452,7 @@ struct fl_graph {
     int64_t n_low = 0, n_hubs = 0, n_seg = 0;
     fl::DBuf items;                // int4[n_items]: work items of the resident kernels
     int64_t n_items = 0;           // 0: the graph is too large for them
-    fl::DBuf part;                 // uint64[n_seg*k]: partial bottom-k of each hub segment (scratch)
+    fl::DBuf part;                 // uint32[n_seg*k]: partial bottom-k of each hub segment (scratch)
     // A graph that is a disjoint union of parts (batched instances): vertex v
     // of the part starting at vbase[v] has local id v - vbase[v], and ranks
     // and priorities are those of the local id, so every part is solved
@@ -545,24 +464,24 @@ struct fl_graph {
     fl::DBuf rid, inv;             // int32[n] or empty
     bool relabelled = false;
     int64_t n_parts = 0;           // 0: not a union
-    fl::DBuf U;                    // uint64[kUW]: the kUW smallest ranks, ascending (kEmpty padded)
-    uint64_t ulim = 0;             // largest entry of U
-    fl::DBuf DM[2];                // uint64[kUSlices][n][4]: hop delta masks over U, slice-major
+    int64_t max_part = 0;          // union: vertices of the largest part
+    fl::DBuf ord;                  // uint32[n]: ordinal of each vertex's rank (unions: among the local ids)
+    fl::DBuf ord_rid;              // int32: rank id of each ordinal
+    fl::DBuf DM[2];                // uint64[kUSlices][n][4]: hop delta masks, slice-major
     fl::DBuf PM;                   // uint64[n_seg*kUWords]: partial masks of hub segments (scratch)
     fl::DBuf seg_flag;             // uint8[n_seg]: the segment had a neighbour that gained entries (scratch)
     fl::DBuf PH;                   // uint64[n_seg]: OR of the segment's neighbours' delta heads (scratch)
-    fl::DBuf F[2], H[2];           // uint64[n]: smallest new rank of the hop (kEmpty: none), delta bits over U[0..63]
-    fl::DBuf W;                    // uint64[n]: own sketch's mask over U[0..63] of head vertices, else 0
+    fl::DBuf F[2];                 // uint32[n]: smallest new ordinal of the hop (all ones: none)
+    fl::DBuf H[2];                 // uint64[n]: delta bits over the ordinals 0..63
+    fl::DBuf W;                    // uint64[n]: own sketch's mask over the ordinals 0..63 of head vertices, else 0
     fl::DBuf fbm;                  // uint32[n/32+1]: frontier bitmap of the previous hop
-    fl::DBuf URid;                 // int32[kUW]: rank id of the vertex of each entry of U
-    uint64_t hlim = 0;             // U[min(63, |U| - 1)]
     // sketches
     int k = 0;
     uint64_t seed = 0;
     int built = 0;
     uint64_t generation = 0;       // bumped by every build
-    fl::DBuf S, Scnt;              // uint64[n*k], uint8[n]
-    fl::DBuf D[2], Dcnt[2];        // hop deltas (ranks), counts
+    fl::DBuf S, Scnt;              // uint32[n*k] ordinals (weighted graphs: uint64[n*k] ranks), uint8[n]
+    fl::DBuf D[2], Dcnt[2];        // hop deltas (ordinals), counts
     fl::DBuf frontier[2];          // int32[n]
     fl::DBuf stamp;                // uint32[n]
     fl::DBuf vg, ve;               // int32[n] per-vertex running group / entry counts
@@ -765,7 +684,7 @@ int relax_reserve(fl_graph* g);
 int relabel_graph(fl_graph* g);
 template <class T>
 int permute_vertices(const fl_graph* g, const T* in, T* out, int64_t reps, bool to_internal, cudaStream_t st);
-int sketch_rows_original(const fl_graph* g, uint64_t* out);
+int sketch_ranks_original(const fl_graph* g, uint64_t* out);
 int ads_original(fl_graph* g, int64_t* gofs_o, int64_t* eofs_o, uint32_t* ginfo_o, double* gwt_o, int32_t* eid_o);
 
 }  // namespace fl

@@ -303,13 +303,16 @@ __global__ void k_gather_map(const T* __restrict__ in, const int32_t* __restrict
     }
 }
 
-// Sketch rows in original order: out[o*k + j] = S[inv[o]*k + j].
-__global__ void k_gather_rows(const uint64_t* __restrict__ S, const int32_t* __restrict__ inv, int64_t n, int k,
-                              uint64_t* __restrict__ out) {
+// Sketch rows as ranks, in original order: out[o*k + j] = the rank of ordinal
+// S[inv[o]*k + j] (inv NULL: of S[o*k + j]).
+__global__ void k_rank_rows(const uint32_t* __restrict__ S, const int32_t* __restrict__ ord_rid,
+                            const int32_t* __restrict__ inv, uint64_t seed, int64_t n, int k,
+                            uint64_t* __restrict__ out) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n * k; t += stride) {
         const int64_t o = t / k, j = t - o * k;
-        out[t] = S[(int64_t)inv[o] * k + j];
+        const uint32_t x = S[(inv ? (int64_t)inv[o] : o) * k + j];
+        out[t] = x == 0xffffffffu ? kEmpty : vertex_rank(seed, ord_rid[x]);
     }
 }
 
@@ -446,9 +449,10 @@ template int permute_vertices<double>(const fl_graph*, const double*, double*, i
 template int permute_vertices<uint8_t>(const fl_graph*, const uint8_t*, uint8_t*, int64_t, bool, cudaStream_t);
 template int permute_vertices<int32_t>(const fl_graph*, const int32_t*, int32_t*, int64_t, bool, cudaStream_t);
 
-int sketch_rows_original(const fl_graph* g, uint64_t* out) {
-    FL_LAUNCH(kProfOther, k_gather_rows<<<grid_for(g->n * g->k, 256), 256, 0, g->stream>>>(
-                              g->S.as<uint64_t>(), g->inv.as<int32_t>(), g->n, g->k, out));
+int sketch_ranks_original(const fl_graph* g, uint64_t* out) {
+    FL_LAUNCH(kProfOther, k_rank_rows<<<grid_for(g->n * g->k, 256), 256, 0, g->stream>>>(
+                              g->S.as<uint32_t>(), g->ord_rid.as<int32_t>(),
+                              g->relabelled ? g->inv.as<int32_t>() : nullptr, g->seed, g->n, g->k, out));
     FL_CUDA(cudaGetLastError());
     return FL_OK;
 }

@@ -2,10 +2,18 @@
 // propagation (Section 3.3, Algorithm 2 for unweighted graphs), with HIP
 // weights computed where each entry joins a sketch.
 //
+// Ranks enter a sketch only by their order, so the hops work on ordinals: the
+// ranks r(v) are sorted once, and a vertex is known by the place of its rank
+// (32 bits in place of 64 in every list, load, shuffle and compare, and the
+// small ranks that the masks below cover are simply the ordinals below kUW).
+// The rank itself is computed again where an HIP weight or an export needs it.
+//
 // Data layout (k <= 32):
-//   S[v*k + i]        current sketch of v, ascending ranks, kEmpty padding
-//   Scnt[v]           number of ranks in S[v]
-//   D[p][v*k + i]     entries v gained at the previous / current hop (ranks)
+//   ord[v]            ordinal of vertex v's rank (in a union: of its local id's)
+//   ord_rid[o]        rank id of ordinal o
+//   S[v*k + i]        current sketch of v, ascending ordinals, kNil padding
+//   Scnt[v]           number of ordinals in S[v]
+//   D[p][v*k + i]     entries v gained at the previous / current hop, kNil padding
 //   Dcnt[p][v]        their number (0 = v is not in the frontier)
 //   staging           one group slot per work item of every hop (v, hop, HIP
 //                     weight, counts) and k entry slots; compacted into the
@@ -18,6 +26,14 @@
 // candidates in scratch (k_hop_hub_segments), and one group per hub merges
 // the partials into the hub's sketch (k_hop_hubs).  Bottom-k of a union is the
 // bottom-k of the union of bottom-k's, so the split does not change results.
+//
+// What bounds the hops: instructions in the list merges (hops 1-3 of an R-MAT
+// graph, all of an Erdos-Renyi graph's), the chain column -> bitmap -> mask
+// word in the mask and head merges.  Per build, against 64-bit ranks and
+// half-warp groups that diverged: non-hub vertices of R-MAT 24 (k = 16) 49.2
+// -> 32.1 ms, hub segments 9.8 -> 7.1; R-MAT 20 (k = 32) 5.4 -> 3.6; 64
+// Erdos-Renyi graphs (k = 32) 14.9 -> 7.0.  The sort of the ranks adds 0.3 ms
+// at 2^20 vertices, 2.0 at 2^24.
 #include <algorithm>
 #include <cstdio>
 #include <vector>
@@ -39,201 +55,188 @@ __host__ __device__ __forceinline__ uint32_t pack_info(int hop, int cnt, int cou
 }
 
 constexpr int kMaxHops = 65535;
+constexpr uint32_t kNil = 0xffffffffu;  // empty sketch or list slot
+constexpr int64_t kCountMax = 16384;    // more ranks than this go through the radix sort
 
-// ------------------------------------------------------------------ small-rank masks
-// U = the kUW smallest ranks of the graph, ascending.  Every rank <= U[last]
-// is an entry of U, so once a sketch is full and its k-th rank is <= U[last]
-// ("saturated"), all its entries and every candidate that can still enter it
-// are entries of U: the sketch is a kUW-bit mask over U, and one hop is
-// S_h(v) = lowest k bits of (S_{h-1}(v) | OR_{u in N(v)} D_{h-1}(u)), with
-// D_{h-1}(u) kept as a mask beside its list.  Candidates above U[last] are
-// above the k-th rank and drop out either way, so the mask update is the
-// list merge exactly.  Masks are merged in 256-bit slices from the smallest
-// ranks up, stopping once k bits are kept: a sketch whose k-th rank lies in
-// the first slice reads 32 bytes per neighbour.
+// ------------------------------------------------------------------ groups in lockstep
+// A group is G consecutive lanes (16 or 32) that work on one vertex.  The two
+// half-warp groups of a warp run in lockstep: every lane of the warp executes
+// every group operation, a group without work carries empty ranges and empty
+// lists through it, and branches are taken by the whole warp.  (Groups that
+// diverge are executed one after the other, which cost half the issue slots.)
+// A G-lane list holds up to G ordinals, one per lane, ascending, kNil after.
 
-struct Mask4 {  // one 256-bit slice
-    uint64_t w0 = 0, w1 = 0, w2 = 0, w3 = 0;
-    __device__ __forceinline__ void set(int i) {
-        const uint64_t b = 1ULL << (i & 63);
-        const int q = i >> 6;
-        w0 |= q == 0 ? b : 0ULL;
-        w1 |= q == 1 ? b : 0ULL;
-        w2 |= q == 2 ? b : 0ULL;
-        w3 |= q == 3 ? b : 0ULL;
+template <int G>
+struct Lock {
+    int l;      // lane within the group
+    int shift;  // position of the group's bits in a warp ballot
+    __device__ __forceinline__ Lock() {
+        const int lane = lane_id();
+        l = lane & (G - 1);
+        shift = lane & ~(G - 1);
     }
-    __device__ __forceinline__ void load(const uint64_t* __restrict__ p) {
-        const ulonglong2 a = __ldg(reinterpret_cast<const ulonglong2*>(p));
-        const ulonglong2 b = __ldg(reinterpret_cast<const ulonglong2*>(p) + 1);
-        w0 |= a.x;
-        w1 |= a.y;
-        w2 |= b.x;
-        w3 |= b.y;
-    }
-    __device__ __forceinline__ void add(const Mask4& o) {
-        w0 |= o.w0;
-        w1 |= o.w1;
-        w2 |= o.w2;
-        w3 |= o.w3;
-    }
-    __device__ __forceinline__ uint64_t word(int q) const {
-        return q == 0 ? w0 : (q == 1 ? w1 : (q == 2 ? w2 : w3));
-    }
-    __device__ __forceinline__ bool operator==(const Mask4& o) const {
-        return w0 == o.w0 && w1 == o.w1 && w2 == o.w2 && w3 == o.w3;
-    }
-    __device__ __forceinline__ bool empty() const { return (w0 | w1 | w2 | w3) == 0; }
-    __device__ __forceinline__ int count() const {
-        return __popcll(w0) + __popcll(w1) + __popcll(w2) + __popcll(w3);
-    }
+    __device__ __forceinline__ unsigned mine(unsigned b) const { return G == 32 ? b : (b >> shift) & 0xffffu; }
+    __device__ __forceinline__ unsigned ballot(bool p) const { return mine(__ballot_sync(kFull, p)); }
+    __device__ __forceinline__ unsigned below() const { return (1u << l) - 1u; }  // the lanes before this one
+    template <class T>
+    __device__ __forceinline__ T shfl(T x, int src) const { return __shfl_sync(kFull, x, src, G); }
+    template <class T>
+    __device__ __forceinline__ T shfl_xor(T x, int m) const { return __shfl_xor_sync(kFull, x, m, G); }
+    template <class T>
+    __device__ __forceinline__ T shfl_up(T x, int d) const { return __shfl_up_sync(kFull, x, d, G); }
 };
 
-// Lowest m set bits of x (m < popcount(x)).
-__device__ __forceinline__ uint64_t keep_lowest64(uint64_t x, int m) {
-    const unsigned lo = (unsigned)x, hi = (unsigned)(x >> 32);
-    const int c = __popc(lo);
-    const int p = m < c ? nth_set_bit(lo, m) : 32 + nth_set_bit(hi, m - c);
-    return x & ((1ULL << p) - 1ULL);
+__device__ __forceinline__ bool warp_any(bool p) { return __any_sync(kFull, p); }
+
+template <int G>
+__device__ __forceinline__ uint32_t lock_sort(const Lock<G>& g, uint32_t x) {
+#pragma unroll
+    for (int k = 2; k <= G; k <<= 1) {
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            const uint32_t y = g.shfl_xor(x, j);
+            const bool up = (g.l & k) == 0 || k == G;
+            const bool low = (g.l & j) == 0;
+            x = low == up ? min(x, y) : max(x, y);
+        }
+    }
+    return x;
 }
 
-__device__ __forceinline__ uint64_t lowest_word(uint64_t x, int& left) {
-    const int c = __popcll(x);
-    const uint64_t r = left <= 0 ? 0ULL : (c > left ? keep_lowest64(x, left) : x);
-    left -= c;
+// Entries of the list L below x (0..G) and whether x is one of them.
+template <int G>
+__device__ __forceinline__ int lock_find(const Lock<G>& g, uint32_t L, uint32_t x, bool& member) {
+    int pos = 0;
+#pragma unroll
+    for (int s = G / 2; s > 0; s >>= 1)
+        if (g.shfl(L, pos + s - 1) < x) pos += s;
+    const uint32_t y = g.shfl(L, pos);
+    member = y == x;
+    return pos + (y < x ? 1 : 0);
+}
+
+template <int G>
+__device__ __forceinline__ uint64_t lock_or64(const Lock<G>& g, uint64_t x) {
+    unsigned lo = (unsigned)x, hi = (unsigned)(x >> 32);
+    if (G == 32) {
+        lo = __reduce_or_sync(kFull, lo);
+        hi = __reduce_or_sync(kFull, hi);
+    } else {
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) {
+            lo |= g.shfl_xor(lo, o);
+            hi |= g.shfl_xor(hi, o);
+        }
+    }
+    return ((uint64_t)hi << 32) | lo;
+}
+
+// ------------------------------------------------------------------ small-ordinal masks
+// A sketch whose k-th ordinal is below kUW ("saturated") holds only ordinals
+// below kUW, and so does every candidate that can still enter it: the sketch
+// is a kUW-bit mask, and one hop is S_h(v) = lowest k bits of (S_{h-1}(v) |
+// OR_{u in N(v)} D_{h-1}(u)), with D_{h-1}(u) kept as a mask beside its list.
+// Candidates at or above kUW are above the k-th ordinal and drop out either
+// way, so the mask update is the list merge exactly.  Masks are merged in
+// 256-bit slices from the smallest ordinals up, stopping once k bits are kept:
+// a sketch whose k-th ordinal lies in the first slice reads 32 bytes per
+// neighbour.
+
+constexpr int kSliceWords = 8;  // 32-bit words of a slice
+
+// Lane l's word l mod 8 of the OR over the group of the lanes' slices: each
+// exchange halves the words a lane still holds (8 shuffles for 16 lanes, 40
+// for the OR of every word on every lane).
+template <int G>
+__device__ __forceinline__ uint32_t slice_or(const Lock<G>& g, const uint32_t (&w)[kSliceWords]) {
+    uint32_t a[4], b[2];
+    const bool h4 = (g.l & 4) != 0, h2 = (g.l & 2) != 0, h1 = (g.l & 1) != 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) a[i] = (h4 ? w[i + 4] : w[i]) | g.shfl_xor(h4 ? w[i] : w[i + 4], 4);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) b[i] = (h2 ? a[i + 2] : a[i]) | g.shfl_xor(h2 ? a[i] : a[i + 2], 2);
+    uint32_t r = (h1 ? b[1] : b[0]) | g.shfl_xor(h1 ? b[0] : b[1], 1);
+    r |= g.shfl_xor(r, 8);
+    if (G == 32) r |= g.shfl_xor(r, 16);
     return r;
 }
 
-// Keep the lowest k set bits of the slice.
-__device__ __forceinline__ void mask_lowest(Mask4& m, int k) {
-    int left = k;
-    m.w0 = lowest_word(m.w0, left);
-    m.w1 = lowest_word(m.w1, left);
-    m.w2 = lowest_word(m.w2, left);
-    m.w3 = lowest_word(m.w3, left);
-}
-
-// Index of the j-th set bit (0-based) of the slice; j < count().
-__device__ __forceinline__ int mask_nth(const Mask4& m, int j) {
-    const int c0 = __popcll(m.w0), c1 = __popcll(m.w1), c2 = __popcll(m.w2);
-    int q = 0;
-    uint64_t x = m.w0;
-    if (j >= c0) { j -= c0; q = 1; x = m.w1;
-        if (j >= c1) { j -= c1; q = 2; x = m.w2;
-            if (j >= c2) { j -= c2; q = 3; x = m.w3; } } }
-    const unsigned lo = (unsigned)x;
-    const int c = __popc(lo);
-    const int p = j < c ? nth_set_bit(lo, j) : 32 + nth_set_bit((unsigned)(x >> 32), j - c);
-    return q * 64 + p;
-}
-
-// Position of rank x in U (-1 when x > ulim: not an entry).
-__device__ __forceinline__ int u_pos(const uint64_t* sU, uint64_t ulim, uint64_t x) {
-    if (x > ulim) return -1;
-    int pos = 0;
+// The lane's entry `x` into its words of slice q.
+__device__ __forceinline__ void slice_set(uint32_t (&w)[kSliceWords], uint32_t x, int q) {
+    const uint32_t bit = (x >> 8) == (uint32_t)q ? 1u << (x & 31) : 0u;
 #pragma unroll
-    for (int s = kUW / 2; s > 0; s >>= 1)
-        if (sU[pos + s - 1] < x) pos += s;
-    return pos;
+    for (int i = 0; i < kSliceWords; ++i)
+        if (((x >> 5) & 7) == (uint32_t)i) w[i] |= bit;
 }
 
+// Slice q of a merged mask (r: lane l holds word l mod 8): its lowest `left`
+// bits go to the lanes base, base + 1, ... of sk.  Returns the bits taken.
 template <int G>
-__device__ __forceinline__ void grp_or(const Grp<G>& g, Mask4& m) {
+__device__ __forceinline__ int slice_emit(const Lock<G>& g, uint32_t r, int q, int base, int left, uint32_t& sk) {
+    const int c = __popc(r);
+    int incl = c;
 #pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) {
-        m.w0 |= g.shfl_xor(m.w0, o);
-        m.w1 |= g.shfl_xor(m.w1, o);
-        m.w2 |= g.shfl_xor(m.w2, o);
-        m.w3 |= g.shfl_xor(m.w3, o);
+    for (int s = 1; s < 8; s <<= 1) {
+        const int y = __shfl_up_sync(kFull, incl, s, 8);
+        if ((g.l & 7) >= s) incl += y;
     }
+    const int take = min(g.shfl(incl, 7), left);
+    const int j = g.l - base;
+    int wl = 0;
+#pragma unroll
+    for (int s = 4; s > 0; s >>= 1)
+        if (g.shfl(incl, wl + s - 1) <= j) wl += s;
+    const uint32_t word = g.shfl(r, wl);
+    const int before = g.shfl(incl - c, wl);
+    if (j >= 0 && j < take) sk = (uint32_t)(q * 256 + wl * 32 + nth_set_bit(word, j - before));
+    return max(take, 0);
 }
 
-// Slice q of the mask of the lanes' U positions (-1 = none).
-template <int G>
-__device__ __forceinline__ Mask4 slice_mask(const Grp<G>& g, int idx, int q) {
-    Mask4 m;
-    if (idx >= 0 && (idx >> 8) == q) m.set(idx & 255);
-    grp_or(g, m);
-    return m;
-}
-
-// Saturated merge, slice by slice from the smallest ranks: first = the OR of
-// the candidates' slice 0, src(q) gives it for q >= 1; idx is the lane's old
-// entry's U position.  Lanes j < k receive the new sketch in sk_new; returns
-// whether it changed.
-template <int G, class Src>
-__device__ __forceinline__ bool merge_slices(const Grp<G>& g, int k, const uint64_t* sU, int idx, const Mask4& first,
-                                             Src src, uint64_t& sk_new) {
-    int left = k, base = 0, own_seen = 0;
-    bool changed = false;
-    sk_new = kEmpty;
-    for (int q = 0; q < kUSlices && left > 0; ++q) {
-        const Mask4 own = slice_mask(g, idx, q);
-        Mask4 m = q == 0 ? first : src(q);
-        m.add(own);
-        mask_lowest(m, left);
-        changed |= !(m == own);
-        own_seen += own.count();
-        const int c = m.count();
-        if (g.l >= base && g.l < base + c) sk_new = sU[q * 256 + mask_nth(m, g.l - base)];
-        base += c;
-        left -= c;
-    }
-    return changed || own_seen < k;
-}
+// ------------------------------------------------------------------ per-hop inputs and outputs
 
 // Per-group hop counters in shared memory, one slot per group, updated by
 // the group's lane 0 without atomics and flushed once at the end of a kernel
-// (the hop kernels run at the register limit; counters in registers cost
-// spills in the merge loops).  32-bit: a group adds at most 32 * kHubDeg
-// per vertex it processes (hub degrees go to the global counters directly)
-// and, with the grids of the hop kernels, processes at most 2^31 / 77824 <
-// 2^16 work items.
+// (counters in registers cost spills in the merge loops).  32-bit: a group
+// adds at most 32 * kHubDeg per vertex it processes (hub degrees go to the
+// global counters directly) and, with the grids of the hop kernels, processes
+// at most 2^31 / 77824 < 2^16 work items.
 enum { kCFront, kCMerges, kCMerging, kCDelta, kCNew, kNCtr };
-__shared__ unsigned s_hop_ctr[256 / 16][kNCtr];
 
-struct HopCounters {
-    unsigned long long cand = 0;  // per lane: neighbour-delta words read
+// Shared memory of a hop kernel (256 threads).
+struct HopShared {
+    unsigned ctr[256 / 16][kNCtr];
+    uint32_t x[8][32];           // per warp: merged candidates by place
+    uint32_t mask[256 / 16][32];  // per group: a delta mask
 };
 
-template <int G>
-__device__ __forceinline__ void hop_ctr_init(const Grp<G>& g) {
-    if (g.l == 0)
-        for (int i = 0; i < kNCtr; ++i) s_hop_ctr[threadIdx.x / G][i] = 0;
-}
-// lane 0 of the group only
-template <int G>
-__device__ __forceinline__ void hop_ctr_add(int field, unsigned x) {
-    s_hop_ctr[threadIdx.x / G][field] += x;
-}
-
-// Per-hop inputs and outputs of the merge kernels (p = previous hop's
-// buffers, read-only during a hop; c = this hop's).  Besides each vertex's
-// delta list D and delta mask DM, two dense per-vertex words make the
-// per-edge reads small and cache-friendly:
-//   F[u]  the smallest rank u gained at the hop (kEmpty: none), the filter of
-//         the list and slice merges: a neighbour whose F is not below the
-//         vertex's k-th rank cannot change its sketch;
-//   H[u]  the bits of u's delta mask over U[0..63] (word 0 of DM);
-// and W[v], the mask over U[0..63] of v's own sketch once the sketch is full
-// and its k-th rank is at most U[63] ("head" vertices; 0 otherwise).  A head
-// vertex takes S_h(v) = lowest k bits of (W[v] | OR_u H[u]): every candidate
-// that can still enter is among U[0..63], so this is the list merge's result.
-// Frontier membership for the counters comes from a bitmap of the previous
-// hop's frontier (n/8 bytes, cache-resident).
+// p = previous hop's buffers, read-only during a hop; c = this hop's.  Besides
+// each vertex's delta list D (padded with kNil) and delta mask DM, two dense
+// per-vertex words make the per-edge reads small and cache-friendly:
+//   F[u]  the smallest ordinal u gained at the hop (kNil: none), the filter of
+//         the list merge: a neighbour whose F is not below the vertex's k-th
+//         ordinal cannot change its sketch;
+//   H[u]  the bits of u's delta mask over the ordinals 0..63 (word 0 of DM);
+// and W[v], the mask of v's own sketch once the sketch is full and its k-th
+// ordinal is below 64 ("head" vertices; 0 otherwise).  A head vertex takes
+// S_h(v) = lowest k bits of (W[v] | OR_u H[u]): every candidate that can still
+// enter is below 64, so this is the list merge's result.  Frontier membership
+// comes from a bitmap of the previous hop's frontier (n/8 bytes,
+// cache-resident).
 struct HopIO {
     const int64_t* __restrict__ rowp;
     const int32_t* __restrict__ cols;
     int k;
     int hop;
     uint64_t seed;
-    uint64_t* __restrict__ S;
+    const uint32_t* __restrict__ ord;        // ordinal of each vertex
+    const int32_t* __restrict__ rid_of;      // rank id of each ordinal
+    uint32_t* __restrict__ S;
     uint8_t* __restrict__ Scnt;
-    const uint64_t* __restrict__ Dp;
-    const uint8_t* __restrict__ Dcp;
-    uint64_t* __restrict__ Dc;
+    const uint32_t* __restrict__ Dp;
+    uint32_t* __restrict__ Dc;
     uint8_t* __restrict__ Dcc;
-    const uint64_t* __restrict__ Fp;
-    uint64_t* __restrict__ Fc;
+    const uint32_t* __restrict__ Fp;
+    uint32_t* __restrict__ Fc;
     const uint64_t* __restrict__ Hp;
     uint64_t* __restrict__ Hc;
     uint64_t* __restrict__ W;
@@ -245,10 +248,6 @@ struct HopIO {
     int32_t* __restrict__ ve;
     int32_t* __restrict__ stg_ent;
     StgGroup* __restrict__ stg_grp;
-    const uint64_t* __restrict__ U;
-    const int32_t* __restrict__ URid;  // rank id of the vertex of each U rank
-    uint64_t ulim;                     // U's largest entry
-    uint64_t hlim;                     // U[min(63, |U| - 1)]: the head's largest rank
     IdMap ids;
     Counters* ctr;
 };
@@ -266,32 +265,22 @@ __device__ __forceinline__ int nth_bit64(uint64_t x, int n) {
 
 // The lowest k set bits of x.
 __device__ __forceinline__ uint64_t lowest_k64(uint64_t x, int k) {
-    return __popcll(x) <= k ? x : keep_lowest64(x, k);
+    return __popcll(x) <= k ? x : x & ((1ULL << nth_bit64(x, k)) - 1ULL);
 }
 
-template <int G>
-__device__ __forceinline__ uint64_t grp_or64(const Grp<G>& g, uint64_t x) {
-#pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) x |= g.shfl_xor(x, o);
-    return x;
-}
-
-// Index of word w of vertex v's delta mask in the slice-major layout (each
-// 256-bit slice of all vertices is one dense array, so that the hot slices
-// of high-degree vertices share cache lines).
+// Word w of vertex v's delta mask in the slice-major layout (each 256-bit
+// slice of all vertices is one dense array, so that the hot slices of
+// high-degree vertices share cache lines).
 __device__ __forceinline__ int64_t dm_word(int64_t n, int64_t v, int w) {
     return ((int64_t)(w >> 2) * n + v) * 4 + (w & 3);
 }
 
-// Slice q of the OR of the delta masks of the neighbours in [e0, e1) that
-// gained entries at the previous hop (frontier bitmap; lane-parallel, four
-// columns per lane in flight, then reduced over the group); `front` tells
-// whether there is such a neighbour.
+// The lanes' shares of slice q of the delta masks of the neighbours in
+// [e0, e1) that gained entries at the previous hop are ORed into w (four
+// columns per lane in flight); `front`: the lane saw such a neighbour.
 template <int G>
-__device__ __forceinline__ Mask4 gather_masks(const Grp<G>& g, const HopIO& io, int64_t e0, int64_t e1, int q,
-                                              bool& front, unsigned long long& cand) {
-    Mask4 acc;
-    bool f = false;
+__device__ __forceinline__ void gather_slice(const Lock<G>& g, const HopIO& io, int64_t e0, int64_t e1, int q,
+                                             uint32_t (&w)[kSliceWords], bool& front, unsigned& cand) {
     const uint64_t* __restrict__ slice = io.DMp + (int64_t)q * io.n * 4;
     for (int64_t e = e0 + g.l; e < e1; e += 4 * G) {
         int32_t u[4];
@@ -303,25 +292,29 @@ __device__ __forceinline__ Mask4 gather_masks(const Grp<G>& g, const HopIO& io, 
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             if (in[j]) {
-                acc.load(slice + (int64_t)u[j] * 4);
-                f = true;
-                cand += 4ULL;
+                const uint4* p = reinterpret_cast<const uint4*>(slice + (int64_t)u[j] * 4);
+                const uint4 a = __ldg(p), b = __ldg(p + 1);
+                w[0] |= a.x;
+                w[1] |= a.y;
+                w[2] |= a.z;
+                w[3] |= a.w;
+                w[4] |= b.x;
+                w[5] |= b.y;
+                w[6] |= b.z;
+                w[7] |= b.w;
+                front = true;
+                cand += 4u;
             }
         }
     }
-    grp_or(g, acc);
-    front = g.ballot(f) != 0;
-    return acc;
 }
 
-// OR of the delta heads H[u] of the neighbours in [e0, e1) that are in the
-// previous hop's frontier (four columns per lane in flight); `front` tells
-// whether there is such a neighbour.
+// OR over the lane's share of the delta heads H[u] of the neighbours in
+// [e0, e1) that are in the previous hop's frontier.
 template <int G>
-__device__ __forceinline__ uint64_t gather_heads(const Grp<G>& g, const HopIO& io, int64_t e0, int64_t e1,
-                                                 bool& front, unsigned long long& cand) {
+__device__ __forceinline__ uint64_t gather_heads(const Lock<G>& g, const HopIO& io, int64_t e0, int64_t e1,
+                                                 bool& front, unsigned& cand) {
     uint64_t acc = 0;
-    bool f = false;
     for (int64_t e = e0 + g.l; e < e1; e += 4 * G) {
         int32_t u[4];
 #pragma unroll
@@ -333,28 +326,25 @@ __device__ __forceinline__ uint64_t gather_heads(const Grp<G>& g, const HopIO& i
         for (int j = 0; j < 4; ++j) {
             if (in[j]) {
                 acc |= __ldg(&io.Hp[u[j]]);
-                f = true;
-                cand += 1ULL;
+                front = true;
+                cand += 1u;
             }
         }
     }
-    front = g.ballot(f) != 0;
-    return grp_or64(g, acc);
+    return acc;
 }
 
 // ------------------------------------------------------------------ hop 0
 
-// Hop 0: S_0(v) = {r(v)} and v's ADS group at distance 0.  (Hop 1 recomputes
-// the neighbours' ranks from their ids, so no hop-0 delta list or mask is
-// stored; the group's single entry is v itself, written by the compaction.)
-__global__ void k_rank_init(int64_t n, int k, uint64_t seed, uint64_t* __restrict__ S,
+// Hop 0: S_0(v) = {ord(v)} and v's ADS group at distance 0.  (Hop 1 reads the
+// neighbours' ordinals, so no hop-0 delta list or mask is stored; the group's
+// single entry is v itself, written by the compaction.)
+__global__ void k_rank_init(int64_t n, int k, const uint32_t* __restrict__ ord, uint32_t* __restrict__ S,
                             uint8_t* __restrict__ Scnt, StgGroup* __restrict__ stg_grp,
-                            int32_t* __restrict__ vg, int32_t* __restrict__ ve, IdMap ids, Counters* ctr) {
+                            int32_t* __restrict__ vg, int32_t* __restrict__ ve) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
-        uint64_t r = vertex_rank(seed, rank_id(ids, v));
-        if (r == kEmpty) atomicOr(&ctr->error, 1ULL);
-        S[v * k] = r;
+        S[v * k] = ord[v];
         Scnt[v] = 1;
         StgGroup gr;
         gr.wt = 1.0;  // a one-vertex ball: fewer than k ranks (k >= 2)
@@ -370,147 +360,171 @@ __global__ void k_rank_init(int64_t n, int k, uint64_t seed, uint64_t* __restric
 
 // ------------------------------------------------------------------ group sketch updates
 
-// Running sketch of one group: list `sk` (k valid lanes), its size `cnt` and
-// the filter `tau` (= sk[k-1] when full, else `tau_base`: kEmpty for a
-// vertex's own sketch, the vertex's old k-th rank for a hub partial).
+// Running sketch of one group: list `sk` (k valid lanes) and the filter `tau`:
+// its k-th ordinal (kNil while it is not full), at most `tau_base` (kNil for a
+// vertex's own sketch, the vertex's old k-th ordinal for a hub partial).
 template <int G>
 struct Sketch {
-    uint64_t sk;
-    int cnt;
-    uint64_t tau;
-    uint64_t tau_base;
-    __device__ __forceinline__ void retau(const Grp<G>& g, int k) {
-        uint64_t kth = g.shfl(sk, k - 1);
-        tau = cnt == k ? kth : tau_base;
-    }
+    uint32_t sk, tau, tau_base;
+    __device__ __forceinline__ void retau(const Lock<G>& g, int k) { tau = min(g.shfl(sk, k - 1), tau_base); }
 };
 
-// Insert one rank x (uniform over the group, x < tau) unless present.
+// Insert one ordinal per group (x uniform over the group; groups without
+// `want` keep their sketch).
 template <int G>
-__device__ __forceinline__ void insert_one(const Grp<G>& g, int k, uint64_t x, Sketch<G>& s) {
-    if (g.ballot(s.sk == x)) return;
-    int p = __popc(g.ballot(s.sk < x));
-    uint64_t up = g.shfl_up(s.sk, 1);
-    s.sk = (g.l > p) ? up : ((g.l == p) ? x : s.sk);
-    if (g.l >= k) s.sk = kEmpty;
-    if (s.cnt < k) ++s.cnt;
+__device__ __forceinline__ void insert_one(const Lock<G>& g, int k, uint32_t x, bool want, Sketch<G>& s) {
+    const bool dup = g.ballot(s.sk == x) != 0;
+    const int p = __popc(g.ballot(s.sk < x));
+    const uint32_t up = g.shfl_up(s.sk, 1);
+    if (want && !dup) {
+        s.sk = g.l > p ? up : (g.l == p ? x : s.sk);
+        if (g.l >= k) s.sk = kNil;
+    }
     s.retau(g, k);
 }
 
-// Merge a batch of candidates (one per lane, kEmpty = none; unsorted, may
-// repeat or already be in the sketch) keeping the k smallest distinct ranks.
+// Merge candidates, ascending over the lanes that have one (kNil: none; no
+// repeats among them): each lane finds its place in the sketch by search,
+// candidates already there drop out, and the others take the places
+// (entries below) + (kept candidates before); the sketch's entries fill the
+// places left.  Candidates pass through shared memory to their places.
 template <int G>
-__device__ __forceinline__ void merge_batch(const Grp<G>& g, int k, uint64_t buf, Sketch<G>& s) {
-    buf = grp_sort(g, buf);
-    uint64_t prev = g.shfl_up(buf, 1);
-    bool dup = g.l > 0 && prev == buf;
-    bool in_sk = grp_member(g, s.sk, buf);
-    unsigned keep = g.ballot(buf != kEmpty && !dup && !in_sk);
-    if (!keep) return;
-    buf = grp_compact(g, buf, keep, kEmpty);
-    uint64_t m = grp_merge_low(g, s.sk, buf);
-    s.sk = g.l < k ? m : kEmpty;
-    s.cnt = __popc(g.ballot(s.sk != kEmpty));
+__device__ __forceinline__ void merge_sorted(const Lock<G>& g, int k, uint32_t x, Sketch<G>& s, uint32_t* sx) {
+    bool member;
+    const int pos = lock_find(g, s.sk, x, member);
+    const bool keep = x != kNil && !member;
+    const unsigned km = __ballot_sync(kFull, keep);
+    if (!km) return;
+    const int dest = pos + __popc(g.mine(km) & g.below());
+    const bool fits = keep && dest < G;
+    const unsigned occ = g.mine(__reduce_or_sync(kFull, fits ? 1u << (dest + g.shift) : 0u));
+    if (fits) sx[g.shift + dest] = x;
+    __syncwarp();
+    const uint32_t old = g.shfl(s.sk, g.l - __popc(occ & g.below()));
+    const uint32_t nv = (occ >> g.l) & 1u ? sx[g.shift + g.l] : old;
+    __syncwarp();
+    s.sk = g.l < k ? nv : kNil;
     s.retau(g, k);
 }
 
-// Merge an ascending list of distinct candidates (lanes 0.., kEmpty after)
-// into the sketch: drop the ones already present, then one bitonic merge.
+// Merge a sorted list: the entries below tau form a prefix, absorbed by one or
+// two insertions or one merge.
 template <int G>
-__device__ __forceinline__ void merge_sorted(const Grp<G>& g, int k, uint64_t x, Sketch<G>& s) {
-    const bool in_sk = grp_member(g, s.sk, x);
-    const unsigned have = g.ballot(x != kEmpty);
-    const unsigned keep = g.ballot(x != kEmpty && !in_sk);
-    if (!keep) return;
-    if (keep != have) x = grp_compact(g, x, keep, kEmpty);
-    const uint64_t m = grp_merge_low(g, s.sk, x);
-    s.sk = g.l < k ? m : kEmpty;
-    s.cnt = __popc(g.ballot(s.sk != kEmpty));
-    s.retau(g, k);
-}
-
-// Absorb one batch of candidates: filter by tau, then insert one by one when
-// few survive, else merge the whole batch.
-template <int G>
-__device__ __forceinline__ void absorb(const Grp<G>& g, int k, uint64_t x, Sketch<G>& s) {
-    unsigned m = g.ballot(x < s.tau);
-    if (!m) return;
-    if (__popc(m) <= 2) {
-        while (m) {
-            int j = __ffs(m) - 1;
-            m &= m - 1;
-            uint64_t xj = g.shfl(x, j);
-            if (xj < s.tau) insert_one(g, k, xj, s);
+__device__ __forceinline__ void merge_list(const Lock<G>& g, int k, uint32_t x, Sketch<G>& s, uint32_t* sx) {
+    const bool in = x < s.tau;
+    const unsigned b = __ballot_sync(kFull, in);
+    if (!b) return;
+    const int c = __popc(g.mine(b));
+    if (!warp_any(c > 2)) {
+        insert_one(g, k, g.shfl(x, 0), c > 0, s);
+        if (warp_any(c > 1)) {
+            const uint32_t x1 = g.shfl(x, 1);
+            insert_one(g, k, x1, c > 1 && x1 < s.tau, s);
         }
     } else {
-        merge_batch(g, k, x < s.tau ? x : kEmpty, s);
+        merge_sorted(g, k, in ? x : kNil, s, sx);
     }
 }
 
-// Absorb the candidates of CSR entries [e0, e1): at hop 1 the neighbours' own
-// ranks (recomputed from their ids), later the entries each neighbour gained
-// at the previous hop.  Lane j of the group owns neighbour j of a chunk of G
-// neighbours and loads its smallest new rank F[u] (independent loads into a
-// dense array that also filter whole lists).  Each neighbour whose smallest
-// new rank is below the filter then has its list loaded across the group;
-// the entries below the filter form an ascending prefix, absorbed by 1-2
-// insertions or one bitonic merge.  `front`: some neighbour gained entries.
+// Absorb one batch of candidates (one per lane, kNil = none; unsorted, may
+// repeat or already be in the sketch): filter by tau, then insert one by one
+// when few survive, else sort and merge.
 template <int G>
-__device__ __forceinline__ void gather_range(const Grp<G>& g, const HopIO& io, int64_t e0, int64_t e1,
-                                             Sketch<G>& s, bool& front, unsigned long long& cand) {
-    const int k = io.k;
-    bool fr = false;
-    // the next chunk's columns are loaded while this chunk merges
-    int32_t u_next = e0 + g.l < e1 ? __ldcs(&io.cols[e0 + g.l]) : 0;
-    for (int64_t cb = e0; cb < e1; cb += G) {
-        const int64_t e = cb + g.l;
-        const bool in = e < e1;
-        const int32_t u = u_next;
-        u_next = e + G < e1 ? __ldcs(&io.cols[e + G]) : 0;
-        if (io.hop == 1) {
-            absorb(g, k, in ? vertex_rank(io.seed, rank_id(io.ids, u)) : kEmpty, s);
-            continue;
+__device__ __forceinline__ void absorb(const Lock<G>& g, int k, uint32_t x, Sketch<G>& s, uint32_t* sx) {
+    unsigned m = g.ballot(x < s.tau);
+    if (!warp_any(m != 0)) return;
+    if (!warp_any(__popc(m) > 3)) {
+        while (warp_any(m != 0)) {
+            const uint32_t y = g.shfl(x, m ? __ffs(m) - 1 : 0);
+            insert_one(g, k, y, m != 0 && y < s.tau, s);
+            m &= m - 1;
         }
-        const uint64_t first = in ? __ldg(&io.Fp[u]) : kEmpty;
-        fr |= first != kEmpty;
-        cand += first != kEmpty ? 1ULL : 0ULL;
-        // list lengths of the neighbours that pass the filter, loaded together
-        const int c = first < s.tau ? (int)__ldg(&io.Dcp[u]) : 0;
+    } else {
+        x = lock_sort(g, x < s.tau ? x : kNil);
+        const uint32_t prev = g.shfl_up(x, 1);
+        merge_sorted(g, k, g.l > 0 && prev == x ? kNil : x, s, sx);
+    }
+}
+
+// Absorb the candidates of CSR entries [e0, e1) (e0 >= e1: none): at hop 1 the
+// neighbours' own ordinals, later the entries each neighbour gained at the
+// previous hop.  Lane j of the group owns neighbour j of a chunk of G
+// neighbours and loads its smallest new ordinal F[u] (independent loads into a
+// dense array that also filter whole lists).  The lists of the neighbours that
+// pass are loaded across the group, four in flight, and merged one after the
+// other.  `front`: the lane saw a neighbour that gained entries.
+template <int G>
+__device__ __forceinline__ void gather_lists(const Lock<G>& g, const HopIO& io, int64_t e0, int64_t e1,
+                                             Sketch<G>& s, bool& front, unsigned& cand, uint32_t* sx) {
+    const int k = io.k;
+    if (io.hop == 1) {
+        front |= e0 < e1;
+        for (int64_t cb = e0; warp_any(cb < e1); cb += 2 * G) {
+            const int64_t e = cb + g.l;
+            const int32_t u0 = e < e1 ? __ldcs(&io.cols[e]) : -1, u1 = e + G < e1 ? __ldcs(&io.cols[e + G]) : -1;
+            const uint32_t x0 = u0 >= 0 ? __ldg(&io.ord[u0]) : kNil, x1 = u1 >= 0 ? __ldg(&io.ord[u1]) : kNil;
+            absorb(g, k, x0, s, sx);
+            absorb(g, k, x1, s, sx);
+        }
+        return;
+    }
+    // the next chunk's columns are loaded while this chunk merges
+    int32_t u_next = e0 + g.l < e1 ? __ldcs(&io.cols[e0 + g.l]) : -1;
+    for (int64_t cb = e0; warp_any(cb < e1); cb += G) {
+        const int32_t u = u_next;
+        const int64_t e = cb + G + g.l;
+        u_next = e < e1 ? __ldcs(&io.cols[e]) : -1;
+        const uint32_t first = u >= 0 ? __ldg(&io.Fp[u]) : kNil;
+        front |= first != kNil;
+        cand += first != kNil ? 1u : 0u;
         unsigned live = g.ballot(first < s.tau);
-        while (live) {
-            const int j = __ffs(live) - 1;
-            live &= live - 1;
-            const int cj = g.shfl(c, j);
-            const uint64_t fj = g.shfl(first, j);
-            if (!(fj < s.tau)) continue;  // the filter tightened since the first loads
-            if (cj == 1) {
-                insert_one(g, k, fj, s);
-                continue;
+        while (warp_any(live != 0)) {
+            uint32_t x[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int j = live ? __ffs(live) - 1 : 0;
+                const int32_t uj = g.shfl(u, j);
+                x[q] = live && g.l < k ? __ldg(&io.Dp[(int64_t)uj * k + g.l]) : kNil;
+                live &= live - 1;
             }
-            const int uj = g.shfl(u, j);
-            uint64_t x = (g.l > 0 && g.l < cj) ? __ldg(&io.Dp[(int64_t)uj * k + g.l]) : kEmpty;
-            cand += (g.l > 0 && g.l < cj) ? 1ULL : 0ULL;
-            if (g.l == 0) x = fj;
-            const unsigned pm = g.ballot(x < s.tau);  // an ascending prefix of the list
-            if (__popc(pm) <= 2) {
-                insert_one(g, k, fj, s);
-                if (pm & 2u) {
-                    const uint64_t x1 = g.shfl(x, 1);
-                    if (x1 < s.tau) insert_one(g, k, x1, s);
-                }
-            } else {
-                merge_sorted(g, k, x < s.tau ? x : kEmpty, s);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                cand += x[q] != kNil ? 1u : 0u;
+                merge_list(g, k, x[q], s, sx);
             }
+            live &= g.ballot(first < s.tau);  // the filter tightened since
         }
     }
-    front = io.hop == 1 || g.ballot(fr) != 0;
+}
+
+// Saturated merge, slice by slice from the smallest ordinals: src(q, w) ORs
+// the candidates' shares of slice q into w, `old` is the lane's old entry.
+// Lanes j < k receive the new sketch; groups that are not `on` keep theirs.
+template <int G, class Src>
+__device__ __forceinline__ void merge_slices(const Lock<G>& g, int k, bool on, Src src, uint32_t& sk) {
+    const uint32_t old = sk;
+    uint32_t nw = kNil;
+    int left = on ? k : 0, base = 0;
+    for (int q = 0; q < kUSlices && warp_any(left > 0); ++q) {
+        uint32_t w[kSliceWords];
+#pragma unroll
+        for (int i = 0; i < kSliceWords; ++i) w[i] = 0u;
+        if (left > 0) {
+            slice_set(w, old, q);
+            src(q, w);
+        }
+        const int c = slice_emit(g, slice_or(g, w), q, base, left, nw);
+        base += c;
+        left -= c;
+    }
+    if (on) sk = nw;
 }
 
 // Record a changed vertex's ADS group in staging slot `slot` and count it
 // (lane 0 of the group).
 template <int G>
-__device__ __forceinline__ void stage_group(const HopIO& io, int32_t v, int64_t deg, int64_t slot, int dcnt,
-                                            int counted, double wt) {
+__device__ __forceinline__ void stage_group(const HopIO& io, HopShared& sh, int32_t v, int64_t deg, int64_t slot,
+                                            int dcnt, int counted, double wt) {
     StgGroup gr;
     gr.wt = wt;
     gr.v = v;
@@ -520,100 +534,124 @@ __device__ __forceinline__ void stage_group(const HopIO& io, int32_t v, int64_t 
     io.vg[v] = gr.gidx + 1;
     io.ve[v] = gr.eidx + dcnt;
     io.stg_grp[slot] = gr;
-    hop_ctr_add<G>(kCFront, 1u);
-    hop_ctr_add<G>(kCNew, (unsigned)dcnt);
+    unsigned* c = sh.ctr[threadIdx.x / G];
+    c[kCFront] += 1u;
+    c[kCNew] += (unsigned)dcnt;
     if (deg <= kHubDeg) {
-        hop_ctr_add<G>(kCMerges, (unsigned)deg);
-        hop_ctr_add<G>(kCDelta, (unsigned)(deg * dcnt));
+        c[kCMerges] += (unsigned)deg;
+        c[kCDelta] += (unsigned)(deg * dcnt);
     }
 }
 
+// Rank of the vertex with ordinal o, and that vertex in v's part.
+__device__ __forceinline__ uint64_t rank_of(const HopIO& io, uint32_t o) {
+    return vertex_rank(io.seed, (int64_t)__ldg(&io.rid_of[o]));
+}
+__device__ __forceinline__ int32_t vertex_of(const HopIO& io, uint32_t o, int32_t v) {
+    return (int32_t)internal_of(io.ids, (int64_t)__ldg(&io.rid_of[o]), v);
+}
 
-// Write the results of vertex v after a list or slice merge: new sketch, the
-// entries it gained (list, mask, head word, smallest one, for the next hop),
-// its own head mask once the sketch is a head sketch, and its staged ADS
-// group in work slot `slot`.  Returns the number of entries gained (0: the
-// sketch is unchanged).
+// Write the results of vertex v (groups that are `on`) after a list or slice
+// merge: new sketch, the entries it gained (list, mask, head word, smallest
+// one, for the next hop), its own head mask once the sketch is a head sketch,
+// and its staged ADS group in work slot `slot`.  Returns the number of entries
+// gained (0: the sketch is unchanged).
 template <int G>
-__device__ __forceinline__ int finish_vertex(const Grp<G>& g, const HopIO& io, int32_t v, int64_t deg, uint64_t old,
-                                             const Sketch<G>& s, int64_t slot, const uint64_t* sU) {
+__device__ __forceinline__ int finish_vertex(const Lock<G>& g, const HopIO& io, HopShared& sh, bool on, int32_t v,
+                                             int64_t deg, uint32_t old, uint32_t sk, int64_t slot) {
     const int k = io.k;
-    const bool valid = g.l < k && s.sk != kEmpty;
-    const bool was_there = grp_member(g, old, s.sk);
-    const unsigned newm = g.ballot(valid && !was_there);
+    const bool valid = g.l < k && sk != kNil;
+    bool was_there;
+    lock_find(g, old, sk, was_there);
+    const unsigned newm = g.ballot(on && valid && !was_there);
     const int dcnt = __popc(newm);
-    if (dcnt == 0) {
-        if (g.l == 0) io.stg_grp[slot].info = 0;  // empty slot
-        return 0;
+    if (on && dcnt == 0 && g.l == 0) io.stg_grp[slot].info = 0;  // empty slot
+    if (!warp_any(dcnt > 0)) return 0;
+    const bool wr = dcnt > 0, is_new = (newm >> g.l) & 1u;
+    uint32_t* m = sh.mask[threadIdx.x / G];
+    m[g.l] = 0u;
+    if (G == 16) m[g.l + 16] = 0u;
+    __syncwarp();
+    if (is_new && sk < (uint32_t)kUW) atomicOr(&m[sk >> 5], 1u << (sk & 31));
+    __syncwarp();
+    if (wr) {
+        if (g.l < k) io.S[(int64_t)v * k + g.l] = sk;
+        if (is_new) {
+            const int at = __popc(newm & g.below());
+            io.Dc[(int64_t)v * k + at] = sk;
+            io.stg_ent[slot * k + at] = vertex_of(io, sk, v);
+        }
+        if (g.l < k && g.l >= dcnt) io.Dc[(int64_t)v * k + g.l] = kNil;
+        if (g.l < kUWords)
+            io.DMc[dm_word(io.n, v, g.l)] = ((uint64_t)m[2 * g.l + 1] << 32) | m[2 * g.l];
     }
     const int cnt_new = __popc(g.ballot(valid));
-    if (g.l < k) io.S[(int64_t)v * k + g.l] = s.sk;
-    const uint64_t dv = grp_compact(g, s.sk, newm, kEmpty);
-    if (g.l < dcnt) {
-        io.Dc[(int64_t)v * k + g.l] = dv;
-        io.stg_ent[slot * k + g.l] = (int32_t)internal_of(io.ids, (int64_t)rank_vertex(io.seed, dv), v);
+    const uint32_t kth = g.shfl(sk, k - 1);
+    const uint32_t least = g.shfl(sk, wr ? __ffs(newm) - 1 : 0);
+    // a full sketch whose k-th ordinal is below 64 becomes a head vertex
+    const bool head = wr && cnt_new == k && kth < 64u;
+    if (warp_any(head)) {
+        const uint64_t own = lock_or64(g, valid && sk < 64u ? 1ULL << sk : 0ULL);
+        if (head && g.l == 0) io.W[v] = own;
     }
-    // delta mask over U: lane w < kUWords builds word w
-    const int di = g.l < dcnt ? u_pos(sU, io.ulim, dv) : -1;
-    uint64_t word = 0;
-    for (int j = 0; j < dcnt; ++j) {
-        const int ij = g.shfl(di, j);
-        if (ij >= 0 && (ij >> 6) == g.l) word |= 1ULL << (ij & 63);
-    }
-    if (g.l < kUWords) io.DMc[dm_word(io.n, v, g.l)] = word;
-    const uint64_t kth = g.shfl(s.sk, k - 1);
-    // a full sketch whose k-th rank is in U's head becomes a head vertex
-    if (cnt_new == k && kth <= io.hlim) {
-        const int p = g.l < k ? u_pos(sU, io.ulim, s.sk) : -1;
-        const uint64_t own = grp_or64(g, p >= 0 ? 1ULL << p : 0ULL);
-        if (g.l == 0) io.W[v] = own;
-    }
-    if (g.l == 0) {
-        io.Fc[v] = dv;    // lane 0 holds the smallest new rank
-        io.Hc[v] = word;  // lane 0 built word 0
+    if (wr && g.l == 0) {
+        io.Fc[v] = least;
+        io.Hc[v] = ((uint64_t)m[1] << 32) | m[0];
         io.Scnt[v] = (uint8_t)cnt_new;
         io.Dcc[v] = (uint8_t)dcnt;
         const int counted = cnt_new < k ? dcnt : __popc(newm & ((1u << (k - 1)) - 1u));
-        stage_group<G>(io, v, deg, slot, dcnt, counted, hip_weight(cnt_new, k, kth));
+        stage_group<G>(io, sh, v, deg, slot, dcnt, counted,
+                       cnt_new < k ? 1.0 : hip_weight(cnt_new, k, rank_of(io, kth)));
     }
+    __syncwarp();
     return dcnt;
 }
 
-// Write the results of head vertex v whose new sketch is the mask nw over
-// U[0..63] (k bits) with gained bits delta (nonzero); the same outputs as
-// finish_vertex.
+// Write the results of head vertex v whose new sketch is the mask nw over the
+// ordinals 0..63 (k bits) with gained bits delta (nonzero); the same outputs
+// as finish_vertex.
 template <int G>
-__device__ __forceinline__ void finish_head(const Grp<G>& g, const HopIO& io, int32_t v, int64_t deg, uint64_t nw,
-                                            uint64_t delta, int64_t slot, const uint64_t* sU,
-                                            const int32_t* sURid) {
+__device__ __forceinline__ void finish_head(const Lock<G>& g, const HopIO& io, HopShared& sh, int32_t v, int64_t deg,
+                                            uint64_t nw, uint64_t delta, int64_t slot) {
     const int k = io.k;
     const int dcnt = __popcll(delta);
-    if (g.l < k) io.S[(int64_t)v * k + g.l] = sU[nth_bit64(nw, g.l)];
-    if (g.l < dcnt) {
-        const int p = nth_bit64(delta, g.l);
-        io.Dc[(int64_t)v * k + g.l] = sU[p];
-        io.stg_ent[slot * k + g.l] = (int32_t)internal_of(io.ids, (int64_t)sURid[p], v);
+    if (g.l < k) {
+        io.S[(int64_t)v * k + g.l] = (uint32_t)nth_bit64(nw, g.l);
+        uint32_t x = kNil;
+        if (g.l < dcnt) {
+            x = (uint32_t)nth_bit64(delta, g.l);
+            io.stg_ent[slot * k + g.l] = vertex_of(io, x, v);
+        }
+        io.Dc[(int64_t)v * k + g.l] = x;
     }
     if (g.l < kUWords) io.DMc[dm_word(io.n, v, g.l)] = g.l == 0 ? delta : 0ULL;
     if (g.l == 0) {
-        const int top = 63 - __clzll(nw);  // the k-th smallest rank's position
+        const int top = 63 - __clzll(nw);  // the k-th ordinal
         io.W[v] = nw;
-        io.Fc[v] = sU[__ffsll(delta) - 1];
+        io.Fc[v] = (uint32_t)(__ffsll(delta) - 1);
         io.Hc[v] = delta;
         io.Dcc[v] = (uint8_t)dcnt;
         const int counted = dcnt - (int)((delta >> top) & 1ULL);
-        stage_group<G>(io, v, deg, slot, dcnt, counted, hip_weight(k, k, sU[top]));
+        stage_group<G>(io, sh, v, deg, slot, dcnt, counted, hip_weight(k, k, rank_of(io, (uint32_t)top)));
     }
 }
 
 template <int G>
-__device__ __forceinline__ void flush_counters(const Grp<G>& g, HopCounters hc, Counters* ctr) {
+__device__ __forceinline__ void ctr_init(const Lock<G>& g, HopShared& sh) {
+    if (g.l == 0)
+        for (int i = 0; i < kNCtr; ++i) sh.ctr[threadIdx.x / G][i] = 0;
+    __syncwarp();
+}
+
+template <int G>
+__device__ __forceinline__ void flush_counters(const Lock<G>& g, const HopShared& sh, unsigned cand, Counters* ctr) {
     // candidate reads are counted per lane; the other counters by lane 0
+    unsigned long long reads = cand;
 #pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) hc.cand += g.shfl_xor(hc.cand, o);
+    for (int o = 16; o > 0; o >>= 1) reads += __shfl_xor_sync(kFull, reads, o);
+    if (lane_id() == 0 && reads) atomicAdd(&ctr->cand_reads, reads);
     if (g.l == 0) {
-        const unsigned* c = s_hop_ctr[threadIdx.x / G];
-        if (hc.cand) atomicAdd(&ctr->cand_reads, hc.cand);
+        const unsigned* c = sh.ctr[threadIdx.x / G];
         if (c[kCFront]) atomicAdd(&ctr->frontier, (unsigned long long)c[kCFront]);
         if (c[kCMerges]) atomicAdd(&ctr->merges, (unsigned long long)c[kCMerges]);
         if (c[kCMerging]) atomicAdd(&ctr->merging, (unsigned long long)c[kCMerging]);
@@ -622,241 +660,223 @@ __device__ __forceinline__ void flush_counters(const Grp<G>& g, HopCounters hc, 
     }
 }
 
-// U and the rank ids of its entries, staged in shared memory by every hop kernel.
-__device__ __forceinline__ void load_tables(uint64_t* sU, int32_t* sURid, const HopIO& io) {
-    for (int i = threadIdx.x; i < kUW; i += blockDim.x) {
-        sU[i] = io.U[i];
-        sURid[i] = io.URid[i];
-    }
-    __syncthreads();
-}
-
 // ------------------------------------------------------------------ hop kernels
 
 // Non-hub vertices: S_h(v) = bottom-k(S_{h-1}(v) U union_{u in N(v)} D_{h-1}(u)),
 // by the head merge (head vertices), the mask merge (other saturated
-// sketches) or the list merge.
+// sketches) or the list merge.  The groups of a warp take part in each merge
+// that one of them needs.
 template <int G>
 __global__ void __launch_bounds__(256, 4) k_hop_vertices(const int32_t* __restrict__ list, int64_t n_list, HopIO io) {
-    __shared__ uint64_t sU[kUW];
-    __shared__ int32_t sURid[kUW];
-    load_tables(sU, sURid, io);
-    const Grp<G> g;
+    __shared__ HopShared sh;
+    const Lock<G> g;
+    uint32_t* sx = sh.x[threadIdx.x >> 5];
     const int k = io.k;
     const int64_t groups = ((int64_t)gridDim.x * blockDim.x) / G;
-    HopCounters hc;
-    hop_ctr_init(g);
-    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G; i < n_list; i += groups) {
-        const int32_t v = list[i];
-        const int64_t beg = io.rowp[v], end = io.rowp[v + 1];
-        const uint64_t wv = io.hop > 1 ? io.W[v] : 0ULL;
+    unsigned cand = 0;
+    ctr_init(g, sh);
+    const int64_t first = ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) / G;  // the warp's first group
+    for (int64_t i0 = first; i0 < n_list; i0 += groups) {
+        const int64_t i = i0 + g.shift / G;
+        const bool on = i < n_list;
+        const int32_t v = on ? list[i] : 0;
+        const int64_t beg = on ? io.rowp[v] : 0, end = on ? io.rowp[v + 1] : 0;
+        const uint64_t wv = on && io.hop > 1 ? io.W[v] : 0ULL;
         bool front = false;
-        if (wv != 0) {
-            // head vertex: the head merge
-            const uint64_t acc = gather_heads(g, io, beg, end, front, hc.cand);
-            if (g.l == 0 && front) hop_ctr_add<G>(kCMerging, 1u);
-            const uint64_t nw = lowest_k64(wv | acc, k);
-            const uint64_t delta = nw & ~wv;
-            if (delta == 0) {
-                if (g.l == 0) io.stg_grp[i].info = 0;  // unchanged: empty slot
-                continue;
+        if (warp_any(wv != 0)) {
+            // head vertices: the head merge
+            const bool head = wv != 0;
+            const uint64_t acc = lock_or64(g, gather_heads(g, io, beg, head ? end : beg, front, cand));
+            if (head) {
+                const uint64_t nw = lowest_k64(wv | acc, k);
+                const uint64_t delta = nw & ~wv;
+                if (delta != 0) finish_head(g, io, sh, v, end - beg, nw, delta, i);
+                else if (g.l == 0) io.stg_grp[i].info = 0;  // unchanged: empty slot
             }
-            finish_head(g, io, v, end - beg, nw, delta, i, sU, sURid);
-            continue;
         }
-        const uint64_t old = g.l < k ? io.S[(int64_t)v * k + g.l] : kEmpty;
-        Sketch<G> s;
-        s.sk = old;
-        s.cnt = io.Scnt[v];
-        s.tau_base = kEmpty;
-        s.retau(g, k);
-        const bool sat = io.hop > 1 && s.cnt == k && s.tau <= io.ulim;
-        if (sat) {
-            // saturated: mask merge over the neighbours whose smallest new
-            // rank is below the k-th rank
-            const Mask4 first = gather_masks(g, io, beg, end, 0, front, hc.cand);
-            if (g.l == 0 && front) hop_ctr_add<G>(kCMerging, 1u);
-            if (!front) {
-                if (g.l == 0) io.stg_grp[i].info = 0;  // unchanged: empty slot
-                continue;
+        const bool rest = on && wv == 0;
+        if (warp_any(rest)) {
+            const uint32_t old = rest && g.l < k ? io.S[(int64_t)v * k + g.l] : kNil;
+            Sketch<G> s;
+            s.sk = old;
+            s.tau_base = kNil;
+            s.retau(g, k);
+            const bool sat = rest && io.hop > 1 && s.tau < (uint32_t)kUW;
+            if (warp_any(sat))  // saturated: mask merge
+                merge_slices(
+                    g, k, sat,
+                    [&](int q, uint32_t(&w)[kSliceWords]) { gather_slice(g, io, beg, end, q, w, front, cand); }, s.sk);
+            if (warp_any(rest && !sat)) {
+                s.retau(g, k);
+                gather_lists(g, io, beg, rest && !sat ? end : beg, s, front, cand, sx);
             }
-            const int idx = g.l < k ? u_pos(sU, io.ulim, old) : -1;
-            uint64_t sk_new;
-            bool fq;
-            const bool changed = merge_slices(
-                g, k, sU, idx, first, [&](int q) { return gather_masks(g, io, beg, end, q, fq, hc.cand); },
-                sk_new);
-            if (!changed) {
-                if (g.l == 0) io.stg_grp[i].info = 0;  // unchanged: empty slot
-                continue;
-            }
-            s.sk = sk_new;
-            s.cnt = k;
-        } else {
-            gather_range(g, io, beg, end, s, front, hc.cand);
-            if (g.l == 0 && front) hop_ctr_add<G>(kCMerging, 1u);
+            finish_vertex(g, io, sh, rest, v, end - beg, old, s.sk, i);
         }
-        finish_vertex(g, io, v, end - beg, old, s, i, sU);
+        if (g.ballot(front) != 0 && g.l == 0) sh.ctr[threadIdx.x / G][kCMerging] += 1u;
     }
-    flush_counters(g, hc, io.ctr);
+    __syncwarp();
+    flush_counters(g, sh, cand, io.ctr);
 }
 
 // Hub segments: partial results of one segment, written per segment -- the
 // OR of its neighbours' delta heads (head hubs), the slices of their delta
-// masks up to the hub's k-th rank (other saturated hubs), or the bottom-k of
-// its candidates below the hub's old k-th rank (list hubs).
+// masks up to the hub's k-th ordinal (other saturated hubs), or the bottom-k
+// of its candidates below the hub's old k-th ordinal (list hubs).
 template <int G>
 __global__ void __launch_bounds__(256) k_hop_hub_segments(const int32_t* __restrict__ hubs,
-                                                          const int64_t* __restrict__ hub_seg,
-                                                          const int32_t* __restrict__ seg_hub, int64_t n_seg,
-                                                          uint64_t* __restrict__ part, uint64_t* __restrict__ PM,
-                                                          uint64_t* __restrict__ PH, uint8_t* __restrict__ seg_flag,
-                                                          const uint32_t* __restrict__ hub_stamp, uint32_t sparse_hop,
-                                                          HopIO io) {
-    __shared__ uint64_t sU[kUW];
-    __shared__ int32_t sURid[kUW];
-    load_tables(sU, sURid, io);
-    const Grp<G> g;
+                                                             const int64_t* __restrict__ hub_seg,
+                                                             const int32_t* __restrict__ seg_hub, int64_t n_seg,
+                                                             uint32_t* __restrict__ part, uint32_t* __restrict__ PM,
+                                                             uint64_t* __restrict__ PH, uint8_t* __restrict__ seg_flag,
+                                                             const uint32_t* __restrict__ hub_stamp,
+                                                             uint32_t sparse_hop, HopIO io) {
+    __shared__ HopShared sh;
+    const Lock<G> g;
+    uint32_t* sx = sh.x[threadIdx.x >> 5];
     const int k = io.k;
     const int64_t groups = ((int64_t)gridDim.x * blockDim.x) / G;
-    HopCounters hc;
-    hop_ctr_init(g);
-    for (int64_t sidx = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G; sidx < n_seg; sidx += groups) {
-        const int32_t h = seg_hub[sidx];
-        const int32_t v = hubs[h];
-        if (sparse_hop && hub_stamp[v] != sparse_hop) {
+    unsigned cand = 0;
+    ctr_init(g, sh);
+    const int64_t first = ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) / G;
+    for (int64_t i0 = first; i0 < n_seg; i0 += groups) {
+        const int64_t sidx = i0 + g.shift / G;
+        bool on = sidx < n_seg;
+        const int32_t h = on ? seg_hub[sidx] : 0;
+        const int32_t v = on ? hubs[h] : 0;
+        if (on && sparse_hop && hub_stamp[v] != sparse_hop) {
             // sparse hop: no neighbour of this hub gained entries
             if (g.l == 0) seg_flag[sidx] = 0;
-            continue;
+            on = false;
         }
-        const int64_t e0 = io.rowp[v] + (sidx - hub_seg[h]) * kSeg;
-        const int64_t e1 = min(e0 + (int64_t)kSeg, io.rowp[v + 1]);
+        const int64_t e0 = on ? io.rowp[v] + (sidx - hub_seg[h]) * kSeg : 0;
+        const int64_t e1 = on ? min(e0 + (int64_t)kSeg, io.rowp[v + 1]) : 0;
+        const bool head = on && io.hop > 1 && io.W[v] != 0;
         bool front = false;
-        if (io.hop > 1 && io.W[v] != 0) {
-            const uint64_t acc = gather_heads(g, io, e0, e1, front, hc.cand);
-            if (g.l == 0) {
-                PH[sidx] = acc;
-                seg_flag[sidx] = front ? 1 : 0;
-            }
-            continue;
+        if (warp_any(head)) {
+            const uint64_t acc = lock_or64(g, gather_heads(g, io, e0, head ? e1 : e0, front, cand));
+            if (head && g.l == 0) PH[sidx] = acc;
         }
-        const uint64_t kth_old = io.S[(int64_t)v * k + k - 1];
-        const bool sat = io.hop > 1 && io.Scnt[v] == k && kth_old <= io.ulim;
-        if (sat) {
-            // saturated hub: partial masks of the segment, the slices up to
-            // the one holding the hub's k-th rank (the merge stops there)
-            const int top = u_pos(sU, io.ulim, kth_old) >> 8;
-            for (int q = 0; q <= top; ++q) {
-                bool fq;
-                const Mask4 m = gather_masks(g, io, e0, e1, q, fq, hc.cand);
-                if (q == 0) front = fq;
-                if (g.l < 4) PM[sidx * kUWords + q * 4 + g.l] = m.word(g.l);
+        const bool rest = on && !head;
+        if (warp_any(rest)) {
+            const uint32_t kth_old = rest ? io.S[(int64_t)v * k + k - 1] : kNil;  // kNil: not full
+            const bool sat = rest && io.hop > 1 && kth_old < (uint32_t)kUW;
+            if (warp_any(sat)) {
+                // saturated hub: partial masks of the segment, the slices up to
+                // the one holding the hub's k-th ordinal (the merge stops there)
+                const int top = sat ? (int)(kth_old >> 8) : -1;
+                for (int q = 0; warp_any(q <= top); ++q) {
+                    uint32_t w[kSliceWords];
+#pragma unroll
+                    for (int j = 0; j < kSliceWords; ++j) w[j] = 0u;
+                    if (q <= top) gather_slice(g, io, e0, e1, q, w, front, cand);
+                    const uint32_t r = slice_or(g, w);
+                    if (q <= top && g.l < kSliceWords) PM[sidx * 2 * kUWords + q * kSliceWords + g.l] = r;
+                }
             }
-            if (g.l == 0) seg_flag[sidx] = front ? 1 : 0;
-            continue;
+            if (warp_any(rest && !sat)) {
+                Sketch<G> s;
+                s.sk = kNil;
+                s.tau_base = kth_old;
+                s.tau = kth_old;
+                gather_lists(g, io, e0, rest && !sat ? e1 : e0, s, front, cand, sx);
+                if (rest && !sat && g.l < k) part[sidx * k + g.l] = s.sk;
+            }
         }
-        Sketch<G> s;
-        s.sk = kEmpty;
-        s.cnt = 0;
-        s.tau_base = io.Scnt[v] == k ? kth_old : kEmpty;
-        s.tau = s.tau_base;
-        gather_range(g, io, e0, e1, s, front, hc.cand);
-        if (g.l < k) part[sidx * k + g.l] = s.sk;
-        if (g.l == 0) seg_flag[sidx] = front ? 1 : 0;
+        const bool any = g.ballot(front) != 0;
+        if (on && g.l == 0) seg_flag[sidx] = any ? 1 : 0;
     }
-    flush_counters(g, hc, io.ctr);
-}
-
-// Did some segment of hub h have a neighbour that gained entries?
-template <int G>
-__device__ __forceinline__ bool hub_merged(const Grp<G>& g, const int64_t* __restrict__ hub_seg,
-                                           const uint8_t* __restrict__ seg_flag, int64_t h) {
-    bool any = false;
-    for (int64_t sidx = hub_seg[h] + g.l; sidx < hub_seg[h + 1]; sidx += G) any |= seg_flag[sidx] != 0;
-    return g.ballot(any) != 0;
+    __syncwarp();
+    flush_counters(g, sh, cand, io.ctr);
 }
 
 // Hubs: merge the partial results of all segments into the hub's sketch.
 template <int G>
 __global__ void __launch_bounds__(256) k_hop_hubs(const int32_t* __restrict__ hubs, int64_t n_hubs,
-                                                  const int64_t* __restrict__ hub_seg,
-                                                  const uint64_t* __restrict__ part, const uint64_t* __restrict__ PM,
-                                                  const uint64_t* __restrict__ PH,
-                                                  const uint8_t* __restrict__ seg_flag,
-                                                  const uint32_t* __restrict__ hub_stamp, uint32_t sparse_hop,
-                                                  int64_t slot0, HopIO io) {
-    __shared__ uint64_t sU[kUW];
-    __shared__ int32_t sURid[kUW];
-    load_tables(sU, sURid, io);
-    const Grp<G> g;
+                                                     const int64_t* __restrict__ hub_seg,
+                                                     const uint32_t* __restrict__ part, const uint32_t* __restrict__ PM,
+                                                     const uint64_t* __restrict__ PH,
+                                                     const uint8_t* __restrict__ seg_flag,
+                                                     const uint32_t* __restrict__ hub_stamp, uint32_t sparse_hop,
+                                                     int64_t slot0, HopIO io) {
+    __shared__ HopShared sh;
+    const Lock<G> g;
+    uint32_t* sx = sh.x[threadIdx.x >> 5];
     const int k = io.k;
     const int64_t groups = ((int64_t)gridDim.x * blockDim.x) / G;
-    HopCounters hc;
-    hop_ctr_init(g);
-    for (int64_t h = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G; h < n_hubs; h += groups) {
-        const int32_t v = hubs[h];
+    ctr_init(g, sh);
+    const int64_t first = ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) / G;
+    for (int64_t i0 = first; i0 < n_hubs; i0 += groups) {
+        const int64_t h = i0 + g.shift / G;
+        bool on = h < n_hubs;
+        const int32_t v = on ? hubs[h] : 0;
         const int64_t slot = slot0 + h;
-        if (sparse_hop && hub_stamp[v] != sparse_hop) {
+        if (on && sparse_hop && hub_stamp[v] != sparse_hop) {
             if (g.l == 0) io.stg_grp[slot].info = 0;  // unchanged: empty slot
-            continue;
+            on = false;
         }
-        const int64_t deg = io.rowp[v + 1] - io.rowp[v];
-        const bool any = hub_merged(g, hub_seg, seg_flag, h);
-        if (g.l == 0 && any) hop_ctr_add<G>(kCMerging, 1u);
-        const uint64_t wv = io.hop > 1 ? io.W[v] : 0ULL;
+        const int64_t deg = on ? io.rowp[v + 1] - io.rowp[v] : 0;
+        const int64_t s0 = on ? hub_seg[h] : 0, s1 = on ? hub_seg[h + 1] : 0;
+        bool any = false;
+        for (int64_t q = s0 + g.l; q < s1; q += G) any |= seg_flag[q] != 0;
+        any = g.ballot(any) != 0;
+        if (any && g.l == 0) sh.ctr[threadIdx.x / G][kCMerging] += 1u;
+        const uint64_t wv = on && io.hop > 1 ? io.W[v] : 0ULL;
         int dc = 0;
-        if (wv != 0) {
+        if (warp_any(wv != 0)) {
             uint64_t acc = 0;
-            for (int64_t sidx = hub_seg[h] + g.l; sidx < hub_seg[h + 1]; sidx += G) acc |= PH[sidx];
-            acc = grp_or64(g, acc);
-            const uint64_t nw = lowest_k64(wv | acc, k);
-            const uint64_t delta = nw & ~wv;
-            if (delta != 0) {
-                finish_head(g, io, v, deg, nw, delta, slot, sU, sURid);
+            if (wv != 0)
+                for (int64_t q = s0 + g.l; q < s1; q += G) acc |= PH[q];
+            acc = lock_or64(g, acc);
+            if (wv != 0) {
+                const uint64_t nw = lowest_k64(wv | acc, k);
+                const uint64_t delta = nw & ~wv;
+                if (delta != 0) finish_head(g, io, sh, v, deg, nw, delta, slot);
+                else if (g.l == 0) io.stg_grp[slot].info = 0;  // unchanged: empty slot
                 dc = __popcll(delta);
-            } else if (g.l == 0) {
-                io.stg_grp[slot].info = 0;  // unchanged: empty slot
             }
-        } else {
-            const uint64_t old = g.l < k ? io.S[(int64_t)v * k + g.l] : kEmpty;
+        }
+        const bool rest = on && wv == 0;
+        if (warp_any(rest)) {
+            const uint32_t old = rest && g.l < k ? io.S[(int64_t)v * k + g.l] : kNil;
             Sketch<G> s;
             s.sk = old;
-            s.cnt = io.Scnt[v];
-            s.tau_base = kEmpty;
+            s.tau_base = kNil;
             s.retau(g, k);
-            bool changed = true;
-            if (io.hop > 1 && s.cnt == k && s.tau <= io.ulim) {
-                // saturated hub: OR of the segments' partial masks
-                const int idx = g.l < k ? u_pos(sU, io.ulim, old) : -1;
-                auto part_slice = [&](int q) {
-                    Mask4 m;
-                    for (int64_t sidx = hub_seg[h] + g.l; sidx < hub_seg[h + 1]; sidx += G)
-                        m.load(PM + sidx * kUWords + q * 4);
-                    grp_or(g, m);
-                    return m;
-                };
-                uint64_t sk_new;
-                changed = merge_slices(g, k, sU, idx, part_slice(0), part_slice, sk_new);
-                s.sk = sk_new;
-                s.cnt = k;
-            } else {
-                for (int64_t sidx = hub_seg[h]; sidx < hub_seg[h + 1]; ++sidx) {
-                    const uint64_t x = g.l < k ? part[sidx * k + g.l] : kEmpty;
-                    absorb(g, k, x, s);
-                }
+            const bool sat = rest && io.hop > 1 && s.tau < (uint32_t)kUW;
+            if (warp_any(sat))  // saturated hub: OR of the segments' partial masks
+                merge_slices(
+                    g, k, sat,
+                    [&](int q, uint32_t(&w)[kSliceWords]) {
+                        for (int64_t x = s0 + g.l; x < s1; x += G) {
+                            const uint4* p = reinterpret_cast<const uint4*>(PM + x * 2 * kUWords + q * kSliceWords);
+                            const uint4 a = p[0], b = p[1];
+                            w[0] |= a.x;
+                            w[1] |= a.y;
+                            w[2] |= a.z;
+                            w[3] |= a.w;
+                            w[4] |= b.x;
+                            w[5] |= b.y;
+                            w[6] |= b.z;
+                            w[7] |= b.w;
+                        }
+                    },
+                    s.sk);
+            if (warp_any(rest && !sat)) {
+                s.retau(g, k);
+                const int64_t end = rest && !sat ? s1 : s0;
+                for (int64_t q = s0; warp_any(q < end); ++q)
+                    merge_list(g, k, q < end && g.l < k ? part[q * k + g.l] : kNil, s, sx);
             }
-            if (changed) {
-                dc = finish_vertex(g, io, v, deg, old, s, slot, sU);
-            } else if (g.l == 0) {
-                io.stg_grp[slot].info = 0;  // unchanged: empty slot
-            }
+            const int got = finish_vertex(g, io, sh, rest, v, deg, old, s.sk, slot);
+            if (rest) dc = got;
         }
         if (dc && g.l == 0) {
             atomicAdd(&io.ctr->merges, (unsigned long long)deg);
             atomicAdd(&io.ctr->delta_next, (unsigned long long)(deg * dc));
         }
     }
-    flush_counters(g, hc, io.ctr);
+    __syncwarp();
+    flush_counters(g, sh, 0u, io.ctr);
 }
 
 // Sparse hops: the non-hub part of N(frontier).  Warp per frontier vertex;
@@ -1051,8 +1071,7 @@ int build_work_lists(fl_graph* g) {
 // vertices, and of those whose sketch is saturated (read by the mask merge).
 // Runs before the hop kernels change the sketches.
 __global__ void k_hop_census(const int32_t* __restrict__ list, int64_t n_list, const int64_t* __restrict__ rowp,
-                             const uint64_t* __restrict__ S, const uint8_t* __restrict__ Scnt, int k, int hop,
-                             uint64_t ulim, const uint32_t* __restrict__ stamp, uint32_t sparse_hop, Counters* ctr) {
+                             const uint32_t* __restrict__ S, int k, int hop, const uint32_t* __restrict__ stamp, uint32_t sparse_hop, Counters* ctr) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     unsigned long long sc = 0, mk = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_list; i += stride) {
@@ -1060,7 +1079,7 @@ __global__ void k_hop_census(const int32_t* __restrict__ list, int64_t n_list, c
         if (sparse_hop && stamp[v] != sparse_hop) continue;  // a hub the hop skips
         const unsigned long long d = (unsigned long long)(rowp[v + 1] - rowp[v]);
         sc += d;
-        if (hop > 1 && Scnt[v] == k && S[(int64_t)v * k + k - 1] <= ulim) mk += d;
+        if (hop > 1 && S[(int64_t)v * k + k - 1] < (uint32_t)kUW) mk += d;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -1073,51 +1092,128 @@ __global__ void k_hop_census(const int32_t* __restrict__ list, int64_t n_list, c
     }
 }
 
-// ------------------------------------------------------------------ small-rank table
+// ------------------------------------------------------------------ ordinals
 
-constexpr int kSelCap = 4096;  // candidates sorted in one block
-
-// Ranks below T -> buf (first kSelCap of them); their number -> *cnt.
-__global__ void k_small_ranks(int64_t n, uint64_t seed, uint64_t T, IdMap ids,
-                              uint64_t* __restrict__ buf, unsigned long long* __restrict__ cnt) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += stride) {
-        const int64_t v = base + lane_id();
-        const uint64_t r = v < n ? vertex_rank(seed, rank_id(ids, v)) : kEmpty;
-        const long long at = warp_append(v < n && r < T, cnt);
-        if (at >= 0 && at < kSelCap) buf[at] = r;
-    }
-}
-
-// Sort the m <= kSelCap candidates (bitonic, one block) and keep the w smallest.
-__global__ void __launch_bounds__(1024) k_sort_small(const uint64_t* __restrict__ buf, int m, int w,
-                                                     uint64_t* __restrict__ U) {
-    __shared__ uint64_t a[kSelCap];
-    for (int i = threadIdx.x; i < kSelCap; i += blockDim.x) a[i] = i < m ? buf[i] : kEmpty;
-    __syncthreads();
-    for (int size = 2; size <= kSelCap; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int i = threadIdx.x; i < kSelCap; i += blockDim.x) {
-                const int j = i ^ stride;
-                if (j > i) {
-                    const bool asc = (i & size) == 0;
-                    const uint64_t x = a[i], y = a[j];
-                    if ((x > y) == asc) {
-                        a[i] = y;
-                        a[j] = x;
-                    }
-                }
-            }
-            __syncthreads();
+// Few ranks: each one's ordinal is the number of ranks below its own.  A block
+// places 64 ids, two per lane; its warps share the scan of all ranks, computed
+// into shared memory a tile at a time.  (Ranks are a bijection of the ids.)
+__global__ void __launch_bounds__(1024) k_ordinals_small(int m, uint64_t seed, int32_t* __restrict__ ord_rid,
+                                                         Counters* ctr) {
+    constexpr int kTile = 2048;
+    __shared__ uint64_t key[kTile];
+    __shared__ int below[32][64];
+    const int lane = lane_id(), warp = threadIdx.x >> 5;
+    const int i0 = blockIdx.x * 64 + lane, i1 = i0 + 32;
+    const uint64_t r0 = vertex_rank(seed, i0), r1 = vertex_rank(seed, i1);
+    int c0 = 0, c1 = 0;
+    for (int t = 0; t < m; t += kTile) {
+        const int cnt = min(kTile, m - t);
+        __syncthreads();
+        for (int j = threadIdx.x; j < cnt; j += 1024) key[j] = vertex_rank(seed, t + j);
+        __syncthreads();
+#pragma unroll 4
+        for (int j = warp; j < cnt; j += 32) {
+            const uint64_t x = key[j];
+            c0 += x < r0;
+            c1 += x < r1;
         }
     }
-    for (int i = threadIdx.x; i < kUW; i += blockDim.x) U[i] = i < w ? a[i] : kEmpty;
+    below[warp][lane] = c0;
+    below[warp][lane + 32] = c1;
+    __syncthreads();
+    if (threadIdx.x < 64) {
+        const int i = blockIdx.x * 64 + threadIdx.x;
+        int o = 0;
+        for (int w = 0; w < 32; ++w) o += below[w][threadIdx.x];
+        if (i < m) {
+            ord_rid[o] = i;
+            if (vertex_rank(seed, i) == kEmpty) atomicOr(&ctr->error, 1ULL);
+        }
+    }
 }
 
-// Rank id of the vertex of each rank of U (-1 for padding).
-__global__ void k_rank_ids(const uint64_t* __restrict__ U, int w, uint64_t seed, int32_t* __restrict__ URid) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < kUW) URid[i] = i < w ? (int32_t)rank_vertex(seed, U[i]) : -1;
+__global__ void k_rank_pairs(int64_t m, uint64_t seed, uint64_t* __restrict__ key, uint32_t* __restrict__ val,
+                             Counters* ctr) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += stride) {
+        const uint64_t r = vertex_rank(seed, i);
+        key[i] = r;
+        val[i] = (uint32_t)i;
+        if (r == kEmpty) atomicOr(&ctr->error, 1ULL);
+    }
+}
+
+// Ranks sorted by their bits from `shift` up: every id to its place, the few
+// runs that these bits leave equal in the order of the whole rank.
+__global__ void k_rank_place(const uint64_t* __restrict__ key, const uint32_t* __restrict__ val, int64_t m, int shift,
+                             int32_t* __restrict__ ord_rid) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += stride) {
+        const uint64_t r = key[i];
+        int64_t at = i;
+        for (int64_t j = i - 1; j >= 0 && (key[j] >> shift) == (r >> shift); --j) at -= key[j] > r;
+        for (int64_t j = i + 1; j < m && (key[j] >> shift) == (r >> shift); ++j) at += key[j] < r;
+        ord_rid[at] = (int32_t)val[i];
+    }
+}
+
+// ord[inv[rid]] = o (inv NULL: ord[rid] = o)
+__global__ void k_ord_scatter(const int32_t* __restrict__ ord_rid, int64_t m, const int32_t* __restrict__ inv,
+                              uint32_t* __restrict__ ord) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; o < m; o += stride) {
+        const int32_t r = ord_rid[o];
+        ord[inv ? inv[r] : r] = (uint32_t)o;
+    }
+}
+
+__global__ void k_ord_gather(const uint32_t* __restrict__ of_rid, const int32_t* __restrict__ rid, int64_t n,
+                             uint32_t* __restrict__ ord) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) ord[v] = of_rid[rid[v]];
+}
+
+// g->ord_rid and g->ord.  The rank ids of a union are its parts' local ids
+// (below the largest part's size).  A reserved rank sets ctr->error.  Scratch:
+// the delta masks, written later (128 bytes per vertex).
+static int build_ordinals(fl_graph* g) {
+    const int64_t n = g->n, m = g->max_part > 0 ? g->max_part : n;
+    cudaStream_t st = g->stream;
+    Counters* ctr = g->ctr.as<Counters>();
+    FL_TRY(dalloc(g->ord, (size_t)n * 4));
+    FL_TRY(dalloc(g->ord_rid, (size_t)m * 4));
+    int32_t* ord_rid = g->ord_rid.as<int32_t>();
+    if (m <= kCountMax) {
+        FL_LAUNCH(kProfSketchOther, k_ordinals_small<<<(unsigned)((m + 63) / 64), 1024, 0, st>>>((int)m, g->seed,
+                                                                                              ord_rid, ctr));
+    } else {
+        SortPairs<uint64_t> p;
+        p.key[0] = g->DM[0].as<uint64_t>();
+        p.key[1] = p.key[0] + m;
+        p.val[0] = reinterpret_cast<uint32_t*>(p.key[1] + m);
+        p.val[1] = p.val[0] + m;
+        int lg = 0, shift[kSortDigits];
+        while ((1LL << lg) < m) ++lg;
+        // equal leading lg + 16 bits: about m / 2^17 pairs
+        const int nd = digit_windows(~0ULL, lg + 16, shift);
+        FL_LAUNCH(kProfSketchOther, k_rank_pairs<<<grid_for(m, 256), 256, 0, st>>>(m, g->seed, p.key[0], p.val[0],
+                                                                                 ctr));
+        FL_TRY(sort_pairs(p, m, shift, nd, st, g->scratch, kProfSketchOther, &ctr->error));
+        FL_LAUNCH(kProfSketchOther, k_rank_place<<<grid_for(m, 256), 256, 0, st>>>(p.key[p.cur], p.val[p.cur], m,
+                                                                                 shift[0], ord_rid));
+    }
+    if (g->max_part > 0) {
+        uint32_t* of_rid = g->DM[1].as<uint32_t>();
+        FL_LAUNCH(kProfSketchOther, k_ord_scatter<<<grid_for(m, 256), 256, 0, st>>>(ord_rid, m, nullptr, of_rid));
+        FL_LAUNCH(kProfSketchOther, k_ord_gather<<<grid_for(n, 256), 256, 0, st>>>(of_rid, g->rid.as<int32_t>(), n,
+                                                                                 g->ord.as<uint32_t>()));
+    } else {
+        FL_LAUNCH(kProfSketchOther, k_ord_scatter<<<grid_for(m, 256), 256, 0, st>>>(
+                                        ord_rid, m, g->relabelled ? g->inv.as<int32_t>() : nullptr,
+                                        g->ord.as<uint32_t>()));
+    }
+    FL_CUDA(cudaGetLastError());
+    return FL_OK;
 }
 
 // The frontier of the previous hop as a bitmap: bit v = (Dcnt[v] > 0).
@@ -1128,54 +1224,6 @@ __global__ void k_front_bitmap(const uint8_t* __restrict__ Dcnt, int64_t n, uint
         const unsigned w = __ballot_sync(kFull, v < n && Dcnt[v] > 0);
         if (lane_id() == 0) bm[base >> 5] = w;
     }
-}
-
-// U = the min(kUW, n) smallest vertex ranks: collect the ranks below a
-// threshold expected to pass about 2048 of them (ranks are uniform), widen or
-// narrow it until between min(kUW, n) and kSelCap pass, then sort them.
-static int select_small_ranks(fl_graph* g) {
-    const int64_t n = g->n;
-    cudaStream_t st = g->stream;
-    const int w = (int)std::min<int64_t>(kUW, n);
-    DBuf buf;
-    FL_TRY(dalloc(buf, (size_t)kSelCap * 8 + 256));
-    unsigned long long* cnt = reinterpret_cast<unsigned long long*>(buf.as<char>() + (size_t)kSelCap * 8);
-    uint64_t T = n <= kSelCap / 2 ? kEmpty : (kEmpty / (uint64_t)n) * 2048ULL;
-    unsigned long long c = 0;
-    int rc = FL_OK;
-    for (int it = 0;; ++it) {
-        if (it > 130) { rc = FL_ECUDA; set_error(rc, "small-rank selection did not converge"); break; }
-        cudaError_t e = cudaMemsetAsync(cnt, 0, 8, st);
-        if (e != cudaSuccess) { rc = status_of(e, "small ranks", __FILE__, __LINE__); break; }
-        FL_LAUNCH(kProfSketchOther, k_small_ranks<<<grid_for(n, 256), 256, 0, st>>>(
-                                        n, g->seed, T, idmap_of(g),
-                                        buf.as<uint64_t>(), cnt));
-        e = cudaMemcpyAsync(&c, cnt, 8, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) { rc = status_of(e, "small ranks", __FILE__, __LINE__); break; }
-        if ((int64_t)c < w) {
-            T = T > kEmpty / 2 ? kEmpty : T * 2;
-            continue;
-        }
-        if (c > (unsigned long long)kSelCap) {
-            T = T / 4 * 3;
-            continue;
-        }
-        break;
-    }
-    if (rc == FL_OK) {
-        FL_LAUNCH(kProfSketchOther, k_sort_small<<<1, 1024, 0, st>>>(buf.as<uint64_t>(), (int)c, w,
-                                                                     g->U.as<uint64_t>()));
-        FL_LAUNCH(kProfSketchOther, k_rank_ids<<<(kUW + 255) / 256, 256, 0, st>>>(
-                                        g->U.as<uint64_t>(), w, g->seed, g->URid.as<int32_t>()));
-        cudaError_t e = cudaMemcpyAsync(&g->ulim, g->U.as<uint64_t>() + (w - 1), 8, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(&g->hlim, g->U.as<uint64_t>() + (std::min(w, 64) - 1), 8, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) rc = status_of(e, "small ranks", __FILE__, __LINE__);
-    }
-    dfree_after(st, {&buf});
-    return rc;
 }
 
 // ------------------------------------------------------------------ driver
@@ -1193,14 +1241,15 @@ static int launch_hop(fl_graph* g, int hop, const int32_t* list, int64_t n_list,
     io.k = k;
     io.hop = hop;
     io.seed = g->seed;
-    io.S = g->S.as<uint64_t>();
+    io.ord = g->ord.as<uint32_t>();
+    io.rid_of = g->ord_rid.as<int32_t>();
+    io.S = g->S.as<uint32_t>();
     io.Scnt = g->Scnt.as<uint8_t>();
-    io.Dp = g->D[pin].as<uint64_t>();
-    io.Dcp = g->Dcnt[pin].as<uint8_t>();
-    io.Dc = g->D[pout].as<uint64_t>();
+    io.Dp = g->D[pin].as<uint32_t>();
+    io.Dc = g->D[pout].as<uint32_t>();
     io.Dcc = g->Dcnt[pout].as<uint8_t>();
-    io.Fp = g->F[pin].as<uint64_t>();
-    io.Fc = g->F[pout].as<uint64_t>();
+    io.Fp = g->F[pin].as<uint32_t>();
+    io.Fc = g->F[pout].as<uint32_t>();
     io.Hp = g->H[pin].as<uint64_t>();
     io.Hc = g->H[pout].as<uint64_t>();
     io.W = g->W.as<uint64_t>();
@@ -1212,10 +1261,6 @@ static int launch_hop(fl_graph* g, int hop, const int32_t* list, int64_t n_list,
     io.ve = g->ve.as<int32_t>();
     io.stg_ent = g->stg_ent.as<int32_t>() + slot_base * k;
     io.stg_grp = g->stg_grp.as<StgGroup>() + slot_base;
-    io.U = g->U.as<uint64_t>();
-    io.URid = g->URid.as<int32_t>();
-    io.ulim = g->ulim;
-    io.hlim = g->hlim;
     io.ids = idmap_of(g);
     io.ctr = g->ctr.as<Counters>();
     if (n_list > 0)
@@ -1223,11 +1268,11 @@ static int launch_hop(fl_graph* g, int hop, const int32_t* list, int64_t n_list,
     if (g->n_hubs > 0) {
         FL_LAUNCH(kProfSketchMerge, k_hop_hub_segments<G><<<grid_for(g->n_seg, per_block), 256, 0, st>>>(
                                         g->hub_list.as<int32_t>(), g->hub_seg.as<int64_t>(), g->seg_hub.as<int32_t>(),
-                                        g->n_seg, g->part.as<uint64_t>(), g->PM.as<uint64_t>(), g->PH.as<uint64_t>(),
+                                        g->n_seg, g->part.as<uint32_t>(), g->PM.as<uint32_t>(), g->PH.as<uint64_t>(),
                                         g->seg_flag.as<uint8_t>(), g->stamp.as<uint32_t>(), sparse_hop, io));
         FL_LAUNCH(kProfSketchMerge, k_hop_hubs<G><<<grid_for(g->n_hubs, per_block), 256, 0, st>>>(
                                         g->hub_list.as<int32_t>(), g->n_hubs, g->hub_seg.as<int64_t>(),
-                                        g->part.as<uint64_t>(), g->PM.as<uint64_t>(), g->PH.as<uint64_t>(),
+                                        g->part.as<uint32_t>(), g->PM.as<uint32_t>(), g->PH.as<uint64_t>(),
                                         g->seg_flag.as<uint8_t>(), g->stamp.as<uint32_t>(), sparse_hop, n_list, io));
     }
     FL_CUDA(cudaGetLastError());
@@ -1256,30 +1301,28 @@ int build_sketches(fl_graph* g, int k, uint64_t seed) {
         g->lists_ready = 1;
     }
     const size_t nk = (size_t)n * k;
-    FL_TRY(dalloc(g->S, nk * 8));
+    FL_TRY(dalloc(g->S, nk * 4));
     FL_TRY(dalloc(g->Scnt, (size_t)n));
     for (int p = 0; p < 2; ++p) {
-        FL_TRY(dalloc(g->D[p], nk * 8));
+        FL_TRY(dalloc(g->D[p], nk * 4));
         FL_TRY(dalloc(g->Dcnt[p], (size_t)n));
         FL_TRY(dalloc(g->frontier[p], (size_t)n * 4));
     }
     FL_TRY(dalloc(g->stamp, (size_t)n * 4));
     FL_TRY(dalloc(g->vg, (size_t)n * 4));
     FL_TRY(dalloc(g->ve, (size_t)n * 4));
-    FL_TRY(dalloc(g->part, (size_t)std::max<int64_t>(g->n_seg, 1) * k * 8));
-    FL_TRY(dalloc(g->U, (size_t)kUW * 8));
+    FL_TRY(dalloc(g->part, (size_t)std::max<int64_t>(g->n_seg, 1) * k * 4));
     FL_TRY(dalloc(g->DM[0], (size_t)n * kUWords * 8));
     FL_TRY(dalloc(g->DM[1], (size_t)n * kUWords * 8));
     FL_TRY(dalloc(g->PM, (size_t)std::max<int64_t>(g->n_seg, 1) * kUWords * 8));
     FL_TRY(dalloc(g->PH, (size_t)std::max<int64_t>(g->n_seg, 1) * 8));
     FL_TRY(dalloc(g->seg_flag, (size_t)std::max<int64_t>(g->n_seg, 1)));
     for (int p = 0; p < 2; ++p) {
-        FL_TRY(dalloc(g->F[p], (size_t)n * 8));
+        FL_TRY(dalloc(g->F[p], (size_t)n * 4));
         FL_TRY(dalloc(g->H[p], (size_t)n * 8));
     }
     FL_TRY(dalloc(g->W, (size_t)n * 8));
     FL_TRY(dalloc(g->fbm, ((size_t)(n + 31) / 32 + 1) * 4));
-    FL_TRY(dalloc(g->URid, (size_t)kUW * 4));
     // staging: slots 0..n-1 for hop 0, then one slot per work item of each hop
     const int64_t per_dense = g->n_low + g->n_hubs;
     size_t slot_cap = (size_t)n + (size_t)per_dense * 8 + 1024;
@@ -1293,24 +1336,25 @@ int build_sketches(fl_graph* g, int k, uint64_t seed) {
     DBuf act;  // active list of sparse hops
     FL_TRY(dalloc(act, (size_t)n * 4));
 
-    FL_CUDA(cudaMemsetAsync(g->S.p, 0xff, nk * 8, st));
+    FL_CUDA(cudaMemsetAsync(g->S.p, 0xff, nk * 4, st));
     FL_CUDA(cudaMemsetAsync(g->W.p, 0, (size_t)n * 8, st));
     FL_CUDA(cudaMemsetAsync(g->stamp.p, 0, (size_t)n * 4, st));
     FL_CUDA(cudaMemsetAsync(g->ctr.p, 0, sizeof(Counters), st));
     {
-        int rc0 = select_small_ranks(g);
+        int rc0 = build_ordinals(g);
         if (rc0 != FL_OK) {
             dfree_after(st, {&act});
             return rc0;
         }
     }
     FL_LAUNCH(kProfSketchOther, k_rank_init<<<grid_for(n, 256), 256, 0, st>>>(
-                                    n, k, seed, g->S.as<uint64_t>(), g->Scnt.as<uint8_t>(), g->stg_grp.as<StgGroup>(),
-                                    g->vg.as<int32_t>(), g->ve.as<int32_t>(), idmap_of(g), g->ctr.as<Counters>()));
+                                    n, k, g->ord.as<uint32_t>(), g->S.as<uint32_t>(), g->Scnt.as<uint8_t>(),
+                                    g->stg_grp.as<StgGroup>(), g->vg.as<int32_t>(), g->ve.as<int32_t>()));
     FL_CUDA(cudaGetLastError());
     FL_TRY(read_counters(g));
     if (g->h_ctr->error) {
         dfree_after(st, {&act});
+        if (g->h_ctr->error & kSortError) FL_FAIL(FL_ETIMEOUT, "ordinals: a sort's wait ran out");
         FL_FAIL(FL_EINVAL, "a vertex rank equals the reserved empty-slot value; choose another seed");
     }
     g->hop_scanned.clear();
@@ -1367,7 +1411,7 @@ int build_sketches(fl_graph* g, int k, uint64_t seed) {
         }
         // this hop's outputs read "no new entries" for every vertex that does not change
         FL_CUDA(cudaMemsetAsync(g->Dcnt[pout].p, 0, (size_t)n, st));
-        FL_CUDA(cudaMemsetAsync(g->F[pout].p, 0xff, (size_t)n * 8, st));
+        FL_CUDA(cudaMemsetAsync(g->F[pout].p, 0xff, (size_t)n * 4, st));
         FL_CUDA(cudaMemsetAsync(g->H[pout].p, 0, (size_t)n * 8, st));
         if (hop > 1)
             FL_LAUNCH(kProfSketchOther, k_front_bitmap<<<grid_for(n, 256), 256, 0, st>>>(
@@ -1375,14 +1419,12 @@ int build_sketches(fl_graph* g, int k, uint64_t seed) {
         if (census) {
             if (n_list > 0)
                 FL_LAUNCH(kProfSketchOther, k_hop_census<<<grid_for(n_list, 256), 256, 0, st>>>(
-                                                list, n_list, g->rowp.as<int64_t>(), g->S.as<uint64_t>(),
-                                                g->Scnt.as<uint8_t>(), k, hop, g->ulim, nullptr, 0u,
-                                                g->ctr.as<Counters>()));
+                                                list, n_list, g->rowp.as<int64_t>(), g->S.as<uint32_t>(), k, hop,
+                                                nullptr, 0u, g->ctr.as<Counters>()));
             if (g->n_hubs > 0)
                 FL_LAUNCH(kProfSketchOther, k_hop_census<<<grid_for(g->n_hubs, 256), 256, 0, st>>>(
                                                 g->hub_list.as<int32_t>(), g->n_hubs, g->rowp.as<int64_t>(),
-                                                g->S.as<uint64_t>(), g->Scnt.as<uint8_t>(), k, hop, g->ulim,
-                                                g->stamp.as<uint32_t>(), dense ? 0u : (uint32_t)hop,
+                                                g->S.as<uint32_t>(), k, hop, g->stamp.as<uint32_t>(), dense ? 0u : (uint32_t)hop,
                                                 g->ctr.as<Counters>()));
         }
         if (time_hops) FL_CUDA(cudaEventRecord(g->hop_ev[0], st));
@@ -1473,17 +1515,17 @@ int build_sketches(fl_graph* g, int k, uint64_t seed) {
 }
 
 // ------------------------------------------------------------------ eccentricity bound
-// The minimum rank of a component (S[v][0] at the fixed point) names a root
+// The minimum ordinal of a component (S[v][0] at the fixed point) names a root
 // for every vertex of it; a multi-source BFS from the roots gives d(v, root)
 // and ecc(root), and ecc(v) <= d(v, root) + ecc(root).
 
-__global__ void k_roots(const uint64_t* __restrict__ S, int k, uint64_t seed, int64_t n,
-                        IdMap ids, int32_t* __restrict__ roots, Counters* ctr) {
+__global__ void k_roots(const uint32_t* __restrict__ S, int k, const uint32_t* __restrict__ ord, int64_t n,
+                        int32_t* __restrict__ roots, Counters* ctr) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += stride) {
         int64_t v = base + lane_id();
         bool is_root = false;
-        if (v < n) is_root = (int64_t)rank_vertex(seed, S[v * k]) == rank_id(ids, v);
+        if (v < n) is_root = S[v * k] == ord[v];
         long long at = warp_append(is_root, &ctr->aux0);
         if (at >= 0) roots[at] = (int32_t)v;
     }
@@ -1518,8 +1560,7 @@ int compute_ecc_bound(fl_graph* g) {
         if (e == cudaSuccess) e = cudaMemsetAsync(eccr.p, 0, (size_t)n * 4, st);
         if (e != cudaSuccess) { rc = status_of(e, "ecc init", __FILE__, __LINE__); break; }
         FL_LAUNCH(kProfSketchOther, k_roots<<<grid_for(n, 256), 256, 0, st>>>(
-                                        g->S.as<uint64_t>(), g->k, g->seed, n,
-                                        idmap_of(g), roots.as<int32_t>(),
+                                        g->S.as<uint32_t>(), g->k, g->ord.as<uint32_t>(), n, roots.as<int32_t>(),
                                         g->ctr.as<Counters>()));
         if ((rc = read_counters(g))) break;
         int64_t n_roots = (int64_t)g->h_ctr->aux0;
