@@ -37,7 +37,7 @@ void destroy_graph(fl_graph* g) {
                     &g->S, &g->Scnt, &g->D[0], &g->D[1], &g->Dcnt[0], &g->Dcnt[1], &g->frontier[0],
                     &g->frontier[1], &g->stamp, &g->vg, &g->ve, &g->stg_ent, &g->stg_grp, &g->gofs, &g->eofs,
                     &g->ginfo, &g->gwt, &g->eid, &g->ecc_ub, &g->ctr, &g->scratch,
-                    &g->relax_aux, &g->ord, &g->ord_rid, &g->DM[0], &g->DM[1], &g->PM, &g->seg_flag, &g->PH, &g->F[0], &g->F[1], &g->H[0],
+                    &g->relax_aux, &g->ord, &g->ord_rid, &g->ord_vid, &g->stg_kth, &g->DM[0], &g->DM[1], &g->PM, &g->seg_flag, &g->PH, &g->F[0], &g->F[1], &g->H[0],
                     &g->H[1], &g->W, &g->fbm, &g->vbase, &g->vpart, &g->rid,
                     &g->inv, &g->xbits, &g->xaux, &g->xio, &g->items};
     for (DBuf* b : bufs) dfree_idle(*b);

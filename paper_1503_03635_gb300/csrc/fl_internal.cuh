@@ -74,11 +74,6 @@ __device__ __forceinline__ int64_t rank_id(const IdMap& m, int64_t v) {
     return m.rid ? (int64_t)__ldg(&m.rid[v]) : v;
 }
 
-// Internal id of the vertex with rank id r, in the part of vertex v.
-__device__ __forceinline__ int64_t internal_of(const IdMap& m, int64_t r, int64_t v) {
-    return m.inv ? (int64_t)__ldg(&m.inv[r]) : (m.vbase ? r + (int64_t)__ldg(&m.vbase[v]) : r);
-}
-
 __host__ __device__ constexpr uint64_t inv_odd(uint64_t a) {
     // Newton iteration for the inverse of an odd number mod 2^64
     uint64_t x = a;
@@ -466,7 +461,7 @@ struct fl_graph {
     int64_t n_parts = 0;           // 0: not a union
     int64_t max_part = 0;          // union: vertices of the largest part
     fl::DBuf ord;                  // uint32[n]: ordinal of each vertex's rank (unions: among the local ids)
-    fl::DBuf ord_rid;              // int32: rank id of each ordinal
+    fl::DBuf ord_rid, ord_vid;     // int32: rank id and vertex (unions: local id) of each ordinal
     fl::DBuf DM[2];                // uint64[kUSlices][n][4]: hop delta masks, slice-major
     fl::DBuf PM;                   // uint64[n_seg*kUWords]: partial masks of hub segments (scratch)
     fl::DBuf seg_flag;             // uint8[n_seg]: the segment had a neighbour that gained entries (scratch)
@@ -485,7 +480,7 @@ struct fl_graph {
     fl::DBuf frontier[2];          // int32[n]
     fl::DBuf stamp;                // uint32[n]
     fl::DBuf vg, ve;               // int32[n] per-vertex running group / entry counts
-    fl::DBuf stg_ent;              // int32 staging entries (k per slot)
+    fl::DBuf stg_ent, stg_kth;     // uint32 staging entries (k per slot), k-th ordinals (one per slot)
     fl::DBuf stg_grp;              // staging group records (one per slot)
     size_t stg_grp_cap = 0;        // slots
     int stg_k = 0;

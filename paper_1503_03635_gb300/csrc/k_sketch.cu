@@ -15,9 +15,10 @@
 //   Scnt[v]           number of ordinals in S[v]
 //   D[p][v*k + i]     entries v gained at the previous / current hop, kNil padding
 //   Dcnt[p][v]        their number (0 = v is not in the frontier)
-//   staging           one group slot per work item of every hop (v, hop, HIP
-//                     weight, counts) and k entry slots; compacted into the
-//                     vertex-major ADS after the last hop
+//   staging           one group slot per work item of every hop >= 1 (v, hop,
+//                     counts, the sketch's k-th ordinal) and k entry slots
+//                     (ordinals); compacted into the vertex-major ADS, with
+//                     HIP weights and vertex ids, after the last hop
 //
 // Work decomposition of one hop.  A group of G lanes (G = 16 when k <= 16,
 // else 32) owns one vertex: lane i holds S[v][i].  Non-hub vertices are
@@ -32,7 +33,9 @@
 // word in the mask and head merges.  Per build, against 64-bit ranks and
 // half-warp groups that diverged: non-hub vertices of R-MAT 24 (k = 16) 49.2
 // -> 32.1 ms, hub segments 9.8 -> 7.1; R-MAT 20 (k = 32) 5.4 -> 3.6; 64
-// Erdos-Renyi graphs (k = 32) 14.9 -> 7.0.  The sort of the ranks adds 0.3 ms
+// Erdos-Renyi graphs (k = 32) 14.9 -> 7.0.  With weights and ids left to the
+// compaction and six blocks per SM in place of four (latency of the gathers):
+// 25.5, 2.9 and 6.0 ms.  The sort of the ranks adds 0.3 ms
 // at 2^20 vertices, 2.0 at 2^24.
 #include <algorithm>
 #include <cstdio>
@@ -42,8 +45,9 @@
 
 namespace fl {
 
-struct StgGroup {
-    double wt;      // HIP weight of the counted entries
+// A staged group; its HIP weight is computed at the compaction from its
+// sketch's k-th ordinal (kNil: fewer than k entries), kept beside it.
+struct __align__(16) StgGroup {
     int32_t v;      // vertex
     int32_t gidx;   // index of this group among v's groups
     int32_t eidx;   // index of its first entry among v's entries
@@ -227,9 +231,7 @@ struct HopIO {
     const int32_t* __restrict__ cols;
     int k;
     int hop;
-    uint64_t seed;
     const uint32_t* __restrict__ ord;        // ordinal of each vertex
-    const int32_t* __restrict__ rid_of;      // rank id of each ordinal
     uint32_t* __restrict__ S;
     uint8_t* __restrict__ Scnt;
     const uint32_t* __restrict__ Dp;
@@ -246,9 +248,9 @@ struct HopIO {
     int64_t n;
     int32_t* __restrict__ vg;
     int32_t* __restrict__ ve;
-    int32_t* __restrict__ stg_ent;
+    uint32_t* __restrict__ stg_ent;
+    uint32_t* __restrict__ stg_kth;
     StgGroup* __restrict__ stg_grp;
-    IdMap ids;
     Counters* ctr;
 };
 
@@ -336,23 +338,15 @@ __device__ __forceinline__ uint64_t gather_heads(const Lock<G>& g, const HopIO& 
 
 // ------------------------------------------------------------------ hop 0
 
-// Hop 0: S_0(v) = {ord(v)} and v's ADS group at distance 0.  (Hop 1 reads the
-// neighbours' ordinals, so no hop-0 delta list or mask is stored; the group's
-// single entry is v itself, written by the compaction.)
+// Hop 0: S_0(v) = {ord(v)}.  (Hop 1 reads the neighbours' ordinals, so no
+// hop-0 delta list or mask is stored; v's group at distance 0, the entry v
+// alone, is written by the compaction.)
 __global__ void k_rank_init(int64_t n, int k, const uint32_t* __restrict__ ord, uint32_t* __restrict__ S,
-                            uint8_t* __restrict__ Scnt, StgGroup* __restrict__ stg_grp,
-                            int32_t* __restrict__ vg, int32_t* __restrict__ ve) {
+                            uint8_t* __restrict__ Scnt, int32_t* __restrict__ vg, int32_t* __restrict__ ve) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
         S[v * k] = ord[v];
         Scnt[v] = 1;
-        StgGroup gr;
-        gr.wt = 1.0;  // a one-vertex ball: fewer than k ranks (k >= 2)
-        gr.v = (int32_t)v;
-        gr.gidx = 0;
-        gr.eidx = 0;
-        gr.info = pack_info(0, 1, 1);
-        stg_grp[v] = gr;
         vg[v] = 1;
         ve[v] = 1;
     }
@@ -524,9 +518,8 @@ __device__ __forceinline__ void merge_slices(const Lock<G>& g, int k, bool on, S
 // (lane 0 of the group).
 template <int G>
 __device__ __forceinline__ void stage_group(const HopIO& io, HopShared& sh, int32_t v, int64_t deg, int64_t slot,
-                                            int dcnt, int counted, double wt) {
+                                            int dcnt, int counted, uint32_t kth) {
     StgGroup gr;
-    gr.wt = wt;
     gr.v = v;
     gr.gidx = io.vg[v];
     gr.eidx = io.ve[v];
@@ -534,6 +527,7 @@ __device__ __forceinline__ void stage_group(const HopIO& io, HopShared& sh, int3
     io.vg[v] = gr.gidx + 1;
     io.ve[v] = gr.eidx + dcnt;
     io.stg_grp[slot] = gr;
+    io.stg_kth[slot] = kth;
     unsigned* c = sh.ctr[threadIdx.x / G];
     c[kCFront] += 1u;
     c[kCNew] += (unsigned)dcnt;
@@ -541,14 +535,6 @@ __device__ __forceinline__ void stage_group(const HopIO& io, HopShared& sh, int3
         c[kCMerges] += (unsigned)deg;
         c[kCDelta] += (unsigned)(deg * dcnt);
     }
-}
-
-// Rank of the vertex with ordinal o, and that vertex in v's part.
-__device__ __forceinline__ uint64_t rank_of(const HopIO& io, uint32_t o) {
-    return vertex_rank(io.seed, (int64_t)__ldg(&io.rid_of[o]));
-}
-__device__ __forceinline__ int32_t vertex_of(const HopIO& io, uint32_t o, int32_t v) {
-    return (int32_t)internal_of(io.ids, (int64_t)__ldg(&io.rid_of[o]), v);
 }
 
 // Write the results of vertex v (groups that are `on`) after a list or slice
@@ -579,7 +565,7 @@ __device__ __forceinline__ int finish_vertex(const Lock<G>& g, const HopIO& io, 
         if (is_new) {
             const int at = __popc(newm & g.below());
             io.Dc[(int64_t)v * k + at] = sk;
-            io.stg_ent[slot * k + at] = vertex_of(io, sk, v);
+            io.stg_ent[slot * k + at] = sk;
         }
         if (g.l < k && g.l >= dcnt) io.Dc[(int64_t)v * k + g.l] = kNil;
         if (g.l < kUWords)
@@ -600,8 +586,7 @@ __device__ __forceinline__ int finish_vertex(const Lock<G>& g, const HopIO& io, 
         io.Scnt[v] = (uint8_t)cnt_new;
         io.Dcc[v] = (uint8_t)dcnt;
         const int counted = cnt_new < k ? dcnt : __popc(newm & ((1u << (k - 1)) - 1u));
-        stage_group<G>(io, sh, v, deg, slot, dcnt, counted,
-                       cnt_new < k ? 1.0 : hip_weight(cnt_new, k, rank_of(io, kth)));
+        stage_group<G>(io, sh, v, deg, slot, dcnt, counted, kth);
     }
     __syncwarp();
     return dcnt;
@@ -620,7 +605,7 @@ __device__ __forceinline__ void finish_head(const Lock<G>& g, const HopIO& io, H
         uint32_t x = kNil;
         if (g.l < dcnt) {
             x = (uint32_t)nth_bit64(delta, g.l);
-            io.stg_ent[slot * k + g.l] = vertex_of(io, x, v);
+            io.stg_ent[slot * k + g.l] = x;
         }
         io.Dc[(int64_t)v * k + g.l] = x;
     }
@@ -632,7 +617,7 @@ __device__ __forceinline__ void finish_head(const Lock<G>& g, const HopIO& io, H
         io.Hc[v] = delta;
         io.Dcc[v] = (uint8_t)dcnt;
         const int counted = dcnt - (int)((delta >> top) & 1ULL);
-        stage_group<G>(io, sh, v, deg, slot, dcnt, counted, hip_weight(k, k, rank_of(io, (uint32_t)top)));
+        stage_group<G>(io, sh, v, deg, slot, dcnt, counted, (uint32_t)top);
     }
 }
 
@@ -667,7 +652,7 @@ __device__ __forceinline__ void flush_counters(const Lock<G>& g, const HopShared
 // sketches) or the list merge.  The groups of a warp take part in each merge
 // that one of them needs.
 template <int G>
-__global__ void __launch_bounds__(256, 4) k_hop_vertices(const int32_t* __restrict__ list, int64_t n_list, HopIO io) {
+__global__ void __launch_bounds__(256, 6) k_hop_vertices(const int32_t* __restrict__ list, int64_t n_list, HopIO io) {
     __shared__ HopShared sh;
     const Lock<G> g;
     uint32_t* sx = sh.x[threadIdx.x >> 5];
@@ -676,11 +661,16 @@ __global__ void __launch_bounds__(256, 4) k_hop_vertices(const int32_t* __restri
     unsigned cand = 0;
     ctr_init(g, sh);
     const int64_t first = ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) / G;  // the warp's first group
+    // the next vertex's id and row are loaded while this one merges
+    const int64_t at0 = first + g.shift / G;
+    int32_t v_next = at0 < n_list ? list[at0] : 0;
+    int64_t beg_next = at0 < n_list ? io.rowp[v_next] : 0, end_next = at0 < n_list ? io.rowp[v_next + 1] : 0;
     for (int64_t i0 = first; i0 < n_list; i0 += groups) {
         const int64_t i = i0 + g.shift / G;
-        const bool on = i < n_list;
-        const int32_t v = on ? list[i] : 0;
-        const int64_t beg = on ? io.rowp[v] : 0, end = on ? io.rowp[v + 1] : 0;
+        const bool on = i < n_list, more = i + groups < n_list;
+        const int32_t v = v_next;
+        const int64_t beg = beg_next, end = end_next;
+        v_next = more ? list[i + groups] : 0;
         const uint64_t wv = on && io.hop > 1 ? io.W[v] : 0ULL;
         bool front = false;
         if (warp_any(wv != 0)) {
@@ -710,7 +700,12 @@ __global__ void __launch_bounds__(256, 4) k_hop_vertices(const int32_t* __restri
                 s.retau(g, k);
                 gather_lists(g, io, beg, rest && !sat ? end : beg, s, front, cand, sx);
             }
+            beg_next = more ? io.rowp[v_next] : 0;
+            end_next = more ? io.rowp[v_next + 1] : 0;
             finish_vertex(g, io, sh, rest, v, end - beg, old, s.sk, i);
+        } else {
+            beg_next = more ? io.rowp[v_next] : 0;
+            end_next = more ? io.rowp[v_next + 1] : 0;
         }
         if (g.ballot(front) != 0 && g.l == 0) sh.ctr[threadIdx.x / G][kCMerging] += 1u;
     }
@@ -922,30 +917,67 @@ __global__ void k_collect_frontier(const int32_t* __restrict__ list, int64_t n, 
 
 // ------------------------------------------------------------------ ADS compaction
 
-// Staged groups -> vertex-major ADS.  kp = k rounded up to a power of two; a
-// thread per (slot, entry) pair, so that a slot's entries are copied by
-// adjacent threads (coalesced); the first thread of a slot writes the group.
-// In the hop-0 region the single entry of slot v is v itself.
-__global__ void k_ads_scatter(const StgGroup* __restrict__ stg_grp, int64_t n_slots, int64_t slot_base, int k,
-                              int log2_kp, bool hop0, const int32_t* __restrict__ stg_ent,
-                              const int64_t* __restrict__ gofs, const int64_t* __restrict__ eofs,
-                              uint32_t* __restrict__ ginfo, double* __restrict__ gwt, int32_t* __restrict__ eid) {
+// v's group at distance 0: the entry v alone, a ball of one vertex (k >= 2).
+__global__ void k_ads_hop0(int64_t n, const int64_t* __restrict__ gofs, const int64_t* __restrict__ eofs,
+                           uint32_t* __restrict__ ginfo, double* __restrict__ gwt, int32_t* __restrict__ eid) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int64_t total = n_slots << log2_kp;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += stride) {
-        const int64_t i = t >> log2_kp;
-        const int j = (int)(t & ((1 << log2_kp) - 1));
-        const StgGroup gr = stg_grp[slot_base + i];
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
+        ginfo[gofs[v]] = pack_info(0, 1, 1);
+        gwt[gofs[v]] = 1.0;
+        eid[eofs[v]] = (int32_t)v;
+    }
+}
+
+// Staged groups -> vertex-major ADS, a thread per slot: the group's words and
+// its HIP weight.  (The weight's FP64 division runs on all lanes here; on the
+// one lane per vertex of a hop kernel it kept the FP64 pipe 25-40 % busy.)
+__global__ void k_ads_groups(const StgGroup* __restrict__ stg_grp, const uint32_t* __restrict__ stg_kth,
+                             int64_t n_slots, int k, uint64_t seed, const int32_t* __restrict__ ord_rid,
+                             const int64_t* __restrict__ gofs, uint32_t* __restrict__ ginfo,
+                             double* __restrict__ gwt) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_slots; i += stride) {
+        const StgGroup gr = stg_grp[i];
         if (gr.info == 0) continue;
-        const int cnt = (int)((gr.info >> 16) & 0xff);
-        if (j >= cnt) continue;
-        const int64_t de = eofs[gr.v] + gr.eidx;
-        if (j == 0) {
-            const int64_t dg = gofs[gr.v] + gr.gidx;
-            ginfo[dg] = gr.info;
-            gwt[dg] = gr.wt;
+        const uint32_t kth = stg_kth[i];
+        const int64_t at = gofs[gr.v] + gr.gidx;
+        ginfo[at] = gr.info;
+        gwt[at] = kth == kNil ? 1.0 : hip_weight(k, k, vertex_rank(seed, (int64_t)__ldg(&ord_rid[kth])));
+    }
+}
+
+// Their entries; vid = vertex of each ordinal, a local id in a union.  A warp
+// takes 32 slots and copies their entries end to end, 32 per pass (a lane finds
+// its slot among the running counts): most slots hold far fewer than k entries
+// and many none, so a thread per entry slot was bound by instructions
+// (R-MAT 24, 416 M entries: 3.1 ms).
+__global__ void __launch_bounds__(256) k_ads_entries(const StgGroup* __restrict__ stg_grp, int64_t n_slots, int k,
+                                                     const uint32_t* __restrict__ stg_ent,
+                                                     const int64_t* __restrict__ eofs,
+                                                     const int32_t* __restrict__ vid,
+                                                     const int32_t* __restrict__ vbase, int32_t* __restrict__ eid) {
+    const int lane = lane_id();
+    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t b = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; b < n_slots; b += warps * 32) {
+        StgGroup gr;
+        gr.info = 0;
+        if (b + lane < n_slots) gr = stg_grp[b + lane];
+        const int cnt = (int)((gr.info >> 16) & 0xff);  // 0 for an empty slot
+        const int incl = warp_incl_scan(cnt);
+        const int total = __shfl_sync(kFull, incl, 31);
+        const int64_t dst = cnt ? eofs[gr.v] + gr.eidx : 0;
+        const int32_t base = cnt && vbase ? vbase[gr.v] : 0;
+        for (int p = 0; p < total; p += 32) {
+            const int j = p + lane;
+            int w = 0;  // the slots whose entries all come before the j-th
+#pragma unroll
+            for (int s = 16; s > 0; s >>= 1)
+                if (__shfl_sync(kFull, incl, w + s - 1) <= j) w += s;
+            const int off = j - __shfl_sync(kFull, incl - cnt, w);
+            const int64_t to = __shfl_sync(kFull, dst, w);
+            const int32_t add = __shfl_sync(kFull, base, w);
+            if (j < total) eid[to + off] = __ldg(&vid[stg_ent[(b + w) * k + off]]) + add;
         }
-        eid[de + j] = hop0 ? gr.v : stg_ent[(slot_base + i) * k + j];
     }
 }
 
@@ -1157,13 +1189,14 @@ __global__ void k_rank_place(const uint64_t* __restrict__ key, const uint32_t* _
     }
 }
 
-// ord[inv[rid]] = o (inv NULL: ord[rid] = o)
+// vid[o] = inv[rid], the vertex of ordinal o, and ord[vid[o]] = o (inv NULL: vid = rid)
 __global__ void k_ord_scatter(const int32_t* __restrict__ ord_rid, int64_t m, const int32_t* __restrict__ inv,
-                              uint32_t* __restrict__ ord) {
+                              int32_t* __restrict__ vid, uint32_t* __restrict__ ord) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; o < m; o += stride) {
-        const int32_t r = ord_rid[o];
-        ord[inv ? inv[r] : r] = (uint32_t)o;
+        const int32_t v = inv ? inv[ord_rid[o]] : ord_rid[o];
+        vid[o] = v;
+        ord[v] = (uint32_t)o;
     }
 }
 
@@ -1173,7 +1206,7 @@ __global__ void k_ord_gather(const uint32_t* __restrict__ of_rid, const int32_t*
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) ord[v] = of_rid[rid[v]];
 }
 
-// g->ord_rid and g->ord.  The rank ids of a union are its parts' local ids
+// g->ord_rid, g->ord_vid and g->ord.  The rank ids of a union are its parts' local ids
 // (below the largest part's size).  A reserved rank sets ctr->error.  Scratch:
 // the delta masks, written later (128 bytes per vertex).
 static int build_ordinals(fl_graph* g) {
@@ -1182,6 +1215,7 @@ static int build_ordinals(fl_graph* g) {
     Counters* ctr = g->ctr.as<Counters>();
     FL_TRY(dalloc(g->ord, (size_t)n * 4));
     FL_TRY(dalloc(g->ord_rid, (size_t)m * 4));
+    FL_TRY(dalloc(g->ord_vid, (size_t)m * 4));
     int32_t* ord_rid = g->ord_rid.as<int32_t>();
     if (m <= kCountMax) {
         FL_LAUNCH(kProfSketchOther, k_ordinals_small<<<(unsigned)((m + 63) / 64), 1024, 0, st>>>((int)m, g->seed,
@@ -1204,13 +1238,14 @@ static int build_ordinals(fl_graph* g) {
     }
     if (g->max_part > 0) {
         uint32_t* of_rid = g->DM[1].as<uint32_t>();
-        FL_LAUNCH(kProfSketchOther, k_ord_scatter<<<grid_for(m, 256), 256, 0, st>>>(ord_rid, m, nullptr, of_rid));
+        FL_LAUNCH(kProfSketchOther, k_ord_scatter<<<grid_for(m, 256), 256, 0, st>>>(ord_rid, m, nullptr,
+                                                                                  g->ord_vid.as<int32_t>(), of_rid));
         FL_LAUNCH(kProfSketchOther, k_ord_gather<<<grid_for(n, 256), 256, 0, st>>>(of_rid, g->rid.as<int32_t>(), n,
                                                                                  g->ord.as<uint32_t>()));
     } else {
         FL_LAUNCH(kProfSketchOther, k_ord_scatter<<<grid_for(m, 256), 256, 0, st>>>(
                                         ord_rid, m, g->relabelled ? g->inv.as<int32_t>() : nullptr,
-                                        g->ord.as<uint32_t>()));
+                                        g->ord_vid.as<int32_t>(), g->ord.as<uint32_t>()));
     }
     FL_CUDA(cudaGetLastError());
     return FL_OK;
@@ -1240,9 +1275,7 @@ static int launch_hop(fl_graph* g, int hop, const int32_t* list, int64_t n_list,
     io.cols = g->cols.as<int32_t>();
     io.k = k;
     io.hop = hop;
-    io.seed = g->seed;
     io.ord = g->ord.as<uint32_t>();
-    io.rid_of = g->ord_rid.as<int32_t>();
     io.S = g->S.as<uint32_t>();
     io.Scnt = g->Scnt.as<uint8_t>();
     io.Dp = g->D[pin].as<uint32_t>();
@@ -1259,9 +1292,9 @@ static int launch_hop(fl_graph* g, int hop, const int32_t* list, int64_t n_list,
     io.n = g->n;
     io.vg = g->vg.as<int32_t>();
     io.ve = g->ve.as<int32_t>();
-    io.stg_ent = g->stg_ent.as<int32_t>() + slot_base * k;
+    io.stg_ent = g->stg_ent.as<uint32_t>() + slot_base * k;
+    io.stg_kth = g->stg_kth.as<uint32_t>() + slot_base;
     io.stg_grp = g->stg_grp.as<StgGroup>() + slot_base;
-    io.ids = idmap_of(g);
     io.ctr = g->ctr.as<Counters>();
     if (n_list > 0)
         FL_LAUNCH(kProfSketchMerge, k_hop_vertices<G><<<grid_for(n_list, per_block), 256, 0, st>>>(list, n_list, io));
@@ -1323,12 +1356,13 @@ int build_sketches(fl_graph* g, int k, uint64_t seed) {
     }
     FL_TRY(dalloc(g->W, (size_t)n * 8));
     FL_TRY(dalloc(g->fbm, ((size_t)(n + 31) / 32 + 1) * 4));
-    // staging: slots 0..n-1 for hop 0, then one slot per work item of each hop
+    // staging: one slot per work item of each hop
     const int64_t per_dense = g->n_low + g->n_hubs;
-    size_t slot_cap = (size_t)n + (size_t)per_dense * 8 + 1024;
+    size_t slot_cap = (size_t)per_dense * 8 + 1024;
     if (g->stg_grp_cap < slot_cap || g->stg_k != k) {
         slot_cap = std::max(slot_cap, g->stg_grp_cap);
         FL_TRY(dalloc(g->stg_grp, slot_cap * sizeof(StgGroup)));
+        FL_TRY(dalloc(g->stg_kth, slot_cap * 4));
         FL_TRY(dalloc(g->stg_ent, slot_cap * k * 4));
         g->stg_grp_cap = slot_cap;
         g->stg_k = k;
@@ -1349,7 +1383,7 @@ int build_sketches(fl_graph* g, int k, uint64_t seed) {
     }
     FL_LAUNCH(kProfSketchOther, k_rank_init<<<grid_for(n, 256), 256, 0, st>>>(
                                     n, k, g->ord.as<uint32_t>(), g->S.as<uint32_t>(), g->Scnt.as<uint8_t>(),
-                                    g->stg_grp.as<StgGroup>(), g->vg.as<int32_t>(), g->ve.as<int32_t>()));
+                                    g->vg.as<int32_t>(), g->ve.as<int32_t>()));
     FL_CUDA(cudaGetLastError());
     FL_TRY(read_counters(g));
     if (g->h_ctr->error) {
@@ -1368,9 +1402,7 @@ int build_sketches(fl_graph* g, int k, uint64_t seed) {
         FL_CUDA(cudaEventCreate(&g->hop_ev[0]));
         FL_CUDA(cudaEventCreate(&g->hop_ev[1]));
     }
-    std::vector<std::pair<int64_t, int64_t>> regions;  // (slot base, slots) of each hop
-    regions.push_back({0, n});
-    int64_t used_slots = n;
+    int64_t used_slots = 0;
     int64_t n_front = n;  // hop 0: every vertex gained its own rank
     bool fr_list_ready = false;
     // hop 1: every vertex gained its own rank at hop 0, so each CSR entry is
@@ -1406,6 +1438,7 @@ int build_sketches(fl_graph* g, int k, uint64_t seed) {
         if ((size_t)(used_slots + slots) > g->stg_grp_cap) {
             size_t cap = std::max<size_t>((size_t)(used_slots + slots), g->stg_grp_cap * 3 / 2);
             FL_TRY(dgrow(g->stg_grp, cap * sizeof(StgGroup), (size_t)used_slots * sizeof(StgGroup), st));
+            FL_TRY(dgrow(g->stg_kth, cap * 4, (size_t)used_slots * 4, st));
             FL_TRY(dgrow(g->stg_ent, cap * k * 4, (size_t)used_slots * k * 4, st));
             g->stg_grp_cap = cap;
         }
@@ -1433,7 +1466,6 @@ int build_sketches(fl_graph* g, int k, uint64_t seed) {
         else
             FL_TRY(launch_hop<32>(g, hop, list, n_list, pin, pout, used_slots, !dense));
         if (time_hops) FL_CUDA(cudaEventRecord(g->hop_ev[1], st));
-        regions.push_back({used_slots, slots});
         used_slots += slots;
         FL_TRY(read_counters(g));
         {
@@ -1496,17 +1528,19 @@ int build_sketches(fl_graph* g, int k, uint64_t seed) {
     FL_TRY(dalloc(g->eid, (size_t)std::max<int64_t>(g->n_entries, 1) * 4));
     FL_CUDA(cudaMemcpyAsync(g->gofs.as<int64_t>() + n, &g->n_groups, 8, cudaMemcpyHostToDevice, st));
     FL_CUDA(cudaMemcpyAsync(g->eofs.as<int64_t>() + n, &g->n_entries, 8, cudaMemcpyHostToDevice, st));
-    int log2_kp = 0;
-    while ((1 << log2_kp) < k) ++log2_kp;
-    for (const auto& r : regions)
-        if (r.second > 0) {
-            const bool hop0 = r.first == 0;
-            const int lk = hop0 ? 0 : log2_kp;
-            FL_LAUNCH(kProfSketchOther, k_ads_scatter<<<grid_for(r.second << lk, 256), 256, 0, st>>>(
-                                            g->stg_grp.as<StgGroup>(), r.second, r.first, k, lk, hop0,
-                                            g->stg_ent.as<int32_t>(), g->gofs.as<int64_t>(), g->eofs.as<int64_t>(),
-                                            g->ginfo.as<uint32_t>(), g->gwt.as<double>(), g->eid.as<int32_t>()));
-        }
+    FL_LAUNCH(kProfSketchOther, k_ads_hop0<<<grid_for(n, 256), 256, 0, st>>>(
+                                    n, g->gofs.as<int64_t>(), g->eofs.as<int64_t>(), g->ginfo.as<uint32_t>(),
+                                    g->gwt.as<double>(), g->eid.as<int32_t>()));
+    if (used_slots > 0) {
+        FL_LAUNCH(kProfSketchOther, k_ads_groups<<<grid_for(used_slots, 256), 256, 0, st>>>(
+                                        g->stg_grp.as<StgGroup>(), g->stg_kth.as<uint32_t>(), used_slots, k, seed,
+                                        g->ord_rid.as<int32_t>(), g->gofs.as<int64_t>(), g->ginfo.as<uint32_t>(),
+                                        g->gwt.as<double>()));
+        FL_LAUNCH(kProfSketchOther, k_ads_entries<<<grid_for(used_slots, 256), 256, 0, st>>>(
+                                        g->stg_grp.as<StgGroup>(), used_slots, k, g->stg_ent.as<uint32_t>(),
+                                        g->eofs.as<int64_t>(), g->ord_vid.as<int32_t>(),
+                                        g->max_part > 0 ? g->vbase.as<int32_t>() : nullptr, g->eid.as<int32_t>()));
+    }
     FL_CUDA(cudaGetLastError());
     FL_CUDA(cudaStreamSynchronize(st));
     FL_TRY(compute_ecc_bound(g));
