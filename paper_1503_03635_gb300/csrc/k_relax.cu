@@ -37,24 +37,36 @@ __device__ __forceinline__ bool in_front(const uint32_t* __restrict__ bm, int32_
 // reads the value of a neighbour only when its bit is set; the bitmap (n/8
 // bytes) stays in L2 while the values do not.
 //
-// In a graph made of disjoint parts (batches) the frontier is also counted
-// per part: a part without frontier vertices has no vertex that can change,
-// and pull rounds skip it.  A part whose limit is below `round` no longer
+// In a graph made of disjoint parts (batches) the parts with frontier vertices
+// are flagged: a part without any has no vertex that can change, and pull
+// rounds skip it.  A part whose limit is below `round` no longer
 // needs its values (nothing of it reads them any more) and sits out too.
+//
+// A warp takes kBmWords words in a row, so that it flags a part once: a count
+// per part and word was bound by the atomics on one line (4.2 M vertices in 16
+// parts: 55 us).
+constexpr int kBmWords = 16;
+
 __global__ void k_bitmap(const uint32_t* __restrict__ stamp, uint32_t sv, int64_t n, uint32_t* __restrict__ bm,
                          const int32_t* __restrict__ vpart, int32_t* __restrict__ part_cnt,
                          const int32_t* __restrict__ part_limit, int32_t round) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += stride) {
-        const int64_t v = base + lane_id();
-        const bool in = v < n && stamp[v] == sv && !(part_limit && part_limit[vpart[v]] < round);
-        const unsigned w = __ballot_sync(kFull, in);
-        if (lane_id() == 0) bm[base >> 5] = w;
-        if (vpart && w) {
-            const int32_t p = v < n ? vpart[v] : -1;
-            const unsigned same = __match_any_sync(kFull, p);
-            const int lead = __ffs(same & w) - 1;  // first frontier lane of this part
-            if (in && lane_id() == lead) atomicAdd(&part_cnt[p], __popc(same & w));
+    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; c * 32 * kBmWords < n; c += warps) {
+        int32_t flagged = -1;
+        const int64_t end = min((c + 1) * 32 * kBmWords, n);
+        for (int64_t base = c * 32 * kBmWords; base < end; base += 32) {
+            const int64_t v = base + lane_id();
+            bool in = v < n && stamp[v] == sv;
+            if (vpart && in) {
+                const int32_t p = vpart[v];
+                in = !(part_limit && part_limit[p] < round);
+                if (in && p != flagged) {
+                    part_cnt[p] = 1;
+                    flagged = p;
+                }
+            }
+            const unsigned w = __ballot_sync(kFull, in);
+            if (lane_id() == 0) bm[base >> 5] = w;
         }
     }
 }
@@ -77,6 +89,13 @@ __device__ __forceinline__ bool skipped(const Prune& pr, int32_t u) {
 // the value loads are independent, so each lane keeps up to four dependent-
 // load chains in flight; the columns of the next pass are loaded at the start
 // of a pass, so their DRAM latency overlaps this pass's bitmap and value loads.
+//
+// kAll: every neighbour's value is read, the bitmap is not.  A neighbour whose
+// value did not change offers what it offered in an earlier round, so the
+// result is the same; when most neighbours are in the frontier the bitmap only
+// adds a second gather per edge to rounds that are bound by the gathers (L1
+// wavefronts, 80 % of its peak).
+template <bool kAll>
 __device__ __forceinline__ unsigned long long pull_min(const int32_t* __restrict__ cols, int64_t e0, int64_t e1,
                                                        int step, const uint32_t* __restrict__ bm,
                                                        const unsigned long long* __restrict__ X,
@@ -94,7 +113,7 @@ __device__ __forceinline__ unsigned long long pull_min(const int32_t* __restrict
 #pragma unroll
         for (int j = 0; j < 4; ++j) nx[j] = en + j * step < e1 ? __ldcs(&cols[en + j * step]) : -1;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) f[j] = u[j] >= 0 && in_front(bm, u[j]);
+        for (int j = 0; j < 4; ++j) f[j] = u[j] >= 0 && (kAll || in_front(bm, u[j]));
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             if (f[j]) {
@@ -110,6 +129,7 @@ __device__ __forceinline__ unsigned long long pull_min(const int32_t* __restrict
 // vertex, its neighbours loaded four at a time (column, bitmap and value
 // loads each independent of the others), so that a warp keeps 32 vertices'
 // chains in flight.
+template <bool kAll>
 __global__ void __launch_bounds__(256) k_pull_small(const int32_t* __restrict__ list, int64_t n_list,
                                                     const int64_t* __restrict__ rowp,
                                                     const int32_t* __restrict__ cols, unsigned long long add,
@@ -130,7 +150,7 @@ __global__ void __launch_bounds__(256) k_pull_small(const int32_t* __restrict__ 
         const unsigned long long own = have ? X[v] : ~0ULL;
         const bool work = have && !(settle && own < limit);
         const int64_t beg = work ? rowp[v] : 0, end = work ? rowp[v + 1] : 0;
-        const unsigned long long m = pull_min(cols, beg, end, 1, bm, X, add, limit, own);
+        const unsigned long long m = pull_min<kAll>(cols, beg, end, 1, bm, X, add, limit, own);
         const bool ch = work && m < own;
         if (ch) {
             Xn[v] = m;
@@ -145,6 +165,7 @@ __global__ void __launch_bounds__(256) k_pull_small(const int32_t* __restrict__ 
 // Pull round over the other non-hub vertices: four vertices per warp, eight
 // lanes per vertex striding over its neighbours; the lanes meet again at the
 // reduction.
+template <bool kAll>
 __global__ void __launch_bounds__(256) k_pull_low(const int32_t* __restrict__ list, int64_t n_list,
                                                   const int64_t* __restrict__ rowp, const int32_t* __restrict__ cols,
                                                   unsigned long long add, unsigned long long limit, bool settle,
@@ -165,7 +186,7 @@ __global__ void __launch_bounds__(256) k_pull_low(const int32_t* __restrict__ li
         const unsigned long long own = have ? X[v] : ~0ULL;
         const bool work = have && !(settle && own < limit);
         const int64_t beg = work ? rowp[v] : 0, end = work ? rowp[v + 1] : 0;
-        unsigned long long m = pull_min(cols, beg + sub, end, 8, bm, X, add, limit, own);
+        unsigned long long m = pull_min<kAll>(cols, beg + sub, end, 8, bm, X, add, limit, own);
 #pragma unroll
         for (int o = 1; o < 8; o <<= 1) m = umin64(m, __shfl_xor_sync(kFull, m, o));
         const bool ch = work && sub == 0 && m < own;
@@ -182,6 +203,7 @@ __global__ void __launch_bounds__(256) k_pull_low(const int32_t* __restrict__ li
 // Pull round over hubs: one warp per segment of kSeg edges.  Xn[v] starts as
 // X[v]; the segments lower it with atomicMin and the one that lowers it first
 // (it sees the old value) flags the hub.
+template <bool kAll>
 __global__ void __launch_bounds__(256) k_pull_segs(const int32_t* __restrict__ seg_hub, int64_t n_seg,
                                                    const int64_t* __restrict__ hub_seg,
                                                    const int32_t* __restrict__ hub_list,
@@ -202,7 +224,7 @@ __global__ void __launch_bounds__(256) k_pull_segs(const int32_t* __restrict__ s
         if ((settle && own < limit) || part_idle(vpart, part_cnt, v) || skipped(pr, v)) continue;
         const int64_t e0 = rowp[v] + (sidx - hub_seg[h]) * kSeg;
         const int64_t e1 = min(e0 + (int64_t)kSeg, rowp[v + 1]);
-        unsigned long long m = pull_min(cols, e0 + lane, e1, 32, bm, X, add, limit, ~0ULL);
+        unsigned long long m = pull_min<kAll>(cols, e0 + lane, e1, 32, bm, X, add, limit, ~0ULL);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) m = umin64(m, __shfl_xor_sync(kFull, m, o));
         if (lane == 0 && m < own) {
@@ -347,6 +369,12 @@ __global__ void k_collect_stamped(const uint32_t* __restrict__ stamp, uint32_t s
 }
 
 constexpr int64_t kPushAlways = 4096;  // smaller frontiers push without counting their edges
+// A pull reads every neighbour's value when frontier * kAllDiv >= the listed
+// vertices.  R-MAT, 4.2 M vertices, a cover round of a query: 160 us (hub
+// segments) and 268 us (the others) with the bitmap, 125 and 222 without; a
+// round with 30 % of the vertices in the frontier 160 and 268 against 127 and
+// 225.
+constexpr int64_t kAllDiv = 4;
 
 }  // namespace
 
@@ -450,21 +478,29 @@ int relax_round(fl_graph* g, Relax& r, unsigned long long add, uint32_t sv, int 
     } else {
         unsigned long long* Xn = r.X[r.cur ^ 1];
         const int32_t* vpart = g->n_parts > 0 ? g->vpart.as<int32_t>() : nullptr;
+        // most of the listed vertices changed: read every neighbour's value
+        // (not in a BFS: its frontier leaves out the hubs, reached earlier, that
+        // most edges lead to)
+        const bool all = !r.settle && r.n_front * kAllDiv >= g->n_low + g->n_hubs;
         if (vpart) FL_CUDA(cudaMemsetAsync(r.part_cnt, 0, (size_t)g->n_parts * 4, st));
-        FL_LAUNCH(cls, k_bitmap<<<grid_for(n, 256), 256, 0, st>>>(r.stamp, r.sv_prev, n, r.bm, vpart, r.part_cnt,
-                                                                  vpart ? r.part_limit : nullptr, r.part_round));
+        if (vpart || !all)
+            FL_LAUNCH(cls, k_bitmap<<<grid_for(n, 256 * kBmWords), 256, 0, st>>>(r.stamp, r.sv_prev, n, r.bm, vpart, r.part_cnt,
+                                                                      vpart ? r.part_limit : nullptr, r.part_round));
         FL_CUDA(cudaMemcpyAsync(Xn, X, (size_t)n * 8, cudaMemcpyDeviceToDevice, st));
         FL_CUDA(cudaMemsetAsync(&r.cnt[2], 0, 8, st));
+        auto small = all ? k_pull_small<true> : k_pull_small<false>;
+        auto low = all ? k_pull_low<true> : k_pull_low<false>;
+        auto segs = all ? k_pull_segs<true> : k_pull_segs<false>;
         if (g->n_small > 0)
-            FL_LAUNCH(cls, k_pull_small<<<grid_for(g->n_small, 256), 256, 0, st>>>(
+            FL_LAUNCH(cls, small<<<grid_for(g->n_small, 256), 256, 0, st>>>(
                                g->small_list.as<int32_t>(), g->n_small, rowp, cols, add, r.limit, r.settle, r.bm, X,
                                Xn, r.stamp, sv, &r.cnt[2], vpart, r.part_cnt, r.prune));
         if (g->n_mid > 0)
-            FL_LAUNCH(cls, k_pull_low<<<grid_for((g->n_mid + 3) / 4, 8), 256, 0, st>>>(
+            FL_LAUNCH(cls, low<<<grid_for((g->n_mid + 3) / 4, 8), 256, 0, st>>>(
                                g->mid_list.as<int32_t>(), g->n_mid, rowp, cols, add, r.limit, r.settle, r.bm, X, Xn,
                                r.stamp, sv, &r.cnt[2], vpart, r.part_cnt, r.prune));
         if (g->n_seg > 0)
-            FL_LAUNCH(cls, k_pull_segs<<<grid_for(g->n_seg, 8), 256, 0, st>>>(
+            FL_LAUNCH(cls, segs<<<grid_for(g->n_seg, 8), 256, 0, st>>>(
                                g->seg_hub.as<int32_t>(), g->n_seg, g->hub_seg.as<int64_t>(), hub_list, rowp, cols, add,
                                r.limit, r.settle, r.bm, X, Xn, r.stamp, sv, &r.cnt[2], vpart, r.part_cnt,
                                r.prune));
