@@ -549,6 +549,13 @@ struct fl_solve {
 
 namespace fl {
 
+// Shares of the keys in a counting kernel of m keys (a block per 64 keys and
+// share): about eight blocks of 256 threads per SM, at least 512 keys each.
+inline unsigned count_shares(int64_t m) {
+    const int64_t groups = (m + 63) / 64, want = (152 * 8 + groups - 1) / groups, most = (m + 511) / 512;
+    return (unsigned)(want < most ? want : most);
+}
+
 // ----------------------------------------------------------------- kernel launchers
 // (implemented in the .cu files; all run on g->stream)
 

@@ -1127,41 +1127,45 @@ __global__ void k_hop_census(const int32_t* __restrict__ list, int64_t n_list, c
 // ------------------------------------------------------------------ ordinals
 
 // Few ranks: each one's ordinal is the number of ranks below its own.  A block
-// places 64 ids, two per lane; its warps share the scan of all ranks, computed
-// into shared memory a tile at a time.  (Ranks are a bijection of the ids.)
-__global__ void __launch_bounds__(1024) k_ordinals_small(int m, uint64_t seed, int32_t* __restrict__ ord_rid,
-                                                         Counters* ctr) {
-    constexpr int kTile = 2048;
+// counts for 64 ids, two per lane, over its share of the ranks (blockIdx.y of
+// gridDim.y), computed into shared memory a tile at a time.  (Ranks are a
+// bijection of the ids.)
+__global__ void __launch_bounds__(256) k_count_ranks(int m, uint64_t seed, uint32_t* __restrict__ of_rid,
+                                                     Counters* ctr) {
+    constexpr int kTile = 512;
     __shared__ uint64_t key[kTile];
-    __shared__ int below[32][64];
+    __shared__ int below[64];
     const int lane = lane_id(), warp = threadIdx.x >> 5;
     const int i0 = blockIdx.x * 64 + lane, i1 = i0 + 32;
     const uint64_t r0 = vertex_rank(seed, i0), r1 = vertex_rank(seed, i1);
+    const int t0 = (int)((int64_t)m * blockIdx.y / gridDim.y), t1 = (int)((int64_t)m * (blockIdx.y + 1) / gridDim.y);
     int c0 = 0, c1 = 0;
-    for (int t = 0; t < m; t += kTile) {
-        const int cnt = min(kTile, m - t);
+    if (threadIdx.x < 64) below[threadIdx.x] = 0;
+    for (int t = t0; t < t1; t += kTile) {
+        const int cnt = min(kTile, t1 - t);
         __syncthreads();
-        for (int j = threadIdx.x; j < cnt; j += 1024) key[j] = vertex_rank(seed, t + j);
+        for (int j = threadIdx.x; j < cnt; j += 256) key[j] = vertex_rank(seed, t + j);
         __syncthreads();
 #pragma unroll 4
-        for (int j = warp; j < cnt; j += 32) {
+        for (int j = warp; j < cnt; j += 8) {
             const uint64_t x = key[j];
             c0 += x < r0;
             c1 += x < r1;
         }
     }
-    below[warp][lane] = c0;
-    below[warp][lane + 32] = c1;
+    atomicAdd(&below[lane], c0);
+    atomicAdd(&below[lane + 32], c1);
     __syncthreads();
-    if (threadIdx.x < 64) {
-        const int i = blockIdx.x * 64 + threadIdx.x;
-        int o = 0;
-        for (int w = 0; w < 32; ++w) o += below[w][threadIdx.x];
-        if (i < m) {
-            ord_rid[o] = i;
-            if (vertex_rank(seed, i) == kEmpty) atomicOr(&ctr->error, 1ULL);
-        }
+    const int i = blockIdx.x * 64 + threadIdx.x;
+    if (threadIdx.x < 64 && i < m) {
+        atomicAdd(&of_rid[i], (uint32_t)below[threadIdx.x]);
+        if (blockIdx.y == 0 && vertex_rank(seed, i) == kEmpty) atomicOr(&ctr->error, 1ULL);
     }
+}
+
+__global__ void k_place_ranks(const uint32_t* __restrict__ of_rid, int m, int32_t* __restrict__ ord_rid) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < m) ord_rid[of_rid[i]] = i;
 }
 
 __global__ void k_rank_pairs(int64_t m, uint64_t seed, uint64_t* __restrict__ key, uint32_t* __restrict__ val,
@@ -1218,8 +1222,12 @@ static int build_ordinals(fl_graph* g) {
     FL_TRY(dalloc(g->ord_vid, (size_t)m * 4));
     int32_t* ord_rid = g->ord_rid.as<int32_t>();
     if (m <= kCountMax) {
-        FL_LAUNCH(kProfSketchOther, k_ordinals_small<<<(unsigned)((m + 63) / 64), 1024, 0, st>>>((int)m, g->seed,
-                                                                                              ord_rid, ctr));
+        uint32_t* place = g->DM[1].as<uint32_t>();
+        FL_CUDA(cudaMemsetAsync(place, 0, (size_t)m * 4, st));
+        FL_LAUNCH(kProfSketchOther, k_count_ranks<<<dim3((unsigned)((m + 63) / 64), count_shares(m)), 256, 0, st>>>(
+                                        (int)m, g->seed, place, ctr));
+        FL_LAUNCH(kProfSketchOther, k_place_ranks<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(place, (int)m,
+                                                                                              ord_rid));
     } else {
         SortPairs<uint64_t> p;
         p.key[0] = g->DM[0].as<uint64_t>();

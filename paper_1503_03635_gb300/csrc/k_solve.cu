@@ -527,8 +527,8 @@ int compute_radii_multi(const fl_graph* src, fl_graph* g, int64_t R, const doubl
 
 // ------------------------------------------------------------------ keys (r_f, pi_f)
 
-// Up to kRankMax candidates are ordered by counting (k_rank_keys), more by the
-// radix sort.  Measured (uniform and log-uniform costs): see k_rank_keys.
+// Up to kRankMax candidates are ordered by counting (k_count_keys), more by the
+// radix sort.
 constexpr int64_t kRankMax = 16384;
 
 __global__ void k_candidates(const double* __restrict__ r, int64_t n, uint64_t seed,
@@ -576,44 +576,71 @@ __global__ void k_candidates(const double* __restrict__ r, int64_t n, uint64_t s
 }
 
 // Few candidates: each one's place in key order is the number of keys below
-// its own.  A block places 64 candidates, two per lane; its warps share the
-// scan of all keys, staged in shared memory 512 at a time (every lane reads
-// the same key: a broadcast).  Equal keys (parts of a batch with equal
-// part-local ids) keep their input order.  Quadratic, but one launch and no
-// pass over memory but the keys: bound by integer compares.
+// its own.  A block counts for 64 candidates, two per lane, over its share of
+// the keys (blockIdx.y of gridDim.y shares), staged in shared memory a tile at
+// a time; its warps share the tile (every lane reads the same key: a
+// broadcast).  Equal keys (parts of a batch with equal part-local ids) keep
+// their input order.  Quadratic, but no pass over memory but the keys: bound by
+// integer compares, one borrow chain over (radius, priority, index) each, and
+// by how evenly the blocks fill the SMs (10^4 keys: 101 us with one share of
+// all keys, 157 blocks on 152 SMs, and compares word by word; 41 us now).
 constexpr int kRankTile = 512;
 
-__global__ void __launch_bounds__(256) k_rank_keys(const uint64_t* __restrict__ hi, const uint64_t* __restrict__ lo,
-                                                   const uint32_t* __restrict__ val, int m,
-                                                   uint32_t* __restrict__ sorted) {
+// -1 when (hi, lo, at) is below (h, l, i), else 0.
+__device__ __forceinline__ int key_below(uint64_t hi, uint64_t lo, unsigned at, uint64_t h, uint64_t l, unsigned i) {
+    int r;
+    asm("{\n\t"
+        ".reg .u32 t, a, b, c, d;\n\t"
+        "sub.cc.u32 t, %1, %2;\n\t"
+        "mov.b64 {a, b}, %3;\n\t"
+        "mov.b64 {c, d}, %4;\n\t"
+        "subc.cc.u32 t, a, c;\n\t"
+        "subc.cc.u32 t, b, d;\n\t"
+        "mov.b64 {a, b}, %5;\n\t"
+        "mov.b64 {c, d}, %6;\n\t"
+        "subc.cc.u32 t, a, c;\n\t"
+        "subc.cc.u32 t, b, d;\n\t"
+        "subc.u32 %0, 0, 0;\n\t"
+        "}"
+        : "=r"(r)
+        : "r"(at), "r"(i), "l"(lo), "l"(l), "l"(hi), "l"(h));
+    return r;
+}
+
+__global__ void __launch_bounds__(256) k_count_keys(const uint64_t* __restrict__ hi, const uint64_t* __restrict__ lo,
+                                                    int m, unsigned* __restrict__ place) {
     __shared__ ulonglong2 key[kRankTile];
-    __shared__ int below[8][64];
+    __shared__ int below[64];
     const int lane = lane_id(), warp = threadIdx.x >> 5;
     const int i0 = blockIdx.x * 64 + lane, i1 = i0 + 32;
     const uint64_t h0 = i0 < m ? hi[i0] : 0, l0 = i0 < m ? lo[i0] : 0;
     const uint64_t h1 = i1 < m ? hi[i1] : 0, l1 = i1 < m ? lo[i1] : 0;
+    const int t0 = (int)((int64_t)m * blockIdx.y / gridDim.y), t1 = (int)((int64_t)m * (blockIdx.y + 1) / gridDim.y);
     int c0 = 0, c1 = 0;
-    for (int t = 0; t < m; t += kRankTile) {
-        const int cnt = min(kRankTile, m - t);
+    if (threadIdx.x < 64) below[threadIdx.x] = 0;
+    for (int t = t0; t < t1; t += kRankTile) {
+        const int cnt = min(kRankTile, t1 - t);
         __syncthreads();
         for (int j = threadIdx.x; j < cnt; j += 256) key[j] = make_ulonglong2(hi[t + j], lo[t + j]);
         __syncthreads();
+#pragma unroll 4
         for (int j = warp; j < cnt; j += 8) {
             const ulonglong2 k = key[j];
-            const int at = t + j;
-            c0 += (k.x < h0) | ((k.x == h0) & ((k.y < l0) | ((k.y == l0) & (at < i0))));
-            c1 += (k.x < h1) | ((k.x == h1) & ((k.y < l1) | ((k.y == l1) & (at < i1))));
+            c0 -= key_below(k.x, k.y, (unsigned)(t + j), h0, l0, (unsigned)i0);
+            c1 -= key_below(k.x, k.y, (unsigned)(t + j), h1, l1, (unsigned)i1);
         }
     }
-    below[warp][lane] = c0;
-    below[warp][lane + 32] = c1;
+    atomicAdd(&below[lane], c0);
+    atomicAdd(&below[lane + 32], c1);
     __syncthreads();
-    if (threadIdx.x < 64) {
-        const int i = blockIdx.x * 64 + threadIdx.x;
-        int rank = 0;
-        for (int w = 0; w < 8; ++w) rank += below[w][threadIdx.x];
-        if (i < m) sorted[rank] = val[i];
-    }
+    if (threadIdx.x < 64 && blockIdx.x * 64 + threadIdx.x < m)
+        atomicAdd(&place[blockIdx.x * 64 + threadIdx.x], (unsigned)below[threadIdx.x]);
+}
+
+__global__ void k_place_keys(const unsigned* __restrict__ place, const uint32_t* __restrict__ val, int m,
+                             uint32_t* __restrict__ sorted) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < m) sorted[place[i]] = val[i];
 }
 
 __device__ __forceinline__ uint64_t priority_of(uint64_t seed, const IdMap& ids, uint32_t f) {
@@ -893,8 +920,13 @@ int sort_candidates(fl_solve* s, int64_t* m_out, const uint32_t** sorted) {
     *sorted = p.val[0];
     if (m <= 1) return FL_OK;
     if (m <= kRankMax) {
-        FL_LAUNCH(kProfKeys, k_rank_keys<<<(unsigned)((m + 63) / 64), 256, 0, st>>>(
-                                 p.key[0], s->key_lo.as<uint64_t>(), p.val[0], (int)m, p.val[1]));
+        unsigned* place = reinterpret_cast<unsigned*>(p.key[1]);
+        const int groups = (int)((m + 63) / 64);
+        FL_CUDA(cudaMemsetAsync(place, 0, (size_t)m * 4, st));
+        FL_LAUNCH(kProfKeys, k_count_keys<<<dim3(groups, count_shares(m)), 256, 0, st>>>(
+                                 p.key[0], s->key_lo.as<uint64_t>(), (int)m, place));
+        FL_LAUNCH(kProfKeys, k_place_keys<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(place, p.val[0], (int)m,
+                                                                                      p.val[1]));
         FL_CUDA(cudaGetLastError());
         *sorted = p.val[1];
         return FL_OK;
@@ -1225,18 +1257,48 @@ int assign_clients(fl_solve* s) {
 
 constexpr int kObjBlocks = 152 * 4;
 
-__global__ void k_objective(int64_t n, const uint8_t* __restrict__ open, const double* __restrict__ cost,
-                            const uint8_t* __restrict__ client, const int32_t* __restrict__ dist,
-                            double* __restrict__ partial, unsigned long long* __restrict__ sums) {
+// Opening cost of the open facilities (per block, a fixed tree), distance sum
+// and unserved clients.  A thread takes four consecutive vertices (the buffers
+// are the solve's own, 256-byte aligned), so that its loads are in flight
+// together, and a block adds up its counts before the atomics (a thread's own
+// atomics on two words took 105 us at 2^20 vertices, now 7).
+__global__ void __launch_bounds__(256) k_objective(int64_t n, const uint8_t* __restrict__ open,
+                                                   const double* __restrict__ cost,
+                                                   const uint8_t* __restrict__ client,
+                                                   const int32_t* __restrict__ dist, double* __restrict__ partial,
+                                                   unsigned long long* __restrict__ sums) {
     __shared__ double red[256];
+    __shared__ unsigned long long s_sum[2];
+    if (threadIdx.x < 2) s_sum[threadIdx.x] = 0;
     double acc = 0.0;
-    unsigned long long ds = 0, un = 0;
+    unsigned long long ds = 0;
+    unsigned un = 0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
-        if (open[v]) acc += cost[v];
-        if (client[v]) {
-            int32_t d = dist[v];
-            if (d < 0) ++un; else ds += (unsigned long long)d;
+    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; 4 * q < n; q += stride) {
+        const int64_t v = 4 * q;
+        uint8_t op[4], cl[4];
+        int32_t d[4];
+        if (v + 4 <= n) {
+            const uchar4 a = reinterpret_cast<const uchar4*>(open)[q], b = reinterpret_cast<const uchar4*>(client)[q];
+            const int4 c = reinterpret_cast<const int4*>(dist)[q];
+            op[0] = a.x, op[1] = a.y, op[2] = a.z, op[3] = a.w;
+            cl[0] = b.x, cl[1] = b.y, cl[2] = b.z, cl[3] = b.w;
+            d[0] = c.x, d[1] = c.y, d[2] = c.z, d[3] = c.w;
+        } else {
+            for (int j = 0; j < 4; ++j) {
+                const bool in = v + j < n;
+                op[j] = in ? open[v + j] : 0;
+                cl[j] = in ? client[v + j] : 0;
+                d[j] = in ? dist[v + j] : 0;
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (op[j]) acc += cost[v + j];
+            if (cl[j]) {
+                if (d[j] < 0) ++un;
+                else ds += (unsigned long long)d[j];
+            }
         }
     }
     red[threadIdx.x] = acc;
@@ -1245,9 +1307,16 @@ __global__ void k_objective(int64_t n, const uint8_t* __restrict__ open, const d
         if ((int)threadIdx.x < s2) red[threadIdx.x] += red[threadIdx.x + s2];
         __syncthreads();
     }
+    un = __reduce_add_sync(kFull, un);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ds += __shfl_xor_sync(kFull, ds, o);
+    if (lane_id() == 0) {
+        atomicAdd(&s_sum[0], ds);
+        atomicAdd(&s_sum[1], (unsigned long long)un);
+    }
+    __syncthreads();
     if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
-    if (ds) atomicAdd(&sums[0], ds);
-    if (un) atomicAdd(&sums[1], un);
+    if (threadIdx.x < 2 && s_sum[threadIdx.x]) atomicAdd(&sums[threadIdx.x], s_sum[threadIdx.x]);
 }
 
 int objective(fl_solve* s, double* obj, int64_t* dist_sum, int64_t* n_unserved) {
