@@ -327,7 +327,7 @@ int fl_export_sketches(fl_graph* g, uint64_t* S, int32_t* cnt, int mem_kind) {
     if (bad_kind(mem_kind)) FL_FAIL(FL_EINVAL, "bad mem_kind");
     ProfScope ps(g);
     cudaStream_t st = g->stream;
-    if (S && !g->wts.p) {  // ordinals of an unweighted build
+    if (S) {  // ranks of the ordinals, in original order
         DBuf tmp;
         FL_TRY(dalloc(tmp, (size_t)g->n * g->k * 8));
         int rc = sketch_ranks_original(g, tmp.as<uint64_t>());
@@ -336,8 +336,6 @@ int fl_export_sketches(fl_graph* g, uint64_t* S, int32_t* cnt, int mem_kind) {
         dfree(tmp);
         if (rc) return rc;
         if (e != cudaSuccess) return status_of(e, "export sketches", __FILE__, __LINE__);
-    } else {
-        FL_TRY(copy_out(S, g->S.p, (size_t)g->n * g->k * 8, mem_kind, st));
     }
     if (cnt) {
         DBuf tmp;

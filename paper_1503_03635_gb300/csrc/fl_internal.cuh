@@ -142,55 +142,6 @@ __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 __device__ __forceinline__ uint64_t umin64(uint64_t a, uint64_t b) { return a < b ? a : b; }
 __device__ __forceinline__ uint64_t umax64(uint64_t a, uint64_t b) { return a < b ? b : a; }
 
-// Bitonic sort of one value per lane, ascending across lanes.
-__device__ __forceinline__ uint64_t warp_sort(uint64_t x) {
-    const int lane = lane_id();
-#pragma unroll
-    for (int k = 2; k <= 32; k <<= 1) {
-#pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            uint64_t y = __shfl_xor_sync(kFull, x, j);
-            bool up = (lane & k) == 0 || k == 32;
-            bool low = (lane & j) == 0;
-            x = (low == up) ? umin64(x, y) : umax64(x, y);
-        }
-    }
-    return x;
-}
-
-// The 32 smallest of two ascending lane lists, ascending (bitonic merge).
-__device__ __forceinline__ uint64_t warp_merge_low(uint64_t a, uint64_t b) {
-    const int lane = lane_id();
-    uint64_t br = __shfl_sync(kFull, b, 31 - lane);
-    uint64_t c = umin64(a, br);
-#pragma unroll
-    for (int j = 16; j > 0; j >>= 1) {
-        uint64_t y = __shfl_xor_sync(kFull, c, j);
-        c = (lane & j) ? umax64(c, y) : umin64(c, y);
-    }
-    return c;
-}
-
-// Number of entries of ascending lane list L that are < x (0..32).
-__device__ __forceinline__ int warp_lower_bound(uint64_t L, uint64_t x) {
-    int pos = 0;
-#pragma unroll
-    for (int s = 16; s > 0; s >>= 1) {
-        uint64_t y = __shfl_sync(kFull, L, pos + s - 1);
-        if (y < x) pos += s;
-    }
-    uint64_t last = __shfl_sync(kFull, L, 31);
-    if (pos == 31 && last < x) pos = 32;
-    return pos;
-}
-
-// Is x one of the entries of ascending lane list L?
-__device__ __forceinline__ bool warp_member(uint64_t L, uint64_t x) {
-    int pos = warp_lower_bound(L, x);
-    uint64_t y = __shfl_sync(kFull, L, pos & 31);
-    return pos < 32 && y == x;
-}
-
 // HIP weight of a group whose ball holds cnt ranks with k-th smallest kth:
 // 1 while the ball has fewer than k vertices, else 1 / Pr[rank < k-th] =
 // 2^64 / kth (one IEEE division).
@@ -214,16 +165,6 @@ __device__ __forceinline__ int nth_set_bit(unsigned m, int n) {
         }
     }
     return pos;
-}
-
-// Gather the values of lanes in `keep` to lanes 0..popc(keep)-1 (order kept),
-// the rest get `fill`.
-__device__ __forceinline__ uint64_t warp_compact(uint64_t x, unsigned keep, uint64_t fill) {
-    const int lane = lane_id();
-    int total = __popc(keep);
-    int src = lane < total ? nth_set_bit(keep, lane) : 0;
-    uint64_t y = __shfl_sync(kFull, x, src);
-    return lane < total ? y : fill;
 }
 
 __device__ __forceinline__ int warp_incl_scan(int x) {
@@ -277,6 +218,167 @@ __device__ __forceinline__ long long block_append(bool pred, unsigned long long*
     }
     __syncthreads();
     return pred ? (long long)(sh.off[warp] + __popc(m & ((1u << lane) - 1u))) : -1LL;
+}
+
+// ----------------------------------------------------------------- groups in lockstep
+// A group is G consecutive lanes (16 or 32) that work on one vertex.  The two
+// half-warp groups of a warp run in lockstep: every lane of the warp executes
+// every group operation, a group without work carries empty ranges and empty
+// lists through it, and branches are taken by the whole warp.  (Groups that
+// diverge are executed one after the other, which cost half the issue slots.)
+// A G-lane list holds up to G ordinals, one per lane, ascending, kNil after.
+
+constexpr uint32_t kNil = 0xffffffffu;  // empty sketch or list slot
+
+template <int G>
+struct Lock {
+    int l;      // lane within the group
+    int shift;  // position of the group's bits in a warp ballot
+    __device__ __forceinline__ Lock() {
+        const int lane = lane_id();
+        l = lane & (G - 1);
+        shift = lane & ~(G - 1);
+    }
+    __device__ __forceinline__ unsigned mine(unsigned b) const { return G == 32 ? b : (b >> shift) & 0xffffu; }
+    __device__ __forceinline__ unsigned ballot(bool p) const { return mine(__ballot_sync(kFull, p)); }
+    __device__ __forceinline__ unsigned below() const { return (1u << l) - 1u; }  // the lanes before this one
+    template <class T>
+    __device__ __forceinline__ T shfl(T x, int src) const { return __shfl_sync(kFull, x, src, G); }
+    template <class T>
+    __device__ __forceinline__ T shfl_xor(T x, int m) const { return __shfl_xor_sync(kFull, x, m, G); }
+    template <class T>
+    __device__ __forceinline__ T shfl_up(T x, int d) const { return __shfl_up_sync(kFull, x, d, G); }
+};
+
+__device__ __forceinline__ bool warp_any(bool p) { return __any_sync(kFull, p); }
+
+template <int G>
+__device__ __forceinline__ uint32_t lock_sort(const Lock<G>& g, uint32_t x) {
+#pragma unroll
+    for (int k = 2; k <= G; k <<= 1) {
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            const uint32_t y = g.shfl_xor(x, j);
+            const bool up = (g.l & k) == 0 || k == G;
+            const bool low = (g.l & j) == 0;
+            x = low == up ? min(x, y) : max(x, y);
+        }
+    }
+    return x;
+}
+
+// Entries of the list L below x (0..G) and whether x is one of them.
+template <int G>
+__device__ __forceinline__ int lock_find(const Lock<G>& g, uint32_t L, uint32_t x, bool& member) {
+    int pos = 0;
+#pragma unroll
+    for (int s = G / 2; s > 0; s >>= 1)
+        if (g.shfl(L, pos + s - 1) < x) pos += s;
+    const uint32_t y = g.shfl(L, pos);
+    member = y == x;
+    return pos + (y < x ? 1 : 0);
+}
+
+template <int G>
+__device__ __forceinline__ uint64_t lock_or64(const Lock<G>& g, uint64_t x) {
+    unsigned lo = (unsigned)x, hi = (unsigned)(x >> 32);
+    if (G == 32) {
+        lo = __reduce_or_sync(kFull, lo);
+        hi = __reduce_or_sync(kFull, hi);
+    } else {
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) {
+            lo |= g.shfl_xor(lo, o);
+            hi |= g.shfl_xor(hi, o);
+        }
+    }
+    return ((uint64_t)hi << 32) | lo;
+}
+
+// Running sketch of one group: list `sk` (k valid lanes) and the filter `tau`:
+// its k-th ordinal (kNil while it is not full), at most `tau_base` (kNil for a
+// vertex's own sketch, the vertex's old k-th ordinal for a hub partial).
+template <int G>
+struct Sketch {
+    uint32_t sk, tau, tau_base;
+    __device__ __forceinline__ void retau(const Lock<G>& g, int k) { tau = min(g.shfl(sk, k - 1), tau_base); }
+};
+
+// Insert one ordinal per group (x uniform over the group; groups without
+// `want` keep their sketch).
+template <int G>
+__device__ __forceinline__ void insert_one(const Lock<G>& g, int k, uint32_t x, bool want, Sketch<G>& s) {
+    const bool dup = g.ballot(s.sk == x) != 0;
+    const int p = __popc(g.ballot(s.sk < x));
+    const uint32_t up = g.shfl_up(s.sk, 1);
+    if (want && !dup) {
+        s.sk = g.l > p ? up : (g.l == p ? x : s.sk);
+        if (g.l >= k) s.sk = kNil;
+    }
+    s.retau(g, k);
+}
+
+// Merge candidates, ascending over the lanes that have one (kNil: none; no
+// repeats among them): each lane finds its place in the sketch by search,
+// candidates already there drop out, and the others take the places
+// (entries below) + (kept candidates before); the sketch's entries fill the
+// places left.  Candidates pass through shared memory to their places.
+template <int G>
+__device__ __forceinline__ void merge_sorted(const Lock<G>& g, int k, uint32_t x, Sketch<G>& s, uint32_t* sx) {
+    bool member;
+    const int pos = lock_find(g, s.sk, x, member);
+    const bool keep = x != kNil && !member;
+    const unsigned km = __ballot_sync(kFull, keep);
+    if (!km) return;
+    const int dest = pos + __popc(g.mine(km) & g.below());
+    const bool fits = keep && dest < G;
+    const unsigned occ = g.mine(__reduce_or_sync(kFull, fits ? 1u << (dest + g.shift) : 0u));
+    if (fits) sx[g.shift + dest] = x;
+    __syncwarp();
+    const uint32_t old = g.shfl(s.sk, g.l - __popc(occ & g.below()));
+    const uint32_t nv = (occ >> g.l) & 1u ? sx[g.shift + g.l] : old;
+    __syncwarp();
+    s.sk = g.l < k ? nv : kNil;
+    s.retau(g, k);
+}
+
+// Merge a sorted list: the entries below tau form a prefix, absorbed by one or
+// two insertions or one merge.
+template <int G>
+__device__ __forceinline__ void merge_list(const Lock<G>& g, int k, uint32_t x, Sketch<G>& s, uint32_t* sx) {
+    const bool in = x < s.tau;
+    const unsigned b = __ballot_sync(kFull, in);
+    if (!b) return;
+    const int c = __popc(g.mine(b));
+    if (!warp_any(c > 2)) {
+        insert_one(g, k, g.shfl(x, 0), c > 0, s);
+        if (warp_any(c > 1)) {
+            const uint32_t x1 = g.shfl(x, 1);
+            insert_one(g, k, x1, c > 1 && x1 < s.tau, s);
+        }
+    } else {
+        merge_sorted(g, k, in ? x : kNil, s, sx);
+    }
+}
+
+// Absorb one batch of candidates (one per lane, kNil = none; unsorted, may
+// repeat or already be in the sketch): filter by tau, then insert one by one
+// when few survive, else sort and merge.
+template <int G>
+__device__ __forceinline__ void absorb(const Lock<G>& g, int k, uint32_t x, Sketch<G>& s, uint32_t* sx) {
+    unsigned m = g.ballot(x < s.tau);
+    if (!warp_any(m != 0)) return;
+    if (!warp_any(__popc(m) > 3)) {
+        while (warp_any(m != 0)) {
+            const uint32_t y = g.shfl(x, m ? __ffs(m) - 1 : 0);
+            insert_one(g, k, y, m != 0 && y < s.tau, s);
+            m &= m - 1;
+        }
+    } else {
+        x = lock_sort(g, x < s.tau ? x : kNil);
+        const uint32_t prev = g.shfl_up(x, 1);
+        merge_sorted(g, k, g.l > 0 && prev == x ? kNil : x, s, sx);
+    }
 }
 
 // ----------------------------------------------------------------- resident kernels
@@ -475,7 +577,7 @@ struct fl_graph {
     uint64_t seed = 0;
     int built = 0;
     uint64_t generation = 0;       // bumped by every build
-    fl::DBuf S, Scnt;              // uint32[n*k] ordinals (weighted graphs: uint64[n*k] ranks), uint8[n]
+    fl::DBuf S, Scnt;              // uint32[n*k] ordinals, uint8[n]
     fl::DBuf D[2], Dcnt[2];        // hop deltas (ordinals), counts
     fl::DBuf frontier[2];          // int32[n]
     fl::DBuf stamp;                // uint32[n]
@@ -586,6 +688,7 @@ int digit_windows(uint64_t varying, int bits, int* shift);
 int validate_csr(fl_graph* g);
 int build_work_lists(fl_graph* g);
 int build_sketches(fl_graph* g, int k, uint64_t seed);
+int build_ordinals(fl_graph* g, DBuf& tmp);
 // weighted graphs (k_wsketch.cu): length check, and the build in Dijkstra order
 int check_weights(fl_graph* g);
 int pair_reverse_edges(fl_graph* g);

@@ -59,81 +59,7 @@ __host__ __device__ __forceinline__ uint32_t pack_info(int hop, int cnt, int cou
 }
 
 constexpr int kMaxHops = 65535;
-constexpr uint32_t kNil = 0xffffffffu;  // empty sketch or list slot
 constexpr int64_t kCountMax = 16384;    // more ranks than this go through the radix sort
-
-// ------------------------------------------------------------------ groups in lockstep
-// A group is G consecutive lanes (16 or 32) that work on one vertex.  The two
-// half-warp groups of a warp run in lockstep: every lane of the warp executes
-// every group operation, a group without work carries empty ranges and empty
-// lists through it, and branches are taken by the whole warp.  (Groups that
-// diverge are executed one after the other, which cost half the issue slots.)
-// A G-lane list holds up to G ordinals, one per lane, ascending, kNil after.
-
-template <int G>
-struct Lock {
-    int l;      // lane within the group
-    int shift;  // position of the group's bits in a warp ballot
-    __device__ __forceinline__ Lock() {
-        const int lane = lane_id();
-        l = lane & (G - 1);
-        shift = lane & ~(G - 1);
-    }
-    __device__ __forceinline__ unsigned mine(unsigned b) const { return G == 32 ? b : (b >> shift) & 0xffffu; }
-    __device__ __forceinline__ unsigned ballot(bool p) const { return mine(__ballot_sync(kFull, p)); }
-    __device__ __forceinline__ unsigned below() const { return (1u << l) - 1u; }  // the lanes before this one
-    template <class T>
-    __device__ __forceinline__ T shfl(T x, int src) const { return __shfl_sync(kFull, x, src, G); }
-    template <class T>
-    __device__ __forceinline__ T shfl_xor(T x, int m) const { return __shfl_xor_sync(kFull, x, m, G); }
-    template <class T>
-    __device__ __forceinline__ T shfl_up(T x, int d) const { return __shfl_up_sync(kFull, x, d, G); }
-};
-
-__device__ __forceinline__ bool warp_any(bool p) { return __any_sync(kFull, p); }
-
-template <int G>
-__device__ __forceinline__ uint32_t lock_sort(const Lock<G>& g, uint32_t x) {
-#pragma unroll
-    for (int k = 2; k <= G; k <<= 1) {
-#pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            const uint32_t y = g.shfl_xor(x, j);
-            const bool up = (g.l & k) == 0 || k == G;
-            const bool low = (g.l & j) == 0;
-            x = low == up ? min(x, y) : max(x, y);
-        }
-    }
-    return x;
-}
-
-// Entries of the list L below x (0..G) and whether x is one of them.
-template <int G>
-__device__ __forceinline__ int lock_find(const Lock<G>& g, uint32_t L, uint32_t x, bool& member) {
-    int pos = 0;
-#pragma unroll
-    for (int s = G / 2; s > 0; s >>= 1)
-        if (g.shfl(L, pos + s - 1) < x) pos += s;
-    const uint32_t y = g.shfl(L, pos);
-    member = y == x;
-    return pos + (y < x ? 1 : 0);
-}
-
-template <int G>
-__device__ __forceinline__ uint64_t lock_or64(const Lock<G>& g, uint64_t x) {
-    unsigned lo = (unsigned)x, hi = (unsigned)(x >> 32);
-    if (G == 32) {
-        lo = __reduce_or_sync(kFull, lo);
-        hi = __reduce_or_sync(kFull, hi);
-    } else {
-#pragma unroll
-        for (int o = G / 2; o > 0; o >>= 1) {
-            lo |= g.shfl_xor(lo, o);
-            hi |= g.shfl_xor(hi, o);
-        }
-    }
-    return ((uint64_t)hi << 32) | lo;
-}
 
 // ------------------------------------------------------------------ small-ordinal masks
 // A sketch whose k-th ordinal is below kUW ("saturated") holds only ordinals
@@ -353,92 +279,6 @@ __global__ void k_rank_init(int64_t n, int k, const uint32_t* __restrict__ ord, 
 }
 
 // ------------------------------------------------------------------ group sketch updates
-
-// Running sketch of one group: list `sk` (k valid lanes) and the filter `tau`:
-// its k-th ordinal (kNil while it is not full), at most `tau_base` (kNil for a
-// vertex's own sketch, the vertex's old k-th ordinal for a hub partial).
-template <int G>
-struct Sketch {
-    uint32_t sk, tau, tau_base;
-    __device__ __forceinline__ void retau(const Lock<G>& g, int k) { tau = min(g.shfl(sk, k - 1), tau_base); }
-};
-
-// Insert one ordinal per group (x uniform over the group; groups without
-// `want` keep their sketch).
-template <int G>
-__device__ __forceinline__ void insert_one(const Lock<G>& g, int k, uint32_t x, bool want, Sketch<G>& s) {
-    const bool dup = g.ballot(s.sk == x) != 0;
-    const int p = __popc(g.ballot(s.sk < x));
-    const uint32_t up = g.shfl_up(s.sk, 1);
-    if (want && !dup) {
-        s.sk = g.l > p ? up : (g.l == p ? x : s.sk);
-        if (g.l >= k) s.sk = kNil;
-    }
-    s.retau(g, k);
-}
-
-// Merge candidates, ascending over the lanes that have one (kNil: none; no
-// repeats among them): each lane finds its place in the sketch by search,
-// candidates already there drop out, and the others take the places
-// (entries below) + (kept candidates before); the sketch's entries fill the
-// places left.  Candidates pass through shared memory to their places.
-template <int G>
-__device__ __forceinline__ void merge_sorted(const Lock<G>& g, int k, uint32_t x, Sketch<G>& s, uint32_t* sx) {
-    bool member;
-    const int pos = lock_find(g, s.sk, x, member);
-    const bool keep = x != kNil && !member;
-    const unsigned km = __ballot_sync(kFull, keep);
-    if (!km) return;
-    const int dest = pos + __popc(g.mine(km) & g.below());
-    const bool fits = keep && dest < G;
-    const unsigned occ = g.mine(__reduce_or_sync(kFull, fits ? 1u << (dest + g.shift) : 0u));
-    if (fits) sx[g.shift + dest] = x;
-    __syncwarp();
-    const uint32_t old = g.shfl(s.sk, g.l - __popc(occ & g.below()));
-    const uint32_t nv = (occ >> g.l) & 1u ? sx[g.shift + g.l] : old;
-    __syncwarp();
-    s.sk = g.l < k ? nv : kNil;
-    s.retau(g, k);
-}
-
-// Merge a sorted list: the entries below tau form a prefix, absorbed by one or
-// two insertions or one merge.
-template <int G>
-__device__ __forceinline__ void merge_list(const Lock<G>& g, int k, uint32_t x, Sketch<G>& s, uint32_t* sx) {
-    const bool in = x < s.tau;
-    const unsigned b = __ballot_sync(kFull, in);
-    if (!b) return;
-    const int c = __popc(g.mine(b));
-    if (!warp_any(c > 2)) {
-        insert_one(g, k, g.shfl(x, 0), c > 0, s);
-        if (warp_any(c > 1)) {
-            const uint32_t x1 = g.shfl(x, 1);
-            insert_one(g, k, x1, c > 1 && x1 < s.tau, s);
-        }
-    } else {
-        merge_sorted(g, k, in ? x : kNil, s, sx);
-    }
-}
-
-// Absorb one batch of candidates (one per lane, kNil = none; unsorted, may
-// repeat or already be in the sketch): filter by tau, then insert one by one
-// when few survive, else sort and merge.
-template <int G>
-__device__ __forceinline__ void absorb(const Lock<G>& g, int k, uint32_t x, Sketch<G>& s, uint32_t* sx) {
-    unsigned m = g.ballot(x < s.tau);
-    if (!warp_any(m != 0)) return;
-    if (!warp_any(__popc(m) > 3)) {
-        while (warp_any(m != 0)) {
-            const uint32_t y = g.shfl(x, m ? __ffs(m) - 1 : 0);
-            insert_one(g, k, y, m != 0 && y < s.tau, s);
-            m &= m - 1;
-        }
-    } else {
-        x = lock_sort(g, x < s.tau ? x : kNil);
-        const uint32_t prev = g.shfl_up(x, 1);
-        merge_sorted(g, k, g.l > 0 && prev == x ? kNil : x, s, sx);
-    }
-}
 
 // Absorb the candidates of CSR entries [e0, e1) (e0 >= e1: none): at hop 1 the
 // neighbours' own ordinals, later the entries each neighbour gained at the
@@ -1211,26 +1051,27 @@ __global__ void k_ord_gather(const uint32_t* __restrict__ of_rid, const int32_t*
 }
 
 // g->ord_rid, g->ord_vid and g->ord.  The rank ids of a union are its parts' local ids
-// (below the largest part's size).  A reserved rank sets ctr->error.  Scratch:
-// the delta masks, written later (128 bytes per vertex).
-static int build_ordinals(fl_graph* g) {
+// (below the largest part's size).  A reserved rank sets bit 0 of ctr->error,
+// which the caller clears before.  tmp: scratch, 28 bytes per rank id.
+int build_ordinals(fl_graph* g, DBuf& tmp) {
     const int64_t n = g->n, m = g->max_part > 0 ? g->max_part : n;
     cudaStream_t st = g->stream;
     Counters* ctr = g->ctr.as<Counters>();
     FL_TRY(dalloc(g->ord, (size_t)n * 4));
     FL_TRY(dalloc(g->ord_rid, (size_t)m * 4));
     FL_TRY(dalloc(g->ord_vid, (size_t)m * 4));
+    FL_TRY(dalloc(tmp, (size_t)m * 28));
     int32_t* ord_rid = g->ord_rid.as<int32_t>();
+    uint32_t* of_rid = reinterpret_cast<uint32_t*>(tmp.as<char>() + (size_t)m * 24);
     if (m <= kCountMax) {
-        uint32_t* place = g->DM[1].as<uint32_t>();
-        FL_CUDA(cudaMemsetAsync(place, 0, (size_t)m * 4, st));
+        FL_CUDA(cudaMemsetAsync(of_rid, 0, (size_t)m * 4, st));
         FL_LAUNCH(kProfSketchOther, k_count_ranks<<<dim3((unsigned)((m + 63) / 64), count_shares(m)), 256, 0, st>>>(
-                                        (int)m, g->seed, place, ctr));
-        FL_LAUNCH(kProfSketchOther, k_place_ranks<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(place, (int)m,
+                                        (int)m, g->seed, of_rid, ctr));
+        FL_LAUNCH(kProfSketchOther, k_place_ranks<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(of_rid, (int)m,
                                                                                               ord_rid));
     } else {
         SortPairs<uint64_t> p;
-        p.key[0] = g->DM[0].as<uint64_t>();
+        p.key[0] = tmp.as<uint64_t>();
         p.key[1] = p.key[0] + m;
         p.val[0] = reinterpret_cast<uint32_t*>(p.key[1] + m);
         p.val[1] = p.val[0] + m;
@@ -1245,7 +1086,6 @@ static int build_ordinals(fl_graph* g) {
                                                                                  shift[0], ord_rid));
     }
     if (g->max_part > 0) {
-        uint32_t* of_rid = g->DM[1].as<uint32_t>();
         FL_LAUNCH(kProfSketchOther, k_ord_scatter<<<grid_for(m, 256), 256, 0, st>>>(ord_rid, m, nullptr,
                                                                                   g->ord_vid.as<int32_t>(), of_rid));
         FL_LAUNCH(kProfSketchOther, k_ord_gather<<<grid_for(n, 256), 256, 0, st>>>(of_rid, g->rid.as<int32_t>(), n,
@@ -1383,7 +1223,7 @@ int build_sketches(fl_graph* g, int k, uint64_t seed) {
     FL_CUDA(cudaMemsetAsync(g->stamp.p, 0, (size_t)n * 4, st));
     FL_CUDA(cudaMemsetAsync(g->ctr.p, 0, sizeof(Counters), st));
     {
-        int rc0 = build_ordinals(g);
+        int rc0 = build_ordinals(g, g->DM[0]);  // the delta masks are written later
         if (rc0 != FL_OK) {
             dfree_after(st, {&act});
             return rc0;

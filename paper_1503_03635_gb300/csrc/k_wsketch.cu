@@ -35,8 +35,9 @@
 // entries are posted by the whole block, so that no level waits for one warp
 // on a hub.  Bound by the latency of the dependent loads of a post (column,
 // k-th rank, sketch).  R-MAT, 65 k vertices, lengths up to 100, k = 16, 313
-// levels: 115 ms of level kernels and some 15 ms of gaps before, 29 ms now (36
-// with bisections in place of the 8-way search and the 8-wide sketch test).
+// levels: 115 ms of level kernels and some 15 ms of gaps before, 23.6 ms now (36
+// with bisections in place of the 8-way search and the 8-wide sketch test, 29
+// with 64-bit ranks in place of their ordinals).
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -56,16 +57,17 @@ int grid_for(int64_t items, int per_block) {
 }
 
 struct WEnt {
-    int32_t id;
+    uint32_t ord;  // ordinal of the entry's vertex
     int32_t dist;
 };
 
-// One group of the log: vertex, its index among the vertex's groups, and
-// the group's distance, entry count, counted prefix, weight, first entry.
+// One group of the log: vertex, its index among the vertex's groups, and the
+// group's distance, entry count, counted prefix, first entry and the sketch's
+// k-th ordinal, which gives the HIP weight.
 struct WGroup {
-    double wt;
     int32_t v, gidx;
     int32_t dist, cnt, counted, first;
+    uint32_t kth;
 };
 
 struct WArgs {
@@ -74,8 +76,8 @@ struct WArgs {
     const int32_t* wts;
     int k;
     int cap;                 // entries per vertex row
-    uint64_t seed;
-    uint64_t* S;             // n*k
+    const uint32_t* ord;     // n: ordinal of each vertex's rank
+    uint32_t* S;             // n*k: sketches, ascending ordinals, kNil after
     uint8_t* Scnt;           // n
     WEnt* ent;               // n*cap
     int32_t* ecnt;           // n: entries at the start of the level (read)
@@ -110,27 +112,39 @@ constexpr int kWQueue = 32;   // of them, queued per block and level
 
 __device__ __forceinline__ WEnt load_ent(const WEnt* p) {
     const int2 x = __ldcg(reinterpret_cast<const int2*>(p));
-    return WEnt{x.x, x.y};
+    return WEnt{(uint32_t)x.x, x.y};
 }
 
-// Which of the gained ranks (lane j < dcnt of the warp: the j-th) are in the
-// sketch row of k ranks, as a mask per lane (all 32 lanes call; a lane without
-// a row passes NULL), and the row's k-th rank.  Eight ranks are loaded at a
-// time, so that a row costs one or two L2 latencies instead of the five of a
-// bisection.  The row may be rewritten meanwhile: every value read is of the
-// old or the new sketch.
-__device__ __forceinline__ unsigned held_ranks(const uint64_t* row, int k, uint64_t gained, int dcnt, uint64_t* kth) {
+// Which of the gained ordinals (lane j < dcnt of the warp: the j-th) are in the
+// sketch row of k, as a mask per lane (all 32 lanes call; a lane without a row
+// passes NULL), and the row's k-th ordinal.  Eight are loaded at a time (as two
+// 16-byte words where rows are aligned), so that a row costs one or two L2
+// latencies instead of the five of a bisection.  The row may be rewritten
+// meanwhile: every value read is of the old or the new sketch.
+__device__ __forceinline__ unsigned held_ranks(const uint32_t* row, int k, uint32_t gained, int dcnt, uint32_t* kth) {
     unsigned held = 0;
-    uint64_t last = kEmpty;
+    uint32_t last = kNil;
     for (int c = 0; c < k; c += 8) {
-        uint64_t y[8];
+        uint32_t y[8];
+        if ((k & 3) == 0) {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) y[q] = row && c + q < k ? __ldcg(&row[c + q]) : kEmpty;
+            for (int q = 0; q < 8; q += 4) {
+                uint4 a = make_uint4(kNil, kNil, kNil, kNil);
+                if (row && c + q < k) a = __ldcg(reinterpret_cast<const uint4*>(row + c + q));
+                y[q] = a.x;
+                y[q + 1] = a.y;
+                y[q + 2] = a.z;
+                y[q + 3] = a.w;
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) y[q] = row && c + q < k ? __ldcg(&row[c + q]) : kNil;
+        }
 #pragma unroll
         for (int q = 0; q < 8; ++q)
             if (c + q == k - 1) last = y[q];
         for (int j = 0; j < dcnt; ++j) {
-            const uint64_t x = __shfl_sync(kFull, gained, j);
+            const uint32_t x = __shfl_sync(kFull, gained, j);
             bool hit = false;
 #pragma unroll
             for (int q = 0; q < 8; ++q) hit |= y[q] == x;
@@ -161,11 +175,11 @@ __device__ __forceinline__ int first_at(const WEnt* row, int have, int32_t x) {
 
 // The ranks gained by v at level L (lane j < dcnt: the j-th, ascending) go to
 // the entries e0 + first, + step, ... of its row (all 32 lanes call).
-__device__ __forceinline__ void post_row(const WArgs& a, int64_t e0, int64_t e1, int first, int step, uint64_t gained,
+__device__ __forceinline__ void post_row(const WArgs& a, int64_t e0, int64_t e1, int first, int step, uint32_t gained,
                                          int dcnt, int64_t L) {
     for (int64_t b = e0 + first; b < e1; b += step) {
         const int64_t e = b + lane_id();
-        const uint64_t* row = nullptr;
+        const uint32_t* row = nullptr;
         int32_t u = 0;
         int64_t lv = 0;
         if (e < e1) {
@@ -174,11 +188,11 @@ __device__ __forceinline__ void post_row(const WArgs& a, int64_t e0, int64_t e1,
             if (lv > 65535) atomicOr(&a.c->err, 2ULL);
             else row = a.S + (int64_t)u * a.k;
         }
-        uint64_t kth;
+        uint32_t kth;
         const unsigned held = held_ranks(row, a.k, gained, dcnt, &kth);
         bool want = false;
         for (int j = 0; j < dcnt; ++j) {
-            const uint64_t x = __shfl_sync(kFull, gained, j);
+            const uint32_t x = __shfl_sync(kFull, gained, j);
             want |= x < kth && !((held >> j) & 1u);
         }
         if (want && row) {
@@ -193,11 +207,14 @@ __device__ __forceinline__ void post_row(const WArgs& a, int64_t e0, int64_t e1,
 }
 
 __global__ void __launch_bounds__(kResThreads, 1) k_wbuild(WArgs a) {
-    __shared__ uint64_t s_gained[kWQueue][32];
+    __shared__ uint32_t s_gained[kWQueue][32];
+    __shared__ uint32_t s_x[kResWarps][32];  // per warp: merged candidates by place
     __shared__ int32_t s_v[kWQueue];
     __shared__ int s_cnt[kWQueue];
     __shared__ unsigned s_queued, s_next;
     WCtl* c = a.c;
+    const Lock<32> g;
+    uint32_t* sx = s_x[threadIdx.x >> 5];
     const int lane = lane_id(), k = a.k;
     const int64_t tid = (int64_t)blockIdx.x * kResThreads + threadIdx.x, threads = (int64_t)gridDim.x * kResThreads;
     // item i to warp i / gridDim of block i mod gridDim: neighbours in a list go to different blocks
@@ -206,7 +223,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_wbuild(WArgs a) {
     if (threadIdx.x == 0) s_queued = 0;
 
     // v gained ranks at level L: post them, or leave a long row to the block
-    auto post = [&](int32_t v, int64_t e0, int64_t e1, uint64_t gained, int dcnt, int64_t L) {
+    auto post = [&](int32_t v, int64_t e0, int64_t e1, uint32_t gained, int dcnt, int64_t L) {
         if (e1 - e0 > kWLong) {
             unsigned at = 0;
             if (lane == 0) at = atomicAdd(&s_queued, 1u);
@@ -235,26 +252,26 @@ __global__ void __launch_bounds__(kResThreads, 1) k_wbuild(WArgs a) {
     };
 
     // level 0: every vertex's own rank
-    for (int64_t i = tid; i < a.n * k; i += threads) a.S[i] = i % k == 0 ? vertex_rank(a.seed, i / k) : kEmpty;
+    for (int64_t i = tid; i < a.n * k; i += threads) a.S[i] = i % k == 0 ? a.ord[i / k] : kNil;
     for (int64_t v = tid; v < a.n; v += threads) {
-        a.ent[v * a.cap] = WEnt{(int32_t)v, 0};
+        a.ent[v * a.cap] = WEnt{a.ord[v], 0};
         a.Scnt[v] = 1;
         a.ecnt[v] = 1;
         a.gcnt[v] = 1;
         WGroup gr;
-        gr.wt = 1.0;  // a ball of one vertex (k >= 2)
         gr.v = (int32_t)v;
         gr.gidx = 0;
         gr.dist = 0;
         gr.cnt = 1;
         gr.counted = 1;
         gr.first = 0;
+        gr.kth = kNil;  // a ball of one vertex (k >= 2)
         a.glog[v] = gr;
     }
     if (tid == 0) c->glog_n = (unsigned long long)a.n;
     if (!end_pass(&c->bar, pass, 0, &total)) return;
     for (int64_t v = item0; v < a.n; v += warps)
-        post((int32_t)v, __ldg(&a.rowp[v]), __ldg(&a.rowp[v + 1]), lane == 0 ? vertex_rank(a.seed, v) : kEmpty, 1, 0);
+        post((int32_t)v, __ldg(&a.rowp[v]), __ldg(&a.rowp[v + 1]), lane == 0 ? a.ord[v] : kNil, 1, 0);
     post_queued(0);
     if (!end_pass(&c->bar, pass, 0, &total)) return;
 
@@ -298,11 +315,12 @@ __global__ void __launch_bounds__(kResThreads, 1) k_wbuild(WArgs a) {
         }
         for (int64_t i = item0; i < n_prev; i += warps) {
             const int32_t v = __ldcg(&a.act[par][i]);
-            const uint64_t s_old = lane < k ? __ldcg(&a.S[(int64_t)v * k + lane]) : kEmpty;
+            const uint32_t s_old = lane < k ? __ldcg(&a.S[(int64_t)v * k + lane]) : kNil;
             const int64_t e0 = __ldg(&a.rowp[v]), e1 = __ldg(&a.rowp[v + 1]);
-            uint64_t s = s_old;
-            int cnt = __popc(__ballot_sync(kFull, s_old != kEmpty));
-            uint64_t kth = __shfl_sync(kFull, s, k - 1);  // kEmpty while the sketch is not full
+            Sketch<32> s;
+            s.sk = s_old;
+            s.tau_base = kNil;
+            s.retau(g, k);
             uint32_t* mk = a.marks + (int64_t)slot * a.mwords;
             const int64_t w1 = (e1 + 31) >> 5;
             for (int64_t wb = e0 >> 5; wb < w1; wb += 32) {
@@ -345,45 +363,25 @@ __global__ void __launch_bounds__(kResThreads, 1) k_wbuild(WArgs a) {
                     }
                     // each lane offers its entry's candidates one per round
                     for (;;) {
-                        uint64_t r = kEmpty;
+                        uint32_t r = kNil;
                         if (at < have) {
                             const WEnt en = load_ent(&row[at]);
                             ++at;
-                            if (en.dist == x) r = vertex_rank(a.seed, en.id);
+                            if (en.dist == x) r = en.ord;
                             else at = have;
                         }
-                        if (!__any_sync(kFull, r != kEmpty)) break;
-                        unsigned m = __ballot_sync(kFull, r < kth);
-                        if (__popc(m) <= 4) {
-                            for (; m; m &= m - 1) {
-                                const uint64_t y = __shfl_sync(kFull, r, __ffs(m) - 1);
-                                if (y >= kth || __ballot_sync(kFull, s == y)) continue;
-                                const int p = __popc(__ballot_sync(kFull, s < y));
-                                const uint64_t up = __shfl_up_sync(kFull, s, 1);
-                                s = lane > p ? up : (lane == p ? y : s);
-                                if (lane >= k) s = kEmpty;
-                                if (cnt < k) ++cnt;
-                                kth = __shfl_sync(kFull, s, k - 1);
-                            }
-                            continue;
-                        }
-                        if (r >= kth) r = kEmpty;
-                        if (warp_member(s, r)) r = kEmpty;  // already held
-                        r = warp_sort(r);
-                        const uint64_t prev = __shfl_up_sync(kFull, r, 1);
-                        const bool keep = r != kEmpty && (lane == 0 || prev != r);
-                        r = warp_compact(r, __ballot_sync(kFull, keep), kEmpty);
-                        s = warp_merge_low(s, r);
-                        if (lane >= k) s = kEmpty;
-                        cnt = __popc(__ballot_sync(kFull, s != kEmpty));
-                        kth = __shfl_sync(kFull, s, k - 1);
+                        if (!__any_sync(kFull, r != kNil)) break;
+                        absorb(g, k, r, s, sx);
                     }
                 }
             }
             // the entries gained at distance L: in the new sketch, not in the old
             // (every lane takes part in the membership shuffles)
-            const bool held = warp_member(s_old, s);
-            const bool fresh = s != kEmpty && !held;
+            bool held;
+            lock_find(g, s_old, s.sk, held);
+            const bool fresh = s.sk != kNil && !held;
+            const int cnt = __popc(__ballot_sync(kFull, s.sk != kNil));
+            const uint32_t kth = __shfl_sync(kFull, s.sk, k - 1);
             const unsigned fm = __ballot_sync(kFull, fresh);
             const int32_t base = __ldcg(&a.ecnt[v]);
             const int dcnt = __popc(fm);
@@ -397,9 +395,9 @@ __global__ void __launch_bounds__(kResThreads, 1) k_wbuild(WArgs a) {
             const int counted = __popc(fm & (cnt < k ? kFull : ((1u << (k - 1)) - 1u)));
             if (fresh) {
                 const int at = base + __popc(fm & ((1u << lane) - 1u));
-                a.ent[(int64_t)v * a.cap + at] = WEnt{(int32_t)rank_vertex(a.seed, s), (int32_t)L};
+                a.ent[(int64_t)v * a.cap + at] = WEnt{s.sk, (int32_t)L};
             }
-            if (lane < k) a.S[(int64_t)v * k + lane] = s;
+            if (lane < k) a.S[(int64_t)v * k + lane] = s.sk;
             if (lane == 0) {
                 a.ecnt_n[v] = base + dcnt;
                 a.Scnt[v] = (uint8_t)cnt;
@@ -407,20 +405,21 @@ __global__ void __launch_bounds__(kResThreads, 1) k_wbuild(WArgs a) {
                 const unsigned long long gi = atomicAdd(&c->glog_n, 1ULL);
                 if (gi < a.glog_cap) {
                     WGroup gr;
-                    gr.wt = hip_weight(cnt, k, kth);
                     gr.v = v;
                     gr.gidx = __ldcg(&a.gcnt[v]);
                     gr.dist = (int32_t)L;
                     gr.cnt = dcnt;
                     gr.counted = counted;
                     gr.first = base;
+                    gr.kth = kth;
                     a.glog[gi] = gr;
                     a.gcnt[v] = gr.gidx + 1;
                 } else {
                     atomicOr(&c->err, 4ULL);
                 }
             }
-            post(v, e0, e1, warp_compact(s, fm, kEmpty), dcnt, L);
+            const uint32_t mine_g = __shfl_sync(kFull, s.sk, lane < dcnt ? nth_set_bit(fm, lane) : 0);
+            post(v, e0, e1, lane < dcnt ? mine_g : kNil, dcnt, L);
         }
         post_queued(L);
         if (!end_pass(&c->bar, pass, 0, &total)) return;
@@ -428,22 +427,24 @@ __global__ void __launch_bounds__(kResThreads, 1) k_wbuild(WArgs a) {
 }
 
 // Vertex-major ADS from the group log and the rows.
-__global__ void k_wgroups(const WGroup* __restrict__ glog, int64_t m, const int64_t* __restrict__ gofs,
+__global__ void k_wgroups(const WGroup* __restrict__ glog, int64_t m, int k, uint64_t seed,
+                          const int32_t* __restrict__ ord_rid, const int64_t* __restrict__ gofs,
                           uint32_t* __restrict__ ginfo, double* __restrict__ gwt) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += stride) {
         const WGroup gr = glog[i];
         const int64_t at = gofs[gr.v] + gr.gidx;
         ginfo[at] = (uint32_t)gr.dist | ((uint32_t)gr.cnt << 16) | ((uint32_t)gr.counted << 24);
-        gwt[at] = gr.wt;
+        gwt[at] = gr.kth == kNil ? 1.0 : hip_weight(k, k, vertex_rank(seed, (int64_t)ord_rid[gr.kth]));
     }
 }
 
 __global__ void k_wentries(const WEnt* __restrict__ ent, int cap, const int32_t* __restrict__ ecnt,
-                           const int64_t* __restrict__ eofs, int64_t n, int32_t* __restrict__ eid) {
+                           const int64_t* __restrict__ eofs, const int32_t* __restrict__ ord_rid, int64_t n,
+                           int32_t* __restrict__ eid) {
     const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < n; v += warps)
-        for (int j = lane_id(); j < ecnt[v]; j += 32) eid[eofs[v] + j] = ent[v * cap + j].id;
+        for (int j = lane_id(); j < ecnt[v]; j += 32) eid[eofs[v] + j] = ord_rid[ent[v * cap + j].ord];
 }
 
 __global__ void k_wmaxlen(const int32_t* __restrict__ w, int64_t nnz, unsigned long long* __restrict__ out,
@@ -634,9 +635,18 @@ int build_sketches_weighted(fl_graph* g, int k, uint64_t seed) {
     const int64_t mwords = (nnz + 31) / 32;
     DBuf ent, ecnt, ecnt_n, gcnt, glog, ring, pend, act, cnt, marks;
     int rc = FL_OK;
+    FL_CUDA(cudaMemsetAsync(g->ctr.p, 0, sizeof(Counters), st));
+    if ((rc = build_ordinals(g, ent)) || (rc = read_counters(g))) {
+        dfree_after(st, {&ent});
+        return rc;
+    }
+    if (g->h_ctr->error & kSortError) {
+        dfree_after(st, {&ent});
+        FL_FAIL(FL_ETIMEOUT, "ordinals: a sort's wait ran out");
+    }
     for (;;) {
         const unsigned long long glog_cap = (unsigned long long)n * (unsigned long long)cap;
-        if ((rc = dalloc(g->S, (size_t)n * k * 8)) || (rc = dalloc(g->Scnt, (size_t)n)) ||
+        if ((rc = dalloc(g->S, (size_t)n * k * 4)) || (rc = dalloc(g->Scnt, (size_t)n)) ||
             (rc = dalloc(ent, (size_t)n * cap * sizeof(WEnt))) || (rc = dalloc(ecnt, (size_t)n * 4)) ||
             (rc = dalloc(ecnt_n, (size_t)n * 4)) ||
             (rc = dalloc(gcnt, (size_t)n * 4)) ||
@@ -651,8 +661,8 @@ int build_sketches_weighted(fl_graph* g, int k, uint64_t seed) {
         a.wts = g->wts.as<int32_t>();
         a.k = k;
         a.cap = (int)cap;
-        a.seed = seed;
-        a.S = g->S.as<uint64_t>();
+        a.ord = g->ord.as<uint32_t>();
+        a.S = g->S.as<uint32_t>();
         a.Scnt = g->Scnt.as<uint8_t>();
         a.ent = ent.as<WEnt>();
         a.ecnt = ecnt.as<int32_t>();
@@ -723,11 +733,11 @@ int build_sketches_weighted(fl_graph* g, int k, uint64_t seed) {
             (rc = dalloc(g->eid, (size_t)std::max<int64_t>(ne, 1) * 4)))
             break;
         FL_LAUNCH(kProfSketchOther, k_wgroups<<<grid_for(m, 256), 256, 0, st>>>(
-                                        glog.as<WGroup>(), m, g->gofs.as<int64_t>(), g->ginfo.as<uint32_t>(),
-                                        g->gwt.as<double>()));
+                                        glog.as<WGroup>(), m, k, seed, g->ord_rid.as<int32_t>(),
+                                        g->gofs.as<int64_t>(), g->ginfo.as<uint32_t>(), g->gwt.as<double>()));
         FL_LAUNCH(kProfSketchOther, k_wentries<<<grid_for(n, 8), 256, 0, st>>>(
-                                        ent.as<WEnt>(), (int)cap, ecnt.as<int32_t>(), g->eofs.as<int64_t>(), n,
-                                        g->eid.as<int32_t>()));
+                                        ent.as<WEnt>(), (int)cap, ecnt.as<int32_t>(), g->eofs.as<int64_t>(),
+                                        g->ord_rid.as<int32_t>(), n, g->eid.as<int32_t>()));
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) { rc = status_of(e, "weighted build", __FILE__, __LINE__); break; }
