@@ -643,7 +643,7 @@ struct fl_solve {
     int64_t n_cand = 0, n_open = 0, mis_rounds = 0;
     // opening phase with eps > 0: per-vertex iterations and scratch, the grid
     // tables, one iteration's selection inputs, statistics of the last run
-    fl::DBuf eps, eps_tab, eps_r, eps_c;
+    fl::DBuf eps, eps_tab, eps_ev, eps_r, eps_c;
     double eps_gamma = -1.0, eps_alpha0 = 0.0;
     int64_t eps_iterations = 0, eps_events = 0, eps_groups = 0;
     int have_eps = 0;

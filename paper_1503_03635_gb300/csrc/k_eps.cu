@@ -21,7 +21,15 @@
 // first at which a client freezes by binary search over (1 + eps) alpha_j.
 // The next event is the smallest of them; its openings and freezings are
 // applied and the search repeats.  The result is the iteration-by-iteration
-// loop's.
+// loop's.  Freezing a client can only lower q_j(f), so the iteration found for
+// a facility is a lower bound at every later event: a facility is looked at
+// again only while its bound is not above the next event found so far, and
+// most keep their bound.  Distances to the open set only fall, so an event
+// spreads from the facilities it opened alone.  The whole event loop is one
+// resident kernel, some seven grid barriers per event.  R-MAT, 65 k vertices,
+// eps = 0.1, 58 events: a full search per facility, a BFS from every open
+// facility, and four looks by the host per event took about 10 ms, the kernel
+// takes 2.4.
 //
 // Selection: H joins a client c to an open facility f iff alpha(c) =
 // alpha(f) and d(c, f) <= (1 + eps) alpha(c), so facilities opened in
@@ -150,7 +158,7 @@ struct EpsADS {
 // q_j(f) by the closed form (see the top of this file).
 __device__ double eps_q(const EpsADS& a, int64_t f, int32_t j, const double* __restrict__ grid, double onepe,
                         const int32_t* __restrict__ shell, int32_t nshell, const uint8_t* __restrict__ client,
-                        const int32_t* __restrict__ cli_iter) {
+                        const int32_t* cli_iter) {
     double q = 0.0;
     int64_t e = a.eofs[f];
     for (int64_t gi = a.gofs[f]; gi < a.gofs[f + 1]; ++gi) {
@@ -161,7 +169,8 @@ __device__ double eps_q(const EpsADS& a, int64_t f, int32_t j, const double* __r
         for (int i = 0; i < counted; ++i) {
             const int32_t w = a.eid[e + i];
             if (!client[w]) continue;
-            const int32_t jw = cli_iter[w] >= 0 ? cli_iter[w] : j;
+            const int32_t ji = __ldcg(&cli_iter[w]);  // written by the kernel that calls this
+            const int32_t jw = ji >= 0 ? ji : j;
             if (sj > jw) continue;  // the client's shell is beyond its radius
             q = __dadd_rn(q, __dmul_rn(wt, __dsub_rn(__dmul_rn(onepe, grid[jw]), grid[sj])));
         }
@@ -170,94 +179,200 @@ __device__ double eps_q(const EpsADS& a, int64_t f, int32_t j, const double* __r
     return q;
 }
 
-// First iteration in (jcur, J] at which each unopened facility opens, given
-// the current frozen clients (kNever: none); the smallest into *jmin.
-__global__ void k_eps_next_open(const int32_t* __restrict__ fac, int64_t n_fac, const int32_t* __restrict__ fac_iter,
-                                const double* __restrict__ cost, EpsADS a, const double* __restrict__ grid,
-                                double onepe, const int32_t* __restrict__ shell, int32_t nshell,
-                                const uint8_t* __restrict__ client, const int32_t* __restrict__ cli_iter, int32_t jcur,
-                                int32_t J, int32_t* __restrict__ nxt, int32_t* __restrict__ jmin) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_fac; i += stride) {
-        const int32_t f = fac[i];
-        if (fac_iter[f] >= 0) continue;
-        const double c = cost[f];
-        int32_t res = kNever;
-        if (jcur < J && eps_q(a, f, J, grid, onepe, shell, nshell, client, cli_iter) >= c) {
-            int32_t lo = jcur + 1, hi = J;
-            while (lo < hi) {
-                const int32_t mid = lo + (hi - lo) / 2;
-                if (eps_q(a, f, mid, grid, onepe, shell, nshell, client, cli_iter) >= c) hi = mid;
-                else lo = mid + 1;
+// Control block of the event loop (device, zero at its start).
+struct EpsCtl {
+    GridBar bar;                   // its err: 2: more events than iterations; 4: the level cap
+    int32_t jmin[3];               // next event's iteration (event number mod 3)
+    unsigned pad;
+    unsigned long long cnt[4];     // frontier list lengths (number of the pass mod 4)
+    long long events, jcur;
+};
+
+constexpr int kELong = 512;   // longer rows are spread by the whole block
+constexpr int kEQueue = 128;  // of them, queued per block and level
+
+struct EpsArgs {
+    const int64_t* rowp;
+    const int32_t* cols;
+    int64_t n;
+    const int32_t* fac;
+    int64_t n_fac;
+    const double* cost;
+    const uint8_t* client;
+    const double* gam;
+    EpsADS ads;
+    const double* grid;
+    const double* reach;
+    const int32_t* shell;
+    double onepe;
+    int32_t nshell, J;
+    int32_t* fac_iter;
+    int32_t* cli_iter;
+    int32_t* nxt;       // lower bound on the iteration at which each facility opens
+    uint32_t* dist;     // hops to the open set (all ones: none in reach)
+    int32_t* list[2];
+    int2* openings;     // (iteration, facilities opened) of each event
+    long long unfrozen;
+    int64_t cap;        // BFS levels at most (a search from every open facility would need one more than the largest distance)
+    EpsCtl* c;
+};
+
+// The events: see the top of this file.
+__global__ void __launch_bounds__(kResThreads, 1) k_eps_events(EpsArgs a) {
+    __shared__ int32_t s_v[kEQueue];
+    __shared__ unsigned s_queued;
+    EpsCtl* c = a.c;
+    const int lane = lane_id();
+    const int64_t tid = (int64_t)blockIdx.x * kResThreads + threadIdx.x, threads = (int64_t)gridDim.x * kResThreads;
+    const int64_t item0 = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x, warps = threads >> 5;
+    unsigned pass = 0, total = 0, lists = 0;  // lists: frontier lists filled
+    long long unopened = a.n_fac, unfrozen = a.unfrozen, events = 0;
+    int32_t jcur = 0;
+    if (threadIdx.x == 0) s_queued = 0;
+    for (int64_t i = tid; i < a.n_fac; i += threads) a.nxt[a.fac[i]] = 1;
+    if (tid < 3) c->jmin[tid] = kNever;
+    if (!end_pass(&c->bar, pass, 0, &total)) return;
+
+    auto q = [&](int32_t f, int32_t j) {
+        return eps_q(a.ads, f, j, a.grid, a.onepe, a.shell, a.nshell, a.client, a.cli_iter);
+    };
+    // u at distance L through a frontier vertex: into the list of the next level
+    auto offer = [&](int64_t e, int64_t end, uint32_t L) {
+        bool fresh = false;
+        int32_t u = 0;
+        if (e < end) {
+            u = __ldg(&a.cols[e]);
+            if (__ldcg(&a.dist[u]) > L) fresh = atomicMin(&a.dist[u], L) > L;
+        }
+        const long long at = warp_append(fresh, &c->cnt[lists & 3]);
+        if (at >= 0) a.list[lists & 1][at] = u;
+        return fresh;
+    };
+    while (unopened > 0 && unfrozen > 0) {
+        int32_t* jmin = &c->jmin[events % 3];  // holds the next freezing
+        if (tid == 0) c->jmin[(events + 1) % 3] = kNever;
+        // ---- the next opening
+        if (jcur < a.J)
+            for (int64_t i = tid; i < a.n_fac; i += threads) {
+                const int32_t f = a.fac[i];
+                if (__ldcg(&a.fac_iter[f]) >= 0) continue;
+                const int32_t lb = max(__ldcg(&a.nxt[f]), jcur + 1), top = min(a.J, __ldcg(jmin));
+                if (lb > top) continue;
+                const double cf = a.cost[f];
+                int32_t res;
+                if (q(f, lb) >= cf) {
+                    res = lb;
+                } else if (lb == top || !(q(f, top) >= cf)) {
+                    a.nxt[f] = top < a.J ? top + 1 : kNever;  // a bound, above this event
+                    continue;
+                } else {
+                    int32_t lo = lb + 1, hi = top;
+                    while (lo < hi) {
+                        const int32_t mid = lo + (hi - lo) / 2;
+                        if (q(f, mid) >= cf) hi = mid;
+                        else lo = mid + 1;
+                    }
+                    res = lo;
+                }
+                a.nxt[f] = res;
+                atomicMin(jmin, res);
             }
-            res = lo;
-            atomicMin(jmin, res);
+        if (!end_pass(&c->bar, pass, 0, &total)) return;
+        const int32_t js = __ldcg(jmin);
+        if (js == kNever) {
+            jcur = a.J;  // nothing changes any more up to the last radius of the grid
+            break;
         }
-        nxt[f] = res;
-    }
-}
-
-// First iteration in (jcur, J] at which each unfrozen client that reaches a
-// facility freezes, given the distances to the open facilities.
-__global__ void k_eps_next_freeze(const uint8_t* __restrict__ client, const double* __restrict__ gam,
-                                  const int32_t* __restrict__ cli_iter, const int32_t* __restrict__ dist, int64_t n,
-                                  const double* __restrict__ reach, int32_t jcur, int32_t J,
-                                  int32_t* __restrict__ jmin) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
-        if (!client[v] || cli_iter[v] >= 0 || !(gam[v] < INFINITY) || dist[v] < 0 || jcur >= J) continue;
-        const double d = (double)dist[v];
-        if (!(reach[J] >= d)) continue;
-        int32_t lo = jcur + 1, hi = J;
-        while (lo < hi) {
-            const int32_t mid = lo + (hi - lo) / 2;
-            if (reach[mid] >= d) hi = mid;
-            else lo = mid + 1;
+        ++events;
+        if (events > (long long)a.J + 1) {
+            if (tid == 0) c->bar.err = 2;
+            return;
         }
-        atomicMin(jmin, lo);
-    }
-}
-
-// Open the facilities of iteration j; list every open facility (for the
-// distances to the open set).
-__global__ void k_eps_open(const int32_t* __restrict__ fac, int64_t n_fac, const int32_t* __restrict__ nxt, int32_t j,
-                           int32_t* __restrict__ fac_iter, int32_t* __restrict__ open_list,
-                           unsigned long long* __restrict__ cnt) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n_fac; base += stride) {
-        const int64_t i = base + lane_id();
-        const int32_t f = i < n_fac ? fac[i] : 0;
-        bool is_open = false, opened = false;
-        if (i < n_fac) {
-            if (fac_iter[f] < 0 && nxt[f] == j) {
-                fac_iter[f] = j;
-                opened = true;
+        // ---- its facilities open (a bound equal to js was confirmed above)
+        unsigned opened = 0;
+        if (tid == 0) c->cnt[(lists + 1) & 3] = 0;
+        for (int64_t b = (tid >> 5) * 32; b < a.n_fac; b += warps * 32) {
+            const int32_t f = b + lane < a.n_fac ? a.fac[b + lane] : -1;
+            const bool now = f >= 0 && __ldcg(&a.fac_iter[f]) < 0 && __ldcg(&a.nxt[f]) == js;
+            if (now) {
+                a.fac_iter[f] = js;
+                a.dist[f] = 0u;
+                ++opened;
             }
-            is_open = fac_iter[f] >= 0;
+            const long long at = warp_append(now, &c->cnt[lists & 3]);
+            if (at >= 0) a.list[lists & 1][at] = f;
         }
-        const long long at = warp_append(is_open, &cnt[0]);
-        if (at >= 0) open_list[at] = f;
-        const unsigned m = __ballot_sync(kFull, opened);
-        if (lane_id() == 0 && m) atomicAdd(&cnt[1], (unsigned long long)__popc(m));
-    }
-}
-
-// Freeze the unfrozen clients with an open facility within (1 + eps) alpha_j.
-__global__ void k_eps_freeze(const uint8_t* __restrict__ client, const double* __restrict__ gam,
-                             int32_t* __restrict__ cli_iter, const int32_t* __restrict__ dist, int64_t n, double reach_j,
-                             int32_t j, unsigned long long* __restrict__ cnt) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    unsigned long long c = 0;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
-        if (!client[v] || cli_iter[v] >= 0 || !(gam[v] < INFINITY) || dist[v] < 0) continue;
-        if ((double)dist[v] <= reach_j) {
-            cli_iter[v] = j;
-            ++c;
+        if (!end_pass(&c->bar, pass, opened, &total)) return;
+        if (tid == 0) a.openings[events - 1] = make_int2(js, (int)total);
+        unopened -= (long long)total;
+        // ---- distances to the open set
+        for (uint32_t L = 1; total; ++L) {
+            const int32_t* list = a.list[lists & 1];
+            const int64_t n_front = (int64_t)total;
+            ++lists;
+            if (tid == 0) c->cnt[(lists + 1) & 3] = 0;
+            unsigned found = 0;
+            for (int64_t i = item0; i < n_front; i += warps) {
+                const int32_t v = __ldcg(&list[i]);
+                const int64_t beg = __ldg(&a.rowp[v]), end = __ldg(&a.rowp[v + 1]);
+                if (end - beg > kELong) {
+                    unsigned at = 0;
+                    if (lane == 0) at = atomicAdd(&s_queued, 1u);
+                    at = __shfl_sync(kFull, at, 0);
+                    if (at < kEQueue) {
+                        if (lane == 0) s_v[at] = v;
+                        continue;
+                    }
+                }
+                for (int64_t e = beg; e < end; e += 32) found += offer(e + lane, end, L);
+            }
+            __syncthreads();
+            const int queued = (int)min(s_queued, (unsigned)kEQueue);
+            for (int x = 0; x < queued; ++x) {
+                const int64_t end = __ldg(&a.rowp[s_v[x] + 1]);
+                for (int64_t e = __ldg(&a.rowp[s_v[x]]) + (threadIdx.x & ~31); e < end; e += kResThreads)
+                    found += offer(e + lane, end, L);
+            }
+            __syncthreads();
+            if (threadIdx.x == 0) s_queued = 0;
+            if (!end_pass(&c->bar, pass, found, &total)) return;
         }
+        ++lists;
+        // ---- its clients freeze; the next freezing of the others
+        unsigned frozen = 0;
+        int32_t next = kNever;
+        const double reach_j = __ldg(&a.reach[js]);
+        for (int64_t v = tid; v < a.n; v += threads) {
+            const uint32_t du = __ldcg(&a.dist[v]);
+            if ((int32_t)du < 0) continue;
+            if ((int64_t)du >= a.cap) atomicOr(&c->bar.err, 4u);
+            if (!a.client[v] || __ldcg(&a.cli_iter[v]) >= 0 || !(a.gam[v] < INFINITY)) continue;
+            const double d = (double)du;
+            if (d <= reach_j) {
+                a.cli_iter[v] = js;
+                ++frozen;
+            } else if (js < a.J && __ldg(&a.reach[a.J]) >= d) {
+                int32_t lo = js + 1, hi = min(a.J, next);
+                if (!(__ldg(&a.reach[hi]) >= d)) continue;  // later than this thread's earliest
+                while (lo < hi) {
+                    const int32_t mid = lo + (hi - lo) / 2;
+                    if (__ldg(&a.reach[mid]) >= d) hi = mid;
+                    else lo = mid + 1;
+                }
+                next = lo;
+            }
+        }
+        next = (int32_t)__reduce_min_sync(kFull, (unsigned)next);
+        if (lane == 0 && next != kNever) atomicMin(&c->jmin[events % 3], next);
+        if (!end_pass(&c->bar, pass, frozen, &total)) return;
+        if (__ldcg(&c->bar.err)) return;
+        unfrozen -= (long long)total;
+        jcur = js;
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(kFull, c, o);
-    if (lane_id() == 0 && c) atomicAdd(cnt, c);
+    if (tid == 0) {
+        c->events = events;
+        c->jcur = jcur;
+    }
 }
 
 // The facility list (finite costs).
@@ -330,7 +445,7 @@ int open_facilities_eps(fl_solve* s, double eps) {
     const double onepe = 1.0 + eps;
     const double* cost = s->cost.as<double>();
     const uint8_t* client = s->client.as<uint8_t>();
-    // scratch: fac_iter, cli_iter, nxt, facility list, open list, dist, label
+    // scratch: fac_iter, cli_iter, nxt, facility list, dist, two frontier lists
     // (int32); gamma (double); M[2] (uint64); selected (uint8); counters
     DBuf& E = s->eps;
     const size_t i32n = (size_t)n * 4;
@@ -343,15 +458,13 @@ int open_facilities_eps(fl_solve* s, double eps) {
     int32_t* cli_iter = fac_iter + n;
     int32_t* nxt = cli_iter + n;
     int32_t* fac = nxt + n;
-    int32_t* open_list = fac + n;
-    int32_t* dist = open_list + n;
-    int32_t* label = dist + n;
+    int32_t* dist = fac + n;
+    int32_t* list[2] = {dist + n, dist + 2 * n};  // frontier lists
     double* gam = reinterpret_cast<double*>(base + off_gam);
     unsigned long long* M[2] = {reinterpret_cast<unsigned long long*>(base + off_M),
                                 reinterpret_cast<unsigned long long*>(base + off_M) + n};
     uint8_t* acc = reinterpret_cast<uint8_t*>(base + off_acc);
     unsigned long long* ctr = reinterpret_cast<unsigned long long*>(base + off_ctr);
-    int32_t* jmin = reinterpret_cast<int32_t*>(ctr + 16);
     FL_CUDA(cudaMemsetAsync(fac_iter, 0xff, i32n * 2, st));
     FL_CUDA(cudaMemsetAsync(dist, 0xff, i32n, st));
     FL_CUDA(cudaMemsetAsync(acc, 0, (size_t)n, st));
@@ -406,7 +519,7 @@ int open_facilities_eps(fl_solve* s, double eps) {
     if (h[1] == 0) return finish();  // no client reaches a facility
     double gamma = 0.0;
     std::memcpy(&gamma, &h[0], 8);
-    int64_t unfrozen = (int64_t)h[1];
+    const int64_t unfrozen = (int64_t)h[1];
     s->eps_gamma = gamma;
 
     // the grid of radii, (1 + eps) alpha_j, and the shell of every hop distance
@@ -446,43 +559,62 @@ int open_facilities_eps(fl_solve* s, double eps) {
     ads.eid = g->eid.as<int32_t>();
 
     // events: the next iteration at which a facility opens or a client freezes
-    int64_t unopened = nF;
-    int32_t jcur = 0;
     std::vector<std::pair<int32_t, int64_t>> openings;  // (iteration, facilities opened)
-    while (unopened > 0 && unfrozen > 0) {
-        if (s->eps_events > (int64_t)J + 1) FL_FAIL(FL_ETIMEOUT, "epsilon phase: more events than iterations");
-        const int32_t never = kNever;
-        FL_CUDA(cudaMemcpyAsync(jmin, &never, 4, cudaMemcpyHostToDevice, st));
-        FL_LAUNCH(kProfMis, k_eps_next_open<<<grid_for(nF, 128), 128, 0, st>>>(
-                                fac, nF, fac_iter, cost, ads, grid_d, onepe, shell_d, nshell, client, cli_iter, jcur,
-                                J, nxt, jmin));
-        FL_LAUNCH(kProfMis, k_eps_next_freeze<<<grid_for(n, 256), 256, 0, st>>>(client, gam, cli_iter, dist, n,
-                                                                                  reach_d, jcur, J, jmin));
-        int32_t js = kNever;
-        FL_CUDA(cudaMemcpyAsync(&js, jmin, 4, cudaMemcpyDeviceToHost, st));
+    {
+        EpsArgs a;
+        a.rowp = g->rowp.as<int64_t>();
+        a.cols = g->cols.as<int32_t>();
+        a.n = n;
+        a.fac = fac;
+        a.n_fac = nF;
+        a.cost = cost;
+        a.client = client;
+        a.gam = gam;
+        a.ads = ads;
+        a.grid = grid_d;
+        a.reach = reach_d;
+        a.shell = shell_d;
+        a.onepe = onepe;
+        a.nshell = nshell;
+        a.J = J;
+        a.fac_iter = fac_iter;
+        a.cli_iter = cli_iter;
+        a.nxt = nxt;
+        a.dist = reinterpret_cast<uint32_t*>(dist);
+        a.list[0] = list[0];
+        a.list[1] = list[1];
+        a.unfrozen = unfrozen;
+        a.cap = g->sched.level_cap > 0 ? g->sched.level_cap : n + 2;
+        const size_t ctl_b = (sizeof(EpsCtl) + 255) & ~(size_t)255;
+        FL_TRY(dalloc(s->eps_ev, ctl_b + ((size_t)J + 2) * sizeof(int2)));
+        a.c = s->eps_ev.as<EpsCtl>();
+        a.openings = reinterpret_cast<int2*>(s->eps_ev.as<char>() + ctl_b);
+        FL_CUDA(cudaMemsetAsync(a.c, 0, sizeof(EpsCtl), st));
+        int dev = 0, sms = 0;
+        FL_CUDA(cudaGetDevice(&dev));
+        FL_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(sms, n / 64));
+        void* args[] = {&a};
+        cudaError_t le = cudaSuccess;
+        FL_LAUNCH(kProfMis, le = cudaLaunchCooperativeKernel((const void*)k_eps_events, dim3(blocks),
+                                                             dim3(kResThreads), args, 0, st));
+        FL_CUDA(le);
+        EpsCtl hc{};
+        FL_CUDA(cudaMemcpyAsync(&hc, a.c, sizeof(EpsCtl), cudaMemcpyDeviceToHost, st));
         FL_CUDA(cudaStreamSynchronize(st));
-        if (js == kNever) {
-            jcur = J;  // nothing changes any more up to the last radius of the grid
-            break;
+        if (hc.bar.err & 2u) FL_FAIL(FL_ETIMEOUT, "epsilon phase: more events than iterations");
+        if (hc.bar.err & 4u) FL_FAIL(FL_ETIMEOUT, "BFS reached its level cap");
+        if (hc.bar.err) FL_FAIL(FL_ETIMEOUT, "epsilon phase: a barrier wait ran out");
+        std::vector<int2> ev((size_t)hc.events);
+        if (hc.events > 0) {
+            FL_CUDA(cudaMemcpyAsync(ev.data(), a.openings, ev.size() * sizeof(int2), cudaMemcpyDeviceToHost, st));
+            FL_CUDA(cudaStreamSynchronize(st));
         }
-        ++s->eps_events;
-        FL_CUDA(cudaMemsetAsync(&ctr[9], 0, 24, st));
-        FL_LAUNCH(kProfMis, k_eps_open<<<grid_for(nF, 256), 256, 0, st>>>(fac, nF, nxt, js, fac_iter, open_list,
-                                                                            &ctr[9]));
-        FL_TRY(read_u64(&ctr[9], h, 2, st));
-        const int64_t n_open_all = (int64_t)h[0], opened = (int64_t)h[1];
-        if (opened > 0) {
-            unopened -= opened;
-            openings.push_back({js, opened});
-            FL_TRY(msbfs(g, open_list, n_open_all, label, dist, s->X, s->stamp, s->fr, s->frval, kProfMis));
-        }
-        FL_LAUNCH(kProfMis, k_eps_freeze<<<grid_for(n, 256), 256, 0, st>>>(client, gam, cli_iter, dist, n,
-                                                                             reach[js], js, &ctr[11]));
-        FL_TRY(read_u64(&ctr[11], h, 1, st));
-        unfrozen -= (int64_t)h[0];
-        jcur = js;
+        for (const int2& o : ev)
+            if (o.y > 0) openings.push_back({o.x, (int64_t)o.y});
+        s->eps_events = hc.events;
+        s->eps_iterations = hc.jcur;
     }
-    s->eps_iterations = jcur;
 
     // selection: one lexicographically-first MIS per iteration that opened
     // two or more facilities; the others' facilities are selected directly

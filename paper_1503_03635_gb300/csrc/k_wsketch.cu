@@ -35,9 +35,9 @@
 // entries are posted by the whole block, so that no level waits for one warp
 // on a hub.  Bound by the latency of the dependent loads of a post (column,
 // k-th rank, sketch).  R-MAT, 65 k vertices, lengths up to 100, k = 16, 313
-// levels: 115 ms of level kernels and some 15 ms of gaps before, 23.6 ms now (36
-// with bisections in place of the 8-way search and the 8-wide sketch test, 29
-// with 64-bit ranks in place of their ordinals).
+// levels: 115 ms of level kernels and some 15 ms of gaps before, 23.6 ms now
+// (36 with bisections in place of the 8-way search and the 8-wide sketch test,
+// 29 with 64-bit ranks in place of their ordinals).
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
