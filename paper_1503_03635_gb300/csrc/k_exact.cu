@@ -14,9 +14,11 @@
 // frontier's row entries against the entries of rows that still need bits:
 //   bottom-up: every vertex that some running source has not reached ORs
 //     its neighbours' frontier words and keeps the new bits.  Rows longer
-//     than 32 entries get a whole warp (8 neighbours x 4 words per step,
-//     stopping once every needed bit is in); shorter rows get 4 lanes, one
-//     word each, so the 4 words of a neighbour are one 32-byte sector.
+//     than 32 entries get a whole warp (8 neighbours x 4 words, four of them
+//     in flight, stopping once every needed bit is in) and rows longer than
+//     1024 a whole block (a warp on the largest hub was most of a level);
+//     shorter rows get 4 lanes, one word each, so the 4 words of a neighbour
+//     are one 32-byte sector.
 //   top-down (sparse frontiers, e.g. the sources themselves): the frontier
 //     rows, cut into work items of 256 entries (so a hub's row is spread
 //     over many warps), OR their bits into the neighbours' next words
@@ -34,6 +36,7 @@ namespace {
 constexpr int kXW = 4;          // 64-bit words of source bits per vertex
 constexpr int kXS = 64 * kXW;   // sources per sweep
 constexpr int kXHeavy = 32;     // rows longer than this get a whole warp
+constexpr int kXHuge = 1024;    // ... and longer than this a whole block
 constexpr int kXBlocks = 152 * 8;
 
 enum XMode { kXSizes = 0, kXRadius = 1 };
@@ -78,10 +81,11 @@ __global__ void k_x_map(const int32_t* __restrict__ src, int64_t n_src, const in
     }
 }
 
-// Vertices with short rows (<= kXHeavy entries, isolated ones included) and
-// with long rows.
+// Vertices with short rows (<= kXHeavy entries, isolated ones included), with
+// long rows, and with rows above kXHuge entries (from the end of `heavy`).
 __global__ void k_x_lists(const int64_t* __restrict__ rowp, int64_t n, int32_t* __restrict__ light,
-                          int32_t* __restrict__ heavy, unsigned long long* n_light, unsigned long long* n_heavy) {
+                          int32_t* __restrict__ heavy, unsigned long long* n_light, unsigned long long* n_heavy,
+                          unsigned long long* n_huge) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += stride) {
         const int64_t v = base + lane_id();
@@ -89,8 +93,10 @@ __global__ void k_x_lists(const int64_t* __restrict__ rowp, int64_t n, int32_t* 
         const int64_t deg = valid ? rowp[v + 1] - rowp[v] : 0;
         const long long a = warp_append(valid && deg <= kXHeavy, n_light);
         if (a >= 0) light[a] = (int32_t)v;
-        const long long b = warp_append(valid && deg > kXHeavy, n_heavy);
+        const long long b = warp_append(valid && deg > kXHeavy && deg <= kXHuge, n_heavy);
         if (b >= 0) heavy[b] = (int32_t)v;
+        const long long c = warp_append(valid && deg > kXHuge, n_huge);
+        if (c >= 0) heavy[n - 1 - c] = (int32_t)v;
     }
 }
 
@@ -267,8 +273,8 @@ __global__ void __launch_bounds__(256) k_x_light(const int32_t* __restrict__ lis
 }
 
 // Bottom-up level for vertices with long rows: a warp per vertex, lane
-// (t, w) reads word w of neighbours t, t+8, ...; every 256 entries the warp
-// stops if its OR already holds every bit the vertex needs.
+// (t, w) reads word w of neighbours t, t+8, ..., four in flight; every 128
+// entries the warp stops if its OR already holds every bit the vertex needs.
 __global__ void __launch_bounds__(256) k_x_heavy(const int32_t* __restrict__ list, int64_t n_list,
                                                  const int64_t* __restrict__ rowp, const int32_t* __restrict__ cols,
                                                  const unsigned long long* __restrict__ cur,
@@ -298,18 +304,21 @@ __global__ void __launch_bounds__(256) k_x_heavy(const int32_t* __restrict__ lis
             deg = end - beg;
             int64_t stop = end;
             unsigned long long acc = 0;
-            for (int64_t b0 = beg; b0 < end; b0 += 16) {
-                const int64_t e0 = b0 + t, e1 = b0 + 8 + t;
-                if (e0 < end) acc |= __ldg(&cur[(int64_t)__ldg(&cols[e0]) * kXW + w]);
-                if (e1 < end) acc |= __ldg(&cur[(int64_t)__ldg(&cols[e1]) * kXW + w]);
-                if (((b0 - beg) & 255) == 240) {
+            for (int64_t b0 = beg; b0 < end; b0 += 32) {
+                int32_t u[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) u[j] = b0 + 8 * j + t < end ? __ldg(&cols[b0 + 8 * j + t]) : -1;
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (u[j] >= 0) acc |= __ldg(&cur[(int64_t)u[j] * kXW + w]);
+                if (((b0 - beg) & 127) == 96) {
                     unsigned long long a = acc;
                     a |= __shfl_xor_sync(kFull, a, 4);
                     a |= __shfl_xor_sync(kFull, a, 8);
                     a |= __shfl_xor_sync(kFull, a, 16);
                     if (__all_sync(kFull, (a & need) == need)) {
                         acc = a;
-                        stop = b0 + 16 < end ? b0 + 16 : end;
+                        stop = b0 + 32 < end ? b0 + 32 : end;
                         break;
                     }
                 }
@@ -340,6 +349,91 @@ __global__ void __launch_bounds__(256) k_x_heavy(const int32_t* __restrict__ lis
         const unsigned long long cv = (!pred || pred[v]) ? nx : 0ULL;
 #pragma unroll
         for (int j = 0; j < 8; ++j) c[j] += (unsigned)((cv >> (8 * j + t)) & 1ULL);
+    }
+    x_flush(c, any, m, s_cnt, s_any, st);
+}
+
+// Bottom-up level for the longest rows: a block per vertex, 1024 entries per
+// step (lane (t, w) of warp p reads word w of entries 64 j + 8 p + t), stopping
+// like k_x_heavy.
+__global__ void __launch_bounds__(256) k_x_huge(const int32_t* __restrict__ list, int64_t n_list,
+                                                const int64_t* __restrict__ rowp, const int32_t* __restrict__ cols,
+                                                const unsigned long long* __restrict__ cur,
+                                                unsigned long long* __restrict__ nxt, unsigned long long* vis,
+                                                const uint8_t* __restrict__ pred, int32_t* __restrict__ next_front,
+                                                XState* __restrict__ st) {
+    __shared__ unsigned s_cnt[kXS];
+    __shared__ unsigned long long s_any[kXW];
+    __shared__ unsigned long long s_acc[2][8][kXW];
+    for (int i = threadIdx.x; i < kXS; i += blockDim.x) s_cnt[i] = 0;
+    if (threadIdx.x < kXW) s_any[threadIdx.x] = 0;
+    __syncthreads();
+    const int lane = lane_id(), warp = threadIdx.x >> 5;
+    const int w = lane & 3, t = lane >> 2;
+    const unsigned long long act = st->active[w];
+    unsigned c[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    unsigned long long any = 0;
+    XSums m;
+    int par = 0;
+    for (int64_t i = blockIdx.x; i < n_list; i += gridDim.x) {
+        const int32_t v = __ldg(&list[i]);
+        const unsigned long long vw = vis[(int64_t)v * kXW + w];
+        const unsigned long long need = act & ~vw;
+        unsigned long long nx = 0;
+        int64_t deg = 0;
+        if (__any_sync(kFull, need != 0)) {  // the same in every warp
+            const int64_t beg = __ldg(&rowp[v]), end = __ldg(&rowp[v + 1]);
+            deg = end - beg;
+            int64_t b0 = beg;
+            unsigned long long acc = 0;
+            for (bool more = true; more;) {
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                    int32_t u[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int64_t e = b0 + 64 * (4 * h + j) + 8 * warp + t;
+                        u[j] = e < end ? __ldg(&cols[e]) : -1;
+                    }
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (u[j] >= 0) acc |= __ldg(&cur[(int64_t)u[j] * kXW + w]);
+                }
+                acc |= __shfl_xor_sync(kFull, acc, 4);
+                acc |= __shfl_xor_sync(kFull, acc, 8);
+                acc |= __shfl_xor_sync(kFull, acc, 16);
+                if (t == 0) s_acc[par][warp][w] = acc;
+                __syncthreads();
+#pragma unroll
+                for (int p = 0; p < 8; ++p) acc |= s_acc[par][p][w];
+                par ^= 1;  // the other buffer was last read before this step's barrier
+                b0 = b0 + 1024 < end ? b0 + 1024 : end;
+                more = b0 < end && !__all_sync(kFull, (acc & need) == need);
+            }
+            nx = acc & need;
+            if (threadIdx.x == 0) {
+                ++m.rows;
+                m.entries += (unsigned long long)(b0 - beg);
+            }
+        }
+        if (warp == 0) {
+            if (t == 0) {
+                nxt[(int64_t)v * kXW + w] = nx;
+                if (nx) vis[(int64_t)v * kXW + w] = vw | nx;
+            }
+            any |= nx;
+            const bool got = __any_sync(kFull, nx != 0);
+            const bool left = __any_sync(kFull, (need & ~nx) != 0);
+            const long long at = warp_append(lane == 0 && got, &st->n_next);
+            if (at >= 0) {
+                next_front[at] = v;
+                m.fr_edges += (unsigned long long)deg;
+            }
+            if (lane == 0 && left) m.rem_edges += (unsigned long long)deg;
+            const unsigned long long cv = (!pred || pred[v]) ? nx : 0ULL;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) c[j] += (unsigned)((cv >> (8 * j + t)) & 1ULL);
+        }
     }
     x_flush(c, any, m, s_cnt, s_any, st);
 }
@@ -608,10 +702,13 @@ int run_sweeps(fl_graph* g, int mode, int64_t n_src, const int32_t* src, int64_t
     const int32_t* cols = g->cols.as<int32_t>();
 
     FL_CUDA(cudaMemsetAsync(g->ctr.p, 0, sizeof(Counters), st));
-    FL_LAUNCH(cls, k_x_lists<<<blocks_for(n, 256), 256, 0, st>>>(rowp, n, light, heavy, &ctr->aux0, &ctr->aux3));
+    FL_LAUNCH(cls, k_x_lists<<<blocks_for(n, 256), 256, 0, st>>>(rowp, n, light, heavy, &ctr->aux0, &ctr->aux3,
+                                                               &ctr->frontier));
     FL_CUDA(cudaGetLastError());
     FL_TRY(read_counters(g));
     const int64_t n_light = (int64_t)g->h_ctr->aux0, n_heavy = (int64_t)g->h_ctr->aux3;
+    const int64_t n_huge = (int64_t)g->h_ctr->frontier;
+    const int32_t* huge = heavy + n - n_huge;
     const int grid_l = blocks_for(n_light, 64);  // 8 warps x 8 vertices per block pass
     const int grid_h = blocks_for(n_heavy, 8);   // 8 warps x 1 vertex
 
@@ -649,6 +746,9 @@ int run_sweeps(fl_graph* g, int mode, int64_t n_src, const int32_t* src, int64_t
                 FL_LAUNCH(cls, k_x_td_finish<<<blocks_for(n, 64), 256, 0, st>>>(n, rowp, buf[c ^ 1], vis, pred,
                                                                                 front[fc ^ 1], xs));
             } else {
+                if (n_huge > 0)
+                    FL_LAUNCH(cls, k_x_huge<<<blocks_for(n_huge, 1), 256, 0, st>>>(
+                                       huge, n_huge, rowp, cols, buf[c], buf[c ^ 1], vis, pred, front[fc ^ 1], xs));
                 if (n_heavy > 0)
                     FL_LAUNCH(cls, k_x_heavy<<<grid_h, 256, 0, st>>>(heavy, n_heavy, rowp, cols, buf[c], buf[c ^ 1],
                                                                      vis, pred, front[fc ^ 1], xs));
