@@ -5,8 +5,12 @@
 // distance in place of the HIP estimate).
 //
 // Exact sizes come from a bit-parallel breadth-first search.  One sweep
-// serves 256 sources; every vertex holds 4 words of source bits for
-// "visited", "frontier" and "next".  A source stops when its question is
+// serves 64 W sources; every vertex holds W words of source bits for
+// "visited", "frontier" and "next".  W is 4, 8 or 16, the smallest that takes
+// the sources left (graphs above kXWideN vertices: 4, for their scratch): a
+// level's launches and its look by the host serve four times the sources at
+// W = 16, and a neighbour is one 128-byte line instead of four 32-byte sectors
+// in four sweeps.  A source stops when its question is
 // answered -- ball sizes at the largest distance asked for or when its
 // component is exhausted, a radius when the walk of Eq. 1 has its root --
 // and its bit is masked out of every later level.  Each level runs in one of
@@ -14,11 +18,10 @@
 // frontier's row entries against the entries of rows that still need bits:
 //   bottom-up: every vertex that some running source has not reached ORs
 //     its neighbours' frontier words and keeps the new bits.  Rows longer
-//     than 32 entries get a whole warp (8 neighbours x 4 words, four of them
-//     in flight, stopping once every needed bit is in) and rows longer than
-//     1024 a whole block (a warp on the largest hub was most of a level);
-//     shorter rows get 4 lanes, one word each, so the 4 words of a neighbour
-//     are one 32-byte sector.
+//     than 32 entries get a whole warp (32 / W neighbours x W words at a time,
+//     several in flight, stopping once every needed bit is in) and rows longer
+//     than 1024 a whole block (a warp on the largest hub was most of a level);
+//     shorter rows get W lanes, one word each.
 //   top-down (sparse frontiers, e.g. the sources themselves): the frontier
 //     rows, cut into work items of 256 entries (so a hub's row is spread
 //     over many warps), OR their bits into the neighbours' next words
@@ -26,6 +29,7 @@
 //     "visited" and counts them.
 // Both directions count the new bits per source under the predicate and
 // list the next frontier with its row entries.
+#include <algorithm>
 #include <cmath>
 
 #include "fl_internal.cuh"
@@ -33,21 +37,24 @@
 namespace fl {
 namespace {
 
-constexpr int kXW = 4;          // 64-bit words of source bits per vertex
-constexpr int kXS = 64 * kXW;   // sources per sweep
+constexpr int kXMaxW = 16;      // 64-bit words of source bits per vertex, at most
+constexpr int64_t kXWideN = 1 << 20;  // larger graphs take W = 4
 constexpr int kXHeavy = 32;     // rows longer than this get a whole warp
 constexpr int kXHuge = 1024;    // ... and longer than this a whole block
 constexpr int kXBlocks = 152 * 8;
+constexpr int kXLevelBlocks = 152 * 4;  // level kernels: each warp flushes its counts once
 
 enum XMode { kXSizes = 0, kXRadius = 1 };
 
 // State of one sweep (device).
+template <int W>
 struct XState {
-    unsigned long long active[kXW];  // sources still searching
-    unsigned long long any[kXW];     // sources that reached a vertex at this level
-    unsigned long long cnt[kXS];     // this level's newly reached vertices under the predicate
-    long long N[kXS];                // sizes: running ball size; radius: N_j
-    long long G[kXS], Gp[kXS];       // radius: G_{j+1} and G_j of the walk
+    static constexpr int kS = 64 * W;  // sources
+    unsigned long long active[W];    // sources still searching
+    unsigned long long any[W];       // sources that reached a vertex at this level
+    unsigned long long cnt[kS];      // this level's newly reached vertices under the predicate
+    long long N[kS];                 // sizes: running ball size; radius: N_j
+    long long G[kS], Gp[kS];         // radius: G_{j+1} and G_j of the walk
     unsigned long long rows, entries;  // rows scanned and their entries read (this sweep, cumulative)
     unsigned long long n_next;       // this level: vertices listed in the next frontier
     unsigned long long fr_edges;     // this level: row entries of the next frontier
@@ -59,10 +66,10 @@ struct XSums {
     unsigned long long rows = 0, entries = 0, fr_edges = 0, rem_edges = 0;
 };
 
-int blocks_for(int64_t items, int64_t per_block) {
+int blocks_for(int64_t items, int64_t per_block, int most = kXBlocks) {
     int64_t b = (items + per_block - 1) / per_block;
     if (b < 1) b = 1;
-    if (b > kXBlocks) b = kXBlocks;
+    if (b > most) b = most;
     return (int)b;
 }
 
@@ -121,16 +128,17 @@ __global__ void k_x_facilities(const double* __restrict__ cost, int64_t n, int32
 
 // Start of a sweep: the sources' own bits in "visited" and "frontier"
 // (which the host cleared), the sources as the first frontier list, cleared
-// counters.  One block of kXS threads.
+// counters.  One block of 64 W threads.
+template <int W>
 __global__ void k_x_seed(const int32_t* __restrict__ src, int64_t nb, const int64_t* __restrict__ rowp,
                          unsigned long long* __restrict__ vis, unsigned long long* __restrict__ cur,
-                         int32_t* __restrict__ front, XState* __restrict__ st) {
+                         int32_t* __restrict__ front, XState<W>* __restrict__ st) {
     const int s = threadIdx.x;
     st->cnt[s] = 0;
     st->N[s] = 0;
     st->G[s] = 0;
     st->Gp[s] = 0;
-    if (s < kXW) {
+    if (s < W) {
         const int64_t m = nb - 64LL * s;  // sources in word s
         st->active[s] = m <= 0 ? 0ULL : (m >= 64 ? ~0ULL : ((1ULL << m) - 1ULL));
         st->any[s] = 0;
@@ -144,28 +152,70 @@ __global__ void k_x_seed(const int32_t* __restrict__ src, int64_t nb, const int6
     if (s < nb) {
         const int32_t v = src[s];
         const unsigned long long bit = 1ULL << (s & 63);
-        atomicOr(&vis[(int64_t)v * kXW + (s >> 6)], bit);
-        atomicOr(&cur[(int64_t)v * kXW + (s >> 6)], bit);
+        atomicOr(&vis[(int64_t)v * W + (s >> 6)], bit);
+        atomicOr(&cur[(int64_t)v * W + (s >> 6)], bit);
         front[s] = v;  // a source listed twice is harmless
         atomicAdd(&st->fr_edges, (unsigned long long)(rowp[v + 1] - rowp[v]));
     }
 }
 
+// Shared memory of a level kernel: counts per source, bit b of word w at
+// [b * W + w] (the lanes of a group count different words: no bank conflicts).
+template <int W>
+struct XShared {
+    unsigned cnt[64 * W];
+    unsigned long long any[W];
+};
 
-// Per-lane counters of one word's bits -> the sweep's per-source counts
-// (lane (q, w) owns bits 8j + q of word w, j = 0..7), the OR of the new
-// bits and the level's sums.  Every thread of the block calls.
-__device__ __forceinline__ void x_flush(const unsigned (&c)[8], unsigned long long any, XSums m, unsigned* s_cnt,
-                                        unsigned long long* s_any, XState* st) {
-    const int lane = lane_id();
-    const int w = lane & 3, q = lane >> 2;
+template <int W>
+__device__ __forceinline__ void x_init(XShared<W>& sh) {
+    for (int i = threadIdx.x; i < 64 * W; i += blockDim.x) sh.cnt[i] = 0;
+    if (threadIdx.x < W) sh.any[threadIdx.x] = 0;
+    __syncthreads();
+}
+
+// Per-bit counts of the words that a lane adds, as five bit planes (a carry
+// chain of ten operations per word, where a ballot per bit took 64 for the
+// warp): up to 31 words between two flushes.
+struct XPlanes {
+    unsigned long long p[5] = {0, 0, 0, 0, 0};
+    int n = 0;
+    __device__ __forceinline__ void add(unsigned long long x) {
 #pragma unroll
-    for (int j = 0; j < 8; ++j)
-        if (c[j]) atomicAdd(&s_cnt[w * 64 + 8 * j + q], c[j]);
-    any |= __shfl_xor_sync(kFull, any, 4);
-    any |= __shfl_xor_sync(kFull, any, 8);
-    any |= __shfl_xor_sync(kFull, any, 16);
-    if (lane < kXW && any) atomicOr(&s_any[lane], any);
+        for (int i = 0; i < 5; ++i) {
+            const unsigned long long c = p[i] & x;
+            p[i] ^= x;
+            x = c;
+        }
+        ++n;
+    }
+    // to the block's counts of word w; rot spreads the lanes that share w (all 32 lanes call)
+    template <int W>
+    __device__ __forceinline__ void flush(XShared<W>& sh, int w, int rot) {
+        n = 0;
+        if (!__any_sync(kFull, (p[0] | p[1] | p[2] | p[3] | p[4]) != 0)) return;
+        for (int i = 0; i < 64; ++i) {
+            const int b = (i + rot) & 63;
+            const unsigned c = (unsigned)((p[0] >> b) & 1) | ((unsigned)((p[1] >> b) & 1) << 1) |
+                               ((unsigned)((p[2] >> b) & 1) << 2) | ((unsigned)((p[3] >> b) & 1) << 3) |
+                               ((unsigned)((p[4] >> b) & 1) << 4);
+            if (c) atomicAdd(&sh.cnt[b * W + w], c);
+        }
+#pragma unroll
+        for (int i = 0; i < 5; ++i) p[i] = 0;
+    }
+};
+
+// End of a level kernel: the lanes' counts, the OR of the new bits (lane w
+// mod W holds word w) and the level's sums.  Every thread of the block calls.
+template <int W>
+__device__ __forceinline__ void x_flush(XPlanes& c, unsigned long long any, XSums m, XShared<W>& sh, XState<W>* st) {
+    const int lane = lane_id();
+    const int q = lane / W;
+    c.flush(sh, lane & (W - 1), q * (64 * W / 32) + q);
+#pragma unroll
+    for (int o = W; o < 32; o <<= 1) any |= __shfl_xor_sync(kFull, any, o);
+    if (lane < W && any) atomicOr(&sh.any[lane], any);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         m.rows += __shfl_xor_sync(kFull, m.rows, o);
@@ -180,57 +230,50 @@ __device__ __forceinline__ void x_flush(const unsigned (&c)[8], unsigned long lo
         if (m.rem_edges) atomicAdd(&st->rem_edges, m.rem_edges);
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < kXS; i += blockDim.x)
-        if (s_cnt[i]) atomicAdd(&st->cnt[i], (unsigned long long)s_cnt[i]);
-    if (threadIdx.x < kXW && s_any[threadIdx.x]) atomicOr(&st->any[threadIdx.x], s_any[threadIdx.x]);
+    for (int i = threadIdx.x; i < 64 * W; i += blockDim.x)
+        if (sh.cnt[i]) atomicAdd(&st->cnt[(i & (W - 1)) * 64 + i / W], (unsigned long long)sh.cnt[i]);
+    if (threadIdx.x < W && sh.any[threadIdx.x]) atomicOr(&st->any[threadIdx.x], sh.any[threadIdx.x]);
 }
 
-// Counts bit b of word w of cv over the warp's 8 vertices (lanes w, w+4,
-// ..., w+28 hold word w) into the owning lanes' counters.
-__device__ __forceinline__ void x_count_quads(unsigned long long cv, unsigned (&c)[8]) {
-    const int lane = lane_id();
-    const unsigned wm = 0x11111111u << (lane & 3);
-    const int q = lane >> 2;
-#pragma unroll
-    for (int b = 0; b < 64; ++b) {
-        const unsigned bal = __ballot_sync(kFull, (cv >> b) & 1ULL);
-        if (q == (b & 7)) c[b >> 3] += __popc(bal & wm);
-    }
+// Does some lane of this lane's group of W hold true?  (mask: a ballot)
+template <int W>
+__device__ __forceinline__ bool group_any(unsigned mask) {
+    constexpr unsigned kGroup = (1u << W) - 1u;
+    return ((mask >> (lane_id() & ~(W - 1))) & kGroup) != 0;
 }
 
-// Bottom-up level for vertices with short rows: 4 lanes per vertex (lane w
-// holds word w), 8 vertices per warp; each lane loads every fourth column of
-// the row and the quad shares them, so 8 neighbours' words are in flight.
+// Bottom-up level for vertices with short rows: W lanes per vertex (lane w
+// holds word w), 32 / W vertices per warp; the lanes of a group load the row's
+// columns together and share them, so several neighbours' words are in flight.
+template <int W>
 __global__ void __launch_bounds__(256) k_x_light(const int32_t* __restrict__ list, int64_t n_list,
                                                  const int64_t* __restrict__ rowp, const int32_t* __restrict__ cols,
                                                  const unsigned long long* __restrict__ cur,
                                                  unsigned long long* __restrict__ nxt, unsigned long long* vis,
                                                  const uint8_t* __restrict__ pred, int32_t* __restrict__ next_front,
-                                                 XState* __restrict__ st) {
-    __shared__ unsigned s_cnt[kXS];
-    __shared__ unsigned long long s_any[kXW];
-    for (int i = threadIdx.x; i < kXS; i += blockDim.x) s_cnt[i] = 0;
-    if (threadIdx.x < kXW) s_any[threadIdx.x] = 0;
-    __syncthreads();
+                                                 XState<W>* __restrict__ st) {
+    __shared__ XShared<W> sh;
+    x_init(sh);
+    constexpr int kLoads = W == 4 ? 2 : 1;  // columns per lane and step
     const int lane = lane_id();
-    const int w = lane & 3, q = lane >> 2;
-    const unsigned qm = 0xFu << (lane & ~3);
+    const int w = lane & (W - 1), q = lane / W;
+    const unsigned qm = ((1u << W) - 1u) << (lane & ~(W - 1));
     const unsigned long long act = st->active[w];
-    unsigned c[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    XPlanes c;
     unsigned long long any = 0;
     XSums m;
-    const int64_t stride = ((int64_t)gridDim.x * blockDim.x) >> 2;
-    for (int64_t base = (((int64_t)blockIdx.x * blockDim.x) + (threadIdx.x & ~31)) >> 2; base < n_list;
+    const int64_t stride = ((int64_t)gridDim.x * blockDim.x) / W;
+    for (int64_t base = (((int64_t)blockIdx.x * blockDim.x) + (threadIdx.x & ~31)) / W; base < n_list;
          base += stride) {
         const int64_t i = base + q;
         const bool valid = i < n_list;
         const int32_t v = valid ? __ldg(&list[i]) : 0;
-        const unsigned long long vw = valid ? vis[(int64_t)v * kXW + w] : ~0ULL;
+        const unsigned long long vw = valid ? vis[(int64_t)v * W + w] : ~0ULL;
         const unsigned long long need = act & ~vw;
         const unsigned nb = __ballot_sync(kFull, need != 0);
         unsigned long long nx = 0;
         int64_t deg = 0;
-        if ((nb >> (lane & ~3)) & 0xFu) {  // some word of this vertex still needs bits
+        if (group_any<W>(nb)) {  // some word of this vertex still needs bits
             const int64_t beg = __ldg(&rowp[v]), end = __ldg(&rowp[v + 1]);
             deg = end - beg;
             if (w == 0) {
@@ -238,64 +281,61 @@ __global__ void __launch_bounds__(256) k_x_light(const int32_t* __restrict__ lis
                 m.entries += (unsigned long long)deg;
             }
             unsigned long long acc = 0;
-            for (int64_t e0 = beg; e0 < end; e0 += 8) {
-                const int64_t ea = e0 + w, eb = e0 + 4 + w;
-                const int32_t ua = ea < end ? __ldg(&cols[ea]) : -1;
-                const int32_t ub = eb < end ? __ldg(&cols[eb]) : -1;
+            for (int64_t e0 = beg; e0 < end; e0 += kLoads * W) {
+                int32_t u[kLoads];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int32_t x = __shfl_sync(qm, ua, j, 4);
-                    const int32_t y = __shfl_sync(qm, ub, j, 4);
-                    if (x >= 0) acc |= __ldg(&cur[(int64_t)x * kXW + w]);
-                    if (y >= 0) acc |= __ldg(&cur[(int64_t)y * kXW + w]);
+                for (int l = 0; l < kLoads; ++l) u[l] = e0 + l * W + w < end ? __ldg(&cols[e0 + l * W + w]) : -1;
+#pragma unroll
+                for (int j = 0; j < kLoads * W; ++j) {
+                    const int32_t x = __shfl_sync(qm, u[j / W], j & (W - 1), W);
+                    if (x >= 0) acc |= __ldg(&cur[(int64_t)x * W + w]);
                 }
             }
             nx = acc & need;
         }
         if (valid) {
-            nxt[(int64_t)v * kXW + w] = nx;
-            if (nx) vis[(int64_t)v * kXW + w] = vw | nx;
+            nxt[(int64_t)v * W + w] = nx;
+            if (nx) vis[(int64_t)v * W + w] = vw | nx;
         }
         any |= nx;
         // the vertex joins the next frontier; or still needs bits afterwards
-        const bool got = (__ballot_sync(kFull, nx != 0) >> (lane & ~3)) & 0xFu;
-        const bool left = (__ballot_sync(kFull, (need & ~nx) != 0) >> (lane & ~3)) & 0xFu;
+        const bool got = group_any<W>(__ballot_sync(kFull, nx != 0));
+        const bool left = group_any<W>(__ballot_sync(kFull, (need & ~nx) != 0));
         const long long at = warp_append(w == 0 && got, &st->n_next);
         if (at >= 0) {
             next_front[at] = v;
             m.fr_edges += (unsigned long long)deg;
         }
         if (w == 0 && left) m.rem_edges += (unsigned long long)deg;
-        const unsigned long long cv = (valid && (!pred || pred[v])) ? nx : 0ULL;
-        if (__ballot_sync(kFull, cv != 0)) x_count_quads(cv, c);
+        c.add((valid && (!pred || pred[v])) ? nx : 0ULL);
+        if (c.n == 31) c.flush(sh, w, q * (64 * W / 32) + q);
     }
-    x_flush(c, any, m, s_cnt, s_any, st);
+    x_flush(c, any, m, sh, st);
 }
 
-// Bottom-up level for vertices with long rows: a warp per vertex, lane
-// (t, w) reads word w of neighbours t, t+8, ..., four in flight; every 128
+// Bottom-up level for vertices with long rows: a warp per vertex, lane (t, w)
+// reads word w of neighbours t, t + 32 / W, ..., kUnroll in flight; every 128
 // entries the warp stops if its OR already holds every bit the vertex needs.
+template <int W>
 __global__ void __launch_bounds__(256) k_x_heavy(const int32_t* __restrict__ list, int64_t n_list,
                                                  const int64_t* __restrict__ rowp, const int32_t* __restrict__ cols,
                                                  const unsigned long long* __restrict__ cur,
                                                  unsigned long long* __restrict__ nxt, unsigned long long* vis,
                                                  const uint8_t* __restrict__ pred, int32_t* __restrict__ next_front,
-                                                 XState* __restrict__ st) {
-    __shared__ unsigned s_cnt[kXS];
-    __shared__ unsigned long long s_any[kXW];
-    for (int i = threadIdx.x; i < kXS; i += blockDim.x) s_cnt[i] = 0;
-    if (threadIdx.x < kXW) s_any[threadIdx.x] = 0;
-    __syncthreads();
+                                                 XState<W>* __restrict__ st) {
+    __shared__ XShared<W> sh;
+    x_init(sh);
+    constexpr int kT = 32 / W, kUnroll = W == 4 ? 4 : 8, kStep = kT * kUnroll;
     const int lane = lane_id();
-    const int w = lane & 3, t = lane >> 2;
+    const int w = lane & (W - 1), t = lane / W;
     const unsigned long long act = st->active[w];
-    unsigned c[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    XPlanes c;
     unsigned long long any = 0;
     XSums m;
     const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t i = (((int64_t)blockIdx.x * blockDim.x) + threadIdx.x) >> 5; i < n_list; i += warps) {
         const int32_t v = __ldg(&list[i]);
-        const unsigned long long vw = vis[(int64_t)v * kXW + w];
+        const unsigned long long vw = vis[(int64_t)v * W + w];
         const unsigned long long need = act & ~vw;
         unsigned long long nx = 0;
         int64_t deg = 0;
@@ -304,28 +344,26 @@ __global__ void __launch_bounds__(256) k_x_heavy(const int32_t* __restrict__ lis
             deg = end - beg;
             int64_t stop = end;
             unsigned long long acc = 0;
-            for (int64_t b0 = beg; b0 < end; b0 += 32) {
-                int32_t u[4];
+            for (int64_t b0 = beg; b0 < end; b0 += kStep) {
+                int32_t u[kUnroll];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) u[j] = b0 + 8 * j + t < end ? __ldg(&cols[b0 + 8 * j + t]) : -1;
+                for (int j = 0; j < kUnroll; ++j) u[j] = b0 + kT * j + t < end ? __ldg(&cols[b0 + kT * j + t]) : -1;
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (u[j] >= 0) acc |= __ldg(&cur[(int64_t)u[j] * kXW + w]);
-                if (((b0 - beg) & 127) == 96) {
+                for (int j = 0; j < kUnroll; ++j)
+                    if (u[j] >= 0) acc |= __ldg(&cur[(int64_t)u[j] * W + w]);
+                if (((b0 - beg) & 127) == 128 - kStep) {
                     unsigned long long a = acc;
-                    a |= __shfl_xor_sync(kFull, a, 4);
-                    a |= __shfl_xor_sync(kFull, a, 8);
-                    a |= __shfl_xor_sync(kFull, a, 16);
+#pragma unroll
+                    for (int o = W; o < 32; o <<= 1) a |= __shfl_xor_sync(kFull, a, o);
                     if (__all_sync(kFull, (a & need) == need)) {
                         acc = a;
-                        stop = b0 + 32 < end ? b0 + 32 : end;
+                        stop = b0 + kStep < end ? b0 + kStep : end;
                         break;
                     }
                 }
             }
-            acc |= __shfl_xor_sync(kFull, acc, 4);
-            acc |= __shfl_xor_sync(kFull, acc, 8);
-            acc |= __shfl_xor_sync(kFull, acc, 16);
+#pragma unroll
+            for (int o = W; o < 32; o <<= 1) acc |= __shfl_xor_sync(kFull, acc, o);
             nx = acc & need;
             if (lane == 0) {
                 ++m.rows;
@@ -333,8 +371,8 @@ __global__ void __launch_bounds__(256) k_x_heavy(const int32_t* __restrict__ lis
             }
         }
         if (t == 0) {
-            nxt[(int64_t)v * kXW + w] = nx;
-            if (nx) vis[(int64_t)v * kXW + w] = vw | nx;
+            nxt[(int64_t)v * W + w] = nx;
+            if (nx) vis[(int64_t)v * W + w] = vw | nx;
         }
         any |= nx;
         const bool got = __any_sync(kFull, nx != 0);
@@ -345,39 +383,36 @@ __global__ void __launch_bounds__(256) k_x_heavy(const int32_t* __restrict__ lis
             m.fr_edges += (unsigned long long)deg;
         }
         if (lane == 0 && left) m.rem_edges += (unsigned long long)deg;
-        // every lane holds its word's new bits; lane (t, w) counts bits 8j + t
-        const unsigned long long cv = (!pred || pred[v]) ? nx : 0ULL;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) c[j] += (unsigned)((cv >> (8 * j + t)) & 1ULL);
+        // every lane holds its word's new bits; the first group counts them
+        c.add(t == 0 && (!pred || pred[v]) ? nx : 0ULL);
+        if (c.n == 31) c.flush(sh, w, 0);
     }
-    x_flush(c, any, m, s_cnt, s_any, st);
+    x_flush(c, any, m, sh, st);
 }
 
-// Bottom-up level for the longest rows: a block per vertex, 1024 entries per
-// step (lane (t, w) of warp p reads word w of entries 64 j + 8 p + t), stopping
-// like k_x_heavy.
+// Bottom-up level for the longest rows: a block per vertex, sixteen
+// neighbours' words per lane and step, stopping like k_x_heavy.
+template <int W>
 __global__ void __launch_bounds__(256) k_x_huge(const int32_t* __restrict__ list, int64_t n_list,
                                                 const int64_t* __restrict__ rowp, const int32_t* __restrict__ cols,
                                                 const unsigned long long* __restrict__ cur,
                                                 unsigned long long* __restrict__ nxt, unsigned long long* vis,
                                                 const uint8_t* __restrict__ pred, int32_t* __restrict__ next_front,
-                                                XState* __restrict__ st) {
-    __shared__ unsigned s_cnt[kXS];
-    __shared__ unsigned long long s_any[kXW];
-    __shared__ unsigned long long s_acc[2][8][kXW];
-    for (int i = threadIdx.x; i < kXS; i += blockDim.x) s_cnt[i] = 0;
-    if (threadIdx.x < kXW) s_any[threadIdx.x] = 0;
-    __syncthreads();
+                                                XState<W>* __restrict__ st) {
+    __shared__ XShared<W> sh;
+    __shared__ unsigned long long s_acc[2][8][W];
+    x_init(sh);
+    constexpr int kT = 32 / W, kRow = 8 * kT, kStep = 16 * kRow;
     const int lane = lane_id(), warp = threadIdx.x >> 5;
-    const int w = lane & 3, t = lane >> 2;
+    const int w = lane & (W - 1), t = lane / W;
     const unsigned long long act = st->active[w];
-    unsigned c[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    XPlanes c;
     unsigned long long any = 0;
     XSums m;
     int par = 0;
     for (int64_t i = blockIdx.x; i < n_list; i += gridDim.x) {
         const int32_t v = __ldg(&list[i]);
-        const unsigned long long vw = vis[(int64_t)v * kXW + w];
+        const unsigned long long vw = vis[(int64_t)v * W + w];
         const unsigned long long need = act & ~vw;
         unsigned long long nx = 0;
         int64_t deg = 0;
@@ -392,22 +427,21 @@ __global__ void __launch_bounds__(256) k_x_huge(const int32_t* __restrict__ list
                     int32_t u[4];
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        const int64_t e = b0 + 64 * (4 * h + j) + 8 * warp + t;
+                        const int64_t e = b0 + kRow * (4 * h + j) + kT * warp + t;
                         u[j] = e < end ? __ldg(&cols[e]) : -1;
                     }
 #pragma unroll
                     for (int j = 0; j < 4; ++j)
-                        if (u[j] >= 0) acc |= __ldg(&cur[(int64_t)u[j] * kXW + w]);
+                        if (u[j] >= 0) acc |= __ldg(&cur[(int64_t)u[j] * W + w]);
                 }
-                acc |= __shfl_xor_sync(kFull, acc, 4);
-                acc |= __shfl_xor_sync(kFull, acc, 8);
-                acc |= __shfl_xor_sync(kFull, acc, 16);
+#pragma unroll
+                for (int o = W; o < 32; o <<= 1) acc |= __shfl_xor_sync(kFull, acc, o);
                 if (t == 0) s_acc[par][warp][w] = acc;
                 __syncthreads();
 #pragma unroll
                 for (int p = 0; p < 8; ++p) acc |= s_acc[par][p][w];
                 par ^= 1;  // the other buffer was last read before this step's barrier
-                b0 = b0 + 1024 < end ? b0 + 1024 : end;
+                b0 = b0 + kStep < end ? b0 + kStep : end;
                 more = b0 < end && !__all_sync(kFull, (acc & need) == need);
             }
             nx = acc & need;
@@ -418,8 +452,8 @@ __global__ void __launch_bounds__(256) k_x_huge(const int32_t* __restrict__ list
         }
         if (warp == 0) {
             if (t == 0) {
-                nxt[(int64_t)v * kXW + w] = nx;
-                if (nx) vis[(int64_t)v * kXW + w] = vw | nx;
+                nxt[(int64_t)v * W + w] = nx;
+                if (nx) vis[(int64_t)v * W + w] = vw | nx;
             }
             any |= nx;
             const bool got = __any_sync(kFull, nx != 0);
@@ -430,12 +464,11 @@ __global__ void __launch_bounds__(256) k_x_huge(const int32_t* __restrict__ list
                 m.fr_edges += (unsigned long long)deg;
             }
             if (lane == 0 && left) m.rem_edges += (unsigned long long)deg;
-            const unsigned long long cv = (!pred || pred[v]) ? nx : 0ULL;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) c[j] += (unsigned)((cv >> (8 * j + t)) & 1ULL);
+            c.add(t == 0 && (!pred || pred[v]) ? nx : 0ULL);
+            if (c.n == 31) c.flush(sh, w, 0);
         }
     }
-    x_flush(c, any, m, s_cnt, s_any, st);
+    x_flush(c, any, m, sh, st);
 }
 
 // Top-down level, step 1: the frontier rows as work items of at most
@@ -443,9 +476,10 @@ __global__ void __launch_bounds__(256) k_x_huge(const int32_t* __restrict__ list
 // many warps.  A vertex without running bits gives none.
 constexpr int kXSeg = 256;
 
+template <int W>
 __global__ void k_x_td_items(const int32_t* __restrict__ front, int64_t n_front, const int64_t* __restrict__ rowp,
                              const unsigned long long* __restrict__ cur, unsigned long long* __restrict__ items,
-                             XState* __restrict__ st) {
+                             XState<W>* __restrict__ st) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int lane = lane_id();
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n_front; base += stride) {
@@ -454,9 +488,10 @@ __global__ void k_x_td_items(const int32_t* __restrict__ front, int64_t n_front,
         int32_t u = 0;
         if (i < n_front) {
             u = __ldg(&front[i]);
-            const int64_t o = (int64_t)u * kXW;
-            const bool live = ((__ldg(&cur[o]) & st->active[0]) | (__ldg(&cur[o + 1]) & st->active[1]) |
-                               (__ldg(&cur[o + 2]) & st->active[2]) | (__ldg(&cur[o + 3]) & st->active[3])) != 0;
+            unsigned long long running = 0;
+#pragma unroll
+            for (int w = 0; w < W; ++w) running |= __ldg(&cur[(int64_t)u * W + w]) & st->active[w];
+            const bool live = running != 0;
             const int64_t deg = __ldg(&rowp[u + 1]) - __ldg(&rowp[u]);
             segs = live ? (int)((deg + kXSeg - 1) / kXSeg) : 0;
         }
@@ -470,15 +505,18 @@ __global__ void k_x_td_items(const int32_t* __restrict__ front, int64_t n_front,
 }
 
 // Step 2: a warp per work item, lane (t, w) takes word w of the row owner's
-// running bits to entries t, t+8, ...: the bits a neighbour has not visited
+// running bits to entries t, t + 32 / W, ...: the bits a neighbour has not visited
 // go into its next words (atomicOr; the host cleared them).
+template <int W>
 __global__ void __launch_bounds__(256) k_x_td(const unsigned long long* __restrict__ items,
                                               const int64_t* __restrict__ rowp, const int32_t* __restrict__ cols,
                                               const unsigned long long* __restrict__ cur,
                                               unsigned long long* __restrict__ nxt,
-                                              const unsigned long long* __restrict__ vis, XState* __restrict__ st) {
+                                              const unsigned long long* __restrict__ vis,
+                                              XState<W>* __restrict__ st) {
+    constexpr int kT = 32 / W;
     const int lane = lane_id();
-    const int w = lane & 3, t = lane >> 2;
+    const int w = lane & (W - 1), t = lane / W;
     const unsigned long long act = st->active[w];
     const int64_t n_items = (int64_t)st->n_next;
     unsigned long long rows = 0, entries = 0;
@@ -487,7 +525,7 @@ __global__ void __launch_bounds__(256) k_x_td(const unsigned long long* __restri
         const unsigned long long it = __ldg(&items[i]);
         const int32_t u = (int32_t)(it >> 32);
         const int64_t seg = (int64_t)(it & 0xffffffffULL);
-        const unsigned long long bits = __ldg(&cur[(int64_t)u * kXW + w]) & act;
+        const unsigned long long bits = __ldg(&cur[(int64_t)u * W + w]) & act;
         const int64_t row_end = __ldg(&rowp[u + 1]);
         const int64_t beg = __ldg(&rowp[u]) + seg * kXSeg;
         const int64_t end = beg + kXSeg < row_end ? beg + kXSeg : row_end;
@@ -496,12 +534,12 @@ __global__ void __launch_bounds__(256) k_x_td(const unsigned long long* __restri
             entries += (unsigned long long)(end - beg);
         }
 #pragma unroll 4
-        for (int64_t b0 = beg; b0 < end; b0 += 8) {
+        for (int64_t b0 = beg; b0 < end; b0 += kT) {
             const int64_t e = b0 + t;
             if (e < end) {
                 const int32_t v = __ldg(&cols[e]);
-                const unsigned long long nb = bits & ~__ldg(&vis[(int64_t)v * kXW + w]);
-                if (nb) atomicOr(&nxt[(int64_t)v * kXW + w], nb);
+                const unsigned long long nb = bits & ~__ldg(&vis[(int64_t)v * W + w]);
+                if (nb) atomicOr(&nxt[(int64_t)v * W + w], nb);
             }
         }
     }
@@ -516,42 +554,41 @@ __global__ void __launch_bounds__(256) k_x_td(const unsigned long long* __restri
     }
 }
 
-// Step 3, over every vertex (4 lanes per vertex): fold the new bits into
+// Step 3, over every vertex (W lanes per vertex): fold the new bits into
 // "visited", count them, list the next frontier and its row entries.
+template <int W>
 __global__ void __launch_bounds__(256) k_x_td_finish(int64_t n, const int64_t* __restrict__ rowp,
                                                      const unsigned long long* __restrict__ nxt,
                                                      unsigned long long* vis, const uint8_t* __restrict__ pred,
-                                                     int32_t* __restrict__ next_front, XState* __restrict__ st) {
-    __shared__ unsigned s_cnt[kXS];
-    __shared__ unsigned long long s_any[kXW];
-    for (int i = threadIdx.x; i < kXS; i += blockDim.x) s_cnt[i] = 0;
-    if (threadIdx.x < kXW) s_any[threadIdx.x] = 0;
-    __syncthreads();
+                                                     int32_t* __restrict__ next_front, XState<W>* __restrict__ st) {
+    __shared__ XShared<W> sh;
+    x_init(sh);
     const int lane = lane_id();
-    const int w = lane & 3, q = lane >> 2;
-    unsigned c[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    const int w = lane & (W - 1), q = lane / W;
+    XPlanes c;
     unsigned long long any = 0;
     XSums m;
-    const int64_t stride = ((int64_t)gridDim.x * blockDim.x) >> 2;
-    for (int64_t base = (((int64_t)blockIdx.x * blockDim.x) + (threadIdx.x & ~31)) >> 2; base < n; base += stride) {
+    const int64_t stride = ((int64_t)gridDim.x * blockDim.x) / W;
+    for (int64_t base = (((int64_t)blockIdx.x * blockDim.x) + (threadIdx.x & ~31)) / W; base < n; base += stride) {
         const int64_t v = base + q;
         const bool valid = v < n;
-        const unsigned long long nx = valid ? nxt[v * kXW + w] : 0ULL;
-        if (nx) vis[v * kXW + w] |= nx;
+        const unsigned long long nx = valid ? nxt[v * W + w] : 0ULL;
+        const unsigned some = __ballot_sync(kFull, nx != 0);
+        if (!some) continue;
+        if (nx) vis[v * W + w] |= nx;
         any |= nx;
-        const bool got = (__ballot_sync(kFull, nx != 0) >> (lane & ~3)) & 0xFu;
-        const long long at = warp_append(w == 0 && got, &st->n_next);
+        const long long at = warp_append(w == 0 && group_any<W>(some), &st->n_next);
         if (at >= 0) {
             next_front[at] = (int32_t)v;
             m.fr_edges += (unsigned long long)(__ldg(&rowp[v + 1]) - __ldg(&rowp[v]));
         }
-        const unsigned long long cv = (valid && (!pred || pred[v])) ? nx : 0ULL;
-        if (__ballot_sync(kFull, cv != 0)) x_count_quads(cv, c);
+        c.add((valid && (!pred || pred[v])) ? nx : 0ULL);
+        if (c.n == 31) c.flush(sh, w, q * (64 * W / 32) + q);
     }
-    x_flush(c, any, m, s_cnt, s_any, st);
+    x_flush(c, any, m, sh, st);
 }
 
-// End of a level (one block of kXS threads, thread s = source s of the
+// End of a level (one block of 64 W threads, thread s = source s of the
 // sweep): fold the level's counts into each running source and stop the
 // sources that are answered.  Level 0 is the source itself.
 //   sizes:  N += (new vertices at this distance under the predicate);
@@ -562,27 +599,28 @@ __global__ void __launch_bounds__(256) k_x_td_finish(int64_t n, const int64_t* _
 //           level that reaches nothing means j-1 was the eccentricity L and
 //           r = L + (c - G_L) / N_L (+inf when N_L = 0).  N and G are exact
 //           integers; each FP64 step is one IEEE operation.
-__global__ void k_x_finish(XState* __restrict__ st, int mode, int64_t level, const int32_t* __restrict__ src,
+template <int W>
+__global__ void k_x_finish(XState<W>* __restrict__ st, int mode, int64_t level, const int32_t* __restrict__ src,
                            const uint8_t* __restrict__ pred, const double* __restrict__ cost, int64_t D,
                            int64_t* __restrict__ sizes, double* __restrict__ radius, Counters* ctr) {
-    __shared__ unsigned s_bal[kXS / 32];
+    __shared__ unsigned s_bal[2 * W];
     const int s = threadIdx.x;
     const int w = s >> 6;
     const unsigned long long bit = 1ULL << (s & 63);
     bool act = (st->active[w] & bit) != 0;
     if (act) {
         const int32_t v = src[s];
-        long long W;
+        long long fresh;
         bool found;
         if (level == 0) {
-            W = (!pred || pred[v]) ? 1 : 0;
+            fresh = (!pred || pred[v]) ? 1 : 0;
             found = true;
         } else {
-            W = (long long)st->cnt[s];
+            fresh = (long long)st->cnt[s];
             found = (st->any[w] & bit) != 0;
         }
         if (mode == kXSizes) {
-            const long long N = st->N[s] + W;
+            const long long N = st->N[s] + fresh;
             st->N[s] = N;
             int64_t* row = sizes + (int64_t)s * (D + 1);
             row[level] = N;
@@ -600,7 +638,7 @@ __global__ void k_x_finish(XState* __restrict__ st, int mode, int64_t level, con
                 if (N > 0) r = __dadd_rn((double)(level - 1), __ddiv_rn(__dsub_rn(c, (double)st->Gp[s]), (double)N));
                 act = false;
             } else {
-                const long long N = st->N[s] + W;
+                const long long N = st->N[s] + fresh;
                 const long long G = st->G[s];
                 const long long Gn = G + N;
                 st->N[s] = N;
@@ -620,13 +658,13 @@ __global__ void k_x_finish(XState* __restrict__ st, int mode, int64_t level, con
     const unsigned bal = __ballot_sync(kFull, act);
     if (lane_id() == 0) s_bal[s >> 5] = bal;
     __syncthreads();
-    if (s < kXW) {
+    if (s < W) {
         st->active[s] = (unsigned long long)s_bal[2 * s] | ((unsigned long long)s_bal[2 * s + 1] << 32);
         st->any[s] = 0;
     }
     if (s == 0) {
         unsigned long long tot = 0;
-        for (int i = 0; i < kXS / 32; ++i) tot += __popc(s_bal[i]);
+        for (int i = 0; i < 2 * W; ++i) tot += __popc(s_bal[i]);
         ctr->aux0 = tot;
         ctr->scanned = st->rows;
         ctr->cand_reads = st->entries;
@@ -674,114 +712,152 @@ __global__ void __launch_bounds__(256) k_x_estimates(const int32_t* __restrict__
     }
 }
 
-// Sweeps of kXS sources over src[0, n_src) (internal ids).
+// Scratch of the sweeps of one call.
+struct XScratch {
+    unsigned long long* vis;
+    unsigned long long* buf[2];
+    int32_t *light, *heavy;
+    const int32_t* huge;
+    int32_t* front[2];
+    unsigned long long* items;
+    size_t n_items;
+    void* state;
+    int64_t n_light, n_heavy, n_huge;
+};
+
+// One sweep of nb <= 64 W sources; rows: the sizes of its first source.
+template <int W>
+int run_sweep(fl_graph* g, const XScratch& x, int mode, int64_t nb, const int32_t* src, int64_t D,
+              const uint8_t* pred, const double* cost, int64_t* rows, double* radius) {
+    cudaStream_t st = g->stream;
+    const int64_t n = g->n, nnz = g->nnz;
+    const int cls = kProfExact;
+    const size_t words = (size_t)n * W;
+    const int kS = 64 * W;
+    Counters* ctr = g->ctr.as<Counters>();
+    const int64_t* rowp = g->rowp.as<int64_t>();
+    const int32_t* cols = g->cols.as<int32_t>();
+    XState<W>* xs = static_cast<XState<W>*>(x.state);
+    unsigned long long* vis = x.vis;
+    unsigned long long* buf[2] = {vis + words, vis + 2 * words};
+    int32_t* front[2] = {x.front[0], x.front[1]};
+    const int grid_l = blocks_for(x.n_light, 256 / W, kXLevelBlocks);
+    const int grid_h = blocks_for(x.n_heavy, 8, kXLevelBlocks);  // 8 warps x 1 vertex
+    // a bottom-up level rewrites the next words of every vertex; a
+    // top-down level gets them cleared first
+    FL_CUDA(cudaMemsetAsync(vis, 0, words * 8, st));
+    FL_CUDA(cudaMemsetAsync(buf[0], 0, words * 8, st));
+    int c = 0, fc = 0;
+    FL_LAUNCH(cls, k_x_seed<W><<<1, kS, 0, st>>>(src, nb, rowp, vis, buf[0], front[0], xs));
+    FL_LAUNCH(cls, k_x_finish<W><<<1, kS, 0, st>>>(xs, mode, 0, src, pred, cost, D, rows, radius, ctr));
+    FL_CUDA(cudaGetLastError());
+    FL_TRY(read_counters(g));
+    int64_t n_front = (int64_t)g->h_ctr->frontier;
+    int64_t fr_edges = (int64_t)g->h_ctr->merges;
+    int64_t rem = nnz;  // entries of rows that may still need bits
+    unsigned long long rows_prev = 0, entries_prev = 0;
+    for (int64_t level = 1; g->h_ctr->aux0 > 0; ++level) {
+        if (level > n + 1) FL_FAIL(FL_ETIMEOUT, "exact search did not finish");
+        // top-down when the frontier's rows are much shorter than the
+        // rows bottom-up would scan, and their work items fit
+        const bool td = 2 * fr_edges < rem && n_front + fr_edges / kXSeg + 1 <= (int64_t)x.n_items;
+        if (td) {
+            FL_CUDA(cudaMemsetAsync(buf[c ^ 1], 0, words * 8, st));
+            // work items (their count in st->n_next), then the pushes;
+            // k_x_td_finish restarts n_next for the next frontier
+            FL_LAUNCH(cls, k_x_td_items<W><<<blocks_for(n_front, 256), 256, 0, st>>>(front[fc], n_front, rowp,
+                                                                                    buf[c], x.items, xs));
+            const int64_t most = n_front + fr_edges / kXSeg;  // work items at most
+            FL_LAUNCH(cls, k_x_td<W><<<blocks_for(most, 8), 256, 0, st>>>(x.items, rowp, cols, buf[c], buf[c ^ 1],
+                                                                          vis, xs));
+            FL_CUDA(cudaMemsetAsync(&xs->n_next, 0, 8, st));
+            FL_LAUNCH(cls, k_x_td_finish<W><<<blocks_for(n, 256 / W, kXLevelBlocks), 256, 0, st>>>(
+                               n, rowp, buf[c ^ 1], vis, pred, front[fc ^ 1], xs));
+        } else {
+            if (x.n_huge > 0)
+                FL_LAUNCH(cls, k_x_huge<W><<<blocks_for(x.n_huge, 1, kXLevelBlocks), 256, 0, st>>>(
+                                   x.huge, x.n_huge, rowp, cols, buf[c], buf[c ^ 1], vis, pred, front[fc ^ 1], xs));
+            if (x.n_heavy > 0)
+                FL_LAUNCH(cls, k_x_heavy<W><<<grid_h, 256, 0, st>>>(x.heavy, x.n_heavy, rowp, cols, buf[c],
+                                                                    buf[c ^ 1], vis, pred, front[fc ^ 1], xs));
+            if (x.n_light > 0)
+                FL_LAUNCH(cls, k_x_light<W><<<grid_l, 256, 0, st>>>(x.light, x.n_light, rowp, cols, buf[c],
+                                                                    buf[c ^ 1], vis, pred, front[fc ^ 1], xs));
+        }
+        FL_LAUNCH(cls, k_x_finish<W><<<1, kS, 0, st>>>(xs, mode, level, src, pred, cost, D, rows, radius, ctr));
+        FL_CUDA(cudaGetLastError());
+        c ^= 1;
+        fc ^= 1;
+        FL_TRY(read_counters(g));
+        const int64_t touched = (int64_t)g->h_ctr->frontier;
+        // algorithmic bytes of the level, B = 8 W bytes of bits per vertex.
+        // Bottom-up: every listed vertex reads its list id and visited words
+        // and writes its next words (4 + 2 B); a scanned row reads two offsets
+        // (16) and, per entry, the column and the neighbour's frontier words
+        // (4 + B).  Top-down: a frontier vertex reads its list id, frontier
+        // words and offsets (4 + B + 16); per entry the column and the
+        // neighbour's visited words (4 + B); every vertex reads its next words
+        // (B) and a newly reached one reads and writes its visited words, reads
+        // its offsets and is listed (2 B + 16 + 4).
+        const double B = 8.0 * W;
+        const double d_rows = (double)(g->h_ctr->scanned - rows_prev);
+        const double d_entries = (double)(g->h_ctr->cand_reads - entries_prev);
+        rows_prev = g->h_ctr->scanned;
+        entries_prev = g->h_ctr->cand_reads;
+        g->prof.bytes[cls] += td ? (20.0 + B) * (double)n_front + (4.0 + B) * d_entries + B * (double)n +
+                                       (20.0 + 2.0 * B) * (double)touched
+                                 : (4.0 + 2.0 * B) * (double)n + 16.0 * d_rows + (4.0 + B) * d_entries;
+        n_front = touched;
+        fr_edges = (int64_t)g->h_ctr->merges;
+        if (!td) rem = (int64_t)g->h_ctr->aux3;
+    }
+    return FL_OK;
+}
+
+// Sweeps over src[0, n_src) (internal ids).
 int run_sweeps(fl_graph* g, int mode, int64_t n_src, const int32_t* src, int64_t D, const uint8_t* pred,
                const double* cost, int64_t* sizes, double* radius) {
     cudaStream_t st = g->stream;
     const int64_t n = g->n, nnz = g->nnz;
-    const int cls = kProfExact;
-    const size_t words = (size_t)n * kXW;
-    FL_TRY(dalloc(g->xbits, words * 8 * 3));
-    // int32 lists: light rows (n), heavy rows (n), two frontiers (n + kXS
-    // each: the first frontier lists the sweep's sources, repeats included);
-    // then the top-down work items (uint64, one per kXSeg entries of a
-    // frontier row: at most n + kXS + nnz / kXSeg) and the sweep state
-    const size_t lists = ((size_t)(4 * n + 2 * kXS) * 4 + 255) & ~(size_t)255;
-    const size_t n_items = (size_t)(n + kXS + nnz / kXSeg + 1);
-    const size_t items_b = (n_items * 8 + 255) & ~(size_t)255;
-    FL_TRY(dalloc(g->xaux, lists + items_b + sizeof(XState)));
-    unsigned long long* vis = g->xbits.as<unsigned long long>();
-    unsigned long long* buf[2] = {vis + words, vis + 2 * words};
-    int32_t* light = g->xaux.as<int32_t>();
-    int32_t* heavy = light + n;
-    int32_t* front[2] = {light + 2 * n, light + 3 * n + kXS};
-    unsigned long long* items = reinterpret_cast<unsigned long long*>(g->xaux.as<char>() + lists);
-    XState* xs = reinterpret_cast<XState*>(g->xaux.as<char>() + lists + items_b);
+    // the smallest W that takes what is left
+    auto width = [&](int64_t left) { return left <= 256 || n > kXWideN ? 4 : (left <= 512 ? 8 : 16); };
+    const int w_max = width(n_src);
+    constexpr int64_t kMost = 64 * kXMaxW;
+    FL_TRY(dalloc(g->xbits, (size_t)n * w_max * 8 * 3));
+    // int32 lists: light rows (n), heavy rows from the front and huge ones from
+    // the back (n), two frontiers (n + kMost each: the first frontier lists the
+    // sweep's sources, repeats included); then the top-down work items (uint64,
+    // one per kXSeg entries of a frontier row: at most n + kMost + nnz / kXSeg)
+    // and the sweep state
+    const size_t lists = ((size_t)(4 * n + 2 * kMost) * 4 + 255) & ~(size_t)255;
+    XScratch x;
+    x.n_items = (size_t)(n + kMost + nnz / kXSeg + 1);
+    const size_t items_b = (x.n_items * 8 + 255) & ~(size_t)255;
+    FL_TRY(dalloc(g->xaux, lists + items_b + sizeof(XState<kXMaxW>)));
+    x.vis = g->xbits.as<unsigned long long>();
+    x.light = g->xaux.as<int32_t>();
+    x.heavy = x.light + n;
+    x.front[0] = x.light + 2 * n;
+    x.front[1] = x.light + 3 * n + kMost;
+    x.items = reinterpret_cast<unsigned long long*>(g->xaux.as<char>() + lists);
+    x.state = g->xaux.as<char>() + lists + items_b;
     Counters* ctr = g->ctr.as<Counters>();
-    const int64_t* rowp = g->rowp.as<int64_t>();
-    const int32_t* cols = g->cols.as<int32_t>();
-
     FL_CUDA(cudaMemsetAsync(g->ctr.p, 0, sizeof(Counters), st));
-    FL_LAUNCH(cls, k_x_lists<<<blocks_for(n, 256), 256, 0, st>>>(rowp, n, light, heavy, &ctr->aux0, &ctr->aux3,
-                                                               &ctr->frontier));
+    FL_LAUNCH(kProfExact, k_x_lists<<<blocks_for(n, 256), 256, 0, st>>>(g->rowp.as<int64_t>(), n, x.light, x.heavy,
+                                                                      &ctr->aux0, &ctr->aux3, &ctr->frontier));
     FL_CUDA(cudaGetLastError());
     FL_TRY(read_counters(g));
-    const int64_t n_light = (int64_t)g->h_ctr->aux0, n_heavy = (int64_t)g->h_ctr->aux3;
-    const int64_t n_huge = (int64_t)g->h_ctr->frontier;
-    const int32_t* huge = heavy + n - n_huge;
-    const int grid_l = blocks_for(n_light, 64);  // 8 warps x 8 vertices per block pass
-    const int grid_h = blocks_for(n_heavy, 8);   // 8 warps x 1 vertex
-
-    for (int64_t b0 = 0; b0 < n_src; b0 += kXS) {
-        const int64_t nb = n_src - b0 < kXS ? n_src - b0 : kXS;
+    x.n_light = (int64_t)g->h_ctr->aux0;
+    x.n_heavy = (int64_t)g->h_ctr->aux3;
+    x.n_huge = (int64_t)g->h_ctr->frontier;
+    x.huge = x.heavy + n - x.n_huge;
+    for (int64_t b0 = 0; b0 < n_src;) {
+        const int w = width(n_src - b0);
+        const int64_t nb = std::min<int64_t>(n_src - b0, 64 * w);
         int64_t* rows = sizes ? sizes + b0 * (D + 1) : nullptr;
-        // a bottom-up level rewrites the next words of every vertex; a
-        // top-down level gets them cleared first
-        FL_CUDA(cudaMemsetAsync(vis, 0, words * 8, st));
-        FL_CUDA(cudaMemsetAsync(buf[0], 0, words * 8, st));
-        int c = 0, fc = 0;
-        FL_LAUNCH(cls, k_x_seed<<<1, kXS, 0, st>>>(src + b0, nb, rowp, vis, buf[0], front[0], xs));
-        FL_LAUNCH(cls, k_x_finish<<<1, kXS, 0, st>>>(xs, mode, 0, src + b0, pred, cost, D, rows, radius, ctr));
-        FL_CUDA(cudaGetLastError());
-        FL_TRY(read_counters(g));
-        int64_t n_front = (int64_t)g->h_ctr->frontier;
-        int64_t fr_edges = (int64_t)g->h_ctr->merges;
-        int64_t rem = nnz;  // entries of rows that may still need bits
-        unsigned long long rows_prev = 0, entries_prev = 0;
-        for (int64_t level = 1; g->h_ctr->aux0 > 0; ++level) {
-            if (level > n + 1) FL_FAIL(FL_ETIMEOUT, "exact search did not finish");
-            // top-down when the frontier's rows are much shorter than the
-            // rows bottom-up would scan, and their work items fit
-            const bool td = 2 * fr_edges < rem && n_front + fr_edges / kXSeg + 1 <= (int64_t)n_items;
-            if (td) {
-                FL_CUDA(cudaMemsetAsync(buf[c ^ 1], 0, words * 8, st));
-                // work items (their count in st->n_next), then the pushes;
-                // k_x_td_finish restarts n_next for the next frontier
-                FL_LAUNCH(cls, k_x_td_items<<<blocks_for(n_front, 256), 256, 0, st>>>(front[fc], n_front, rowp,
-                                                                                     buf[c], items, xs));
-                const int64_t most = n_front + fr_edges / kXSeg;  // work items at most
-                FL_LAUNCH(cls, k_x_td<<<blocks_for(most, 8), 256, 0, st>>>(items, rowp, cols, buf[c], buf[c ^ 1], vis,
-                                                                           xs));
-                FL_CUDA(cudaMemsetAsync(&xs->n_next, 0, 8, st));
-                FL_LAUNCH(cls, k_x_td_finish<<<blocks_for(n, 64), 256, 0, st>>>(n, rowp, buf[c ^ 1], vis, pred,
-                                                                                front[fc ^ 1], xs));
-            } else {
-                if (n_huge > 0)
-                    FL_LAUNCH(cls, k_x_huge<<<blocks_for(n_huge, 1), 256, 0, st>>>(
-                                       huge, n_huge, rowp, cols, buf[c], buf[c ^ 1], vis, pred, front[fc ^ 1], xs));
-                if (n_heavy > 0)
-                    FL_LAUNCH(cls, k_x_heavy<<<grid_h, 256, 0, st>>>(heavy, n_heavy, rowp, cols, buf[c], buf[c ^ 1],
-                                                                     vis, pred, front[fc ^ 1], xs));
-                if (n_light > 0)
-                    FL_LAUNCH(cls, k_x_light<<<grid_l, 256, 0, st>>>(light, n_light, rowp, cols, buf[c], buf[c ^ 1],
-                                                                     vis, pred, front[fc ^ 1], xs));
-            }
-            FL_LAUNCH(cls, k_x_finish<<<1, kXS, 0, st>>>(xs, mode, level, src + b0, pred, cost, D, rows, radius, ctr));
-            FL_CUDA(cudaGetLastError());
-            c ^= 1;
-            fc ^= 1;
-            FL_TRY(read_counters(g));
-            const int64_t touched = (int64_t)g->h_ctr->frontier;
-            // algorithmic bytes of the level.  Bottom-up: every listed vertex
-            // reads its list id and visited words and writes its next words
-            // (4 + 32 + 32 B); a scanned row reads two offsets (16 B) and, per
-            // entry, the column and the neighbour's frontier words (4 + 32 B).
-            // Top-down: a frontier vertex reads its list id, frontier words
-            // and offsets (4 + 32 + 16 B); per entry the column and the
-            // neighbour's visited words (4 + 32 B); every vertex reads its
-            // next words (32 B) and a newly reached one reads and writes its
-            // visited words, reads its offsets and is listed (32 + 32 + 16 + 4 B).
-            const double d_rows = (double)(g->h_ctr->scanned - rows_prev);
-            const double d_entries = (double)(g->h_ctr->cand_reads - entries_prev);
-            rows_prev = g->h_ctr->scanned;
-            entries_prev = g->h_ctr->cand_reads;
-            g->prof.bytes[cls] += td ? 52.0 * (double)n_front + 36.0 * d_entries + 32.0 * (double)n +
-                                           84.0 * (double)touched
-                                     : 68.0 * (double)n + 16.0 * d_rows + 36.0 * d_entries;
-            n_front = touched;
-            fr_edges = (int64_t)g->h_ctr->merges;
-            if (!td) rem = (int64_t)g->h_ctr->aux3;
-        }
+        auto sweep = w == 4 ? run_sweep<4> : (w == 8 ? run_sweep<8> : run_sweep<16>);
+        FL_TRY(sweep(g, x, mode, nb, src + b0, D, pred, cost, rows, radius));
+        b0 += nb;
     }
     return FL_OK;
 }
