@@ -19,9 +19,12 @@
 //   bottom-up: every vertex that some running source has not reached ORs
 //     its neighbours' frontier words and keeps the new bits.  Rows longer
 //     than 32 entries get a whole warp (32 / W neighbours x W words at a time,
-//     several in flight, stopping once every needed bit is in) and rows longer
-//     than 1024 a whole block (a warp on the largest hub was most of a level);
-//     shorter rows get W lanes, one word each.
+//     several in flight, stopping once every needed bit is in); rows longer
+//     than 256 are cut into work items of 256 entries, a warp each, that OR
+//     into the row's next words (a warp, or a block, on the largest hub was
+//     most of a level); shorter rows get W lanes, one word each.
+//     A bottom-up level of 1000 sources on an R-MAT graph with 262 k vertices:
+//     light 92 us, heavy 105, items 86 (a block per long row: 552).
 //   top-down (sparse frontiers, e.g. the sources themselves): the frontier
 //     rows, cut into work items of 256 entries (so a hub's row is spread
 //     over many warps), OR their bits into the neighbours' next words
@@ -40,7 +43,8 @@ namespace {
 constexpr int kXMaxW = 16;      // 64-bit words of source bits per vertex, at most
 constexpr int64_t kXWideN = 1 << 20;  // larger graphs take W = 4
 constexpr int kXHeavy = 32;     // rows longer than this get a whole warp
-constexpr int kXHuge = 1024;    // ... and longer than this a whole block
+constexpr int kXSeg = 256;      // entries of a work item
+constexpr int kXHuge = kXSeg;   // rows longer than this are cut into work items
 constexpr int kXBlocks = 152 * 8;
 constexpr int kXLevelBlocks = 152 * 4;  // level kernels: each warp flushes its counts once
 
@@ -89,7 +93,7 @@ __global__ void k_x_map(const int32_t* __restrict__ src, int64_t n_src, const in
 }
 
 // Vertices with short rows (<= kXHeavy entries, isolated ones included), with
-// long rows, and with rows above kXHuge entries (from the end of `heavy`).
+// with long rows, and with rows above kXHuge entries (from the end of `heavy`).
 __global__ void k_x_lists(const int64_t* __restrict__ rowp, int64_t n, int32_t* __restrict__ light,
                           int32_t* __restrict__ heavy, unsigned long long* n_light, unsigned long long* n_heavy,
                           unsigned long long* n_huge) {
@@ -390,83 +394,107 @@ __global__ void __launch_bounds__(256) k_x_heavy(const int32_t* __restrict__ lis
     x_flush(c, any, m, sh, st);
 }
 
-// Bottom-up level for the longest rows: a block per vertex, sixteen
-// neighbours' words per lane and step, stopping like k_x_heavy.
+// Work items of the rows above kXHuge entries (vertex << 32 | segment).
+__global__ void k_x_huge_items(const int32_t* __restrict__ list, int64_t n_list, const int64_t* __restrict__ rowp,
+                               unsigned long long* __restrict__ items, unsigned long long* __restrict__ n_items) {
+    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t i = (((int64_t)blockIdx.x * blockDim.x) + threadIdx.x) >> 5; i < n_list; i += warps) {
+        const int32_t v = list[i];
+        const int segs = (int)((rowp[v + 1] - rowp[v] + kXSeg - 1) / kXSeg);
+        unsigned long long at = 0;
+        if (lane_id() == 0) at = atomicAdd(n_items, (unsigned long long)segs);
+        at = __shfl_sync(kFull, at, 0);
+        for (int j = lane_id(); j < segs; j += 32) items[at + j] = ((unsigned long long)(uint32_t)v << 32) | (unsigned)j;
+    }
+}
+
+// Their next words start empty (W lanes per vertex).
 template <int W>
-__global__ void __launch_bounds__(256) k_x_huge(const int32_t* __restrict__ list, int64_t n_list,
+__global__ void k_x_huge_clear(const int32_t* __restrict__ list, int64_t n_list,
+                               unsigned long long* __restrict__ nxt) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n_list * W; t += stride)
+        nxt[(int64_t)list[t / W] * W + (t & (W - 1))] = 0;
+}
+
+// Bottom-up level, the items: a warp each; lane (t, w) reads word w of
+// neighbours t, t + 32 / W, ..., eight in flight.  An item whose row has every
+// bit it needs is passed over.
+template <int W>
+__global__ void __launch_bounds__(256) k_x_huge(const unsigned long long* __restrict__ items, int64_t n_items,
                                                 const int64_t* __restrict__ rowp, const int32_t* __restrict__ cols,
-                                                const unsigned long long* __restrict__ cur,
-                                                unsigned long long* __restrict__ nxt, unsigned long long* vis,
-                                                const uint8_t* __restrict__ pred, int32_t* __restrict__ next_front,
-                                                XState<W>* __restrict__ st) {
-    __shared__ XShared<W> sh;
-    __shared__ unsigned long long s_acc[2][8][W];
-    x_init(sh);
-    constexpr int kT = 32 / W, kRow = 8 * kT, kStep = 16 * kRow;
-    const int lane = lane_id(), warp = threadIdx.x >> 5;
+                                                const unsigned long long* __restrict__ cur, unsigned long long* nxt,
+                                                const unsigned long long* __restrict__ vis, XState<W>* __restrict__ st) {
+    constexpr int kT = 32 / W, kUnroll = 8, kStep = kT * kUnroll;
+    const int lane = lane_id();
     const int w = lane & (W - 1), t = lane / W;
+    const unsigned long long act = st->active[w];
+    unsigned long long entries = 0;
+    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t i = (((int64_t)blockIdx.x * blockDim.x) + threadIdx.x) >> 5; i < n_items; i += warps) {
+        const unsigned long long it = __ldg(&items[i]);
+        const int32_t v = (int32_t)(it >> 32);
+        const unsigned long long need = act & ~__ldg(&vis[(int64_t)v * W + w]) & ~__ldcg(&nxt[(int64_t)v * W + w]);
+        if (!__any_sync(kFull, need != 0)) continue;
+        const int64_t row_end = __ldg(&rowp[v + 1]);
+        const int64_t beg = __ldg(&rowp[v]) + (int64_t)(uint32_t)it * kXSeg;
+        const int64_t end = beg + kXSeg < row_end ? beg + kXSeg : row_end;
+        unsigned long long acc = 0;
+        for (int64_t b0 = beg; b0 < end; b0 += kStep) {
+            int32_t u[kUnroll];
+#pragma unroll
+            for (int j = 0; j < kUnroll; ++j) u[j] = b0 + kT * j + t < end ? __ldg(&cols[b0 + kT * j + t]) : -1;
+#pragma unroll
+            for (int j = 0; j < kUnroll; ++j)
+                if (u[j] >= 0) acc |= __ldg(&cur[(int64_t)u[j] * W + w]);
+        }
+#pragma unroll
+        for (int o = W; o < 32; o <<= 1) acc |= __shfl_xor_sync(kFull, acc, o);
+        acc &= need;
+        if (t == 0 && acc) atomicOr(&nxt[(int64_t)v * W + w], acc);
+        entries += (unsigned long long)(end - beg);
+    }
+    if (lane == 0 && entries) atomicAdd(&st->entries, entries);
+}
+
+// ... and their vertices: what the warp kernels do after a row (W lanes per vertex).
+template <int W>
+__global__ void __launch_bounds__(256) k_x_huge_done(const int32_t* __restrict__ list, int64_t n_list,
+                                                     const int64_t* __restrict__ rowp,
+                                                     const unsigned long long* __restrict__ nxt,
+                                                     unsigned long long* vis, const uint8_t* __restrict__ pred,
+                                                     int32_t* __restrict__ next_front, XState<W>* __restrict__ st) {
+    __shared__ XShared<W> sh;
+    x_init(sh);
+    const int lane = lane_id();
+    const int w = lane & (W - 1), q = lane / W;
     const unsigned long long act = st->active[w];
     XPlanes c;
     unsigned long long any = 0;
     XSums m;
-    int par = 0;
-    for (int64_t i = blockIdx.x; i < n_list; i += gridDim.x) {
-        const int32_t v = __ldg(&list[i]);
-        const unsigned long long vw = vis[(int64_t)v * W + w];
+    const int64_t stride = ((int64_t)gridDim.x * blockDim.x) / W;
+    for (int64_t base = (((int64_t)blockIdx.x * blockDim.x) + (threadIdx.x & ~31)) / W; base < n_list;
+         base += stride) {
+        const bool valid = base + q < n_list;
+        const int32_t v = valid ? __ldg(&list[base + q]) : 0;
+        const unsigned long long vw = valid ? vis[(int64_t)v * W + w] : ~0ULL;
         const unsigned long long need = act & ~vw;
-        unsigned long long nx = 0;
-        int64_t deg = 0;
-        if (__any_sync(kFull, need != 0)) {  // the same in every warp
-            const int64_t beg = __ldg(&rowp[v]), end = __ldg(&rowp[v + 1]);
-            deg = end - beg;
-            int64_t b0 = beg;
-            unsigned long long acc = 0;
-            for (bool more = true; more;) {
-#pragma unroll
-                for (int h = 0; h < 4; ++h) {
-                    int32_t u[4];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const int64_t e = b0 + kRow * (4 * h + j) + kT * warp + t;
-                        u[j] = e < end ? __ldg(&cols[e]) : -1;
-                    }
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        if (u[j] >= 0) acc |= __ldg(&cur[(int64_t)u[j] * W + w]);
-                }
-#pragma unroll
-                for (int o = W; o < 32; o <<= 1) acc |= __shfl_xor_sync(kFull, acc, o);
-                if (t == 0) s_acc[par][warp][w] = acc;
-                __syncthreads();
-#pragma unroll
-                for (int p = 0; p < 8; ++p) acc |= s_acc[par][p][w];
-                par ^= 1;  // the other buffer was last read before this step's barrier
-                b0 = b0 + kStep < end ? b0 + kStep : end;
-                more = b0 < end && !__all_sync(kFull, (acc & need) == need);
-            }
-            nx = acc & need;
-            if (threadIdx.x == 0) {
-                ++m.rows;
-                m.entries += (unsigned long long)(b0 - beg);
-            }
+        const unsigned long long nx = valid ? nxt[(int64_t)v * W + w] : 0ULL;
+        const unsigned long long deg = valid ? (unsigned long long)(__ldg(&rowp[v + 1]) - __ldg(&rowp[v])) : 0ULL;
+        if (nx) vis[(int64_t)v * W + w] = vw | nx;
+        any |= nx;
+        const bool had = group_any<W>(__ballot_sync(kFull, need != 0));
+        const bool got = group_any<W>(__ballot_sync(kFull, nx != 0));
+        const bool left = group_any<W>(__ballot_sync(kFull, (need & ~nx) != 0));
+        const long long at = warp_append(w == 0 && got, &st->n_next);
+        if (at >= 0) {
+            next_front[at] = v;
+            m.fr_edges += deg;
         }
-        if (warp == 0) {
-            if (t == 0) {
-                nxt[(int64_t)v * W + w] = nx;
-                if (nx) vis[(int64_t)v * W + w] = vw | nx;
-            }
-            any |= nx;
-            const bool got = __any_sync(kFull, nx != 0);
-            const bool left = __any_sync(kFull, (need & ~nx) != 0);
-            const long long at = warp_append(lane == 0 && got, &st->n_next);
-            if (at >= 0) {
-                next_front[at] = v;
-                m.fr_edges += (unsigned long long)deg;
-            }
-            if (lane == 0 && left) m.rem_edges += (unsigned long long)deg;
-            c.add(t == 0 && (!pred || pred[v]) ? nx : 0ULL);
-            if (c.n == 31) c.flush(sh, w, 0);
-        }
+        if (w == 0 && had) ++m.rows;
+        if (w == 0 && left) m.rem_edges += deg;
+        c.add((valid && (!pred || pred[v])) ? nx : 0ULL);
+        if (c.n == 31) c.flush(sh, w, q * (64 * W / 32) + q);
     }
     x_flush(c, any, m, sh, st);
 }
@@ -474,7 +502,6 @@ __global__ void __launch_bounds__(256) k_x_huge(const int32_t* __restrict__ list
 // Top-down level, step 1: the frontier rows as work items of at most
 // kXSeg entries (vertex << 32 | segment), so that a hub's row is spread over
 // many warps.  A vertex without running bits gives none.
-constexpr int kXSeg = 256;
 
 template <int W>
 __global__ void k_x_td_items(const int32_t* __restrict__ front, int64_t n_front, const int64_t* __restrict__ rowp,
@@ -719,7 +746,9 @@ struct XScratch {
     int32_t *light, *heavy;
     const int32_t* huge;
     int32_t* front[2];
-    unsigned long long* items;
+    unsigned long long* huge_items;  // of the huge rows
+    int64_t n_huge_items;
+    unsigned long long* items;       // of a top-down level
     size_t n_items;
     void* state;
     int64_t n_light, n_heavy, n_huge;
@@ -774,9 +803,14 @@ int run_sweep(fl_graph* g, const XScratch& x, int mode, int64_t nb, const int32_
             FL_LAUNCH(cls, k_x_td_finish<W><<<blocks_for(n, 256 / W, kXLevelBlocks), 256, 0, st>>>(
                                n, rowp, buf[c ^ 1], vis, pred, front[fc ^ 1], xs));
         } else {
-            if (x.n_huge > 0)
-                FL_LAUNCH(cls, k_x_huge<W><<<blocks_for(x.n_huge, 1, kXLevelBlocks), 256, 0, st>>>(
-                                   x.huge, x.n_huge, rowp, cols, buf[c], buf[c ^ 1], vis, pred, front[fc ^ 1], xs));
+            if (x.n_huge > 0) {
+                FL_LAUNCH(cls, k_x_huge_clear<W><<<blocks_for(x.n_huge, 256 / W), 256, 0, st>>>(x.huge, x.n_huge,
+                                                                                              buf[c ^ 1]));
+                FL_LAUNCH(cls, k_x_huge<W><<<blocks_for(x.n_huge_items, 8), 256, 0, st>>>(
+                                   x.huge_items, x.n_huge_items, rowp, cols, buf[c], buf[c ^ 1], vis, xs));
+                FL_LAUNCH(cls, k_x_huge_done<W><<<blocks_for(x.n_huge, 256 / W, kXLevelBlocks), 256, 0, st>>>(
+                                   x.huge, x.n_huge, rowp, buf[c ^ 1], vis, pred, front[fc ^ 1], xs));
+            }
             if (x.n_heavy > 0)
                 FL_LAUNCH(cls, k_x_heavy<W><<<grid_h, 256, 0, st>>>(x.heavy, x.n_heavy, rowp, cols, buf[c],
                                                                     buf[c ^ 1], vis, pred, front[fc ^ 1], xs));
@@ -827,20 +861,22 @@ int run_sweeps(fl_graph* g, int mode, int64_t n_src, const int32_t* src, int64_t
     // int32 lists: light rows (n), heavy rows from the front and huge ones from
     // the back (n), two frontiers (n + kMost each: the first frontier lists the
     // sweep's sources, repeats included); then the top-down work items (uint64,
-    // one per kXSeg entries of a frontier row: at most n + kMost + nnz / kXSeg)
-    // and the sweep state
+    // one per kXSeg entries of a frontier row: at most n + kMost + nnz / kXSeg),
+    // those of the huge rows (at most 2 nnz / kXSeg) and the sweep state
     const size_t lists = ((size_t)(4 * n + 2 * kMost) * 4 + 255) & ~(size_t)255;
     XScratch x;
     x.n_items = (size_t)(n + kMost + nnz / kXSeg + 1);
     const size_t items_b = (x.n_items * 8 + 255) & ~(size_t)255;
-    FL_TRY(dalloc(g->xaux, lists + items_b + sizeof(XState<kXMaxW>)));
+    const size_t huge_b = ((size_t)(2 * (nnz / kXSeg) + 1) * 8 + 255) & ~(size_t)255;
+    FL_TRY(dalloc(g->xaux, lists + items_b + huge_b + sizeof(XState<kXMaxW>)));
     x.vis = g->xbits.as<unsigned long long>();
     x.light = g->xaux.as<int32_t>();
     x.heavy = x.light + n;
     x.front[0] = x.light + 2 * n;
     x.front[1] = x.light + 3 * n + kMost;
     x.items = reinterpret_cast<unsigned long long*>(g->xaux.as<char>() + lists);
-    x.state = g->xaux.as<char>() + lists + items_b;
+    x.huge_items = reinterpret_cast<unsigned long long*>(g->xaux.as<char>() + lists + items_b);
+    x.state = g->xaux.as<char>() + lists + items_b + huge_b;
     Counters* ctr = g->ctr.as<Counters>();
     FL_CUDA(cudaMemsetAsync(g->ctr.p, 0, sizeof(Counters), st));
     FL_LAUNCH(kProfExact, k_x_lists<<<blocks_for(n, 256), 256, 0, st>>>(g->rowp.as<int64_t>(), n, x.light, x.heavy,
@@ -851,6 +887,15 @@ int run_sweeps(fl_graph* g, int mode, int64_t n_src, const int32_t* src, int64_t
     x.n_heavy = (int64_t)g->h_ctr->aux3;
     x.n_huge = (int64_t)g->h_ctr->frontier;
     x.huge = x.heavy + n - x.n_huge;
+    x.n_huge_items = 0;
+    if (x.n_huge > 0) {
+        FL_CUDA(cudaMemsetAsync(g->ctr.p, 0, sizeof(Counters), st));
+        FL_LAUNCH(kProfExact, k_x_huge_items<<<blocks_for(x.n_huge, 8), 256, 0, st>>>(
+                                  x.huge, x.n_huge, g->rowp.as<int64_t>(), x.huge_items, &ctr->aux0));
+        FL_CUDA(cudaGetLastError());
+        FL_TRY(read_counters(g));
+        x.n_huge_items = (int64_t)g->h_ctr->aux0;
+    }
     for (int64_t b0 = 0; b0 < n_src;) {
         const int w = width(n_src - b0);
         const int64_t nb = std::min<int64_t>(n_src - b0, 64 * w);

@@ -1,5 +1,5 @@
 """Exact ball sizes and radii where the sweeps can go wrong: rows at the limits
-between the kernels (32 / 33 entries, 1024 / 1025 entries), numbers of sources
+between the kernels and work items (32, 256 and 512 entries), numbers of sources
 around the sweep widths, one source listed many times."""
 import numpy as np
 import pytest
@@ -30,7 +30,7 @@ def _bfs_sizes(rowp, cols, src, D, pred):
     return out
 
 
-@pytest.mark.parametrize("deg", [32, 33, 1024, 1025, 2100])
+@pytest.mark.parametrize("deg", [32, 33, 256, 257, 512, 513, 1025, 2100])
 def test_row_limits(deg):
     n = 2 * deg + 2
     rowp, cols = brute.csr_from_edges(n, [(0, 2 + i) for i in range(deg)] + [(1, 2 + deg // 2 + i) for i in range(deg)])
