@@ -1099,14 +1099,37 @@ int build_ordinals(fl_graph* g, DBuf& tmp) {
     return FL_OK;
 }
 
-// The frontier of the previous hop as a bitmap: bit v = (Dcnt[v] > 0).
-__global__ void k_front_bitmap(const uint8_t* __restrict__ Dcnt, int64_t n, uint32_t* __restrict__ bm) {
+// Start of a hop, in one pass: the previous hop's frontier as a bitmap (bit v =
+// (Dp[v] > 0); Dp NULL at hop 1, where every vertex counts), this hop's
+// outputs at "no new entries" for every vertex that will not change, and the
+// counters at zero.
+__global__ void k_hop_begin(const uint8_t* __restrict__ Dp, int64_t n, uint32_t* __restrict__ bm,
+                            uint8_t* __restrict__ Dc, uint32_t* __restrict__ F, uint64_t* __restrict__ H,
+                            Counters* ctr) {
+    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += stride) {
+    if (tid < (int64_t)(sizeof(Counters) / 8)) reinterpret_cast<unsigned long long*>(ctr)[tid] = 0;
+    for (int64_t base = tid & ~(int64_t)31; base < n; base += stride) {
         const int64_t v = base + lane_id();
-        const unsigned w = __ballot_sync(kFull, v < n && Dcnt[v] > 0);
-        if (lane_id() == 0) bm[base >> 5] = w;
+        if (Dp) {
+            const unsigned w = __ballot_sync(kFull, v < n && Dp[v] > 0);
+            if (lane_id() == 0) bm[base >> 5] = w;
+        }
+        if (v < n) {
+            Dc[v] = 0;
+            F[v] = kNil;
+            H[v] = 0;
+        }
     }
+}
+
+// Ends of the ADS offsets; the totals also to the counters (aux0, aux3).
+__global__ void k_ads_totals(const int32_t* __restrict__ vg, const int32_t* __restrict__ ve, int64_t n,
+                             int64_t* __restrict__ gofs, int64_t* __restrict__ eofs, Counters* ctr) {
+    gofs[n] = gofs[n - 1] + vg[n - 1];
+    eofs[n] = eofs[n - 1] + ve[n - 1];
+    ctr->aux0 = (unsigned long long)gofs[n];
+    ctr->aux3 = (unsigned long long)eofs[n];
 }
 
 // ------------------------------------------------------------------ driver
@@ -1267,8 +1290,10 @@ int build_sketches(fl_graph* g, int k, uint64_t seed) {
         int64_t n_list;
         // dense hops run every non-isolated vertex; sparse hops expand the frontier
         const bool dense = !fr_list_ready;
-        Counters init{};
-        FL_CUDA(cudaMemcpyAsync(g->ctr.p, &init, sizeof(Counters), cudaMemcpyHostToDevice, st));
+        FL_LAUNCH(kProfSketchOther, k_hop_begin<<<grid_for(n, 256), 256, 0, st>>>(
+                                        hop > 1 ? g->Dcnt[pin].as<uint8_t>() : nullptr, n, g->fbm.as<uint32_t>(),
+                                        g->Dcnt[pout].as<uint8_t>(), g->F[pout].as<uint32_t>(),
+                                        g->H[pout].as<uint64_t>(), g->ctr.as<Counters>()));
         if (dense) {
             list = g->low_list.as<int32_t>();
             n_list = g->n_low;
@@ -1290,13 +1315,6 @@ int build_sketches(fl_graph* g, int k, uint64_t seed) {
             FL_TRY(dgrow(g->stg_ent, cap * k * 4, (size_t)used_slots * k * 4, st));
             g->stg_grp_cap = cap;
         }
-        // this hop's outputs read "no new entries" for every vertex that does not change
-        FL_CUDA(cudaMemsetAsync(g->Dcnt[pout].p, 0, (size_t)n, st));
-        FL_CUDA(cudaMemsetAsync(g->F[pout].p, 0xff, (size_t)n * 4, st));
-        FL_CUDA(cudaMemsetAsync(g->H[pout].p, 0, (size_t)n * 8, st));
-        if (hop > 1)
-            FL_LAUNCH(kProfSketchOther, k_front_bitmap<<<grid_for(n, 256), 256, 0, st>>>(
-                                            g->Dcnt[pin].as<uint8_t>(), n, g->fbm.as<uint32_t>()));
         if (census) {
             if (n_list > 0)
                 FL_LAUNCH(kProfSketchOther, k_hop_census<<<grid_for(n_list, 256), 256, 0, st>>>(
@@ -1344,7 +1362,7 @@ int build_sketches(fl_graph* g, int k, uint64_t seed) {
         // a small frontier makes the next hop sparse: collect its list
         fr_list_ready = false;
         if (n_front * g->sched.sparse_div < g->n_low + g->n_hubs) {
-            FL_CUDA(cudaMemsetAsync(&g->ctr.as<Counters>()->aux0, 0, 8, st));
+            // (aux0 is zero since the hop began)
             if (n_list > 0)
                 FL_LAUNCH(kProfSketchExpand, k_collect_frontier<<<grid_for(n_list, 256), 256, 0, st>>>(
                                                  list, n_list, g->Dcnt[pout].as<uint8_t>(),
@@ -1368,14 +1386,16 @@ int build_sketches(fl_graph* g, int k, uint64_t seed) {
     FL_TRY(dalloc(g->eofs, (size_t)(n + 1) * 8));
     FL_TRY(scan_exclusive_i32_to_i64(g->vg.as<int32_t>(), g->gofs.as<int64_t>(), n, st, g->scratch));
     FL_TRY(scan_exclusive_i32_to_i64(g->ve.as<int32_t>(), g->eofs.as<int64_t>(), n, st, g->scratch));
-    FL_TRY(scan_total(g->gofs.as<int64_t>(), g->vg.as<int32_t>(), n, st, &g->n_groups));
-    FL_TRY(scan_total(g->eofs.as<int64_t>(), g->ve.as<int32_t>(), n, st, &g->n_entries));
+    FL_LAUNCH(kProfSketchOther, k_ads_totals<<<1, 1, 0, st>>>(g->vg.as<int32_t>(), g->ve.as<int32_t>(), n,
+                                                              g->gofs.as<int64_t>(), g->eofs.as<int64_t>(),
+                                                              g->ctr.as<Counters>()));
+    FL_TRY(read_counters(g));
+    g->n_groups = (int64_t)g->h_ctr->aux0;
+    g->n_entries = (int64_t)g->h_ctr->aux3;
     g->prof.bytes[kProfSketchMerge] += 12.0 * (double)(g->n_entries - n);
     FL_TRY(dalloc(g->ginfo, (size_t)std::max<int64_t>(g->n_groups, 1) * 4));
     FL_TRY(dalloc(g->gwt, (size_t)std::max<int64_t>(g->n_groups, 1) * 8));
     FL_TRY(dalloc(g->eid, (size_t)std::max<int64_t>(g->n_entries, 1) * 4));
-    FL_CUDA(cudaMemcpyAsync(g->gofs.as<int64_t>() + n, &g->n_groups, 8, cudaMemcpyHostToDevice, st));
-    FL_CUDA(cudaMemcpyAsync(g->eofs.as<int64_t>() + n, &g->n_entries, 8, cudaMemcpyHostToDevice, st));
     FL_LAUNCH(kProfSketchOther, k_ads_hop0<<<grid_for(n, 256), 256, 0, st>>>(
                                     n, g->gofs.as<int64_t>(), g->eofs.as<int64_t>(), g->ginfo.as<uint32_t>(),
                                     g->gwt.as<double>(), g->eid.as<int32_t>()));
@@ -1390,8 +1410,7 @@ int build_sketches(fl_graph* g, int k, uint64_t seed) {
                                         g->max_part > 0 ? g->vbase.as<int32_t>() : nullptr, g->eid.as<int32_t>()));
     }
     FL_CUDA(cudaGetLastError());
-    FL_CUDA(cudaStreamSynchronize(st));
-    FL_TRY(compute_ecc_bound(g));
+    FL_TRY(compute_ecc_bound(g));  // synchronises
     g->built = 1;
     return FL_OK;
 }
