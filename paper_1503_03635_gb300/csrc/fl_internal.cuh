@@ -114,10 +114,10 @@ __host__ __device__ __forceinline__ uint64_t facility_priority(uint64_t seed, in
 
 constexpr unsigned kFull = 0xffffffffu;
 
-// Vertices with more than kHubDeg neighbours are hubs; their edge lists are
-// processed in segments of kSeg edges, one group of lanes per segment.
-constexpr int kHubDeg = 2048;
-constexpr int kSeg = 2048;
+// Vertices with more than fl_graph::seg neighbours are hubs; their edge lists
+// are processed in segments of that many edges, one group of lanes per segment
+// (seg_of in k_sketch.cu).
+constexpr int kMaxSeg = 2048;
 // Non-hub vertices with at most kSmallDeg neighbours are pulled by one thread each.
 constexpr int kSmallDeg = 8;
 // Graphs of at most kResidentEdges CSR entries (and vertices) run their MIS and
@@ -218,6 +218,20 @@ __device__ __forceinline__ long long block_append(bool pred, unsigned long long*
     }
     __syncthreads();
     return pred ? (long long)(sh.off[warp] + __popc(m & ((1u << lane) - 1u))) : -1LL;
+}
+
+// Adds the threads' counts to *counter, one global atomic per block (a launch
+// of thousands of warps that each add to the same word waits for the word, some
+// 2 ns an add).  Every thread of the block calls it, once per launch.
+__device__ __forceinline__ void block_count(unsigned x, unsigned long long* counter) {
+    __shared__ unsigned s_part[32];
+    x = __reduce_add_sync(kFull, x);
+    if (lane_id() == 0) s_part[threadIdx.x >> 5] = x;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const unsigned long long y = __reduce_add_sync(kFull, threadIdx.x < (blockDim.x >> 5) ? s_part[threadIdx.x] : 0u);
+        if (threadIdx.x == 0 && y) atomicAdd(counter, y);
+    }
 }
 
 // ----------------------------------------------------------------- groups in lockstep
@@ -544,6 +558,7 @@ struct fl_graph {
     // kSmallDeg neighbours (a thread each), more (a group of lanes each)
     fl::DBuf small_list, mid_list; // int32[n_small], int32[n_mid]
     int64_t n_small = 0, n_mid = 0;
+    int seg = fl::kMaxSeg;         // longest row that is not a hub's, and edges per hub segment
     fl::DBuf hub_seg;              // int64[n_hubs+1]: first segment of each hub
     fl::DBuf seg_hub;              // int32[n_seg]: hub of each segment
     int64_t n_low = 0, n_hubs = 0, n_seg = 0;

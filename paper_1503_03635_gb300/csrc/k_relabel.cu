@@ -65,7 +65,7 @@ __global__ void k_perm_maps(const uint32_t* __restrict__ perm, const int64_t* __
 // most 8 entries (a sorting network in registers), a warp per row of 9-32
 // (a bitonic network of shuffles), a warp per row of 33-kSortMax (a bitonic
 // network over values held m/32 per lane, in registers and shuffles), and for
-// the longer rows (hubs, kept in their input order) a warp per kSeg entries
+// the longer rows (hubs, kept in their input order) a warp per kMaxSeg entries
 // of the new CSR.
 constexpr int kSortMax = 2048;
 constexpr int32_t kSortPad = 0x7fffffff;  // above every vertex id
@@ -252,16 +252,16 @@ __global__ void __launch_bounds__(kBig ? 32 * kBigWarps : 256, kBig ? 4 : 3) k_r
 }
 
 // Rows [0, i1) (hubs, more than kSortMax entries, kept in input order): a
-// warp per kSeg consecutive entries of the new CSR; a chunk spans at most two
-// rows (every hub row is longer than kSeg).
+// warp per kMaxSeg consecutive entries of the new CSR; a chunk spans at most two
+// rows (every hub row is longer than kMaxSeg).
 __global__ void k_rows_hub(const int64_t* __restrict__ rowp, const int32_t* __restrict__ cols,
                            const int32_t* __restrict__ rid, const int32_t* __restrict__ inv,
                            const int64_t* __restrict__ rowp_new, int64_t i1, int32_t* __restrict__ cols_new) {
     const int lane = lane_id();
     const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int64_t total = rowp_new[i1];
-    for (int64_t c0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kSeg; c0 < total;
-         c0 += warps * kSeg) {
+    for (int64_t c0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kMaxSeg; c0 < total;
+         c0 += warps * kMaxSeg) {
         int64_t lo = 0, hi = i1 - 1;  // the row holding entry c0: last r with rowp_new[r] <= c0
         while (lo < hi) {
             const int64_t mid = (lo + hi + 1) >> 1;
@@ -271,7 +271,7 @@ __global__ void k_rows_hub(const int64_t* __restrict__ rowp, const int32_t* __re
         const int64_t r0 = lo, r1 = lo + 1 < i1 ? lo + 1 : lo;
         const int64_t s0 = rowp_new[r0], s1 = rowp_new[r0 + 1];
         const int64_t o0 = rowp[rid[r0]], o1 = rowp[rid[r1]];
-        const int64_t c1 = c0 + kSeg < total ? c0 + kSeg : total;
+        const int64_t c1 = c0 + kMaxSeg < total ? c0 + kMaxSeg : total;
         for (int64_t p = c0 + lane; p < c1; p += 32) {
             const int64_t src = p < s1 ? o0 + (p - s0) : o1 + (p - s1);
             cols_new[p] = __ldg(&inv[__ldcs(&cols[src])]);
@@ -408,7 +408,7 @@ int relabel_graph(fl_graph* g) {
             const int64_t* rpn = rowp_new.as<int64_t>();
             int32_t* cn = cols_new.as<int32_t>();
             if (c_mid > 0) {
-                const int64_t chunks = (g->nnz + kSeg - 1) / kSeg;  // an upper bound of the hub chunks
+                const int64_t chunks = (g->nnz + kMaxSeg - 1) / kMaxSeg;  // an upper bound of the hub chunks
                 FL_LAUNCH(kProfOther, k_rows_hub<<<grid_for(chunks, 8), 256, 0, st>>>(rp, cl, rid, inv, rpn, c_mid, cn));
             }
             if (c_lo > c_mid)

@@ -10,7 +10,7 @@
 // frontier's values snapshotted first); pull rounds write the second buffer
 // (every vertex reads its frontier neighbours, found in a bitmap; no atomics
 // except per hub segment) and flag changed vertices with the next round's
-// stamp.  Hub edge lists are split into kSeg-edge segments in both.
+// stamp.  Hub edge lists are split into fl_graph::seg-edge segments in both.
 #include <algorithm>
 #include <cstdio>
 
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(256) k_pull_small(const int32_t* __restrict__ 
                                                     const int32_t* __restrict__ vpart,
                                                     const int32_t* __restrict__ part_cnt, Prune pr) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    unsigned long long changed = 0;
+    unsigned changed = 0;
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n_list; base += stride) {
         const int64_t i = base + lane_id();
         const int32_t v = i < n_list ? list[i] : 0;
@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(256) k_pull_small(const int32_t* __restrict__ 
         }
         changed += __popc(__ballot_sync(kFull, ch));
     }
-    if (lane_id() == 0 && changed) atomicAdd(n_changed, changed);
+    block_count(lane_id() == 0 ? changed : 0u, n_changed);
 }
 
 // Pull round over the other non-hub vertices: four vertices per warp, eight
@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(256) k_pull_low(const int32_t* __restrict__ li
     const int lane = lane_id();
     const int sub = lane & 7;
     const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    unsigned long long changed = 0;
+    unsigned changed = 0;
     for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w * 4 < n_list; w += warps) {
         const int64_t i = w * 4 + (lane >> 3);
         const int32_t v = i < n_list ? list[i] : 0;
@@ -197,10 +197,10 @@ __global__ void __launch_bounds__(256) k_pull_low(const int32_t* __restrict__ li
         }
         changed += __popc(__ballot_sync(kFull, ch));
     }
-    if (lane == 0 && changed) atomicAdd(n_changed, changed);
+    block_count(lane == 0 ? changed : 0u, n_changed);
 }
 
-// Pull round over hubs: one warp per segment of kSeg edges.  Xn[v] starts as
+// Pull round over hubs: one warp per segment of fl_graph::seg edges.  Xn[v] starts as
 // X[v]; the segments lower it with atomicMin and the one that lowers it first
 // (it sees the old value) flags the hub.
 template <bool kAll>
@@ -208,6 +208,7 @@ __global__ void __launch_bounds__(256) k_pull_segs(const int32_t* __restrict__ s
                                                    const int64_t* __restrict__ hub_seg,
                                                    const int32_t* __restrict__ hub_list,
                                                    const int64_t* __restrict__ rowp, const int32_t* __restrict__ cols,
+                                                   int seg,
                                                    unsigned long long add, unsigned long long limit, bool settle,
                                                    const uint32_t* __restrict__ bm,
                                                    const unsigned long long* __restrict__ X,
@@ -222,8 +223,8 @@ __global__ void __launch_bounds__(256) k_pull_segs(const int32_t* __restrict__ s
         const int32_t v = hub_list[h];
         const unsigned long long own = X[v];
         if ((settle && own < limit) || part_idle(vpart, part_cnt, v) || skipped(pr, v)) continue;
-        const int64_t e0 = rowp[v] + (sidx - hub_seg[h]) * kSeg;
-        const int64_t e1 = min(e0 + (int64_t)kSeg, rowp[v + 1]);
+        const int64_t e0 = rowp[v] + (sidx - hub_seg[h]) * seg;
+        const int64_t e1 = min(e0 + (int64_t)seg, rowp[v + 1]);
         unsigned long long m = pull_min<kAll>(cols, e0 + lane, e1, 32, bm, X, add, limit, ~0ULL);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) m = umin64(m, __shfl_xor_sync(kFull, m, o));
@@ -244,7 +245,7 @@ __global__ void __launch_bounds__(256) k_pull_segs(const int32_t* __restrict__ s
 __global__ void k_snap_front(const int32_t* __restrict__ fr, const unsigned long long* __restrict__ n_fr,
                              const unsigned long long* __restrict__ X, unsigned long long* __restrict__ frval,
                              unsigned long long* __restrict__ reset_next, const int64_t* __restrict__ rowp,
-                             const int32_t* __restrict__ hub_list, int64_t n_hubs, uint32_t* __restrict__ hub_tag,
+                             const int32_t* __restrict__ hub_list, int64_t n_hubs, int seg, uint32_t* __restrict__ hub_tag,
                              uint32_t tag, unsigned long long* __restrict__ hub_val,
                              unsigned long long* __restrict__ edges) {
     const int64_t n = (int64_t)*n_fr;
@@ -257,7 +258,7 @@ __global__ void k_snap_front(const int32_t* __restrict__ fr, const unsigned long
         frval[i] = x;
         const int64_t d = rowp[v + 1] - rowp[v];
         ed += (unsigned long long)d;
-        if (d > kHubDeg) {
+        if (d > seg) {
             int64_t lo = 0, hi = n_hubs;  // first hub_list entry >= v
             while (lo < hi) {
                 const int64_t mid = (lo + hi) >> 1;
@@ -281,6 +282,7 @@ __global__ void __launch_bounds__(256) k_push_low(const int32_t* __restrict__ fr
                                                   const unsigned long long* __restrict__ frval,
                                                   const unsigned long long* __restrict__ n_fr,
                                                   const int64_t* __restrict__ rowp, const int32_t* __restrict__ cols,
+                                                   int seg,
                                                   unsigned long long add, unsigned long long limit,
                                                   unsigned long long* __restrict__ X,
                                                   uint32_t* __restrict__ stamp, uint32_t sv,
@@ -292,7 +294,7 @@ __global__ void __launch_bounds__(256) k_push_low(const int32_t* __restrict__ fr
     for (int64_t w = (((int64_t)blockIdx.x * blockDim.x) + threadIdx.x) >> 5; w < n; w += warps) {
         const int32_t v = fr[w];
         const int64_t beg = rowp[v], end = rowp[v + 1];
-        if (end - beg > kHubDeg) continue;  // hubs: k_push_segs
+        if (end - beg > seg) continue;  // hubs: k_push_segs
         const unsigned long long val = frval[w] + add;
         for (int64_t cb = beg; cb < end; cb += 32) {
             const int64_t e = cb + lane;
@@ -321,6 +323,7 @@ __global__ void __launch_bounds__(256) k_push_segs(const int32_t* __restrict__ s
                                                    const uint32_t* __restrict__ hub_tag, uint32_t tag,
                                                    const unsigned long long* __restrict__ hub_val,
                                                    const int64_t* __restrict__ rowp, const int32_t* __restrict__ cols,
+                                                   int seg,
                                                    unsigned long long add, unsigned long long limit,
                                                    unsigned long long* __restrict__ X,
                                                    uint32_t* __restrict__ stamp, uint32_t sv,
@@ -333,8 +336,8 @@ __global__ void __launch_bounds__(256) k_push_segs(const int32_t* __restrict__ s
         if (hub_tag[h] != tag) continue;
         const int32_t v = hub_list[h];
         const unsigned long long val = hub_val[h] + add;
-        const int64_t e0 = rowp[v] + (sidx - hub_seg[h]) * kSeg;
-        const int64_t e1 = min(e0 + (int64_t)kSeg, rowp[v + 1]);
+        const int64_t e0 = rowp[v] + (sidx - hub_seg[h]) * seg;
+        const int64_t e1 = min(e0 + (int64_t)seg, rowp[v + 1]);
         for (int64_t cb = e0; cb < e1; cb += 32) {
             const int64_t e = cb + lane;
             bool fresh = false;
@@ -453,7 +456,7 @@ int relax_round(fl_graph* g, Relax& r, unsigned long long add, uint32_t sv, int 
         }
         FL_CUDA(cudaMemsetAsync(r.ecnt, 0, 8, st));
         FL_LAUNCH(cls, k_snap_front<<<grid_for(r.n_front, 256), 256, 0, st>>>(
-                           r.fr[r.fc], &r.cnt[r.fc], X, r.frval, &r.cnt[r.fc ^ 1], rowp, hub_list, g->n_hubs,
+                           r.fr[r.fc], &r.cnt[r.fc], X, r.frval, &r.cnt[r.fc ^ 1], rowp, hub_list, g->n_hubs, g->seg,
                            r.hub_tag, r.sv_prev, r.hub_val, r.ecnt));
         FL_CUDA(cudaGetLastError());
         if (r.n_front >= kPushAlways) {
@@ -463,13 +466,13 @@ int relax_round(fl_graph* g, Relax& r, unsigned long long add, uint32_t sv, int 
         }
     }
     if (!dense) {
-        FL_LAUNCH(cls, k_push_low<<<grid_for(r.n_front, 8), 256, 0, st>>>(r.fr[r.fc], r.frval, &r.cnt[r.fc], rowp, cols,
+        FL_LAUNCH(cls, k_push_low<<<grid_for(r.n_front, 8), 256, 0, st>>>(r.fr[r.fc], r.frval, &r.cnt[r.fc], rowp, cols, g->seg,
                                                                          add, r.limit, X, r.stamp, sv, r.fr[r.fc ^ 1],
                                                                          &r.cnt[r.fc ^ 1], r.prune));
         if (g->n_seg > 0)
             FL_LAUNCH(cls, k_push_segs<<<grid_for(g->n_seg, 8), 256, 0, st>>>(
                                g->seg_hub.as<int32_t>(), g->n_seg, g->hub_seg.as<int64_t>(), hub_list, r.hub_tag,
-                               r.sv_prev, r.hub_val, rowp, cols, add, r.limit, X, r.stamp, sv, r.fr[r.fc ^ 1],
+                               r.sv_prev, r.hub_val, rowp, cols, g->seg, add, r.limit, X, r.stamp, sv, r.fr[r.fc ^ 1],
                                &r.cnt[r.fc ^ 1], r.prune));
         FL_CUDA(cudaGetLastError());
         r.fc ^= 1;
@@ -501,7 +504,7 @@ int relax_round(fl_graph* g, Relax& r, unsigned long long add, uint32_t sv, int 
                                r.stamp, sv, &r.cnt[2], vpart, r.part_cnt, r.prune));
         if (g->n_seg > 0)
             FL_LAUNCH(cls, segs<<<grid_for(g->n_seg, 8), 256, 0, st>>>(
-                               g->seg_hub.as<int32_t>(), g->n_seg, g->hub_seg.as<int64_t>(), hub_list, rowp, cols, add,
+                               g->seg_hub.as<int32_t>(), g->n_seg, g->hub_seg.as<int64_t>(), hub_list, rowp, cols, g->seg, add,
                                r.limit, r.settle, r.bm, X, Xn, r.stamp, sv, &r.cnt[2], vpart, r.part_cnt,
                                r.prune));
         FL_CUDA(cudaGetLastError());
@@ -549,7 +552,7 @@ __global__ void __launch_bounds__(256) k_mark_small(const int32_t* __restrict__ 
                                                     const uint8_t* __restrict__ need, uint32_t b,
                                                     unsigned long long* __restrict__ n_marked) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    unsigned long long marked = 0;
+    unsigned marked = 0;
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n_list; base += stride) {
         const int64_t i = base + lane_id();
         const int32_t v = i < n_list ? list[i] : 0;
@@ -567,7 +570,7 @@ __global__ void __launch_bounds__(256) k_mark_small(const int32_t* __restrict__ 
         }
         marked += __popc(__ballot_sync(kFull, hit));
     }
-    if (lane_id() == 0 && marked) atomicAdd(n_marked, marked);
+    block_count(lane_id() == 0 ? marked : 0u, n_marked);
 }
 
 // Other non-hub vertices: eight lanes each (four per warp), 32 entries of a
@@ -580,7 +583,7 @@ __global__ void __launch_bounds__(256) k_mark_low(const int32_t* __restrict__ li
     const int lane = lane_id();
     const int sub = lane & 7;
     const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    unsigned long long marked = 0;
+    unsigned marked = 0;
     for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w * 4 < n_list; w += warps) {
         const int64_t i = w * 4 + (lane >> 3);
         const int32_t v = i < n_list ? list[i] : 0;
@@ -610,17 +613,16 @@ __global__ void __launch_bounds__(256) k_mark_low(const int32_t* __restrict__ li
             if (!__any_sync(kFull, work)) break;
         }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) marked += __shfl_xor_sync(kFull, marked, o);
-    if (lane == 0 && marked) atomicAdd(n_marked, marked);
+    block_count(marked, n_marked);
 }
 
-// Hubs: a warp per segment of kSeg entries; every segment that finds a marked
+// Hubs: a warp per segment of fl_graph::seg entries; every segment that finds a marked
 // neighbour marks the hub (the count may hold a hub more than once).
 __global__ void __launch_bounds__(256) k_mark_segs(const int32_t* __restrict__ seg_hub, int64_t n_seg,
                                                    const int64_t* __restrict__ hub_seg,
                                                    const int32_t* __restrict__ hub_list,
                                                    const int64_t* __restrict__ rowp, const int32_t* __restrict__ cols,
+                                                   int seg,
                                                    const uint32_t* __restrict__ bm, uint8_t* __restrict__ kr,
                                                    const uint8_t* __restrict__ need, uint32_t b,
                                                    unsigned long long* __restrict__ n_marked) {
@@ -630,8 +632,8 @@ __global__ void __launch_bounds__(256) k_mark_segs(const int32_t* __restrict__ s
         const int32_t h = seg_hub[sidx];
         const int32_t v = hub_list[h];
         if (!unmarked_needed(kr, need, v, b)) continue;
-        const int64_t e0 = rowp[v] + (sidx - hub_seg[h]) * kSeg;
-        const int64_t e1 = min(e0 + (int64_t)kSeg, rowp[v + 1]);
+        const int64_t e0 = rowp[v] + (sidx - hub_seg[h]) * seg;
+        const int64_t e1 = min(e0 + (int64_t)seg, rowp[v + 1]);
         for (int64_t at = e0; at < e1; at += 128) {
             bool hit = false;
             int32_t u[4];
@@ -670,7 +672,7 @@ int mark_round(fl_graph* g, Relax& r, uint8_t* kr, const uint8_t* need, uint32_t
     if (g->n_seg > 0)
         FL_LAUNCH(cls, k_mark_segs<<<grid_for(g->n_seg, 8), 256, 0, st>>>(
                            g->seg_hub.as<int32_t>(), g->n_seg, g->hub_seg.as<int64_t>(), g->hub_list.as<int32_t>(),
-                           rowp, cols, r.bm, kr, need, b, &r.cnt[2]));
+                           rowp, cols, g->seg, r.bm, kr, need, b, &r.cnt[2]));
     FL_CUDA(cudaGetLastError());
     FL_CUDA(cudaMemcpyAsync(r.h_cnt, &r.cnt[2], 8, cudaMemcpyDeviceToHost, st));
     FL_CUDA(cudaStreamSynchronize(st));

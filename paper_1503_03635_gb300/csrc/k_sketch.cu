@@ -22,8 +22,8 @@
 //
 // Work decomposition of one hop.  A group of G lanes (G = 16 when k <= 16,
 // else 32) owns one vertex: lane i holds S[v][i].  Non-hub vertices are
-// processed directly (k_hop_vertices).  Hubs (degree > kHubDeg) are cut into
-// segments of kSeg edges; each segment yields a partial bottom-k of its
+// processed directly (k_hop_vertices).  Hubs (degree > fl_graph::seg) are cut into
+// segments of that many edges; each segment yields a partial bottom-k of its
 // candidates in scratch (k_hop_hub_segments), and one group per hub merges
 // the partials into the hub's sketch (k_hop_hubs).  Bottom-k of a union is the
 // bottom-k of the union of bottom-k's, so the split does not change results.
@@ -127,14 +127,15 @@ __device__ __forceinline__ int slice_emit(const Lock<G>& g, uint32_t r, int q, i
 // Per-group hop counters in shared memory, one slot per group, updated by
 // the group's lane 0 without atomics and flushed once at the end of a kernel
 // (counters in registers cost spills in the merge loops).  32-bit: a group
-// adds at most 32 * kHubDeg per vertex it processes (hub degrees go to the
+// adds at most 32 * kMaxSeg per vertex it processes (hub degrees go to the
 // global counters directly) and, with the grids of the hop kernels, processes
 // at most 2^31 / 77824 < 2^16 work items.
-enum { kCFront, kCMerges, kCMerging, kCDelta, kCNew, kNCtr };
+enum { kCFront, kCMerges, kCMerging, kCDelta, kCNew, kNCtr };  // in the order of flush_counters
 
 // Shared memory of a hop kernel (256 threads).
 struct HopShared {
     unsigned ctr[256 / 16][kNCtr];
+    unsigned cand[8];            // per warp
     uint32_t x[8][32];           // per warp: merged candidates by place
     uint32_t mask[256 / 16][32];  // per group: a delta mask
 };
@@ -157,6 +158,7 @@ struct HopIO {
     const int32_t* __restrict__ cols;
     int k;
     int hop;
+    int seg;                                 // longest row that is not a hub's, and edges per hub segment
     const uint32_t* __restrict__ ord;        // ordinal of each vertex
     uint32_t* __restrict__ S;
     uint8_t* __restrict__ Scnt;
@@ -371,7 +373,7 @@ __device__ __forceinline__ void stage_group(const HopIO& io, HopShared& sh, int3
     unsigned* c = sh.ctr[threadIdx.x / G];
     c[kCFront] += 1u;
     c[kCNew] += (unsigned)dcnt;
-    if (deg <= kHubDeg) {
+    if (deg <= io.seg) {
         c[kCMerges] += (unsigned)deg;
         c[kCDelta] += (unsigned)(deg * dcnt);
     }
@@ -468,20 +470,25 @@ __device__ __forceinline__ void ctr_init(const Lock<G>& g, HopShared& sh) {
     __syncwarp();
 }
 
-template <int G>
-__device__ __forceinline__ void flush_counters(const Lock<G>& g, const HopShared& sh, unsigned cand, Counters* ctr) {
-    // candidate reads are counted per lane; the other counters by lane 0
-    unsigned long long reads = cand;
+// End of a hop kernel (every thread calls): the groups' counters, one atomic
+// per counter and block.  (An atomic per counter and group put 60 k adds on one
+// line: 100 us of a 130 us hop on a graph with 61 k vertices.)
+__device__ __forceinline__ void flush_counters(HopShared& sh, int groups, unsigned cand, Counters* ctr) {
+    cand = __reduce_add_sync(kFull, cand);
+    if (lane_id() == 0) sh.cand[threadIdx.x >> 5] = cand;
+    __syncthreads();
+    if (threadIdx.x < kNCtr) {
+        unsigned long long x = 0;
+        for (int i = 0; i < groups; ++i) x += sh.ctr[i][threadIdx.x];
+        unsigned long long* to[kNCtr] = {&ctr->frontier, &ctr->merges, &ctr->merging, &ctr->delta_next,
+                                         &ctr->new_entries};
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) reads += __shfl_xor_sync(kFull, reads, o);
-    if (lane_id() == 0 && reads) atomicAdd(&ctr->cand_reads, reads);
-    if (g.l == 0) {
-        const unsigned* c = sh.ctr[threadIdx.x / G];
-        if (c[kCFront]) atomicAdd(&ctr->frontier, (unsigned long long)c[kCFront]);
-        if (c[kCMerges]) atomicAdd(&ctr->merges, (unsigned long long)c[kCMerges]);
-        if (c[kCMerging]) atomicAdd(&ctr->merging, (unsigned long long)c[kCMerging]);
-        if (c[kCDelta]) atomicAdd(&ctr->delta_next, (unsigned long long)c[kCDelta]);
-        if (c[kCNew]) atomicAdd(&ctr->new_entries, (unsigned long long)c[kCNew]);
+        for (int c = 0; c < kNCtr; ++c)
+            if (threadIdx.x == c && x) atomicAdd(to[c], x);
+    } else if (threadIdx.x == 32) {
+        unsigned long long x = 0;
+        for (int w = 0; w < 8; ++w) x += sh.cand[w];
+        if (x) atomicAdd(&ctr->cand_reads, x);
     }
 }
 
@@ -549,8 +556,7 @@ __global__ void __launch_bounds__(256, 6) k_hop_vertices(const int32_t* __restri
         }
         if (g.ballot(front) != 0 && g.l == 0) sh.ctr[threadIdx.x / G][kCMerging] += 1u;
     }
-    __syncwarp();
-    flush_counters(g, sh, cand, io.ctr);
+    flush_counters(sh, 256 / G, cand, io.ctr);
 }
 
 // Hub segments: partial results of one segment, written per segment -- the
@@ -583,8 +589,8 @@ __global__ void __launch_bounds__(256) k_hop_hub_segments(const int32_t* __restr
             if (g.l == 0) seg_flag[sidx] = 0;
             on = false;
         }
-        const int64_t e0 = on ? io.rowp[v] + (sidx - hub_seg[h]) * kSeg : 0;
-        const int64_t e1 = on ? min(e0 + (int64_t)kSeg, io.rowp[v + 1]) : 0;
+        const int64_t e0 = on ? io.rowp[v] + (sidx - hub_seg[h]) * io.seg : 0;
+        const int64_t e1 = on ? min(e0 + (int64_t)io.seg, io.rowp[v + 1]) : 0;
         const bool head = on && io.hop > 1 && io.W[v] != 0;
         bool front = false;
         if (warp_any(head)) {
@@ -620,8 +626,7 @@ __global__ void __launch_bounds__(256) k_hop_hub_segments(const int32_t* __restr
         const bool any = g.ballot(front) != 0;
         if (on && g.l == 0) seg_flag[sidx] = any ? 1 : 0;
     }
-    __syncwarp();
-    flush_counters(g, sh, cand, io.ctr);
+    flush_counters(sh, 256 / G, cand, io.ctr);
 }
 
 // Hubs: merge the partial results of all segments into the hub's sketch.
@@ -699,8 +704,13 @@ __global__ void __launch_bounds__(256) k_hop_hubs(const int32_t* __restrict__ hu
             if (warp_any(rest && !sat)) {
                 s.retau(g, k);
                 const int64_t end = rest && !sat ? s1 : s0;
-                for (int64_t q = s0; warp_any(q < end); ++q)
-                    merge_list(g, k, q < end && g.l < k ? part[q * k + g.l] : kNil, s, sx);
+                for (int64_t q = s0; warp_any(q < end); q += 4) {
+                    uint32_t x[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) x[j] = q + j < end && g.l < k ? part[(q + j) * k + g.l] : kNil;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) merge_list(g, k, x[j], s, sx);
+                }
             }
             const int got = finish_vertex(g, io, sh, rest, v, deg, old, s.sk, slot);
             if (rest) dc = got;
@@ -710,8 +720,7 @@ __global__ void __launch_bounds__(256) k_hop_hubs(const int32_t* __restrict__ hu
             atomicAdd(&io.ctr->delta_next, (unsigned long long)(deg * dc));
         }
     }
-    __syncwarp();
-    flush_counters(g, sh, 0u, io.ctr);
+    flush_counters(sh, 256 / G, 0u, io.ctr);
 }
 
 // Sparse hops: the non-hub part of N(frontier).  Warp per frontier vertex;
@@ -719,7 +728,7 @@ __global__ void __launch_bounds__(256) k_hop_hubs(const int32_t* __restrict__ hu
 // stamp = hop too, and the hub kernels skip the others.
 __global__ void k_expand(const int32_t* __restrict__ fr, int64_t n_fr, const int64_t* __restrict__ rowp,
                          const int32_t* __restrict__ cols, uint32_t* __restrict__ stamp, uint32_t hop,
-                         int32_t* __restrict__ act, Counters* ctr) {
+                         int seg, int32_t* __restrict__ act, Counters* ctr) {
     const int lane = lane_id();
     const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t w = (((int64_t)blockIdx.x * blockDim.x) + threadIdx.x) >> 5; w < n_fr; w += warps) {
@@ -731,7 +740,7 @@ __global__ void k_expand(const int32_t* __restrict__ fr, int64_t n_fr, const int
             int32_t v = 0;
             if (e < end) {
                 v = cols[e];
-                if (rowp[v + 1] - rowp[v] <= kHubDeg)
+                if (rowp[v + 1] - rowp[v] <= seg)
                     fresh = atomicExch(&stamp[v], hop) != hop;
                 else
                     stamp[v] = hop;  // a hub with a frontier neighbour: its segments run this hop
@@ -823,14 +832,14 @@ __global__ void __launch_bounds__(256) k_ads_entries(const StgGroup* __restrict_
 
 // ------------------------------------------------------------------ graph work lists
 
-__global__ void k_flag_degree(const int64_t* __restrict__ rowp, int64_t n, int32_t* __restrict__ low,
+__global__ void k_flag_degree(const int64_t* __restrict__ rowp, int64_t n, int seg, int32_t* __restrict__ low,
                               int32_t* __restrict__ hub, int32_t* __restrict__ nseg, int32_t* __restrict__ small) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
         const int64_t d = rowp[v + 1] - rowp[v];
-        low[v] = (d > 0 && d <= kHubDeg) ? 1 : 0;
-        hub[v] = d > kHubDeg ? 1 : 0;
-        nseg[v] = d > kHubDeg ? (int32_t)((d + kSeg - 1) / kSeg) : 0;
+        low[v] = (d > 0 && d <= seg) ? 1 : 0;
+        hub[v] = d > seg ? 1 : 0;
+        nseg[v] = d > seg ? (int32_t)((d + seg - 1) / seg) : 0;
         small[v] = (d > 0 && d <= kSmallDeg) ? 1 : 0;
     }
 }
@@ -884,9 +893,17 @@ static int scan_total(const int64_t* pos, const int32_t* flag, int64_t n, cudaSt
     return FL_OK;
 }
 
+// Longest row that is not cut, and edges per segment.  On a small graph the
+// longest row ends every hop (61 k vertices: hub segments 81 us in hop 1 at
+// 2048, 14 at 256); on larger ones shorter segments only add partial results to
+// merge (all hop kernels, 2^20 vertices, k = 32: 3.4 ms at 2048, 3.5 at 512, 3.9
+// at 256; 2^24, k = 16: 33.6 at 2048, 35.6 at 512).
+static int seg_of(int64_t nnz) { return nnz <= (4 << 20) ? 256 : kMaxSeg; }
+
 // Static work lists of a graph: non-hub non-isolated vertices, hubs and the
 // segment table of the hubs.
 int build_work_lists(fl_graph* g) {
+    g->seg = seg_of(g->nnz);
     const int64_t n = g->n;
     cudaStream_t st = g->stream;
     DBuf low, hub, nseg, low_pos, hub_pos, seg_pos, small, small_pos;
@@ -898,7 +915,7 @@ int build_work_lists(fl_graph* g) {
             (rc = dalloc(small, (size_t)n * 4)) || (rc = dalloc(small_pos, (size_t)n * 8)))
             break;
         FL_LAUNCH(kProfOther, k_flag_degree<<<grid_for(n, 256), 256, 0, st>>>(
-                                  g->rowp.as<int64_t>(), n, low.as<int32_t>(), hub.as<int32_t>(), nseg.as<int32_t>(),
+                                  g->rowp.as<int64_t>(), n, g->seg, low.as<int32_t>(), hub.as<int32_t>(), nseg.as<int32_t>(),
                                   small.as<int32_t>()));
         if ((rc = scan_exclusive_i32_to_i64(low.as<int32_t>(), low_pos.as<int64_t>(), n, st, g->scratch, kProfOther)) ||
             (rc = scan_exclusive_i32_to_i64(hub.as<int32_t>(), hub_pos.as<int64_t>(), n, st, g->scratch, kProfOther)) ||
@@ -1146,6 +1163,7 @@ static int launch_hop(fl_graph* g, int hop, const int32_t* list, int64_t n_list,
     io.cols = g->cols.as<int32_t>();
     io.k = k;
     io.hop = hop;
+    io.seg = g->seg;
     io.ord = g->ord.as<uint32_t>();
     io.S = g->S.as<uint32_t>();
     io.Scnt = g->Scnt.as<uint8_t>();
@@ -1300,7 +1318,7 @@ int build_sketches(fl_graph* g, int k, uint64_t seed) {
         } else {
             FL_LAUNCH(kProfSketchExpand, k_expand<<<grid_for(n_front, 8), 256, 0, st>>>(
                                              g->frontier[pin].as<int32_t>(), n_front, g->rowp.as<int64_t>(),
-                                             g->cols.as<int32_t>(), g->stamp.as<uint32_t>(), (uint32_t)hop,
+                                             g->cols.as<int32_t>(), g->stamp.as<uint32_t>(), (uint32_t)hop, g->seg,
                                              act.as<int32_t>(), g->ctr.as<Counters>()));
             FL_CUDA(cudaGetLastError());
             FL_TRY(read_counters(g));
