@@ -717,54 +717,100 @@ __global__ void k_ordinals(const uint32_t* __restrict__ sorted_f, int64_t m, con
         bcap[f] = b;
         mx = max(mx, b);
     }
-    // the largest ball radius: one atomic per warp
+    // the largest ball radius: one atomic per block
+    __shared__ int s_max;
+    if (threadIdx.x == 0) s_max = 0;
+    __syncthreads();
     mx = (int32_t)__reduce_max_sync(kFull, (unsigned)mx);
-    if (lane_id() == 0 && mx > 0) atomicMax(bmax, (unsigned long long)mx);
+    if (lane_id() == 0 && mx > 0) atomicMax(&s_max, mx);
+    __syncthreads();
+    if (threadIdx.x == 0 && s_max > 0) atomicMax(bmax, (unsigned long long)s_max);
 }
 
 // ------------------------------------------------------------------ MIS rounds (phase iii)
 
 // Bucket sizes by ball radius, the largest radius, and (for a graph made of
-// parts) each part's largest radius; maxima reduced per warp first.
-__global__ void k_bucket_count(const int32_t* __restrict__ ulist, int64_t n_u, const int32_t* __restrict__ bcap,
-                               int32_t* __restrict__ bcount, unsigned long long* __restrict__ tmax,
-                               const int32_t* __restrict__ vpart, int32_t* __restrict__ part_T) {
+// parts) each part's largest radius, gathered per block in shared memory (radii
+// and parts beyond its tables go to the global counts at once): the undecided
+// are in key order, so a warp holds most radii and parts, and its atomics on a
+// few words took 120 us for 4.2 M facilities in 16 parts.
+constexpr int kBuckets = 1024;
+constexpr int kPartTab = 1024;
+
+__global__ void __launch_bounds__(256) k_bucket_count(const int32_t* __restrict__ ulist, int64_t n_u,
+                                                      const int32_t* __restrict__ bcap, int32_t* __restrict__ bcount,
+                                                      unsigned long long* __restrict__ tmax,
+                                                      const int32_t* __restrict__ vpart, int32_t* __restrict__ part_T,
+                                                      int64_t n_parts) {
+    __shared__ int s_cnt[kBuckets];
+    __shared__ int s_part[kPartTab];
+    __shared__ int s_max;
+    for (int i = threadIdx.x; i < kBuckets; i += blockDim.x) s_cnt[i] = 0;
+    if (vpart)
+        for (int i = threadIdx.x; i < kPartTab; i += blockDim.x) s_part[i] = -1;
+    if (threadIdx.x == 0) s_max = 0;
+    __syncthreads();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n_u; base += stride) {
-        const int64_t i = base + lane_id();
-        const bool valid = i < n_u;
-        const int32_t f = valid ? ulist[i] : 0;
-        const int32_t b = valid ? bcap[f] : 0;
-        const unsigned sameb = __match_any_sync(kFull, valid ? b : -1);  // one atomic per bucket and warp
-        if (valid && lane_id() == __ffs(sameb) - 1) atomicAdd(&bcount[b], __popc(sameb));
-        const unsigned mx = __reduce_max_sync(kFull, (unsigned)b);
-        if (lane_id() == 0) atomicMax(tmax, (unsigned long long)mx);
+    int32_t mx = 0;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_u; i += stride) {
+        const int32_t f = ulist[i];
+        const int32_t b = bcap[f];
+        mx = max(mx, b);
+        if (b < kBuckets) atomicAdd(&s_cnt[b], 1);
+        else atomicAdd(&bcount[b], 1);
         if (vpart) {
-            const int32_t p = valid ? vpart[f] : -1;
-            const unsigned same = __match_any_sync(kFull, p);
-            const unsigned pm = __reduce_max_sync(same, (unsigned)b);
-            if (valid && lane_id() == __ffs(same) - 1) atomicMax(&part_T[p], (int)pm);
+            const int32_t p = vpart[f];
+            if (p >= kPartTab) atomicMax(&part_T[p], b);
+            else if (s_part[p] < b) atomicMax(&s_part[p], b);
         }
     }
+    mx = (int32_t)__reduce_max_sync(kFull, (unsigned)mx);
+    if (lane_id() == 0) atomicMax(&s_max, mx);
+    __syncthreads();
+    if (threadIdx.x == 0) atomicMax(tmax, (unsigned long long)s_max);
+    for (int i = threadIdx.x; i < min(s_max + 1, kBuckets); i += blockDim.x)
+        if (s_cnt[i]) atomicAdd(&bcount[i], s_cnt[i]);
+    if (vpart)
+        for (int i = threadIdx.x; i < kPartTab && i < n_parts; i += blockDim.x)
+            if (s_part[i] >= 0) atomicMax(&part_T[i], s_part[i]);
 }
 
-// Facilities to their bucket's range; the lanes of a warp with the same
-// bucket take consecutive places with one atomic.
-__global__ void k_bucket_scatter(const int32_t* __restrict__ ulist, int64_t n_u, const int32_t* __restrict__ bcap,
-                                 int32_t* __restrict__ cursor, int32_t* __restrict__ ubuck) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int lane = lane_id();
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n_u; base += stride) {
-        const int64_t i = base + lane;
-        const bool valid = i < n_u;
-        const int32_t f = valid ? ulist[i] : 0;
-        const int32_t b = valid ? bcap[f] : -1;
-        const unsigned same = __match_any_sync(kFull, b);
-        const int lead = __ffs(same) - 1;
-        int at = 0;
-        if (valid && lane == lead) at = atomicAdd(&cursor[b], __popc(same));
-        at = __shfl_sync(kFull, at, lead);
-        if (valid) ubuck[at + __popc(same & ((1u << lane) - 1u))] = f;
+// Facilities to their bucket's range: a block counts kScatter per thread by
+// bucket, reserves its places with one atomic per bucket and writes them.
+constexpr int kScatter = 8;
+
+__global__ void __launch_bounds__(256) k_bucket_scatter(const int32_t* __restrict__ ulist, int64_t n_u,
+                                                        const int32_t* __restrict__ bcap,
+                                                        int32_t* __restrict__ cursor, int32_t* __restrict__ ubuck) {
+    __shared__ int s_cnt[kBuckets];  // counts, then first places
+    __shared__ int s_top;
+    const int64_t tile = (int64_t)blockDim.x * kScatter;
+    for (int64_t t = blockIdx.x * tile; t < n_u; t += gridDim.x * tile) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < kBuckets; i += blockDim.x) s_cnt[i] = 0;
+        if (threadIdx.x == 0) s_top = 0;
+        __syncthreads();
+        int32_t f[kScatter], b[kScatter], at[kScatter];
+        int top = 0;
+#pragma unroll
+        for (int j = 0; j < kScatter; ++j) {
+            const int64_t i = t + (int64_t)j * blockDim.x + threadIdx.x;
+            f[j] = i < n_u ? ulist[i] : -1;
+            b[j] = f[j] >= 0 ? bcap[f[j]] : -1;
+            at[j] = 0;
+            if (b[j] >= kBuckets) at[j] = atomicAdd(&cursor[b[j]], 1);
+            else if (b[j] >= 0) at[j] = atomicAdd(&s_cnt[b[j]], 1);
+            if (b[j] < kBuckets) top = max(top, b[j]);
+        }
+        top = (int)__reduce_max_sync(kFull, (unsigned)top);
+        if (lane_id() == 0) atomicMax(&s_top, top);
+        __syncthreads();
+        for (int i = threadIdx.x; i <= s_top; i += blockDim.x)
+            if (s_cnt[i]) s_cnt[i] = atomicAdd(&cursor[i], s_cnt[i]);
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kScatter; ++j)
+            if (f[j] >= 0) ubuck[(b[j] < kBuckets ? s_cnt[b[j]] : 0) + at[j]] = f[j];
     }
 }
 
@@ -828,7 +874,7 @@ __global__ void k_claim(const int32_t* __restrict__ touched, const unsigned long
                         unsigned long long* __restrict__ n_new) {
     const int64_t n = (int64_t)*n_touched;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    unsigned long long fresh = 0;
+    unsigned fresh = 0;
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += stride) {
         const int64_t i = base + lane_id();
         bool now = false;
@@ -842,7 +888,7 @@ __global__ void k_claim(const int32_t* __restrict__ touched, const unsigned long
         }
         fresh += __popc(__ballot_sync(kFull, now));
     }
-    if (lane_id() == 0 && fresh) atomicAdd(n_new, fresh);
+    block_count(lane_id() == 0 ? fresh : 0u, n_new);
 }
 
 // Kill sweep decision: an undecided facility with a client claimed in this
@@ -1081,8 +1127,9 @@ int open_facilities(fl_solve* s) {
         FL_CUDA(cudaMemsetAsync(bcount, 0, (bmax + 1) * 4, st));
         FL_CUDA(cudaMemsetAsync(&cnt[4], 0, 8, st));
         if (part_T) FL_CUDA(cudaMemsetAsync(part_T, 0xff, (size_t)g->n_parts * 4, st));  // -1: no undecided facility
-        FL_LAUNCH(kProfMis, k_bucket_count<<<grid_for(n_u, 256), 256, 0, st>>>(
-                                ulist[cu], n_u, s->bcap.as<int32_t>(), bcount, &cnt[4], vpart, part_T));
+        FL_LAUNCH(kProfMis, k_bucket_count<<<std::min(grid_for(n_u, 256), 152 * 4), 256, 0, st>>>(
+                                ulist[cu], n_u, s->bcap.as<int32_t>(), bcount, &cnt[4], vpart, part_T,
+                                g->n_parts));
         FL_CUDA(cudaGetLastError());
         unsigned long long T64 = 0;
         FL_CUDA(cudaMemcpyAsync(&T64, &cnt[4], 8, cudaMemcpyDeviceToHost, st));
@@ -1101,7 +1148,7 @@ int open_facilities(fl_solve* s) {
         const bool prune = T < 255;
         if (prune) FL_CUDA(cudaMemsetAsync(reach, 0, (size_t)n, st));
         FL_CUDA(cudaMemcpyAsync(cursor, hoff.data(), (T + 1) * 4, cudaMemcpyHostToDevice, st));
-        FL_LAUNCH(kProfMis, k_bucket_scatter<<<grid_for(n_u, 256), 256, 0, st>>>(
+        FL_LAUNCH(kProfMis, k_bucket_scatter<<<grid_for(n_u, 256 * kScatter), 256, 0, st>>>(
                                 ulist[cu], n_u, s->bcap.as<int32_t>(), cursor, s->ubuck.as<int32_t>()));
         FL_CUDA(cudaGetLastError());
         const int32_t* ub = s->ubuck.as<int32_t>();
