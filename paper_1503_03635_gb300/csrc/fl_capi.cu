@@ -58,7 +58,7 @@ void destroy_solve(fl_solve* s) {
     DBuf* bufs[] = {&s->cost, &s->client, &s->radii, &s->ord, &s->fac_by_ord, &s->bcap, &s->state, &s->claimed,
                     &s->X, &s->stamp, &s->mval, &s->fr[0], &s->fr[1], &s->frval, &s->touched, &s->ulist,
                     &s->ubuck, &s->bcount, &s->open, &s->assign, &s->dist, &s->key_hi, &s->key_lo,
-                    &s->key_val, &s->key_alt, &s->obj_tmp, &s->part_T, &s->io, &s->eps, &s->eps_tab, &s->eps_ev, &s->eps_r,
+                    &s->key_val, &s->key_alt, &s->obj_tmp, &s->part_T, &s->io, &s->eps, &s->eps_tab, &s->eps_ev, &s->eps_out, &s->eps_r,
                     &s->eps_c, &s->rlist, &s->rctl, &s->reach, &s->kill};
     for (DBuf* b : bufs) dfree_idle(*b);
     delete s;

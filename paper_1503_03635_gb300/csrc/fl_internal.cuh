@@ -658,7 +658,7 @@ struct fl_solve {
     int64_t n_cand = 0, n_open = 0, mis_rounds = 0;
     // opening phase with eps > 0: per-vertex iterations and scratch, the grid
     // tables, one iteration's selection inputs, statistics of the last run
-    fl::DBuf eps, eps_tab, eps_ev, eps_r, eps_c;
+    fl::DBuf eps, eps_tab, eps_ev, eps_out, eps_r, eps_c;
     double eps_gamma = -1.0, eps_alpha0 = 0.0;
     int64_t eps_iterations = 0, eps_events = 0, eps_groups = 0;
     int have_eps = 0;
@@ -712,8 +712,9 @@ int compute_ecc_bound(fl_graph* g);
 
 int check_costs(fl_solve* s);
 int compute_radii(fl_solve* s);
-int sort_candidates(fl_solve* s, int64_t* m_out, const uint32_t** sorted);
+int sort_candidates(fl_solve* s, int64_t* m_out, const uint32_t** sorted, int64_t known = -1);
 int open_facilities(fl_solve* s);
+int open_facilities_queued(fl_solve* s, int64_t known, uint8_t* acc, int* outcome, bool* queued);
 // the greedy MIS and the assignment by weighted distance (k_wsolve.cu)
 int open_facilities_weighted(fl_solve* s);
 int assign_weighted(fl_solve* s);
@@ -725,6 +726,7 @@ void graph_bfs_release(GraphBfs* c);
 // resident kernels of small graphs (k_resident.cu); usable when g->n_items > 0
 int build_items(fl_graph* g);
 int mis_resident(fl_solve* s, int64_t m, bool* done);
+int mis_resident_queue(fl_solve* s, int64_t m, uint8_t* acc, int* outcome);
 int msbfs_resident(fl_graph* g, const int32_t* src, int64_t n_src, int32_t* label, int32_t* dist, DBuf& ctl, int cls);
 
 // Per-vertex pruning of the rounds of a sweep (the MIS cover and gather

@@ -625,19 +625,47 @@ int open_facilities_eps(fl_solve* s, double eps) {
     FL_LAUNCH(kProfMis, k_eps_single<<<grid_for(n, 256), 256, 0, st>>>(fac_iter, n, multi_d, acc));
     FL_TRY(dalloc(s->eps_r, (size_t)n * 8));
     FL_TRY(dalloc(s->eps_c, (size_t)n));
-    for (const auto& o : openings) {
-        if (o.second < 2) continue;
-        ++s->eps_groups;
+    // All groups but the last are queued one behind the other (on graphs whose
+    // selection is one launch), those that one launch did not finish run again
+    // with the host's help; the last one runs like a plain selection and leaves
+    // its log and counts.
+    std::vector<size_t> groups;
+    for (size_t i = 0; i < openings.size(); ++i)
+        if (openings[i].second >= 2) groups.push_back(i);
+    s->eps_groups = (int64_t)groups.size();
+    FL_TRY(dalloc(s->eps_out, groups.size() * 4 + 16));
+    int* outcome = s->eps_out.as<int>();
+    auto select = [&](size_t i, bool queue, bool* queued) -> int {
+        const auto& o = openings[groups[i]];
         FL_LAUNCH(kProfMis, k_eps_group<<<grid_for(n, 256), 256, 0, st>>>(fac_iter, cli_iter, n, o.first,
                                                                             reach[o.first], s->eps_r.as<double>(),
                                                                             s->eps_c.as<uint8_t>()));
         std::swap(s->radii, s->eps_r);
         std::swap(s->client, s->eps_c);
-        const int rc = open_facilities(s);
+        *queued = false;
+        int rc = queue ? open_facilities_queued(s, o.second, acc, outcome + i, queued) : FL_OK;
+        if (rc == FL_OK && !*queued) rc = open_facilities(s);
         std::swap(s->radii, s->eps_r);
         std::swap(s->client, s->eps_c);
         FL_TRY(rc);
-        FL_LAUNCH(kProfMis, k_eps_or<<<grid_for(n, 256), 256, 0, st>>>(s->open.as<uint8_t>(), n, acc));
+        if (!*queued)
+            FL_LAUNCH(kProfMis, k_eps_or<<<grid_for(n, 256), 256, 0, st>>>(s->open.as<uint8_t>(), n, acc));
+        return FL_OK;
+    };
+    std::vector<size_t> waiting;
+    for (size_t i = 0; i < groups.size(); ++i) {
+        const bool last = i + 1 == groups.size();
+        if (last && !waiting.empty()) {
+            std::vector<int> got(groups.size());
+            FL_CUDA(cudaMemcpyAsync(got.data(), outcome, (i + 1) * 4, cudaMemcpyDeviceToHost, st));
+            FL_CUDA(cudaStreamSynchronize(st));
+            bool unused;
+            for (size_t w : waiting)
+                if (got[w] != 1) FL_TRY(select(w, false, &unused));
+        }
+        bool queued = false;
+        FL_TRY(select(i, !last, &queued));
+        if (queued) waiting.push_back(i);
     }
     FL_CUDA(cudaGetLastError());
     return finish();

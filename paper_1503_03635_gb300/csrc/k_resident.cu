@@ -44,6 +44,7 @@ struct Ctl {
     unsigned tmax[2];                 // largest ball radius of the undecided, by round parity
     unsigned hist[2][kMaxBall + 1];   // undecided facilities by ball radius, by round parity
     long long rounds, n_u, n_open, log_n;
+    long long done;                   // 1: the launch ran to its end
 };
 
 struct ItemGraph {
@@ -413,6 +414,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_mis_resident(MisArgs a) {
         c->rounds = rounds;
         c->n_u = n_u;
         c->log_n = min(log_n, a.log_cap);
+        c->done = 1;
     }
 }
 
@@ -542,24 +544,22 @@ static ItemGraph item_graph(const fl_graph* g) {
     return ig;
 }
 
-// The greedy MIS of the m sorted candidates (s->ord, s->fac_by_ord, s->bcap,
-// s->state set) and its open list.  *done = false: not for this kernel (a
-// ball radius above kMaxBall); nothing but scratch was written.
-int mis_resident(fl_solve* s, int64_t m, bool* done) {
+constexpr size_t kCtlBytes = (sizeof(Ctl) + 255) & ~(size_t)255;
+
+// Arguments of the greedy MIS of the m sorted candidates (s->ord,
+// s->fac_by_ord, s->bcap, s->state set), its scratch and a cleared control block.
+static int mis_args(fl_solve* s, int64_t m, MisArgs* out, int* blocks) {
     fl_graph* g = s->g;
     const int64_t n = g->n;
-    cudaStream_t st = g->stream;
-    *done = false;
+    MisArgs& a = *out;
     FL_TRY(dalloc(s->X, (size_t)n * 16));
     FL_TRY(dalloc(s->frval, (size_t)n * 8 + 64));
     FL_TRY(dalloc(s->fr[0], (size_t)n * 4));
     FL_TRY(dalloc(s->claimed, (size_t)n));
     FL_TRY(dalloc(s->rlist, (size_t)g->n_items * 32));
-    const size_t ctl_b = (sizeof(Ctl) + 255) & ~(size_t)255;
     // a greedy round logs at most its buckets, three sweeps and a total
     const long long log_cap = (long long)kRoundsPerLaunch * (4LL * kMaxBall + 8);
-    FL_TRY(dalloc(s->rctl, ctl_b + (size_t)log_cap * 48));
-    MisArgs a;
+    FL_TRY(dalloc(s->rctl, kCtlBytes + (size_t)log_cap * 48));
     a.g = item_graph(g);
     a.items = g->items.as<int4>();
     a.n_items = g->n_items;
@@ -580,21 +580,64 @@ int mis_resident(fl_solve* s, int64_t m, bool* done) {
     a.open = s->open.as<uint8_t>();
     a.open_list = s->ulist.as<int32_t>();
     a.c = s->rctl.as<Ctl>();
-    a.log = reinterpret_cast<long long*>(s->rctl.as<char>() + ctl_b);
+    a.log = reinterpret_cast<long long*>(s->rctl.as<char>() + kCtlBytes);
     a.log_cap = log_cap;
     a.m = m;
     a.resume = 0;
+    FL_TRY(resident_blocks(g->n_items, blocks));
+    FL_CUDA(cudaMemsetAsync(s->rctl.p, 0, sizeof(Ctl), g->stream));
+    return FL_OK;
+}
+
+static cudaError_t mis_launch(const MisArgs& a, int blocks, cudaStream_t st) {
+    void* args[] = {const_cast<MisArgs*>(&a)};
+    return cudaLaunchCooperativeKernel((const void*)k_mis_resident, dim3(blocks), dim3(kResThreads), args, 0, st);
+}
+
+// A finished selection's open set into acc; *outcome = 1 when it finished (in
+// one launch, without an error), else 0 and acc is left alone.
+__global__ void k_mis_take(const Ctl* __restrict__ c, const uint8_t* __restrict__ open, int64_t n,
+                           uint8_t* __restrict__ acc, int* __restrict__ outcome) {
+    const bool done = c->done != 0 && c->n_u == 0 && c->bar.err == 0;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (tid == 0) *outcome = done ? 1 : 0;
+    if (!done) return;
+    for (int64_t v = tid; v < n; v += stride)
+        if (open[v]) acc[v] = 1;
+}
+
+// One launch of the greedy MIS and k_mis_take behind it, without a look by the host.
+int mis_resident_queue(fl_solve* s, int64_t m, uint8_t* acc, int* outcome) {
+    cudaStream_t st = s->g->stream;
+    MisArgs a;
     int blocks = 0;
-    FL_TRY(resident_blocks(g->n_items, &blocks));
-    FL_CUDA(cudaMemsetAsync(s->rctl.p, 0, sizeof(Ctl), st));
+    FL_TRY(mis_args(s, m, &a, &blocks));
+    cudaError_t le = cudaSuccess;
+    FL_LAUNCH(kProfMis, le = mis_launch(a, blocks, st));
+    FL_CUDA(le);
+    FL_LAUNCH(kProfMis, k_mis_take<<<(unsigned)std::min<int64_t>((s->g->n + 255) / 256, 152 * 4), 256, 0, st>>>(
+                            a.c, a.open, s->g->n, acc, outcome));
+    FL_CUDA(cudaGetLastError());
+    return FL_OK;
+}
+
+// The greedy MIS of the m sorted candidates and its open list.  *done = false:
+// not for this kernel (a ball radius above kMaxBall); nothing but scratch was
+// written.
+int mis_resident(fl_solve* s, int64_t m, bool* done) {
+    fl_graph* g = s->g;
+    cudaStream_t st = g->stream;
+    *done = false;
+    MisArgs a;
+    int blocks = 0;
+    FL_TRY(mis_args(s, m, &a, &blocks));
     char* h = reinterpret_cast<char*>(g->h_ctr) + sizeof(Counters);  // pinned
-    const size_t h_b = ctl_b + kFastRows * 48;
-    static_assert(sizeof(Counters) + ((sizeof(Ctl) + 255) & ~(size_t)255) + kFastRows * 48 <= kPinnedBytes, "pinned block");
+    const size_t h_b = kCtlBytes + kFastRows * 48;
+    static_assert(sizeof(Counters) + kCtlBytes + kFastRows * 48 <= kPinnedBytes, "pinned block");
     for (;;) {
-        void* args[] = {&a};
         cudaError_t le = cudaSuccess;
-        FL_LAUNCH(kProfMis, le = cudaLaunchCooperativeKernel((const void*)k_mis_resident, dim3(blocks),
-                                                             dim3(kResThreads), args, 0, st));
+        FL_LAUNCH(kProfMis, le = mis_launch(a, blocks, st));
         FL_CUDA(le);
         FL_CUDA(cudaMemcpyAsync(h, s->rctl.p, h_b, cudaMemcpyDeviceToHost, st));
         FL_CUDA(cudaStreamSynchronize(st));
@@ -605,7 +648,7 @@ int mis_resident(fl_solve* s, int64_t m, bool* done) {
         const size_t at = s->mis_log.size(), rows = (size_t)c->log_n;
         s->mis_log.resize(at + rows * 6);
         if (rows <= (size_t)kFastRows) {
-            std::copy_n(reinterpret_cast<const int64_t*>(h + ctl_b), rows * 6, s->mis_log.begin() + at);
+            std::copy_n(reinterpret_cast<const int64_t*>(h + kCtlBytes), rows * 6, s->mis_log.begin() + at);
         } else {
             FL_CUDA(cudaMemcpyAsync(s->mis_log.data() + at, a.log, rows * 48, cudaMemcpyDeviceToHost, st));
             FL_CUDA(cudaStreamSynchronize(st));

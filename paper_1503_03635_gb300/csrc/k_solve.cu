@@ -939,7 +939,10 @@ __global__ void k_open_list(const uint8_t* __restrict__ state, int64_t n, uint8_
 // length: then the top half of pi_f is sorted first and r_f by all its varying
 // bits after it (each pass keeps the order of the one before), and again the
 // runs that are left are put in order.
-int sort_candidates(fl_solve* s, int64_t* m_out, const uint32_t** sorted) {
+//
+// known: the number of candidates when the caller has it (else -1); a few known
+// ones are ordered without a look by the host.
+int sort_candidates(fl_solve* s, int64_t* m_out, const uint32_t** sorted, int64_t known) {
     fl_graph* g = s->g;
     const int64_t n = g->n;
     cudaStream_t st = g->stream;
@@ -959,8 +962,9 @@ int sort_candidates(fl_solve* s, int64_t* m_out, const uint32_t** sorted) {
     FL_LAUNCH(kProfKeys, k_candidates<<<grid_for(n, 256), 256, 0, st>>>(s->radii.as<double>(), n, g->seed, ids,
                                                    p.key[0], s->key_lo.as<uint64_t>(), p.val[0],
                                                    s->state.as<uint8_t>(), ctr));
-    FL_TRY(read_counters(g));
-    const int64_t m = (int64_t)g->h_ctr->aux0;
+    const bool told = known >= 0 && known <= kRankMax;
+    if (!told) FL_TRY(read_counters(g));
+    const int64_t m = told ? known : (int64_t)g->h_ctr->aux0;
     s->n_cand = m;
     *m_out = m;
     *sorted = p.val[0];
@@ -1017,11 +1021,16 @@ int sort_candidates(fl_solve* s, int64_t* m_out, const uint32_t** sorted) {
     return FL_OK;
 }
 
-int open_facilities(fl_solve* s) {
+// Keys: candidates sorted by (r_f, pi_f) -> ordinals, ball radii and the list
+// of the undecided (s->ulist).  cnt = the counters behind s->frval, cleared:
+// cnt[0], cnt[1] frontier counts; cnt[2] changed count (dense rounds); cnt[3]
+// undecided; cnt[4] largest ball radius; cnt[5] open list; cnt[6] touched.
+// All scratch is solve-owned and grow-only: a cudaFree per solve would
+// synchronise the whole device (and stall other solves on other streams).
+static int candidate_keys(fl_solve* s, int64_t known, int64_t* m, unsigned long long** cnt) {
     fl_graph* g = s->g;
     const int64_t n = g->n;
     cudaStream_t st = g->stream;
-    // -------- keys: candidates sorted by (r_f, pi_f) -> ordinals
     FL_TRY(dalloc(s->ord, (size_t)n * 4));
     FL_TRY(dalloc(s->fac_by_ord, (size_t)n * 4));
     FL_TRY(dalloc(s->bcap, (size_t)n * 4));
@@ -1030,23 +1039,43 @@ int open_facilities(fl_solve* s) {
     FL_TRY(dalloc(s->ulist, (size_t)n * 4 * 2));
     FL_TRY(dalloc(s->open, (size_t)n));
     s->mis_log.clear();
-    unsigned long long* cnt = reinterpret_cast<unsigned long long*>(s->frval.as<char>() + (size_t)n * 8);
-    // cnt[0], cnt[1]: frontier counts; cnt[2]: changed count (dense rounds);
-    // cnt[3]: undecided; cnt[4]: T max; cnt[5]: open list; cnt[6]: touched
-    // solve-owned, grow-only scratch: a cudaFree per solve would synchronise
-    // the whole device (and stall other solves running on other streams)
-    int64_t m = 0;
+    *cnt = reinterpret_cast<unsigned long long*>(s->frval.as<char>() + (size_t)n * 8);
     const uint32_t* sorted = nullptr;
-    FL_TRY(sort_candidates(s, &m, &sorted));
-    int32_t* ulist[2] = {s->ulist.as<int32_t>(), s->ulist.as<int32_t>() + n};
-    FL_CUDA(cudaMemsetAsync(cnt, 0, 64, st));
-    if (m > 0) {
-        FL_LAUNCH(kProfKeys, k_ordinals<<<grid_for(m, 256), 256, 0, st>>>(sorted, m, s->radii.as<double>(),
-                                                     g->ecc_ub.as<int32_t>(), s->ord.as<uint32_t>(),
-                                                     s->fac_by_ord.as<int32_t>(), s->bcap.as<int32_t>(), ulist[0],
-                                                     &cnt[4]));
+    FL_TRY(sort_candidates(s, m, &sorted, known));
+    FL_CUDA(cudaMemsetAsync(*cnt, 0, 64, st));
+    if (*m > 0) {
+        FL_LAUNCH(kProfKeys, k_ordinals<<<grid_for(*m, 256), 256, 0, st>>>(
+                                 sorted, *m, s->radii.as<double>(), g->ecc_ub.as<int32_t>(), s->ord.as<uint32_t>(),
+                                 s->fac_by_ord.as<int32_t>(), s->bcap.as<int32_t>(), s->ulist.as<int32_t>(),
+                                 &(*cnt)[4]));
     }
     FL_CUDA(cudaGetLastError());
+    return FL_OK;
+}
+
+// The selection of `known` candidates on a graph with work items, queued
+// without a look by the host: its open set goes into acc (uint8, OR) and its
+// outcome into *outcome when the device gets there (mis_resident_queue).
+// *queued = false: not for this path.
+int open_facilities_queued(fl_solve* s, int64_t known, uint8_t* acc, int* outcome, bool* queued) {
+    *queued = false;
+    if (!s->g->lists_ready || s->g->n_items == 0 || known > kRankMax) return FL_OK;
+    int64_t m = 0;
+    unsigned long long* cnt = nullptr;
+    FL_TRY(candidate_keys(s, known, &m, &cnt));
+    FL_TRY(mis_resident_queue(s, m, acc, outcome));
+    *queued = true;
+    return FL_OK;
+}
+
+int open_facilities(fl_solve* s) {
+    fl_graph* g = s->g;
+    const int64_t n = g->n;
+    cudaStream_t st = g->stream;
+    int64_t m = 0;
+    unsigned long long* cnt = nullptr;
+    FL_TRY(candidate_keys(s, -1, &m, &cnt));
+    int32_t* ulist[2] = {s->ulist.as<int32_t>(), s->ulist.as<int32_t>() + n};
     if (!g->lists_ready) {
         FL_TRY(build_work_lists(g));
         g->lists_ready = 1;
