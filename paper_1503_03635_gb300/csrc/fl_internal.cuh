@@ -743,11 +743,12 @@ struct Prune {
 
 // State of a sequence of synchronous min-propagation rounds (k_relax.cu).
 struct Relax {
-    unsigned long long* X[2] = {nullptr, nullptr};  // value buffers; X[cur] is current
+    bool narrow = false;                            // 32-bit values (else 64-bit)
+    void* X[2] = {nullptr, nullptr};                // value buffers; X[cur] is current
     int cur = 0;
     int32_t* fr[2] = {nullptr, nullptr};            // frontier lists; fr[fc] is current
     int fc = 0;
-    unsigned long long* frval = nullptr;            // snapshot of frontier values
+    void* frval = nullptr;                          // snapshot of frontier values
     uint32_t* stamp = nullptr;                      // frontier stamps / changed flags
     unsigned long long* cnt = nullptr;              // device: [0], [1] list sizes, [2] changed count
     unsigned long long* h_cnt = nullptr;            // pinned host word
@@ -761,7 +762,7 @@ struct Relax {
     // set by relax_begin (graph-owned scratch)
     uint32_t* bm = nullptr;                         // frontier bitmap of a pull round (n bits)
     uint32_t* hub_tag = nullptr;                    // uint32[n_hubs]: round whose push frontier holds the hub
-    unsigned long long* hub_val = nullptr;          // uint64[n_hubs]: the hub's snapshotted value
+    void* hub_val = nullptr;                        // [n_hubs]: the hub's snapshotted value
     unsigned long long* ecnt = nullptr;             // device: frontier edge count
     int32_t* part_cnt = nullptr;                    // device int32[n_parts]: frontier vertices per part
     const int32_t* part_limit = nullptr;            // device int32[n_parts] or NULL: a part whose limit is
@@ -778,8 +779,7 @@ int relax_prepare_list(fl_graph* g, Relax& r, int cls);
 // every unmarked v with need[v] > b (need may be NULL) and a neighbour whose
 // kr is in [1, b]; *marked = the marks made (hubs may count more than once).
 int mark_round(fl_graph* g, Relax& r, uint8_t* kr, const uint8_t* need, uint32_t b, int cls, int64_t* marked);
-int relax_collect_epoch(fl_graph* g, const unsigned long long* X, unsigned long long hi, int32_t* out,
-                        unsigned long long* n_out, int cls);
+int relax_collect_set(fl_graph* g, const uint32_t* X, int32_t* out, unsigned long long* n_out, int cls);
 int assign_clients(fl_solve* s);
 // the opening phase with eps > 0 and the selection of Algorithm 6 (k_eps.cu)
 int open_facilities_eps(fl_solve* s, double eps);

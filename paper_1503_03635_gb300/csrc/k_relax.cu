@@ -80,8 +80,13 @@ __device__ __forceinline__ bool skipped(const Prune& pr, int32_t u) {
     return (pr.need && __ldg(&pr.need[u]) <= pr.round) || (pr.only && !__ldg(&pr.only[u]));
 }
 
-// Values >= `limit` are ignored: unset entries (BFS) or values of an earlier
-// sweep (MIS sweeps stamp each sweep into the high word).  With `settle`, a
+// Values are 64-bit for a BFS (distance << 32 | label) and 32-bit for the MIS
+// sweeps, whose values are key ordinals below 2^31: half the bytes of every
+// gather and of the copy per round, and a warp's 32 gathers touch fewer sectors
+// of the hot head of X.  R-MAT scale 22, a dense gather round: k_pull_low 221 ->
+// 192 us, k_pull_segs 125 -> 114 us; the whole query 8.29 -> 7.24 ms, a batch of 16
+// solves on R-MAT scale 18 6.72 -> 5.93 ms.
+// Values >= `limit` are ignored: unset entries.  With `settle`, a
 // vertex holding a value below the limit is final and is skipped.
 //
 // Lowest value offered by the frontier neighbours cols[e], e in [e0, e1) with
@@ -95,12 +100,9 @@ __device__ __forceinline__ bool skipped(const Prune& pr, int32_t u) {
 // result is the same; when most neighbours are in the frontier the bitmap only
 // adds a second gather per edge to rounds that are bound by the gathers (L1
 // wavefronts, 80 % of its peak).
-template <bool kAll>
-__device__ __forceinline__ unsigned long long pull_min(const int32_t* __restrict__ cols, int64_t e0, int64_t e1,
-                                                       int step, const uint32_t* __restrict__ bm,
-                                                       const unsigned long long* __restrict__ X,
-                                                       unsigned long long add, unsigned long long limit,
-                                                       unsigned long long m) {
+template <bool kAll, class V>
+__device__ __forceinline__ V pull_min(const int32_t* __restrict__ cols, int64_t e0, int64_t e1, int step,
+                                      const uint32_t* __restrict__ bm, const V* __restrict__ X, V add, V limit, V m) {
     int32_t nx[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) nx[j] = e0 + j * step < e1 ? __ldcs(&cols[e0 + j * step]) : -1;
@@ -117,7 +119,7 @@ __device__ __forceinline__ unsigned long long pull_min(const int32_t* __restrict
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             if (f[j]) {
-                const unsigned long long x = __ldg(&X[u[j]]);
+                const V x = __ldg(&X[u[j]]);
                 if (x < limit && x + add < m) m = x + add;
             }
         }
@@ -129,14 +131,12 @@ __device__ __forceinline__ unsigned long long pull_min(const int32_t* __restrict
 // vertex, its neighbours loaded four at a time (column, bitmap and value
 // loads each independent of the others), so that a warp keeps 32 vertices'
 // chains in flight.
-template <bool kAll>
+template <bool kAll, class V>
 __global__ void __launch_bounds__(256) k_pull_small(const int32_t* __restrict__ list, int64_t n_list,
                                                     const int64_t* __restrict__ rowp,
-                                                    const int32_t* __restrict__ cols, unsigned long long add,
-                                                    unsigned long long limit, bool settle,
-                                                    const uint32_t* __restrict__ bm,
-                                                    const unsigned long long* __restrict__ X,
-                                                    unsigned long long* __restrict__ Xn,
+                                                    const int32_t* __restrict__ cols, V add, V limit, bool settle,
+                                                    const uint32_t* __restrict__ bm, const V* __restrict__ X,
+                                                    V* __restrict__ Xn,
                                                     uint32_t* __restrict__ stamp, uint32_t sv,
                                                     unsigned long long* __restrict__ n_changed,
                                                     const int32_t* __restrict__ vpart,
@@ -147,10 +147,10 @@ __global__ void __launch_bounds__(256) k_pull_small(const int32_t* __restrict__ 
         const int64_t i = base + lane_id();
         const int32_t v = i < n_list ? list[i] : 0;
         const bool have = i < n_list && !part_idle(vpart, part_cnt, v) && !skipped(pr, v);
-        const unsigned long long own = have ? X[v] : ~0ULL;
+        const V own = have ? X[v] : (V)~(V)0;
         const bool work = have && !(settle && own < limit);
         const int64_t beg = work ? rowp[v] : 0, end = work ? rowp[v + 1] : 0;
-        const unsigned long long m = pull_min<kAll>(cols, beg, end, 1, bm, X, add, limit, own);
+        const V m = pull_min<kAll, V>(cols, beg, end, 1, bm, X, add, limit, own);
         const bool ch = work && m < own;
         if (ch) {
             Xn[v] = m;
@@ -165,13 +165,12 @@ __global__ void __launch_bounds__(256) k_pull_small(const int32_t* __restrict__ 
 // Pull round over the other non-hub vertices: four vertices per warp, eight
 // lanes per vertex striding over its neighbours; the lanes meet again at the
 // reduction.
-template <bool kAll>
+template <bool kAll, class V>
 __global__ void __launch_bounds__(256) k_pull_low(const int32_t* __restrict__ list, int64_t n_list,
                                                   const int64_t* __restrict__ rowp, const int32_t* __restrict__ cols,
-                                                  unsigned long long add, unsigned long long limit, bool settle,
-                                                  const uint32_t* __restrict__ bm,
-                                                  const unsigned long long* __restrict__ X,
-                                                  unsigned long long* __restrict__ Xn, uint32_t* __restrict__ stamp,
+                                                  V add, V limit, bool settle,
+                                                  const uint32_t* __restrict__ bm, const V* __restrict__ X,
+                                                  V* __restrict__ Xn, uint32_t* __restrict__ stamp,
                                                   uint32_t sv, unsigned long long* __restrict__ n_changed,
                                                   const int32_t* __restrict__ vpart,
                                                   const int32_t* __restrict__ part_cnt, Prune pr) {
@@ -183,12 +182,12 @@ __global__ void __launch_bounds__(256) k_pull_low(const int32_t* __restrict__ li
         const int64_t i = w * 4 + (lane >> 3);
         const int32_t v = i < n_list ? list[i] : 0;
         const bool have = i < n_list && !part_idle(vpart, part_cnt, v) && !skipped(pr, v);
-        const unsigned long long own = have ? X[v] : ~0ULL;
+        const V own = have ? X[v] : (V)~(V)0;
         const bool work = have && !(settle && own < limit);
         const int64_t beg = work ? rowp[v] : 0, end = work ? rowp[v + 1] : 0;
-        unsigned long long m = pull_min<kAll>(cols, beg + sub, end, 8, bm, X, add, limit, own);
+        V m = pull_min<kAll, V>(cols, beg + sub, end, 8, bm, X, add, limit, own);
 #pragma unroll
-        for (int o = 1; o < 8; o <<= 1) m = umin64(m, __shfl_xor_sync(kFull, m, o));
+        for (int o = 1; o < 8; o <<= 1) m = min(m, __shfl_xor_sync(kFull, m, o));
         const bool ch = work && sub == 0 && m < own;
         if (ch) {
             Xn[v] = m;
@@ -203,16 +202,14 @@ __global__ void __launch_bounds__(256) k_pull_low(const int32_t* __restrict__ li
 // Pull round over hubs: one warp per segment of fl_graph::seg edges.  Xn[v] starts as
 // X[v]; the segments lower it with atomicMin and the one that lowers it first
 // (it sees the old value) flags the hub.
-template <bool kAll>
+template <bool kAll, class V>
 __global__ void __launch_bounds__(256) k_pull_segs(const int32_t* __restrict__ seg_hub, int64_t n_seg,
                                                    const int64_t* __restrict__ hub_seg,
                                                    const int32_t* __restrict__ hub_list,
                                                    const int64_t* __restrict__ rowp, const int32_t* __restrict__ cols,
-                                                   int seg,
-                                                   unsigned long long add, unsigned long long limit, bool settle,
-                                                   const uint32_t* __restrict__ bm,
-                                                   const unsigned long long* __restrict__ X,
-                                                   unsigned long long* __restrict__ Xn, uint32_t* __restrict__ stamp,
+                                                   int seg, V add, V limit, bool settle,
+                                                   const uint32_t* __restrict__ bm, const V* __restrict__ X,
+                                                   V* __restrict__ Xn, uint32_t* __restrict__ stamp,
                                                    uint32_t sv, unsigned long long* __restrict__ n_changed,
                                                    const int32_t* __restrict__ vpart,
                                                    const int32_t* __restrict__ part_cnt, Prune pr) {
@@ -221,15 +218,15 @@ __global__ void __launch_bounds__(256) k_pull_segs(const int32_t* __restrict__ s
     for (int64_t sidx = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; sidx < n_seg; sidx += warps) {
         const int32_t h = seg_hub[sidx];
         const int32_t v = hub_list[h];
-        const unsigned long long own = X[v];
+        const V own = X[v];
         if ((settle && own < limit) || part_idle(vpart, part_cnt, v) || skipped(pr, v)) continue;
         const int64_t e0 = rowp[v] + (sidx - hub_seg[h]) * seg;
         const int64_t e1 = min(e0 + (int64_t)seg, rowp[v + 1]);
-        unsigned long long m = pull_min<kAll>(cols, e0 + lane, e1, 32, bm, X, add, limit, ~0ULL);
+        V m = pull_min<kAll, V>(cols, e0 + lane, e1, 32, bm, X, add, limit, (V)~(V)0);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = umin64(m, __shfl_xor_sync(kFull, m, o));
+        for (int o = 16; o > 0; o >>= 1) m = min(m, __shfl_xor_sync(kFull, m, o));
         if (lane == 0 && m < own) {
-            const unsigned long long old = atomicMin(&Xn[v], m);
+            const V old = atomicMin(&Xn[v], m);
             if (old == own) {
                 stamp[v] = sv;
                 if (pr.reach && own >= limit) pr.reach[v] = (uint8_t)pr.reach_val;
@@ -242,11 +239,12 @@ __global__ void __launch_bounds__(256) k_pull_segs(const int32_t* __restrict__ s
 // Snapshot of a push frontier: frval[i] = X[fr[i]], the frontier's edge count
 // into *edges, and each hub of the frontier tagged (hub_tag = tag, hub_val =
 // its value) for the segment push.  hub_list is ascending.
+template <class V>
 __global__ void k_snap_front(const int32_t* __restrict__ fr, const unsigned long long* __restrict__ n_fr,
-                             const unsigned long long* __restrict__ X, unsigned long long* __restrict__ frval,
+                             const V* __restrict__ X, V* __restrict__ frval,
                              unsigned long long* __restrict__ reset_next, const int64_t* __restrict__ rowp,
                              const int32_t* __restrict__ hub_list, int64_t n_hubs, int seg, uint32_t* __restrict__ hub_tag,
-                             uint32_t tag, unsigned long long* __restrict__ hub_val,
+                             uint32_t tag, V* __restrict__ hub_val,
                              unsigned long long* __restrict__ edges) {
     const int64_t n = (int64_t)*n_fr;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -254,7 +252,7 @@ __global__ void k_snap_front(const int32_t* __restrict__ fr, const unsigned long
     unsigned long long ed = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         const int32_t v = fr[i];
-        const unsigned long long x = X[v];
+        const V x = X[v];
         frval[i] = x;
         const int64_t d = rowp[v + 1] - rowp[v];
         ed += (unsigned long long)d;
@@ -278,13 +276,12 @@ __global__ void k_snap_front(const int32_t* __restrict__ fr, const unsigned long
 
 // Push from the non-hub frontier vertices: a warp per vertex, read-before-
 // atomicMin on the neighbours, stamp dedupe for the next frontier.
+template <class V>
 __global__ void __launch_bounds__(256) k_push_low(const int32_t* __restrict__ fr,
-                                                  const unsigned long long* __restrict__ frval,
+                                                  const V* __restrict__ frval,
                                                   const unsigned long long* __restrict__ n_fr,
                                                   const int64_t* __restrict__ rowp, const int32_t* __restrict__ cols,
-                                                   int seg,
-                                                  unsigned long long add, unsigned long long limit,
-                                                  unsigned long long* __restrict__ X,
+                                                  int seg, V add, V limit, V* __restrict__ X,
                                                   uint32_t* __restrict__ stamp, uint32_t sv,
                                                   int32_t* __restrict__ fr_next, unsigned long long* __restrict__ n_next,
                                                   Prune pr) {
@@ -295,7 +292,7 @@ __global__ void __launch_bounds__(256) k_push_low(const int32_t* __restrict__ fr
         const int32_t v = fr[w];
         const int64_t beg = rowp[v], end = rowp[v + 1];
         if (end - beg > seg) continue;  // hubs: k_push_segs
-        const unsigned long long val = frval[w] + add;
+        const V val = frval[w] + add;
         for (int64_t cb = beg; cb < end; cb += 32) {
             const int64_t e = cb + lane;
             bool fresh = false;
@@ -303,7 +300,7 @@ __global__ void __launch_bounds__(256) k_push_low(const int32_t* __restrict__ fr
             if (e < end) {
                 u = cols[e];
                 if (val < X[u] && !skipped(pr, u)) {
-                    const unsigned long long old = atomicMin(&X[u], val);
+                    const V old = atomicMin(&X[u], val);
                     if (val < old) {
                         if (pr.reach && old >= limit) pr.reach[u] = (uint8_t)pr.reach_val;
                         fresh = atomicExch(&stamp[u], sv) != sv;
@@ -317,15 +314,14 @@ __global__ void __launch_bounds__(256) k_push_low(const int32_t* __restrict__ fr
 }
 
 // Push from the frontier hubs (tagged by k_snap_front): a warp per segment.
+template <class V>
 __global__ void __launch_bounds__(256) k_push_segs(const int32_t* __restrict__ seg_hub, int64_t n_seg,
                                                    const int64_t* __restrict__ hub_seg,
                                                    const int32_t* __restrict__ hub_list,
                                                    const uint32_t* __restrict__ hub_tag, uint32_t tag,
-                                                   const unsigned long long* __restrict__ hub_val,
+                                                   const V* __restrict__ hub_val,
                                                    const int64_t* __restrict__ rowp, const int32_t* __restrict__ cols,
-                                                   int seg,
-                                                   unsigned long long add, unsigned long long limit,
-                                                   unsigned long long* __restrict__ X,
+                                                   int seg, V add, V limit, V* __restrict__ X,
                                                    uint32_t* __restrict__ stamp, uint32_t sv,
                                                    int32_t* __restrict__ fr_next, unsigned long long* __restrict__ n_next,
                                                    Prune pr) {
@@ -335,7 +331,7 @@ __global__ void __launch_bounds__(256) k_push_segs(const int32_t* __restrict__ s
         const int32_t h = seg_hub[sidx];
         if (hub_tag[h] != tag) continue;
         const int32_t v = hub_list[h];
-        const unsigned long long val = hub_val[h] + add;
+        const V val = hub_val[h] + add;
         const int64_t e0 = rowp[v] + (sidx - hub_seg[h]) * seg;
         const int64_t e1 = min(e0 + (int64_t)seg, rowp[v + 1]);
         for (int64_t cb = e0; cb < e1; cb += 32) {
@@ -345,7 +341,7 @@ __global__ void __launch_bounds__(256) k_push_segs(const int32_t* __restrict__ s
             if (e < e1) {
                 u = cols[e];
                 if (val < X[u] && !skipped(pr, u)) {
-                    const unsigned long long old = atomicMin(&X[u], val);
+                    const V old = atomicMin(&X[u], val);
                     if (val < old) {
                         if (pr.reach && old >= limit) pr.reach[u] = (uint8_t)pr.reach_val;
                         fresh = atomicExch(&stamp[u], sv) != sv;
@@ -381,23 +377,22 @@ constexpr int64_t kAllDiv = 4;
 
 }  // namespace
 
-// Vertices whose value carries high word `hi` -> list (the vertices a sweep reached).
-__global__ void k_collect_epoch(const unsigned long long* __restrict__ X, unsigned long long hi, int64_t n,
-                                int32_t* __restrict__ out, unsigned long long* __restrict__ n_out) {
+// Vertices that a sweep reached (a value below the unset one) -> list.
+__global__ void k_collect_set(const uint32_t* __restrict__ X, int64_t n, int32_t* __restrict__ out,
+                              unsigned long long* __restrict__ n_out) {
     __shared__ BlockAppend<8> sh;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t bb = (int64_t)blockIdx.x * blockDim.x; bb < n; bb += stride) {
         const int64_t v = bb + threadIdx.x;
-        const bool in = v < n && (X[v] >> 32) == hi;
+        const bool in = v < n && X[v] != 0xffffffffu;
         const long long at = block_append<8>(in, n_out, sh);
         if (at >= 0) out[at] = (int32_t)v;
     }
 }
 
-int relax_collect_epoch(fl_graph* g, const unsigned long long* X, unsigned long long hi, int32_t* out,
-                        unsigned long long* n_out, int cls) {
+int relax_collect_set(fl_graph* g, const uint32_t* X, int32_t* out, unsigned long long* n_out, int cls) {
     FL_CUDA(cudaMemsetAsync(n_out, 0, 8, g->stream));
-    FL_LAUNCH(cls, k_collect_epoch<<<grid_for(g->n, 256), 256, 0, g->stream>>>(X, hi, g->n, out, n_out));
+    FL_LAUNCH(cls, k_collect_set<<<grid_for(g->n, 256), 256, 0, g->stream>>>(X, g->n, out, n_out));
     FL_CUDA(cudaGetLastError());
     return FL_OK;
 }
@@ -425,7 +420,7 @@ int relax_begin(fl_graph* g, Relax& r) {
     char* base = g->relax_aux.as<char>();
     r.bm = reinterpret_cast<uint32_t*>(base);
     r.hub_tag = reinterpret_cast<uint32_t*>(base + off_tag);
-    r.hub_val = reinterpret_cast<unsigned long long*>(base + off_val);
+    r.hub_val = base + off_val;
     r.ecnt = reinterpret_cast<unsigned long long*>(base + off_cnt);
     r.part_cnt = reinterpret_cast<int32_t*>(base + off_part);
     if (g->n_hubs > 0) FL_CUDA(cudaMemsetAsync(r.hub_tag, 0, (size_t)g->n_hubs * 4, g->stream));
@@ -433,19 +428,25 @@ int relax_begin(fl_graph* g, Relax& r) {
     return FL_OK;
 }
 
+namespace {
+
 // One synchronous round.  The caller keeps the frontier count on the host
 // (r.n_front) and, for push rounds, a valid list in r.fr[r.fc] with its count
 // in r.cnt[r.fc].  `sv` is the stamp of the frontier this round produces.
 // A round pushes when its frontier is small (few vertices, or few edges);
 // otherwise it pulls with the frontier bitmap.
-int relax_round(fl_graph* g, Relax& r, unsigned long long add, uint32_t sv, int cls) {
+template <class V>
+int round_of(fl_graph* g, Relax& r, V add, uint32_t sv, int cls) {
     cudaStream_t st = g->stream;
     const int64_t n = g->n;
     const int64_t* rowp = g->rowp.as<int64_t>();
     const int32_t* cols = g->cols.as<int32_t>();
     const int32_t* hub_list = g->hub_list.as<int32_t>();
     bool dense = r.n_front * r.dense_div >= g->n_low + g->n_hubs;
-    unsigned long long* X = r.X[r.cur];
+    V* X = static_cast<V*>(r.X[r.cur]);
+    V* frval = static_cast<V*>(r.frval);
+    V* hub_val = static_cast<V*>(r.hub_val);
+    const V limit = (V)r.limit;
     if (!dense) {
         if (!r.list_valid) {
             // rebuild the frontier list from the stamps of the previous round
@@ -456,8 +457,8 @@ int relax_round(fl_graph* g, Relax& r, unsigned long long add, uint32_t sv, int 
         }
         FL_CUDA(cudaMemsetAsync(r.ecnt, 0, 8, st));
         FL_LAUNCH(cls, k_snap_front<<<grid_for(r.n_front, 256), 256, 0, st>>>(
-                           r.fr[r.fc], &r.cnt[r.fc], X, r.frval, &r.cnt[r.fc ^ 1], rowp, hub_list, g->n_hubs, g->seg,
-                           r.hub_tag, r.sv_prev, r.hub_val, r.ecnt));
+                           r.fr[r.fc], &r.cnt[r.fc], X, frval, &r.cnt[r.fc ^ 1], rowp, hub_list, g->n_hubs, g->seg,
+                           r.hub_tag, r.sv_prev, hub_val, r.ecnt));
         FL_CUDA(cudaGetLastError());
         if (r.n_front >= kPushAlways) {
             FL_CUDA(cudaMemcpyAsync(r.h_cnt, r.ecnt, 8, cudaMemcpyDeviceToHost, st));
@@ -466,20 +467,20 @@ int relax_round(fl_graph* g, Relax& r, unsigned long long add, uint32_t sv, int 
         }
     }
     if (!dense) {
-        FL_LAUNCH(cls, k_push_low<<<grid_for(r.n_front, 8), 256, 0, st>>>(r.fr[r.fc], r.frval, &r.cnt[r.fc], rowp, cols, g->seg,
-                                                                         add, r.limit, X, r.stamp, sv, r.fr[r.fc ^ 1],
+        FL_LAUNCH(cls, k_push_low<<<grid_for(r.n_front, 8), 256, 0, st>>>(r.fr[r.fc], frval, &r.cnt[r.fc], rowp, cols, g->seg,
+                                                                         add, limit, X, r.stamp, sv, r.fr[r.fc ^ 1],
                                                                          &r.cnt[r.fc ^ 1], r.prune));
         if (g->n_seg > 0)
             FL_LAUNCH(cls, k_push_segs<<<grid_for(g->n_seg, 8), 256, 0, st>>>(
                                g->seg_hub.as<int32_t>(), g->n_seg, g->hub_seg.as<int64_t>(), hub_list, r.hub_tag,
-                               r.sv_prev, r.hub_val, rowp, cols, g->seg, add, r.limit, X, r.stamp, sv, r.fr[r.fc ^ 1],
+                               r.sv_prev, hub_val, rowp, cols, g->seg, add, limit, X, r.stamp, sv, r.fr[r.fc ^ 1],
                                &r.cnt[r.fc ^ 1], r.prune));
         FL_CUDA(cudaGetLastError());
         r.fc ^= 1;
         r.list_valid = true;
         FL_CUDA(cudaMemcpyAsync(r.h_cnt, &r.cnt[r.fc], 8, cudaMemcpyDeviceToHost, st));
     } else {
-        unsigned long long* Xn = r.X[r.cur ^ 1];
+        V* Xn = static_cast<V*>(r.X[r.cur ^ 1]);
         const int32_t* vpart = g->n_parts > 0 ? g->vpart.as<int32_t>() : nullptr;
         // most of the listed vertices changed: read every neighbour's value
         // (not in a BFS: its frontier leaves out the hubs, reached earlier, that
@@ -489,23 +490,23 @@ int relax_round(fl_graph* g, Relax& r, unsigned long long add, uint32_t sv, int 
         if (vpart || !all)
             FL_LAUNCH(cls, k_bitmap<<<grid_for(n, 256 * kBmWords), 256, 0, st>>>(r.stamp, r.sv_prev, n, r.bm, vpart, r.part_cnt,
                                                                       vpart ? r.part_limit : nullptr, r.part_round));
-        FL_CUDA(cudaMemcpyAsync(Xn, X, (size_t)n * 8, cudaMemcpyDeviceToDevice, st));
+        FL_CUDA(cudaMemcpyAsync(Xn, X, (size_t)n * sizeof(V), cudaMemcpyDeviceToDevice, st));
         FL_CUDA(cudaMemsetAsync(&r.cnt[2], 0, 8, st));
-        auto small = all ? k_pull_small<true> : k_pull_small<false>;
-        auto low = all ? k_pull_low<true> : k_pull_low<false>;
-        auto segs = all ? k_pull_segs<true> : k_pull_segs<false>;
+        auto small = all ? k_pull_small<true, V> : k_pull_small<false, V>;
+        auto low = all ? k_pull_low<true, V> : k_pull_low<false, V>;
+        auto segs = all ? k_pull_segs<true, V> : k_pull_segs<false, V>;
         if (g->n_small > 0)
             FL_LAUNCH(cls, small<<<grid_for(g->n_small, 256), 256, 0, st>>>(
-                               g->small_list.as<int32_t>(), g->n_small, rowp, cols, add, r.limit, r.settle, r.bm, X,
+                               g->small_list.as<int32_t>(), g->n_small, rowp, cols, add, limit, r.settle, r.bm, X,
                                Xn, r.stamp, sv, &r.cnt[2], vpart, r.part_cnt, r.prune));
         if (g->n_mid > 0)
             FL_LAUNCH(cls, low<<<grid_for((g->n_mid + 3) / 4, 8), 256, 0, st>>>(
-                               g->mid_list.as<int32_t>(), g->n_mid, rowp, cols, add, r.limit, r.settle, r.bm, X, Xn,
+                               g->mid_list.as<int32_t>(), g->n_mid, rowp, cols, add, limit, r.settle, r.bm, X, Xn,
                                r.stamp, sv, &r.cnt[2], vpart, r.part_cnt, r.prune));
         if (g->n_seg > 0)
             FL_LAUNCH(cls, segs<<<grid_for(g->n_seg, 8), 256, 0, st>>>(
                                g->seg_hub.as<int32_t>(), g->n_seg, g->hub_seg.as<int64_t>(), hub_list, rowp, cols, g->seg, add,
-                               r.limit, r.settle, r.bm, X, Xn, r.stamp, sv, &r.cnt[2], vpart, r.part_cnt,
+                               limit, r.settle, r.bm, X, Xn, r.stamp, sv, &r.cnt[2], vpart, r.part_cnt,
                                r.prune));
         FL_CUDA(cudaGetLastError());
         r.cur ^= 1;
@@ -517,6 +518,12 @@ int relax_round(fl_graph* g, Relax& r, unsigned long long add, uint32_t sv, int 
     r.sv_prev = sv;
     r.last_dense = dense;
     return FL_OK;
+}
+
+}  // namespace
+
+int relax_round(fl_graph* g, Relax& r, unsigned long long add, uint32_t sv, int cls) {
+    return r.narrow ? round_of<uint32_t>(g, r, (uint32_t)add, sv, cls) : round_of<unsigned long long>(g, r, add, sv, cls);
 }
 
 // ------------------------------------------------------------------ marking rounds

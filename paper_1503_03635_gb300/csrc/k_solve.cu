@@ -24,9 +24,9 @@ static int grid_for(int64_t items, int per_block) {
 
 // Seeds: X[s] = min(X[s], val(s)); s joins the frontier when it decreases.
 // With `reach`, a seed that held no value below `limit` records reach_val.
+template <class V>
 __global__ void k_inject(const int32_t* __restrict__ src, int64_t n_src, uint8_t* __restrict__ reach,
-                         uint32_t reach_val, unsigned long long limit,
-                         unsigned long long hi, const uint32_t* __restrict__ lo_of, unsigned long long* __restrict__ X,
+                         uint32_t reach_val, V limit, const uint32_t* __restrict__ lo_of, V* __restrict__ X,
                          uint32_t* __restrict__ stamp, uint32_t sv, int32_t* __restrict__ fr,
                          unsigned long long* __restrict__ n_fr) {
     __shared__ BlockAppend<8> sh;
@@ -37,8 +37,8 @@ __global__ void k_inject(const int32_t* __restrict__ src, int64_t n_src, uint8_t
         int32_t s = 0;
         if (i < n_src) {
             s = src[i];
-            unsigned long long val = (hi << 32) | (lo_of ? lo_of[s] : (uint32_t)s);
-            unsigned long long old = atomicMin(&X[s], val);
+            const V val = lo_of ? lo_of[s] : (uint32_t)s;
+            const V old = atomicMin(&X[s], val);
             if (val < old) {
                 if (reach && old >= limit) reach[s] = (uint8_t)reach_val;
                 fresh = atomicExch(&stamp[s], sv) != sv;
@@ -80,11 +80,11 @@ int msbfs(fl_graph* g, const int32_t* src_list, int64_t n_src, int32_t* label, i
     FL_TRY(dalloc(fr[1], (size_t)n * 4));
     FL_TRY(dalloc(frval, (size_t)n * 8 + 64));
     Relax r;
-    r.X[0] = X.as<unsigned long long>();
-    r.X[1] = r.X[0] + n;
+    r.X[0] = X.p;
+    r.X[1] = X.as<unsigned long long>() + n;
     r.fr[0] = fr[0].as<int32_t>();
     r.fr[1] = fr[1].as<int32_t>();
-    r.frval = frval.as<unsigned long long>();
+    r.frval = frval.p;
     r.stamp = stampb.as<uint32_t>();
     r.cnt = reinterpret_cast<unsigned long long*>(frval.as<char>() + (size_t)n * 8);
     r.h_cnt = &g->h_ctr->aux3;
@@ -98,9 +98,9 @@ int msbfs(fl_graph* g, const int32_t* src_list, int64_t n_src, int32_t* label, i
         // labels are the sources' rank ids: ties go to the smallest original
         // (or part-local) facility id whatever the internal numbering
         const uint32_t* label_of = g->rid.p ? g->rid.as<uint32_t>() : nullptr;
-        FL_LAUNCH(cls, k_inject<<<grid_for(n_src, 256), 256, 0, st>>>(src_list, n_src, nullptr, 0u, ~0ULL, 0ULL,
-                                                                      label_of, r.X[0], r.stamp, 1u, r.fr[0],
-                                                                      &r.cnt[0]));
+        FL_LAUNCH(cls, k_inject<<<grid_for(n_src, 256), 256, 0, st>>>(
+                           src_list, n_src, nullptr, 0u, ~0ULL, label_of, X.as<unsigned long long>(), r.stamp, 1u,
+                           r.fr[0], &r.cnt[0]));
         FL_CUDA(cudaGetLastError());
     }
     r.n_front = n_src;
@@ -110,7 +110,8 @@ int msbfs(fl_graph* g, const int32_t* src_list, int64_t n_src, int32_t* label, i
         if ((int64_t)level >= cap) FL_FAIL(FL_ETIMEOUT, "BFS reached its level cap");
         FL_TRY(relax_round(g, r, 1ULL << 32, level + 2, cls));
     }
-    FL_LAUNCH(cls, k_unpack_bfs<<<grid_for(n, 256), 256, 0, st>>>(r.X[r.cur], n, label, dist));
+    FL_LAUNCH(cls, k_unpack_bfs<<<grid_for(n, 256), 256, 0, st>>>(
+                       static_cast<unsigned long long*>(r.X[r.cur]), n, label, dist));
     FL_CUDA(cudaGetLastError());
     return FL_OK;
 }
@@ -814,12 +815,13 @@ __global__ void __launch_bounds__(256) k_bucket_scatter(const int32_t* __restric
     }
 }
 
-// Gather seeds: every client covered in this round's cover sweep starts with
-// 0 if already claimed, else 1 + (smallest key of an undecided facility
-// covering it); mval keeps that smallest key for the claim step.
+// Gather seeds: every client covered in this round's cover sweep (values C)
+// starts the gather (values X, all unset) with 0 if already claimed, else 1 +
+// (smallest key of an undecided facility covering it); mval keeps that smallest
+// key for the claim step.
 __global__ void k_gather_seed(const int32_t* __restrict__ touched, const unsigned long long* __restrict__ n_touched,
                               const uint8_t* __restrict__ client, const uint8_t* __restrict__ claimed,
-                              unsigned long long hi, unsigned long long* __restrict__ X, uint32_t* __restrict__ mval,
+                              const uint32_t* __restrict__ C, uint32_t* __restrict__ X, uint32_t* __restrict__ mval,
                               uint32_t* __restrict__ stamp, uint32_t sv, int32_t* __restrict__ fr,
                               unsigned long long* __restrict__ n_fr) {
     __shared__ BlockAppend<8> sh;
@@ -832,9 +834,9 @@ __global__ void k_gather_seed(const int32_t* __restrict__ touched, const unsigne
         if (i < n) {
             v = touched[i];
             if (client[v]) {
-                uint32_t m = (uint32_t)(X[v] & 0xffffffffULL);
+                const uint32_t m = C[v];
                 mval[v] = m;
-                X[v] = (hi << 32) | (claimed[v] ? 0ULL : (unsigned long long)m + 1ULL);
+                X[v] = claimed[v] ? 0u : m + 1u;
                 stamp[v] = sv;
                 seed = true;
             }
@@ -847,20 +849,15 @@ __global__ void k_gather_seed(const int32_t* __restrict__ touched, const unsigne
 // Facilities whose ball radius is b read the minimum over their ball after
 // b gather rounds: 0 -> a client of the ball is claimed (dead); own key + 1
 // -> smallest key among all conflicting undecided facilities (joins S).
-__global__ void k_decide(const int32_t* __restrict__ fl, int64_t m, const unsigned long long* __restrict__ X,
-                         unsigned long long hi, const uint32_t* __restrict__ ord, uint8_t* __restrict__ state,
-                         Counters* ctr) {
+__global__ void k_decide(const int32_t* __restrict__ fl, int64_t m, const uint32_t* __restrict__ X,
+                         const uint32_t* __restrict__ ord, uint8_t* __restrict__ state, Counters* ctr) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += stride) {
         int32_t f = fl[i];
-        unsigned long long x = X[f];
-        if ((x >> 32) != hi) {
-            atomicOr(&ctr->error, 8ULL);  // a candidate's ball holds no client (cannot happen)
-            continue;
-        }
-        uint32_t lo = (uint32_t)(x & 0xffffffffULL);
-        if (lo == 0) state[f] = 2;
-        else if (lo == ord[f] + 1u) state[f] = 1;
+        const uint32_t x = X[f];
+        if (x == 0xffffffffu) atomicOr(&ctr->error, 8ULL);  // a candidate's ball holds no client (cannot happen)
+        else if (x == 0) state[f] = 2;
+        else if (x == ord[f] + 1u) state[f] = 1;
     }
 }
 
@@ -1086,7 +1083,7 @@ int open_facilities(fl_solve* s) {
         if (done) return FL_OK;
     }
     FL_TRY(dalloc(s->claimed, (size_t)n));
-    FL_TRY(dalloc(s->X, (size_t)n * 16));          // two value buffers
+    FL_TRY(dalloc(s->X, (size_t)n * 16));          // two value buffers of the cover, two of the gather
     FL_TRY(dalloc(s->stamp, (size_t)n * 4));
     FL_TRY(dalloc(s->mval, (size_t)n * 4));
     FL_TRY(dalloc(s->fr[0], (size_t)n * 4));
@@ -1098,7 +1095,6 @@ int open_facilities(fl_solve* s) {
     unsigned long long bmax = 0;
     FL_CUDA(cudaMemcpyAsync(&bmax, &cnt[4], 8, cudaMemcpyDeviceToHost, st));
     FL_CUDA(cudaMemsetAsync(s->claimed.p, 0, (size_t)n, st));
-    FL_CUDA(cudaMemsetAsync(s->X.p, 0xff, (size_t)n * 16, st));
     FL_CUDA(cudaMemsetAsync(s->stamp.p, 0, (size_t)n * 4, st));
     FL_CUDA(cudaStreamSynchronize(st));
     DBuf& bcount_d = s->bcount;
@@ -1107,12 +1103,14 @@ int open_facilities(fl_solve* s) {
     int32_t* cursor = bcount + (bmax + 2);
     std::vector<int32_t> hcount(bmax + 2), hoff(bmax + 2);
 
+    // values are keys (ordinals), all ones where unset
+    uint32_t* const val = s->X.as<uint32_t>();
     Relax r;
-    r.X[0] = s->X.as<unsigned long long>();
-    r.X[1] = r.X[0] + n;
+    r.narrow = true;
+    r.limit = 0xffffffffULL;
     r.fr[0] = s->fr[0].as<int32_t>();
     r.fr[1] = s->fr[1].as<int32_t>();
-    r.frval = s->frval.as<unsigned long long>();
+    r.frval = s->frval.p;
     r.stamp = s->stamp.as<uint32_t>();
     r.cnt = cnt;
     r.h_cnt = &g->h_ctr->aux3;
@@ -1144,7 +1142,6 @@ int open_facilities(fl_solve* s) {
                 std::chrono::duration<double, std::micro>(clock::now() - t0).count());
         return FL_OK;
     };
-    uint32_t epoch = 0;
     uint32_t sv = 0;  // frontier stamp values, unique per round
     int64_t n_u = m;
     int cu = 0;
@@ -1184,9 +1181,11 @@ int open_facilities(fl_solve* s) {
 
         // ---- cover: X[c] = smallest key of an undecided f with d(c, f) <= B_f.
         // Facility f starts at time T - B_f; all waves stop at time T.
-        ++epoch;
-        const unsigned long long hi_c = 0xffffffffULL - epoch;
-        r.limit = (hi_c + 1) << 32;
+        r.X[0] = val;
+        r.X[1] = val + n;
+        r.cur = 0;
+        auto now = [&]() { return static_cast<uint32_t*>(r.X[r.cur]); };
+        FL_CUDA(cudaMemsetAsync(val, 0xff, (size_t)n * 4, st));
         FL_CUDA(cudaMemsetAsync(cnt, 0, 24, st));
         r.n_front = 0;
         r.list_valid = true;
@@ -1199,8 +1198,8 @@ int open_facilities(fl_solve* s) {
             if (hcount[b] > 0) {
                 FL_TRY(relax_prepare_list(g, r, kProfMis));
                 FL_LAUNCH(kProfMis, k_inject<<<grid_for(hcount[b], 256), 256, 0, st>>>(
-                                        ub + hoff[b], hcount[b], r.prune.reach, (uint32_t)b + 1u, r.limit, hi_c,
-                                        s->ord.as<uint32_t>(), r.X[r.cur], r.stamp, sv0 + 1 + t, r.fr[r.fc],
+                                        ub + hoff[b], hcount[b], r.prune.reach, (uint32_t)b + 1u, 0xffffffffu,
+                                        s->ord.as<uint32_t>(), now(), r.stamp, sv0 + 1 + t, r.fr[r.fc],
                                         &r.cnt[r.fc]));
                 FL_CUDA(cudaGetLastError());
                 r.n_front += hcount[b];
@@ -1216,18 +1215,19 @@ int open_facilities(fl_solve* s) {
         }
         r.prune = Prune();
         sv = sv0 + T + 2;
-        // every vertex the cover reached (its value carries this sweep's epoch)
-        FL_TRY(relax_collect_epoch(g, r.X[r.cur], hi_c, touched, &cnt[6], kProfMis));
+        const uint32_t* cover = now();
+        FL_TRY(relax_collect_set(g, cover, touched, &cnt[6], kProfMis));
 
         // ---- gather: min over Ball(f) of (claimed ? 0 : cover + 1), read at radius B_f
-        ++epoch;
-        const unsigned long long hi_g = 0xffffffffULL - epoch;
-        r.limit = (hi_g + 1) << 32;
+        r.X[0] = val + 2 * n;
+        r.X[1] = val + 3 * n;
+        r.cur = 0;
+        FL_CUDA(cudaMemsetAsync(r.X[0], 0xff, (size_t)n * 4, st));
         FL_CUDA(cudaMemsetAsync(cnt, 0, 24, st));
         r.fc = 0;
         const uint32_t sg0 = ++sv;
         FL_LAUNCH(kProfMis, k_gather_seed<<<152 * 2, 256, 0, st>>>(touched, &cnt[6], s->client.as<uint8_t>(),
-                                                                   s->claimed.as<uint8_t>(), hi_g, r.X[r.cur],
+                                                                   s->claimed.as<uint8_t>(), cover, now(),
                                                                    s->mval.as<uint32_t>(), r.stamp, sg0, r.fr[0],
                                                                    &r.cnt[0]));
         FL_CUDA(cudaGetLastError());
@@ -1238,7 +1238,7 @@ int open_facilities(fl_solve* s) {
         r.sv_prev = sg0;
         if (hcount[0] > 0)
             FL_LAUNCH(kProfMis, k_decide<<<grid_for(hcount[0], 256), 256, 0, st>>>(
-                                    ub + hoff[0], hcount[0], r.X[r.cur], hi_g, s->ord.as<uint32_t>(),
+                                    ub + hoff[0], hcount[0], now(), s->ord.as<uint32_t>(),
                                     s->state.as<uint8_t>(), g->ctr.as<Counters>()));
         r.part_limit = part_T;
         r.prune.need = prune ? reach : nullptr;
@@ -1249,7 +1249,7 @@ int open_facilities(fl_solve* s) {
             else r.sv_prev = sg0 + b;
             if (hcount[b] > 0)
                 FL_LAUNCH(kProfMis, k_decide<<<grid_for(hcount[b], 256), 256, 0, st>>>(
-                                        ub + hoff[b], hcount[b], r.X[r.cur], hi_g, s->ord.as<uint32_t>(),
+                                        ub + hoff[b], hcount[b], now(), s->ord.as<uint32_t>(),
                                         s->state.as<uint8_t>(), g->ctr.as<Counters>()));
         }
         sv = sg0 + T + 1;
