@@ -30,14 +30,21 @@
 // second array, which the next level's first pass copies back.
 //
 // The whole loop is one resident kernel, two grid barriers per level (collect
-// the active vertices; merge and post), in place of three launches and a look
-// at the ring by the host.  A warp per active vertex; rows above kWLong
-// entries are posted by the whole block, so that no level waits for one warp
-// on a hub.  Bound by the latency of the dependent loads of a post (column,
-// k-th rank, sketch).  R-MAT, 65 k vertices, lengths up to 100, k = 16, 313
-// levels: 115 ms of level kernels and some 15 ms of gaps before, 23.6 ms now
-// (36 with bisections in place of the 8-way search and the 8-wide sketch test,
-// 29 with 64-bit ranks in place of their ordinals).
+// the active vertices; merge and post) and a third where hubs were active (post
+// theirs), in place of three launches and a look at the ring by the host.  A
+// warp merges an active vertex; a hub (a row above kWHub entries) is merged by a
+// block, each warp taking every 32nd part of its marks into a copy of the
+// sketch.  Posts are dealt out 32 entries at a time: a hub's to the warps of
+// the grid, those of other rows above kWLong entries to the warps of the block.
+// With a warp per merge and a block per hub's posts, a level of 30 k active
+// vertices waited some 100 us for the block that held the hub (merge 270 k
+// cycles, average of the blocks 100 k; posts 230 k, average 49 k).
+// Bound by the latency of the dependent loads of a merge and of a post (column,
+// row, sketch).  R-MAT, 65 k vertices, lengths up to 100, k = 16, 313 levels:
+// 115 ms of level kernels and some 15 ms of gaps as launches per level, 18.0 ms
+// now (23.2 without the sharing of hubs; 36 with bisections in place of the
+// 8-way search and the 8-wide sketch test, 29 with 64-bit ranks in place of
+// their ordinals, both before it).
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -92,7 +99,9 @@ struct WArgs {
     uint32_t* marks;         // R bitmaps of `mwords` words over the CSR entries
     int64_t mwords;
     unsigned* pend;          // R: nonzero when the slot has activations
-    int32_t* act[2];         // active vertices of the even / odd steps (n each)
+    int32_t* act[2];         // active vertices of the even / odd steps (n each; hubs from the back)
+    uint32_t* hub_gain;      // 32 per hub of the level: the ordinals it gained
+    int32_t* hub_cnt;        // per hub of the level: their number
     int64_t n;
     struct WCtl* c;
 };
@@ -100,15 +109,19 @@ struct WArgs {
 // Control block of the build (device, zero at its start).
 struct WCtl {
     GridBar bar;
-    unsigned long long n_act[2];  // active vertices of the even / odd steps
+    unsigned long long n_act[2];  // active vertices of the even / odd steps, hubs left out
+    unsigned long long n_hub[2];  // active hubs
     unsigned long long glog_n;    // groups logged
     unsigned long long err;       // 1: a row overflowed; 2: a distance above 65535; 4: the group log overflowed
     long long last;               // the largest level that added groups
     long long levels;             // levels run
 };
 
-constexpr int kWLong = 512;   // longer rows are posted by the whole block
-constexpr int kWQueue = 32;   // of them, queued per block and level
+constexpr int kWLong = 32;    // longer rows are posted by the whole block (128: 22.9 ms for 21.9)
+constexpr int kWQueue = 128;  // of them, queued per block and level
+// Rows above are hubs.  2048: 18.4 ms for 18.0; 512 and 256, with a block per
+// hub: 26 and up, a block's shared merge costs more than the warps' own.
+constexpr int kWHub = 1024;
 
 __device__ __forceinline__ WEnt load_ent(const WEnt* p) {
     const int2 x = __ldcg(reinterpret_cast<const int2*>(p));
@@ -209,7 +222,8 @@ __device__ __forceinline__ void post_row(const WArgs& a, int64_t e0, int64_t e1,
 __global__ void __launch_bounds__(kResThreads, 1) k_wbuild(WArgs a) {
     __shared__ uint32_t s_gained[kWQueue][32];
     __shared__ uint32_t s_x[kResWarps][32];  // per warp: merged candidates by place
-    __shared__ int32_t s_v[kWQueue];
+    __shared__ uint32_t s_part[kResWarps][32];  // per warp: its share of a hub's merge
+    __shared__ int64_t s_e0[kWQueue], s_e1[kWQueue];
     __shared__ int s_cnt[kWQueue];
     __shared__ unsigned s_queued, s_next;
     WCtl* c = a.c;
@@ -222,8 +236,8 @@ __global__ void __launch_bounds__(kResThreads, 1) k_wbuild(WArgs a) {
     unsigned pass = 0, total = 0;
     if (threadIdx.x == 0) s_queued = 0;
 
-    // v gained ranks at level L: post them, or leave a long row to the block
-    auto post = [&](int32_t v, int64_t e0, int64_t e1, uint32_t gained, int dcnt, int64_t L) {
+    // the ranks gained at level L go to the row [e0, e1): now, or by the whole block
+    auto post = [&](int64_t e0, int64_t e1, uint32_t gained, int dcnt, int64_t L) {
         if (e1 - e0 > kWLong) {
             unsigned at = 0;
             if (lane == 0) at = atomicAdd(&s_queued, 1u);
@@ -231,7 +245,8 @@ __global__ void __launch_bounds__(kResThreads, 1) k_wbuild(WArgs a) {
             if (at < kWQueue) {
                 s_gained[at][lane] = gained;
                 if (lane == 0) {
-                    s_v[at] = v;
+                    s_e0[at] = e0;
+                    s_e1[at] = e1;
                     s_cnt[at] = dcnt;
                 }
                 return;
@@ -239,13 +254,16 @@ __global__ void __launch_bounds__(kResThreads, 1) k_wbuild(WArgs a) {
         }
         post_row(a, e0, e1, 0, 32, gained, dcnt, L);
     };
+    // the queued rows, 32 entries at a time, dealt to the warps in turn
     auto post_queued = [&](int64_t L) {
         __syncthreads();
         const int queued = (int)min(s_queued, (unsigned)kWQueue);
+        int dealt = 0;
         for (int q = 0; q < queued; ++q) {
-            const int32_t v = s_v[q];
-            post_row(a, __ldg(&a.rowp[v]), __ldg(&a.rowp[v + 1]), (int)(threadIdx.x & ~31u), kResThreads,
-                     s_gained[q][lane], s_cnt[q], L);
+            const int64_t e0 = s_e0[q], e1 = s_e1[q];
+            const int first = (int)((threadIdx.x >> 5) - (unsigned)dealt) & (kResWarps - 1);
+            post_row(a, e0, e1, 32 * first, kResThreads, s_gained[q][lane], s_cnt[q], L);
+            dealt += (int)((e1 - e0 + 31) >> 5);
         }
         __syncthreads();
         if (threadIdx.x == 0) s_queued = 0;
@@ -271,11 +289,11 @@ __global__ void __launch_bounds__(kResThreads, 1) k_wbuild(WArgs a) {
     if (tid == 0) c->glog_n = (unsigned long long)a.n;
     if (!end_pass(&c->bar, pass, 0, &total)) return;
     for (int64_t v = item0; v < a.n; v += warps)
-        post((int32_t)v, __ldg(&a.rowp[v]), __ldg(&a.rowp[v + 1]), lane == 0 ? a.ord[v] : kNil, 1, 0);
+        post(__ldg(&a.rowp[v]), __ldg(&a.rowp[v + 1]), lane == 0 ? a.ord[v] : kNil, 1, 0);
     post_queued(0);
     if (!end_pass(&c->bar, pass, 0, &total)) return;
 
-    int64_t L = 0, n_prev = 0;
+    int64_t L = 0, n_prev = 0, hub_prev = 0;
     for (unsigned step = 0;; ++step) {
         // the next level with activations
         if (threadIdx.x == 0) s_next = ~0u;
@@ -289,7 +307,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_wbuild(WArgs a) {
         const int par = (int)(step & 1);
         // the level before: its new row counts become current
         for (int64_t i = tid; i < n_prev; i += threads) {
-            const int32_t v = __ldcg(&a.act[par ^ 1][i]);
+            const int32_t v = __ldcg(&a.act[par ^ 1][i < hub_prev ? a.n - 1 - i : i - hub_prev]);
             a.ecnt[v] = __ldcg(&a.ecnt_n[v]);
         }
         if (s_next == ~0u) break;
@@ -301,20 +319,34 @@ __global__ void __launch_bounds__(kResThreads, 1) k_wbuild(WArgs a) {
             const uint32_t word = __ldcg(&bm[w]);
             if (!word) continue;
             const bool in = (word >> lane) & 1u;
-            const long long at = warp_append(in, &c->n_act[par]);
-            if (in) a.act[par][at] = (int32_t)(w * 32 + lane);
+            const int64_t v = w * 32 + lane;
+            const bool hub = in && __ldg(&a.rowp[v + 1]) - __ldg(&a.rowp[v]) > kWHub;
+            const long long at = warp_append(in && !hub, &c->n_act[par]);
+            if (in && !hub) a.act[par][at] = (int32_t)v;
+            if (__any_sync(kFull, hub)) {
+                const long long ah = warp_append(hub, &c->n_hub[par]);
+                if (hub) a.act[par][a.n - 1 - ah] = (int32_t)v;
+            }
             mine += in;
             if (lane == 0) bm[w] = 0u;
         }
         if (!end_pass(&c->bar, pass, mine, &total)) return;
         n_prev = (int64_t)total;
+        hub_prev = (int64_t)__ldcg(&c->n_hub[par]);
         if (tid == 0) {
             c->n_act[par ^ 1] = 0;
+            c->n_hub[par ^ 1] = 0;
             a.pend[slot] = 0;  // no post of this level targets its own slot
             ++c->levels;
         }
-        for (int64_t i = item0; i < n_prev; i += warps) {
-            const int32_t v = __ldcg(&a.act[par][i]);
+        // Items [0, hub_prev) are the hubs; up to one per block, a block merges
+        // its hub before its other items.
+        const int64_t by_block = hub_prev <= (int64_t)gridDim.x ? hub_prev : 0;
+        int64_t i = blockIdx.x < by_block ? blockIdx.x : by_block + item0;
+        for (int64_t next; i < n_prev; i = next) {
+            const bool shared = i < by_block, hub = i < hub_prev;
+            next = shared ? by_block + item0 : i + warps;
+            const int32_t v = __ldcg(&a.act[par][hub ? a.n - 1 - i : i - hub_prev]);
             const uint32_t s_old = lane < k ? __ldcg(&a.S[(int64_t)v * k + lane]) : kNil;
             const int64_t e0 = __ldg(&a.rowp[v]), e1 = __ldg(&a.rowp[v + 1]);
             Sketch<32> s;
@@ -323,11 +355,14 @@ __global__ void __launch_bounds__(kResThreads, 1) k_wbuild(WArgs a) {
             s.retau(g, k);
             uint32_t* mk = a.marks + (int64_t)slot * a.mwords;
             const int64_t w1 = (e1 + 31) >> 5;
-            for (int64_t wb = e0 >> 5; wb < w1; wb += 32) {
-                // 32 words of marks at once: their set bits inside [e0, e1) are the delivering entries
+            // the row's marks, 32 words at once (four per warp where the block shares
+            // the row): their set bits inside [e0, e1) are the delivering entries
+            const int span = shared ? 4 : 32;
+            for (int64_t wb = (e0 >> 5) + (shared ? 4 * (threadIdx.x >> 5) : 0); wb < w1;
+                 wb += shared ? 4 * kResWarps : 32) {
                 const int64_t wi = wb + lane;
                 uint32_t bits = 0;
-                if (wi < w1) {
+                if (lane < span && wi < w1) {
                     bits = __ldcg(&mk[wi]);
                     const int64_t first = wi << 5;
                     uint32_t mask = ~0u;
@@ -375,6 +410,12 @@ __global__ void __launch_bounds__(kResThreads, 1) k_wbuild(WArgs a) {
                     }
                 }
             }
+            if (shared) {
+                s_part[threadIdx.x >> 5][lane] = s.sk;
+                __syncthreads();
+                if (threadIdx.x >= 32) continue;
+                for (int w = 1; w < kResWarps; ++w) merge_list(g, k, s_part[w][lane], s, sx);
+            }
             // the entries gained at distance L: in the new sketch, not in the old
             // (every lane takes part in the membership shuffles)
             bool held;
@@ -389,6 +430,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_wbuild(WArgs a) {
                 if (lane == 0) {
                     a.ecnt_n[v] = base;
                     if (fm) atomicOr(&c->err, 1ULL);
+                    if (hub) a.hub_cnt[i] = 0;
                 }
                 continue;
             }
@@ -419,9 +461,40 @@ __global__ void __launch_bounds__(kResThreads, 1) k_wbuild(WArgs a) {
                 }
             }
             const uint32_t mine_g = __shfl_sync(kFull, s.sk, lane < dcnt ? nth_set_bit(fm, lane) : 0);
-            post(v, e0, e1, lane < dcnt ? mine_g : kNil, dcnt, L);
+            if (hub) {
+                a.hub_gain[i * 32 + lane] = lane < dcnt ? mine_g : kNil;
+                if (lane == 0) a.hub_cnt[i] = dcnt;
+            } else {
+                post(e0, e1, lane < dcnt ? mine_g : kNil, dcnt, L);
+            }
         }
         post_queued(L);
+        if (!end_pass(&c->bar, pass, 0, &total)) return;
+        if (hub_prev == 0) continue;
+        // the hubs' rows, 32 entries at a time, dealt to the grid's warps in turn
+        unsigned dealt = 0;  // mod the number of warps
+        for (int64_t h0 = 0; h0 < hub_prev; h0 += 32) {
+            int64_t e0 = 0, e1 = 0;
+            int dcnt = 0;
+            if (h0 + lane < hub_prev) {
+                const int32_t v = __ldcg(&a.act[par][a.n - 1 - (h0 + lane)]);
+                dcnt = __ldcg(&a.hub_cnt[h0 + lane]);
+                e0 = __ldg(&a.rowp[v]);
+                e1 = __ldg(&a.rowp[v + 1]);
+            }
+            for (unsigned m = __ballot_sync(kFull, dcnt > 0); m; m &= m - 1) {
+                const int l = __ffs(m) - 1;
+                const int64_t b0 = __shfl_sync(kFull, e0, l), b1 = __shfl_sync(kFull, e1, l);
+                const unsigned chunks = (unsigned)((b1 - b0 + 31) >> 5);
+                // the first of the row's chunks that is this warp's
+                const unsigned turn = (unsigned)item0 + ((unsigned)item0 < dealt ? (unsigned)warps : 0u) - dealt;
+                dealt += chunks;
+                if (dealt >= (unsigned)warps) dealt %= (unsigned)warps;
+                if (turn >= chunks) continue;
+                post_row(a, b0 + 32 * (int64_t)turn, b1, 0, (int)(32 * warps), __ldcg(&a.hub_gain[(h0 + l) * 32 + lane]),
+                         __shfl_sync(kFull, dcnt, l), L);
+            }
+        }
         if (!end_pass(&c->bar, pass, 0, &total)) return;
     }
 }
@@ -633,7 +706,8 @@ int build_sketches_weighted(fl_graph* g, int k, uint64_t seed) {
     const double expect = (double)k * (1.0 + std::log(std::max(1.0, (double)n / k)));
     int64_t cap = std::min<int64_t>(n, (int64_t)(2.0 * expect) + 64);
     const int64_t mwords = (nnz + 31) / 32;
-    DBuf ent, ecnt, ecnt_n, gcnt, glog, ring, pend, act, cnt, marks;
+    const int64_t hubs_max = nnz / kWHub + 1;
+    DBuf ent, ecnt, ecnt_n, gcnt, glog, ring, pend, act, cnt, marks, hubs;
     int rc = FL_OK;
     FL_CUDA(cudaMemsetAsync(g->ctr.p, 0, sizeof(Counters), st));
     if ((rc = build_ordinals(g, ent)) || (rc = read_counters(g))) {
@@ -652,7 +726,7 @@ int build_sketches_weighted(fl_graph* g, int k, uint64_t seed) {
             (rc = dalloc(gcnt, (size_t)n * 4)) ||
             (rc = dalloc(glog, (size_t)glog_cap * sizeof(WGroup))) ||
             (rc = dalloc(ring, (size_t)R * words * 4 + 16)) || (rc = dalloc(pend, (size_t)R * 4)) ||
-            (rc = dalloc(act, (size_t)n * 8)) || (rc = dalloc(cnt, sizeof(WCtl))) ||
+            (rc = dalloc(act, (size_t)n * 8)) || (rc = dalloc(hubs, (size_t)hubs_max * 33 * 4)) || (rc = dalloc(cnt, sizeof(WCtl))) ||
             (rc = dalloc(marks, (size_t)R * mwords * 4 + 16)))
             break;
         WArgs a;
@@ -676,6 +750,8 @@ int build_sketches_weighted(fl_graph* g, int k, uint64_t seed) {
         a.pend = pend.as<unsigned>();
         a.act[0] = act.as<int32_t>();
         a.act[1] = a.act[0] + n;
+        a.hub_gain = hubs.as<uint32_t>();
+        a.hub_cnt = hubs.as<int32_t>() + hubs_max * 32;
         a.n = n;
         a.c = cnt.as<WCtl>();
         a.rev = g->wrev.as<uint32_t>();
@@ -746,7 +822,7 @@ int build_sketches_weighted(fl_graph* g, int k, uint64_t seed) {
         g->wlevels = hc.levels;
         break;
     }
-    dfree_after(st, {&ent, &ecnt, &ecnt_n, &gcnt, &glog, &ring, &pend, &act, &cnt, &marks});
+    dfree_after(st, {&ent, &ecnt, &ecnt_n, &gcnt, &glog, &ring, &pend, &act, &cnt, &marks, &hubs});
     return rc;
 }
 
