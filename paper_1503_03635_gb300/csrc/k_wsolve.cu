@@ -23,7 +23,8 @@
 // arrivals; times without are passed over.  With three launches per time step
 // a sweep was bound by them and by the largest hub, pushed by one warp: the 24
 // sweeps (2819 times) of an R-MAT graph with 65 k vertices and lengths up to
-// 100 took 45 ms, 13.9 ms now; bound by the barriers and dependent loads.
+// 100 took 45 ms, 12.7 ms now; bound by the barriers (4.5 us per time) and dependent
+// loads.
 //   cover:  facility f enters at time H - B_f with its key ordinal (H = the
 //           largest B_f), so every wave ends at H and the label of v at H is
 //           the smallest key whose ball holds v;
@@ -128,8 +129,8 @@ struct WEntry {
     const uint8_t* mask;
 };
 
-constexpr int kPLong = 512;   // longer rows are pushed by the whole block
-constexpr int kPQueue = 128;  // of them, queued per block and step
+constexpr int kPLong = 32;    // longer rows are pushed by the whole block (512: 13.3 ms of sweeps for 12.7)
+constexpr int kPQueue = 256;  // of them, queued per block and step
 
 // x arrives at v at time t: into the ring.
 __device__ __forceinline__ void send(const WSweep& a, int32_t v, uint32_t x, uint32_t t) {
@@ -169,7 +170,7 @@ __device__ __forceinline__ void push_row(const WSweep& a, int64_t e0, int64_t e1
 // block in step t and cleared in the next one, t': t' <= t + R - 1, so no
 // send of step t' (to times up to t' + R - 1) uses the same of the 2R counters.
 __global__ void __launch_bounds__(kResThreads, 1) k_wsweep(WSweep a, WEntry in, int64_t H, WSweepCtl* c) {
-    __shared__ int32_t s_v[kPQueue];
+    __shared__ int64_t s_e0[kPQueue], s_e1[kPQueue];
     __shared__ uint32_t s_x[kPQueue];
     __shared__ unsigned s_queued, s_next;
     __shared__ long long s_first;
@@ -261,7 +262,8 @@ __global__ void __launch_bounds__(kResThreads, 1) k_wsweep(WSweep a, WEntry in, 
                     at = __shfl_sync(kFull, at, 0);
                     if (at < kPQueue) {
                         if (lane == 0) {
-                            s_v[at] = u;
+                            s_e0[at] = e0;
+                            s_e1[at] = e1;
                             s_x[at] = y;
                         }
                         continue;
@@ -272,9 +274,12 @@ __global__ void __launch_bounds__(kResThreads, 1) k_wsweep(WSweep a, WEntry in, 
         }
         __syncthreads();
         const int queued = (int)min(s_queued, (unsigned)kPQueue);
+        int dealt = 0;  // 32 entries at a time, dealt to the warps in turn
         for (int q = 0; q < queued; ++q) {
-            const int32_t u = s_v[q];
-            push_row(a, __ldg(&a.rowp[u]), __ldg(&a.rowp[u + 1]), (int)(threadIdx.x & ~31u), kResThreads, s_x[q], t, H);
+            const int64_t e0 = s_e0[q], e1 = s_e1[q];
+            const int turn = (int)((threadIdx.x >> 5) - (unsigned)dealt) & (kResWarps - 1);
+            push_row(a, e0, e1, 32 * turn, kResThreads, s_x[q], t, H);
+            dealt += (int)((e1 - e0 + 31) >> 5);
         }
         __syncthreads();
         if (threadIdx.x == 0) s_queued = 0;
