@@ -571,7 +571,7 @@ def run_exact(args):
             "unit": "sources/s", "n_gpus": 1, "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "u64", "data": "synthetic",
             "config": {"workload": "exact", "graph": f"rmat20 (n={n}, nnz={w.nnz})", "sources": len(src),
-                       "max_dist": D, "l2": "bit arrays (96 MB) mostly L2-resident; no flush"},
+                       "max_dist": D, "l2": "bit arrays (403 MB) larger than L2 (no flush)"},
             "roofline": roofline, "gpu_launches": launches, "clocks": clk,
             "accuracy_vs_k": {"samples": "100 vertices per distance 1..20 (Section 5.1)", "by_k": accuracy},
             "exact_radii": {"facilities": len(fac), "seconds": t_exact, "facilities_per_s": len(fac) / t_exact,

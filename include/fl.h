@@ -271,8 +271,9 @@ int fl_mis_log(const fl_solve* s, int64_t cap, int64_t* n_rows, int64_t* rows);
  * (Section 5.1, "Accuracy vs. k", Fig. 1: relative error |S_E - S_ADS| / S_E
  * per distance, against k).  These calls give both sides of that comparison
  * on the GPU and an exact-radius mode of phase (ii).  The exact sizes come
- * from a bit-parallel breadth-first search (256 sources per sweep, 96 bytes
- * of device scratch per vertex, held by the graph), so their cost grows
+ * from a bit-parallel breadth-first search (up to 1024 sources per sweep and
+ * 384 bytes of device scratch per vertex, held by the graph; above 2^20
+ * vertices 256 sources and 96 bytes), so their cost grows
  * with the number of sources times the balls' edges: meant for sampled
  * vertices and small or medium graphs.
  */
@@ -330,10 +331,10 @@ int fl_compute_radii_exact(fl_solve* s, const double* open_cost, const uint8_t* 
  * alg_bytes is filled for FL_PROF_SKETCH_MERGE: per hop, 8 B per merging
  * vertex (row offsets) + 4 B per edge-merge (column) + 8 B per neighbour
  * delta rank read + 16k B per merging vertex (own sketch read and write) +
- * 12 B per new ADS entry; and for FL_PROF_EXACT: per search level, 68 B per
- * vertex (list id, visited words read, next words written) + 16 B per
- * scanned row (offsets) + 36 B per scanned entry (column and the
- * neighbour's frontier words).
+ * 12 B per new ADS entry; and for FL_PROF_EXACT, with B bytes of source bits
+ * per vertex (32, 64 or 128): per bottom-up level, 4 + 2 B per vertex (list id,
+ * visited words read, next words written) + 16 per scanned row (offsets) +
+ * 4 + B per scanned entry (column and the neighbour's frontier words).
  */
 #define FL_PROF_SKETCH_MERGE 0
 #define FL_PROF_SKETCH_EXPAND 1
@@ -435,8 +436,8 @@ int fl_autotune_forget(void);
  *   merging[h-1]      A_h: vertices with at least one such entry;
  *   delta_read[h-1]   neighbour-delta ranks the merge kernels read (filtering
  *                     loads of the list merge; 4 words per neighbour and
- *                     256-bit slice in the mask merge; 0 at hop 1, which
- *                     recomputes its neighbours' ranks);
+ *                     256-bit slice in the mask merge; 0 at hop 1, whose
+ *                     neighbours offer the one ordinal of their own);
  *   delta_sum[h-1]    the sum of |D_{h-1}(u)| over the E_h edge-merges (the
  *                     ranks the paper's messages carry; = E_1 at hop 1);
  *   new_entries[h-1]  |D_h|: ADS entries gained at hop h.
