@@ -1226,7 +1226,7 @@ int open_facilities(fl_solve* s) {
         FL_CUDA(cudaMemsetAsync(cnt, 0, 24, st));
         r.fc = 0;
         const uint32_t sg0 = ++sv;
-        FL_LAUNCH(kProfMis, k_gather_seed<<<152 * 2, 256, 0, st>>>(touched, &cnt[6], s->client.as<uint8_t>(),
+        FL_LAUNCH(kProfMis, k_gather_seed<<<152 * 8, 256, 0, st>>>(touched, &cnt[6], s->client.as<uint8_t>(),
                                                                    s->claimed.as<uint8_t>(), cover, now(),
                                                                    s->mval.as<uint32_t>(), r.stamp, sg0, r.fr[0],
                                                                    &r.cnt[0]));
@@ -1260,7 +1260,7 @@ int open_facilities(fl_solve* s) {
         // ---- claim the balls of this round's winners; keep the undecided
         if (prune) FL_CUDA(cudaMemsetAsync(kill, 0, (size_t)n, st));
         FL_CUDA(cudaMemsetAsync(&cnt[7], 0, 8, st));
-        FL_LAUNCH(kProfMis, k_claim<<<152 * 4, 256, 0, st>>>(s->touched.as<int32_t>(), &cnt[6], s->client.as<uint8_t>(),
+        FL_LAUNCH(kProfMis, k_claim<<<152 * 8, 256, 0, st>>>(s->touched.as<int32_t>(), &cnt[6], s->client.as<uint8_t>(),
                                          s->claimed.as<uint8_t>(), s->mval.as<uint32_t>(),
                                          s->fac_by_ord.as<int32_t>(), s->state.as<uint8_t>(),
                                          prune ? kill : nullptr, &cnt[7]));
