@@ -51,3 +51,13 @@ def test_level_cap_is_refused():
     s.open_facilities_eps(0.5, cost, np.ones(40, np.uint8))
     s.close()
     g.close()
+
+
+@pytest.mark.parametrize("deg", [255, 256, 257, 769])
+def test_gamma_over_rows_at_segment_edges(deg):
+    # one facility, the leaf that comes last in the hubs' rows
+    rowp, cols = _hubs(3, deg)
+    n = len(rowp) - 1
+    cost = np.full(n, np.inf)
+    cost[n - 1] = 2.5
+    _compare(rowp, cols, 8, 3, 0.2, cost, np.ones(n, np.uint8))
