@@ -385,7 +385,10 @@ int fl_hop_stats(const fl_graph* g, int64_t cap, int64_t* n_hops, int64_t* scann
  *   dense_div   a relaxation round (MIS sweeps, BFS levels) pulls when its
  *               frontier * dense_div >= the listed vertices (default 8) ...
  *   edge_div    ... or when its frontier's edges * edge_div >= nnz
- *               (default 16); otherwise it pushes.
+ *               (default 16); otherwise it pushes.  Small graphs run all
+ *               rounds of a sweep in one kernel, which pulls throughout;
+ *               with dense_div or edge_div off its default they run round by
+ *               round like the others.
  *   graph_bfs   1: the assignment BFS runs as one CUDA graph whose
  *               conditional WHILE node repeats one pull level on the device
  *               (no host round trip per level; capped at n + 2 levels,

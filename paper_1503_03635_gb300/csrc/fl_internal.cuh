@@ -525,6 +525,8 @@ struct Sched {
     int edge_div = 16;    // ... or when frontier edges * edge_div >= nnz
     int graph_bfs = 0;    // 1: the assignment BFS runs as one CUDA graph (a device-side level loop)
     int level_cap = 0;    // BFS levels at most (0: n + 2); beyond it FL_ETIMEOUT
+    // dense_div or edge_div set: the caller asks for rounds that these switch
+    bool switches_rounds() const { return dense_div != 8 || edge_div != 16; }
 };
 
 // ----------------------------------------------------------------- graph BFS
@@ -723,7 +725,9 @@ int msbfs(fl_graph* g, const int32_t* src_list, int64_t n_src, int32_t* label, i
 int msbfs_graph(fl_graph* g, const int32_t* src_list, int64_t n_src, int32_t* label, int32_t* dist, DBuf& X,
                 DBuf& stampb, int cls);
 void graph_bfs_release(GraphBfs* c);
-// resident kernels of small graphs (k_resident.cu); usable when g->n_items > 0
+// resident kernels of small graphs (k_resident.cu): graphs with work items whose
+// schedule leaves the round switches alone (a pull has no push to switch to)
+inline bool runs_resident(const fl_graph* g) { return g->n_items > 0 && !g->sched.switches_rounds(); }
 int build_items(fl_graph* g);
 int mis_resident(fl_solve* s, int64_t m, bool* done);
 int mis_resident_queue(fl_solve* s, int64_t m, uint8_t* acc, int* outcome);
