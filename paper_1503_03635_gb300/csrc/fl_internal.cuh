@@ -123,11 +123,25 @@ constexpr int kSmallDeg = 8;
 // Graphs of at most kResidentEdges CSR entries (and vertices) run their MIS and
 // BFS as resident kernels over work items of at most kItemEdges entries.  The
 // kernels read every row each round, the host-driven rounds only what the
-// frontier needs, so the line lies where the reads outgrow the launches.  MIS
+// frontier needs, so the lines lie where the reads outgrow the launches.  MIS
 // with keys, resident against host-driven: Erdos-Renyi 0.08 M entries 0.57 /
 // 3.55 ms, 0.8 M 1.28 / 5.91, 10 M 1.90 / 4.10; R-MAT 1.8 M 0.46 / 1.18, 7.6 M
 // 1.05 / 1.40, 15.5 M 2.65 / 1.90.
+//
+// A round costs a step per item, and a vertex is an item however short its row:
+// graphs of short rows are bounded by their items too.  BFS of an open set,
+// resident against host-driven, by million items: Erdos-Renyi 0.6 0.41 / 0.41
+// ms, 0.8 0.52 / 0.45, 1.0 0.63 / 0.47, 2.0 1.48 / 0.79; square grid, 50 levels, 0.7 1.82 / 2.24,
+// 1.0 2.30 / 2.38, 2.2 4.85 / 3.38 (kResidentBfsItems).  MIS with balls of up to 14 hops:
+// Erdos-Renyi 1.2 2.77 / 4.73, 2.0 6.47 / 5.71; R-MAT 1.2 1.80 / 1.63, 2.0 3.34 / 2.30;
+// grid 1.4 3.38 / 4.74, 2.2 6.19 / 5.69 (kResidentMisItems).  Balls of 50 to 120 hops,
+// whose sweeps are mostly thin: grid 0.7 20.8 / 28.4, 1.0 13.6 / 13.3 and 31.4 /
+// 37.1, 1.4 50.6 / 38.9, 2.2 79.8 / 53.9 (kWideBallItems).
 constexpr int64_t kResidentEdges = 10 << 20;
+constexpr int64_t kResidentBfsItems = 3 << 18;
+constexpr int64_t kResidentMisItems = 3 << 19;
+constexpr int64_t kWideBallItems = 1 << 20;  // above: only balls of at most kNarrowBall hops
+constexpr int kNarrowBall = 16;
 constexpr int kItemEdges = 64;
 // Pinned host block of a graph: its Counters mirror, then scratch of a call.
 constexpr size_t kPinnedBytes = 16384;
@@ -565,7 +579,7 @@ struct fl_graph {
     fl::DBuf seg_hub;              // int32[n_seg]: hub of each segment
     int64_t n_low = 0, n_hubs = 0, n_seg = 0;
     fl::DBuf items;                // int4[n_items]: work items of the resident kernels
-    int64_t n_items = 0;           // 0: the graph is too large for them
+    int64_t n_items = 0;           // 0: the graph is too large for them (kResidentEdges, kResidentMisItems)
     fl::DBuf part;                 // uint32[n_seg*k]: partial bottom-k of each hub segment (scratch)
     // A graph that is a disjoint union of parts (batched instances): vertex v
     // of the part starting at vbase[v] has local id v - vbase[v], and ranks
@@ -727,7 +741,8 @@ int msbfs_graph(fl_graph* g, const int32_t* src_list, int64_t n_src, int32_t* la
 void graph_bfs_release(GraphBfs* c);
 // resident kernels of small graphs (k_resident.cu): graphs with work items whose
 // schedule leaves the round switches alone (a pull has no push to switch to)
-inline bool runs_resident(const fl_graph* g) { return g->n_items > 0 && !g->sched.switches_rounds(); }
+inline bool resident_mis(const fl_graph* g) { return g->n_items > 0 && !g->sched.switches_rounds(); }
+inline bool resident_bfs(const fl_graph* g) { return resident_mis(g) && g->n_items <= kResidentBfsItems; }
 int build_items(fl_graph* g);
 int mis_resident(fl_solve* s, int64_t m, bool* done);
 int mis_resident_queue(fl_solve* s, int64_t m, uint8_t* acc, int* outcome);

@@ -32,14 +32,14 @@ namespace {
 
 constexpr uint32_t kNone = 0xffffffffu;
 constexpr uint64_t kDone = ~0ULL;           // fk of a vertex that is no undecided facility
-constexpr int kMaxBall = 1023;              // larger ball radii take the host-driven rounds
+constexpr int kMaxBall = 1023;              // larger ball radii take the host-driven rounds (kNarrowBall on large graphs)
 constexpr int kRoundsPerLaunch = 32;        // greedy rounds (bounds the log)
 constexpr int kFastRows = 128;              // log rows copied with the control block
 
 // Control block of a launch (device).
 struct Ctl {
     GridBar bar;                      // its err: 1: a barrier wait ran out; 2: a ball without clients; 4: the level cap
-    unsigned deep;                    // 1: a ball radius above kMaxBall (nothing was done)
+    unsigned deep;                    // 1: a ball radius above max_ball (nothing was done)
     unsigned n_list[2];               // items of the current / next greedy round
     unsigned tmax[2];                 // largest ball radius of the undecided, by round parity
     unsigned hist[2][kMaxBall + 1];   // undecided facilities by ball radius, by round parity
@@ -146,6 +146,7 @@ struct MisArgs {
     long long* log;         // rows of 6
     long long log_cap;
     long long m;            // candidates
+    int max_ball;           // largest ball radius that the kernel takes
     int resume;             // 0: first launch; 1: goes on after kRoundsPerLaunch rounds
 };
 
@@ -215,7 +216,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_mis_resident(MisArgs a) {
             unsigned long long f = kDone;
             if (a.state[v] == 0) {
                 const int32_t B = a.bcap[v];
-                if (B > kMaxBall) {
+                if (B > a.max_ball) {
                     deep = 1;
                 } else {
                     f = ((unsigned long long)(uint32_t)B << 32) | a.ord[v];
@@ -578,8 +579,9 @@ int build_items(fl_graph* g) {
         if (e == cudaSuccess) e = cudaMemcpyAsync(&c, cnt.as<int32_t>() + n - 1, 4, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) { rc = status_of(e, "work items", __FILE__, __LINE__); break; }
-        g->n_items = p + c;
+        if (p + c <= kResidentMisItems) g->n_items = p + c;
     } while (0);
+    if (g->n_items == 0) dfree_after(st, {&g->items});
     dfree_after(st, {&cnt, &pos});
     return rc;
 }
@@ -630,6 +632,7 @@ static int mis_args(fl_solve* s, int64_t m, MisArgs* out, int* blocks) {
     a.log = reinterpret_cast<long long*>(s->rctl.as<char>() + kCtlBytes);
     a.log_cap = log_cap;
     a.m = m;
+    a.max_ball = g->n_items > kWideBallItems ? kNarrowBall : kMaxBall;
     a.resume = 0;
     FL_TRY(resident_blocks(g->n_items, blocks));
     FL_CUDA(cudaMemsetAsync(s->rctl.p, 0, sizeof(Ctl), g->stream));
@@ -670,7 +673,7 @@ int mis_resident_queue(fl_solve* s, int64_t m, uint8_t* acc, int* outcome) {
 }
 
 // The greedy MIS of the m sorted candidates and its open list.  *done = false:
-// not for this kernel (a ball radius above kMaxBall); nothing but scratch was
+// not for this kernel (a ball radius above max_ball); nothing but scratch was
 // written.
 int mis_resident(fl_solve* s, int64_t m, bool* done) {
     fl_graph* g = s->g;
