@@ -486,7 +486,7 @@ struct Counters {
     unsigned long long new_entries;  // merge: entries gained this hop (sum of |D_h(v)|)
     unsigned long long key_or;       // keys: OR of the candidates' radius words
     unsigned long long key_orn;      // keys: OR of their complements (a bit set in both varies)
-    unsigned long long key_ties;     // keys: a run of equal radius prefixes too long to order in place
+    unsigned long long key_ties;     // keys: 1: a run of equal prefixes too long to order in place, 2: equal radii out of order
 };
 
 // ----------------------------------------------------------------- profiling
