@@ -1,6 +1,7 @@
 """The resident event loop of the phase with eps > 0 against the oracle where it
-can go wrong: rows at the length that a whole block takes, more long rows than
-a block queues, components without facilities or clients, and the level cap."""
+can go wrong: rows at the length that a whole block takes (one or two in a
+block's queue; more than it holds: test_gpu_eps_queue.py), components without
+facilities or clients, and the level cap."""
 import numpy as np
 import pytest
 

@@ -1,8 +1,8 @@
 """The allocation-free assignment against a plain BFS where its levels can go
-wrong: rows at the edges of the 32-row windows and of the 128-entry steps,
-rows long enough to be taken by a whole block, more long rows than a block
-queues, thin frontiers (push) and wide ones (pull), and graphs whose entries do
-not fill one window."""
+wrong: rows at the edges of the 32-row windows and of the 128-entry steps, thin frontiers
+(push) and wide ones (pull), long rows in levels that pull, and graphs whose
+entries do not fill one window.  (Long rows in levels that push:
+test_gpu_noalloc_push.py.)"""
 import numpy as np
 import pytest
 
