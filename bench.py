@@ -87,6 +87,15 @@ def ncu_traffic(kernel, workload):
     return e["dram_bytes_per_launch"]
 
 
+def merge_model_bytes(hops, k):
+    """Algorithmic bytes of a build's merges (Graph.hop_model rows): row offsets
+    and own sketch (k ordinals of 4 bytes, read and written) per merging vertex, a
+    column and the neighbour's delta ordinals per edge-merge, an ADS id and weight
+    per new entry."""
+    return sum(8 * m["merging"] + 4 * m["edge_merges"] + 4 * m["delta_sum"] + 8 * k * m["merging"]
+               + 12 * m["new_entries"] for m in hops)
+
+
 class Clocks:
     """nvidia-smi clock/throttle sampling during the timed region."""
 
@@ -353,11 +362,7 @@ def run_gpu(args):
                    "changed": h["changed"], "E": m["edge_merges"], "A": m["merging"], "delta_sum": m["delta_sum"],
                    "delta_read": m["delta_read"], "new": m["new_entries"]}
                   for h, m in zip(g.hop_stats(), model)]
-    # algorithmic bytes of one build by the per-hop model: row offsets and own
-    # sketch (read + write) per merging vertex, a column and the neighbour's
-    # delta ranks per edge-merge, an ADS id + weight per new entry
-    model_bytes = sum(8 * m["merging"] + 4 * m["edge_merges"] + 8 * m["delta_sum"] + 16 * w.k * m["merging"]
-                      + 12 * m["new_entries"] for m in model)
+    model_bytes = merge_model_bytes(model, w.k)
     g.profile(False)
     merges_step = stats["edge_merges"]
     value = world * merges_step * args.steps / (ms / 1e3)
@@ -424,7 +429,7 @@ def run_gpu(args):
     peak, peak_kind = measured_peaks()
     mp = prof["sketch_merge"]
     # numerator: the model's bytes of every timed build (the same graph and
-    # seed each step); beside it, the bytes the merge kernels' loads touched
+    # seed each step); beside it, the delta words the merge kernels read
     alg_bytes = model_bytes * args.steps
     achieved = alg_bytes / (mp["ms"] / 1e3) / 1e9 if mp["ms"] > 0 else None
     achieved_reads = mp["alg_bytes"] / (mp["ms"] / 1e3) / 1e9 if mp["ms"] > 0 else None
@@ -434,11 +439,12 @@ def run_gpu(args):
                 "frac": (achieved / peak) if achieved else None, "traffic": traffic,
                 "peak_kind": f"{peak_kind} copy bandwidth", "alg_bytes_per_launch": per_launch_bytes,
                 "alg_bytes_per_build": model_bytes,
-                "alg_model": "per hop: 8 A + 4 E + 8 sum|D_{h-1}(u)| + 16 k A + 12 |D_h| (hop_detail terms)",
+                "alg_model": "per hop: 8 A + 4 E + 4 sum|D_{h-1}(u)| + 8 k A + 12 |D_h| (hop_detail terms)",
                 "achieved_reads": achieved_reads, "frac_reads": (achieved_reads / peak) if achieved_reads else None,
                 "reads_bytes_per_build": mp["alg_bytes"] / args.steps,
-                "reads_model": "as alg_model with the neighbour-delta ranks the kernels' loads read (delta_read) "
-                               "in place of sum|D_{h-1}(u)|",
+                "reads_model": "as alg_model with 8 bytes per delta word that the kernels read (delta_read: mask words, "
+                               "or ordinals of 4 bytes, charged at 8) in place of 4 sum|D_{h-1}(u)|; words used, not "
+                               "sectors moved (traffic)",
                 "launches": mp["launches"], "kernel_ms": mp["ms"],
                 "share_of_step": mp["ms"] / ms if ms > 0 else None}
 

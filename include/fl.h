@@ -330,8 +330,10 @@ int fl_compute_radii_exact(fl_solve* s, const double* open_cost, const uint8_t* 
  * (exact sizes, their estimates, exact-count radii); -1 = all classes.
  * alg_bytes is filled for FL_PROF_SKETCH_MERGE: per hop, 8 B per merging
  * vertex (row offsets) + 4 B per edge-merge (column) + 8 B per neighbour
- * delta rank read + 16k B per merging vertex (own sketch read and write) +
- * 12 B per new ADS entry; and for FL_PROF_EXACT, with B bytes of source bits
+ * delta word read (fl_hop_model's delta_read; mask words have 8 B, the list
+ * merge's words are ordinals of 4 B, so that this term is up to twice what its
+ * loads move) + 8k B per merging vertex (own sketch read and write) + 12 B per
+ * new ADS entry; and for FL_PROF_EXACT, with B bytes of source bits
  * per vertex (32, 64 or 128): per bottom-up level, 4 + 2 B per vertex (list id,
  * visited words read, next words written) + 16 per scanned row (offsets) +
  * 4 + B per scanned entry (column and the neighbour's frontier words).
@@ -437,7 +439,7 @@ int fl_autotune_forget(void);
  *   edge_merges[h-1]  E_h: CSR entries (v, u) whose u gained entries at hop
  *                     h-1 (every entry at hop 1);
  *   merging[h-1]      A_h: vertices with at least one such entry;
- *   delta_read[h-1]   neighbour-delta ranks the merge kernels read (filtering
+ *   delta_read[h-1]   neighbour-delta words the merge kernels read (filtering
  *                     loads of the list merge; 4 words per neighbour and
  *                     256-bit slice in the mask merge; 0 at hop 1, whose
  *                     neighbours offer the one ordinal of their own);

@@ -1369,12 +1369,13 @@ int build_sketches(fl_graph* g, int k, uint64_t seed) {
         next_merges = (int64_t)g->h_ctr->merges;
         next_delta = (int64_t)g->h_ctr->delta_next;
         // algorithmic bytes of this hop's merge: row offsets of each merging
-        // vertex (8 B), frontier columns (4 B per edge-merge), neighbour delta
-        // ranks read (8 B each), own sketch read + write (16k B per merging
-        // vertex); the ADS entries (12 B each) are added after the last hop
+        // vertex (8 B), frontier columns (4 B per edge-merge), delta words read
+        // (8 B each, the size of a mask word; the list merge's are ordinals of
+        // 4 B), own sketch read + write (ordinals: 8k B per merging vertex); the
+        // ADS entries (12 B each) are added after the last hop
         {
-            const double A = (double)g->h_ctr->merging, SD = (double)g->h_ctr->cand_reads;
-            g->prof.bytes[kProfSketchMerge] += 8.0 * A + 4.0 * (double)hop_merges + 8.0 * SD + 16.0 * k * A;
+            const double A = (double)g->h_ctr->merging, R = (double)g->h_ctr->cand_reads;
+            g->prof.bytes[kProfSketchMerge] += 8.0 * A + 4.0 * (double)hop_merges + 8.0 * R + 8.0 * k * A;
         }
         if (n_front == 0) break;
         // a small frontier makes the next hop sparse: collect its list
