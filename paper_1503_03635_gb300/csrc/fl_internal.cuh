@@ -74,33 +74,15 @@ __device__ __forceinline__ int64_t rank_id(const IdMap& m, int64_t v) {
     return m.rid ? (int64_t)__ldg(&m.rid[v]) : v;
 }
 
-__host__ __device__ constexpr uint64_t inv_odd(uint64_t a) {
-    // Newton iteration for the inverse of an odd number mod 2^64
-    uint64_t x = a;
-    for (int i = 0; i < 6; ++i) x *= 2 - a * x;
-    return x;
-}
-
-// SplitMix64 finaliser and its inverse (each step is a bijection on 64 bits).
+// SplitMix64 finaliser (each step is a bijection on 64 bits).
 __host__ __device__ __forceinline__ uint64_t mix64(uint64_t z) {
     z = (z ^ (z >> 30)) * kMul1;
     z = (z ^ (z >> 27)) * kMul2;
     return z ^ (z >> 31);
 }
-__host__ __device__ __forceinline__ uint64_t unmix64(uint64_t y) {
-    y = y ^ (y >> 31) ^ (y >> 62);
-    y *= inv_odd(kMul2);
-    y = y ^ (y >> 27) ^ (y >> 54);
-    y *= inv_odd(kMul1);
-    return y ^ (y >> 30) ^ (y >> 60);
-}
 // r(v): SplitMix64 output v+1 from state `seed`.
 __host__ __device__ __forceinline__ uint64_t vertex_rank(uint64_t seed, int64_t v) {
     return mix64(seed + (uint64_t)(v + 1) * kGamma);
-}
-// the vertex whose rank is x (ranks are a bijection of the counter)
-__host__ __device__ __forceinline__ int64_t rank_vertex(uint64_t seed, uint64_t x) {
-    return (int64_t)((unmix64(x) - seed) * inv_odd(kGamma) - 1);
 }
 // pi(f): SplitMix64 output f+1 from the state given by the first output for `seed`.
 __host__ __device__ __forceinline__ uint64_t facility_priority(uint64_t seed, int64_t f) {
@@ -154,7 +136,6 @@ constexpr int kUWords = kUW / 64;
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 
 __device__ __forceinline__ uint64_t umin64(uint64_t a, uint64_t b) { return a < b ? a : b; }
-__device__ __forceinline__ uint64_t umax64(uint64_t a, uint64_t b) { return a < b ? b : a; }
 
 // HIP weight of a group whose ball holds cnt ranks with k-th smallest kth:
 // 1 while the ball has fewer than k vertices, else 1 / Pr[rank < k-th] =
@@ -492,7 +473,7 @@ struct Counters {
 // ----------------------------------------------------------------- profiling
 // Kernel classes for launch counts and CUDA-event timings.
 enum ProfClass {
-    kProfSketchMerge = 0,  // k_merge_hop
+    kProfSketchMerge = 0,  // the hop kernels (k_hop_*), k_wbuild
     kProfSketchExpand = 1, // k_expand
     kProfSketchOther = 2,  // rank init, ADS compaction, scans, eccentricity bound
     kProfRadius = 3,

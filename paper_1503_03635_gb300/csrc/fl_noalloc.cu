@@ -5,8 +5,8 @@
 // elsewhere would fail or fragment it), and latency-critical loops for which
 // an allocation's implicit device synchronisation is not acceptable.  For
 // them this file offers the assignment step with its scratch memory (BFS
-// values, level stamps, frontiers, counters) in one file-scope device array
-// of fixed size.  The caller passes the graph, the open set and the outputs.
+// values, two frontier lists, three frontier bitmaps, counters) in one
+// file-scope device array of fixed size.  The caller passes the graph, the open set and the outputs.
 //
 // Every GPU that loads the library holds the array until the process exits.
 // All calls share it and it keeps the last call's contents: each call clears

@@ -41,7 +41,11 @@ namespace fl {
 namespace {
 
 constexpr int kXMaxW = 16;      // 64-bit words of source bits per vertex, at most
-constexpr int64_t kXWideN = 1 << 20;  // larger graphs take W = 4
+// Larger graphs take W = 4: a sweep holds 24 W bytes per vertex until the graph is
+// destroyed (96 B at W = 4, 384 at 16; 1.6 GB against 0.4 at 2^22 vertices).  The
+// line is that limit on scratch, not where the speed turns: 1000 sources on R-MAT,
+// W = 4 against 16, 2^20 + 1 vertices 4.3 / 2.8 ms, 2^21 9.7 / 7.8, 2^22 18.2 / 14.3.
+constexpr int64_t kXWideN = 1 << 20;
 constexpr int kXHeavy = 32;     // rows longer than this get a whole warp
 constexpr int kXSeg = 256;      // entries of a work item
 constexpr int kXHuge = kXSeg;   // rows longer than this are cut into work items
@@ -93,7 +97,7 @@ __global__ void k_x_map(const int32_t* __restrict__ src, int64_t n_src, const in
 }
 
 // Vertices with short rows (<= kXHeavy entries, isolated ones included), with
-// with long rows, and with rows above kXHuge entries (from the end of `heavy`).
+// long rows, and with rows above kXHuge entries (from the end of `heavy`).
 __global__ void k_x_lists(const int64_t* __restrict__ rowp, int64_t n, int32_t* __restrict__ light,
                           int32_t* __restrict__ heavy, unsigned long long* n_light, unsigned long long* n_heavy,
                           unsigned long long* n_huge) {

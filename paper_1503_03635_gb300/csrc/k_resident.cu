@@ -443,7 +443,6 @@ __global__ void __launch_bounds__(kResThreads, 1) k_mis_resident(MisArgs a) {
         if (__ldcg(&c->bar.err)) return;
     }
     if (n_u == 0) {  // the open set and its list
-        unsigned opened = 0;
         for (int64_t b = warp0 * 32; b < a.g.n; b += warps * 32) {
             const int64_t v = b + lane;
             const bool o = v < a.g.n && __ldcg(&a.state[v]) == 1;
@@ -455,7 +454,6 @@ __global__ void __launch_bounds__(kResThreads, 1) k_mis_resident(MisArgs a) {
                 at = __shfl_sync(kFull, at, 0);
                 if (o) a.open_list[at + __popc(mk & ((1u << lane) - 1u))] = (int32_t)v;
             }
-            opened += o;
         }
     }
     if (scribe) {
