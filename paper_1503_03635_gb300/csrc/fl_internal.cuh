@@ -111,19 +111,25 @@ constexpr int kSmallDeg = 8;
 // 1.05 / 1.40, 15.5 M 2.65 / 1.90.
 //
 // A round costs a step per item, and a vertex is an item however short its row:
-// graphs of short rows are bounded by their items too.  BFS of an open set,
-// resident against host-driven, by million items: Erdos-Renyi 0.6 0.41 / 0.41
-// ms, 0.8 0.52 / 0.45, 1.0 0.63 / 0.47, 2.0 1.48 / 0.79; square grid, 50 levels, 0.7 1.82 / 2.24,
-// 1.0 2.30 / 2.38, 2.2 4.85 / 3.38 (kResidentBfsItems).  MIS with balls of up to 14 hops:
-// Erdos-Renyi 1.2 2.77 / 4.73, 2.0 6.47 / 5.71; R-MAT 1.2 1.80 / 1.63, 2.0 3.34 / 2.30;
-// grid 1.4 3.38 / 4.74, 2.2 6.19 / 5.69 (kResidentMisItems).  Balls of 50 to 120 hops,
-// whose sweeps are mostly thin: grid 0.7 20.8 / 28.4, 1.0 13.6 / 13.3 and 31.4 /
-// 37.1, 1.4 50.6 / 38.9, 2.2 79.8 / 53.9 (kWideBallItems).
+// graphs of short rows are bounded by their items too (resident against
+// host-driven in ms, by million items).
+//   MIS, balls of up to 64 hops (kResidentMisItems): Erdos-Renyi 1.2 2.77 / 4.73,
+//   1.5 12.9 / 14.1, 2.0 6.47 / 5.71; R-MAT 1.2 1.80 / 1.63, 2.0 3.34 / 2.30; square
+//   grid, 40 to 48 hops, 1.3 16.8 / 19.9 and 19.4 / 20.9, 1.6 22.1 / 22.2.
+//   MIS, larger balls, whose sweeps are mostly thin (kWideBallItems): grid, 70 to
+//   120 hops, 0.7 20.8 / 28.4, 1.0 31.4 / 37.1, 1.1 21.9 / 19.9, 1.3 21.3 / 18.2, 1.6
+//   32.4 / 23.4, 2.2 79.8 / 53.9.
+//   BFS (kResidentBfsItems): R-MAT 1.0 0.46 / 0.51, 1.2 0.41 / 0.40; Erdos-Renyi 0.8
+//   0.52 / 0.45, 1.0 0.63 / 0.47, 2.0 1.48 / 0.79; grid, 50 levels, 0.7 1.82 / 2.24, 1.0
+//   2.30 / 2.38, 2.2 4.85 / 3.38.  Host-driven rounds of a graph made of parts flag
+//   its parts as well: whole batches, replicas of R-MAT 0.96 2.97 / 3.22, 1.3 4.01 /
+//   4.12, union of Erdos-Renyi graphs 1.2 16.8 / 16.4 (kResidentBfsPartItems).
 constexpr int64_t kResidentEdges = 10 << 20;
-constexpr int64_t kResidentBfsItems = 3 << 18;
+constexpr int64_t kResidentBfsItems = 1 << 20;
+constexpr int64_t kResidentBfsPartItems = 5 << 18;
 constexpr int64_t kResidentMisItems = 3 << 19;
 constexpr int64_t kWideBallItems = 1 << 20;  // above: only balls of at most kNarrowBall hops
-constexpr int kNarrowBall = 16;
+constexpr int kNarrowBall = 64;
 constexpr int kItemEdges = 64;
 // Pinned host block of a graph: its Counters mirror, then scratch of a call.
 constexpr size_t kPinnedBytes = 16384;
@@ -723,7 +729,9 @@ void graph_bfs_release(GraphBfs* c);
 // resident kernels of small graphs (k_resident.cu): graphs with work items whose
 // schedule leaves the round switches alone (a pull has no push to switch to)
 inline bool resident_mis(const fl_graph* g) { return g->n_items > 0 && !g->sched.switches_rounds(); }
-inline bool resident_bfs(const fl_graph* g) { return resident_mis(g) && g->n_items <= kResidentBfsItems; }
+inline bool resident_bfs(const fl_graph* g) {
+    return resident_mis(g) && g->n_items <= (g->n_parts > 0 ? kResidentBfsPartItems : kResidentBfsItems);
+}
 int build_items(fl_graph* g);
 int mis_resident(fl_solve* s, int64_t m, bool* done);
 int mis_resident_queue(fl_solve* s, int64_t m, uint8_t* acc, int* outcome);
