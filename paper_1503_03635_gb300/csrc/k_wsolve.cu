@@ -143,9 +143,13 @@ __device__ __forceinline__ void send(const WSweep& a, int32_t v, uint32_t x, uin
 // An arrival that cannot lower u's label is not sent: u's label already holds
 // a value at most x from an arrival at or before t, and that arrival was also
 // kept by u's deadline whenever this one would be.  (A label that drops in
-// this same step does so by an arrival at t.)
+// this same step does so by an arrival at t.)  The same holds for an arrival of
+// time t that is still in the slot (now: the slot's values): the step drains
+// and pushes at once, and an arrival sent past a label that is about to drop is
+// one more time to run.  Star of 1000 vertices, lengths up to 5000, every vertex
+// a source: assignment 1.4 to 2.8 ms without the look at the slot, 0.12 with it.
 __device__ __forceinline__ void push_row(const WSweep& a, int64_t e0, int64_t e1, int first, int step, uint32_t x,
-                                         int64_t t, int64_t H) {
+                                         int64_t t, int64_t H, const uint32_t* now) {
     for (int64_t e = e0 + first + lane_id(); e < e1; e += step) {
         const int32_t u = __ldg(&a.cols[e]);
         const uint32_t lu = __ldcg(&a.lab[u]);
@@ -159,6 +163,8 @@ __device__ __forceinline__ void push_row(const WSweep& a, int64_t e0, int64_t e1
             if (a.first) a.past[u] = 1;
             continue;
         }
+        const uint32_t pu = __ldcg(&now[u]);
+        if (a.first ? pu != kNone : pu <= x) continue;
         send(a, u, x, (uint32_t)t2);
     }
 }
@@ -248,8 +254,8 @@ __global__ void __launch_bounds__(kResThreads, 1) k_wsweep(WSweep a, WEntry in, 
             if (lane < per && i < cnt) {
                 v = __ldcg(&a.plist[slot + i]);
                 x = __ldcg(&a.pend[slot + v]);
-                a.pend[slot + v] = kNone;
                 join = arrive(a, v, x, t);
+                a.pend[slot + v] = kNone;  // after the label: push_row looks at it and then at the slot
             }
             for (unsigned m = __ballot_sync(kFull, join); m; m &= m - 1) {
                 const int l = __ffs(m) - 1;
@@ -269,7 +275,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_wsweep(WSweep a, WEntry in, 
                         continue;
                     }
                 }
-                push_row(a, e0, e1, 0, 32, y, t, H);
+                push_row(a, e0, e1, 0, 32, y, t, H, a.pend + slot);
             }
         }
         __syncthreads();
@@ -278,7 +284,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_wsweep(WSweep a, WEntry in, 
         for (int q = 0; q < queued; ++q) {
             const int64_t e0 = s_e0[q], e1 = s_e1[q];
             const int turn = (int)((threadIdx.x >> 5) - (unsigned)dealt) & (kResWarps - 1);
-            push_row(a, e0, e1, 32 * turn, kResThreads, s_x[q], t, H);
+            push_row(a, e0, e1, 32 * turn, kResThreads, s_x[q], t, H, a.pend + slot);
             dealt += (int)((e1 - e0 + 31) >> 5);
         }
         __syncthreads();
