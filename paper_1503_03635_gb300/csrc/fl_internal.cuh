@@ -735,7 +735,8 @@ inline bool resident_bfs(const fl_graph* g) {
 int build_items(fl_graph* g);
 int mis_resident(fl_solve* s, int64_t m, bool* done);
 int mis_resident_queue(fl_solve* s, int64_t m, uint8_t* acc, int* outcome);
-int msbfs_resident(fl_graph* g, const int32_t* src, int64_t n_src, int32_t* label, int32_t* dist, DBuf& ctl, int cls);
+int msbfs_resident(fl_graph* g, const int32_t* src, int64_t n_src, int32_t* label, int32_t* dist, DBuf& ctl, DBuf& lists,
+                   int cls);
 
 // Per-vertex pruning of the rounds of a sweep (the MIS cover and gather
 // sweeps).  A round that first gives v a value below the limit records

@@ -86,8 +86,8 @@ int scratch_address(unsigned char** out) {
 // What bounds it: the entries of unreached rows, read once per level from L2,
 // and about 40 instructions per 32 entries; then a grid barrier per level.
 // Before, a warp walked each frontier row alone, two launches and a look by
-// the host per level: R-MAT, 500 k vertices, 16 M draws, 1 % open 2.73 ms per
-// call (1.67 ms of it one launch that waits for the largest hub), now 0.34 ms;
+// the host per level: R-MAT, 500 k vertices, 16 M draws, 1 % open 2.62 ms per
+// call (1.67 ms of it one launch that waits for the largest hub), now 0.35 ms;
 // 167 k vertices 0.75 -> 0.20 ms, Erdos-Renyi, 12 k vertices 0.29 -> 0.12 ms.
 constexpr int kPushDiv = 64;
 constexpr int kLongRow = 512;

@@ -45,6 +45,7 @@ struct Ctl {
     unsigned hist[2][kMaxBall + 1];   // undecided facilities by ball radius, by round parity
     long long rounds, n_u, n_open, log_n;
     long long done;                   // 1: the launch ran to its end
+    unsigned long long bfs_n[4];      // BFS: lengths of the frontier lists (level mod 4)
 };
 
 struct ItemGraph {
@@ -466,6 +467,8 @@ __global__ void __launch_bounds__(kResThreads, 1) k_mis_resident(MisArgs a) {
 
 struct BfsArgs {
     ItemGraph g;
+    const int64_t* rowp;
+    int64_t nnz;
     const int4* items;
     int64_t n_items;
     const int32_t* src;
@@ -473,50 +476,166 @@ struct BfsArgs {
     const int32_t* label_of;  // labels of the sources, or NULL (their ids)
     uint32_t* label;
     int32_t* dist;
+    int32_t *list0, *list1;   // frontier lists (levels of even / odd number)
     Ctl* c;
     int64_t cap;              // levels at most
 };
 
+// With kPush, a level whose frontier's vertices and entries are less than
+// 1 / kBfsPushDiv of the graph's items and entries is pushed; where the level
+// before pulled, the frontier is listed first, a pass and a barrier more, for which
+// a pull must take more than kBfsListSteps items per group of lanes.
+constexpr int kBfsPushDiv = 128;
+constexpr int kBfsPushSteps = 4;   // items per group of lanes above which the kernel with pushes runs
+constexpr int kBfsListSteps = 16;
+constexpr int kBfsLong = 512;      // longer rows are pushed by the whole block
+constexpr int kBfsQueue = 256;     // of them, queued per block and level
+
 // Level-synchronous BFS: level L gives every vertex without a distance the
 // smallest label among its neighbours at distance L - 1.  In place: a
 // distance written in this level is L and does not pass for L - 1.
+//
+// A pull reads every item and the rows of every vertex not reached.  On graphs of
+// many levels, or with a few sources beside hubs, that is all rows for a handful
+// of vertices, so thin frontiers push (div 64 costs more than it gives where many
+// rows push to a few hubs).  One kernel of pulls alone | this one: grid of 490 k
+// vertices, 460 levels 9.46 | 2.69 ms, 50 levels 1.27 | 1.08; Erdos-Renyi, 1 M vertices of
+// degree 2, 31 levels 1.47 | 0.82; 50 hubs of 100 k entries, 3 levels 0.70 | 0.20.  A
+// graph whose pulls are a few steps runs without: the code for pushes costs it 1 us a level.
+template <bool kPush>
 __global__ void __launch_bounds__(kResThreads, 1) k_bfs_resident(BfsArgs a) {
-    const int lane = lane_id();
+    __shared__ int32_t s_queue[kBfsQueue];
+    __shared__ unsigned s_queued;
+    Ctl* c = a.c;
+    const int lane = lane_id(), sub = lane & 7;
     const int64_t tid = (int64_t)blockIdx.x * kResThreads + threadIdx.x, threads = (int64_t)gridDim.x * kResThreads;
+    const int64_t group0 = (tid >> 5) * 4, groups = (threads >> 5) * 4;
     unsigned pass = 0, total = 0;
+    if (kPush && threadIdx.x == 0) s_queued = 0;
     for (int64_t v = tid; v < a.g.n; v += threads) {
         a.label[v] = kNone;
         a.dist[v] = -1;
     }
-    if (!end_pass(&a.c->bar, pass, 0, &total)) return;
+    if (!end_pass(&c->bar, pass, 0, &total)) return;
+    // total: with pushes the frontier's vertices and entries, else at least its vertices
+    auto weight = [&](int64_t v) {
+        return kPush ? 1u + (unsigned)(__ldg(&a.rowp[v + 1]) - __ldg(&a.rowp[v])) : 1u;
+    };
+    unsigned reached = 0;
     for (int64_t i = tid; i < a.n_src; i += threads) {
         const int32_t s = a.src[i];
         a.label[s] = (uint32_t)(a.label_of ? a.label_of[s] : s);
         a.dist[s] = 0;
+        if (kPush) reached += weight(s);
     }
-    if (!end_pass(&a.c->bar, pass, 0, &total)) return;
-    total = a.n_src > 0;
+    if (!end_pass(&c->bar, pass, reached, &total)) return;
+    if (!kPush) total = a.n_src > 0;
+    bool listed = true;
+    const int32_t* front = a.src;
+    int64_t n_front = a.n_src;
     for (int64_t L = 1; total; ++L) {
         if (L > a.cap) {
-            if (tid == 0) a.c->bar.err = 4;
+            if (tid == 0) c->bar.err = 4;
             return;
         }
-        unsigned reached = 0;
-        for (int64_t b = (tid >> 5) * 4; b < a.n_items; b += (threads >> 5) * 4) {
-            const int4 it = b + (lane >> 3) < a.n_items ? __ldg(&a.items[b + (lane >> 3)]) : make_int4(-1, 0, 0, 0);
-            const int32_t d = it.x >= 0 ? __ldcg(&a.dist[it.x]) : 0;
-            const bool want = it.x >= 0 && (d < 0 || d == (int32_t)L);
-            const uint32_t low = item_min(a.g, it.y, want ? it.z : it.y, [&](int32_t u) {
-                return __ldcg(&a.dist[u]) == (int32_t)L - 1 ? __ldcg(&a.label[u]) : kNone;
-            });
-            if (want && (lane & 7) == 0 && low != kNone) {
-                if (it.w & kSingle) a.label[it.x] = low;
-                else atomicMin(&a.label[it.x], low);
-                a.dist[it.x] = (int32_t)L;
-                ++reached;
+        int32_t* next = L & 1 ? a.list1 : a.list0;
+        unsigned long long* n_next = &c->bfs_n[L & 3];
+        if (kPush) {
+            if (tid == 0) c->bfs_n[(L + 1) & 3] = 0;  // read last in level L - 2
+            const bool thin = (int64_t)total * kBfsPushDiv < a.nnz + a.n_items;
+            if (thin && !listed && a.n_items > kBfsListSteps * groups) {
+                int32_t* mine = L & 1 ? a.list0 : a.list1;
+                for (int64_t b = (tid >> 5) * 32; b < a.g.n; b += (threads >> 5) * 32) {
+                    const int64_t v = b + lane;
+                    const bool in = v < a.g.n && __ldcg(&a.dist[v]) == (int32_t)L - 1;
+                    const long long at = warp_append(in, &c->bfs_n[(L - 1) & 3]);
+                    if (at >= 0) mine[at] = (int32_t)v;
+                }
+                if (!end_pass(&c->bar, pass, 0, &total)) return;
+                listed = true;
+                front = mine;
+                n_front = (int64_t)__ldcg(&c->bfs_n[(L - 1) & 3]);
+            }
+            listed = listed && thin;  // so is the next level's frontier, then
+        }
+        reached = 0;
+        if (kPush && listed) {
+            // label lab to the vertex of entry e (e >= end: none), all 32 lanes
+            auto offer = [&](int64_t e, int64_t end, uint32_t lab) {
+                bool fresh = false;
+                int32_t u = 0;
+                if (e < end) {
+                    u = __ldg(&a.g.cols[e]);
+                    int32_t d = __ldcg(&a.dist[u]);
+                    if (d < 0) {
+                        d = atomicCAS(&a.dist[u], -1, (int32_t)L);
+                        fresh = d < 0;
+                        if (fresh) d = (int32_t)L;
+                    }
+                    if (d == (int32_t)L && lab < __ldcg(&a.label[u])) atomicMin(&a.label[u], lab);
+                }
+                const long long at = warp_append(fresh, n_next);
+                if (at >= 0) {
+                    next[at] = u;
+                    reached += weight(u);
+                }
+            };
+            for (int64_t b = group0; b < n_front; b += groups) {
+                const int64_t i = b + (lane >> 3);
+                const int32_t v = i < n_front ? __ldcg(&front[i]) : -1;
+                int64_t e = v >= 0 ? __ldg(&a.rowp[v]) : 0;
+                int64_t end = v >= 0 ? __ldg(&a.rowp[v + 1]) : 0;
+                if (end - e > kBfsLong) {
+                    unsigned at = kBfsQueue;
+                    if (sub == 0) at = atomicAdd(&s_queued, 1u);
+                    at = __shfl_sync(0xffu << (lane & 24), at, 0, 8);  // the row's eight lanes
+                    if (at < kBfsQueue) {
+                        if (sub == 0) s_queue[at] = v;
+                        end = e;
+                    }
+                }
+                const uint32_t lab = v >= 0 ? __ldcg(&a.label[v]) : kNone;
+                for (; __any_sync(kFull, e < end); e += 8) offer(e + sub, end, lab);
+            }
+            __syncthreads();
+            const int queued = (int)min(s_queued, (unsigned)kBfsQueue);
+            for (int q = 0; q < queued; ++q) {
+                const int32_t v = s_queue[q];
+                const int64_t end = __ldg(&a.rowp[v + 1]);
+                const uint32_t lab = __ldcg(&a.label[v]);
+                for (int64_t e = __ldg(&a.rowp[v]) + (threadIdx.x & ~31); e < end; e += kResThreads)
+                    offer(e + lane, end, lab);
+            }
+            __syncthreads();
+            if (threadIdx.x == 0) s_queued = 0;
+        } else {
+            for (int64_t b = group0; b < a.n_items; b += groups) {
+                const int4 it = b + (lane >> 3) < a.n_items ? __ldg(&a.items[b + (lane >> 3)]) : make_int4(-1, 0, 0, 0);
+                const int32_t d = it.x >= 0 ? __ldcg(&a.dist[it.x]) : 0;
+                const bool want = it.x >= 0 && (d < 0 || d == (int32_t)L);
+                const uint32_t low = item_min(a.g, it.y, want ? it.z : it.y, [&](int32_t u) {
+                    return __ldcg(&a.dist[u]) == (int32_t)L - 1 ? __ldcg(&a.label[u]) : kNone;
+                });
+                if (want && sub == 0 && low != kNone) {
+                    if (it.w & kSingle) a.label[it.x] = low;
+                    else atomicMin(&a.label[it.x], low);
+                    if (!kPush) {
+                        a.dist[it.x] = (int32_t)L;
+                        ++reached;
+                    } else if (it.w & kSingle) {
+                        a.dist[it.x] = (int32_t)L;
+                        reached += 1u + (unsigned)(it.z - it.y);
+                    } else if (d < 0 && atomicCAS(&a.dist[it.x], -1, (int32_t)L) < 0) {
+                        reached += weight(it.x);
+                    }
+                }
             }
         }
-        if (!end_pass(&a.c->bar, pass, reached, &total)) return;
+        if (!end_pass(&c->bar, pass, reached, &total)) return;
+        if (kPush && listed) {
+            front = next;
+            n_front = (int64_t)__ldcg(n_next);
+        }
     }
 }
 
@@ -717,11 +836,19 @@ int mis_resident(fl_solve* s, int64_t m, bool* done) {
 }
 
 int msbfs_resident(fl_graph* g, const int32_t* src, int64_t n_src, int32_t* label, int32_t* dist, DBuf& ctl,
-                   int cls) {
+                   DBuf& lists, int cls) {
     cudaStream_t st = g->stream;
     FL_TRY(dalloc(ctl, sizeof(Ctl)));
+    int blocks = 0;
+    FL_TRY(resident_blocks(g->n_items, &blocks));
+    const bool push = g->n_items > (int64_t)kBfsPushSteps * blocks * (kResThreads / 8);
+    if (push) FL_TRY(dalloc(lists, (size_t)g->n * 8));
     BfsArgs a;
     a.g = item_graph(g);
+    a.rowp = g->rowp.as<int64_t>();
+    a.nnz = g->nnz;
+    a.list0 = lists.as<int32_t>();
+    a.list1 = a.list0 + g->n;
     a.items = g->items.as<int4>();
     a.n_items = g->n_items;
     a.src = src;
@@ -731,13 +858,11 @@ int msbfs_resident(fl_graph* g, const int32_t* src, int64_t n_src, int32_t* labe
     a.dist = dist;
     a.c = ctl.as<Ctl>();
     a.cap = g->sched.level_cap > 0 ? g->sched.level_cap : g->n + 2;
-    int blocks = 0;
-    FL_TRY(resident_blocks(g->n_items, &blocks));
     FL_CUDA(cudaMemsetAsync(ctl.p, 0, sizeof(Ctl), st));
     void* args[] = {&a};
     cudaError_t le = cudaSuccess;
-    FL_LAUNCH(cls, le = cudaLaunchCooperativeKernel((const void*)k_bfs_resident, dim3(blocks), dim3(kResThreads), args,
-                                                    0, st));
+    const void* kernel = push ? (const void*)k_bfs_resident<true> : (const void*)k_bfs_resident<false>;
+    FL_LAUNCH(cls, le = cudaLaunchCooperativeKernel(kernel, dim3(blocks), dim3(kResThreads), args, 0, st));
     FL_CUDA(le);
     unsigned* h = reinterpret_cast<unsigned*>(g->h_ctr + 1);
     FL_CUDA(cudaMemcpyAsync(h, &a.c->bar.err, 4, cudaMemcpyDeviceToHost, st));

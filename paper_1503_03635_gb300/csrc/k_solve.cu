@@ -73,7 +73,7 @@ int msbfs(fl_graph* g, const int32_t* src_list, int64_t n_src, int32_t* label, i
         FL_TRY(build_work_lists(g));
         g->lists_ready = 1;
     }
-    if (resident_bfs(g)) return msbfs_resident(g, src_list, n_src, label, dist, frval, cls);
+    if (resident_bfs(g)) return msbfs_resident(g, src_list, n_src, label, dist, frval, X, cls);
     FL_TRY(dalloc(X, (size_t)n * 16));
     FL_TRY(dalloc(stampb, (size_t)n * 4));
     FL_TRY(dalloc(fr[0], (size_t)n * 4));
