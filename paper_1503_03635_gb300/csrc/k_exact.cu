@@ -398,17 +398,25 @@ __global__ void __launch_bounds__(256) k_x_heavy(const int32_t* __restrict__ lis
     x_flush(c, any, m, sh, st);
 }
 
-// Work items of the rows above kXHuge entries (vertex << 32 | segment).
+// Work items of the rows above kXHuge entries (vertex << 32 | segment): the rows'
+// first segments, then the others (*n_more of them) in any order.  With few
+// sources a row's first segment often brings all that it needs, and the items
+// after it are passed over: one source on 2 x 2000 vertices, joined completely,
+// 0.28 ms with a row's items side by side, 0.24 now (and one wait of the host less).
 __global__ void k_x_huge_items(const int32_t* __restrict__ list, int64_t n_list, const int64_t* __restrict__ rowp,
-                               unsigned long long* __restrict__ items, unsigned long long* __restrict__ n_items) {
+                               unsigned long long* __restrict__ items, unsigned long long* __restrict__ n_more) {
     const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t i = (((int64_t)blockIdx.x * blockDim.x) + threadIdx.x) >> 5; i < n_list; i += warps) {
         const int32_t v = list[i];
-        const int segs = (int)((rowp[v + 1] - rowp[v] + kXSeg - 1) / kXSeg);
+        const unsigned long long item = (unsigned long long)(uint32_t)v << 32;
+        const int more = (int)((rowp[v + 1] - rowp[v] + kXSeg - 1) / kXSeg) - 1;
         unsigned long long at = 0;
-        if (lane_id() == 0) at = atomicAdd(n_items, (unsigned long long)segs);
+        if (lane_id() == 0) {
+            items[i] = item;
+            at = (unsigned long long)n_list + atomicAdd(n_more, (unsigned long long)more);
+        }
         at = __shfl_sync(kFull, at, 0);
-        for (int j = lane_id(); j < segs; j += 32) items[at + j] = ((unsigned long long)(uint32_t)v << 32) | (unsigned)j;
+        for (int j = lane_id(); j < more; j += 32) items[at + j] = item | (unsigned)(j + 1);
     }
 }
 
@@ -425,7 +433,8 @@ __global__ void k_x_huge_clear(const int32_t* __restrict__ list, int64_t n_list,
 // neighbours t, t + 32 / W, ..., eight in flight.  An item whose row has every
 // bit it needs is passed over.
 template <int W>
-__global__ void __launch_bounds__(256) k_x_huge(const unsigned long long* __restrict__ items, int64_t n_items,
+__global__ void __launch_bounds__(256) k_x_huge(const unsigned long long* __restrict__ items, int64_t n_first,
+                                                const unsigned long long* __restrict__ n_more,
                                                 const int64_t* __restrict__ rowp, const int32_t* __restrict__ cols,
                                                 const unsigned long long* __restrict__ cur, unsigned long long* nxt,
                                                 const unsigned long long* __restrict__ vis, XState<W>* __restrict__ st) {
@@ -434,6 +443,7 @@ __global__ void __launch_bounds__(256) k_x_huge(const unsigned long long* __rest
     const int w = lane & (W - 1), t = lane / W;
     const unsigned long long act = st->active[w];
     unsigned long long entries = 0;
+    const int64_t n_items = n_first + (int64_t)*n_more;
     const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t i = (((int64_t)blockIdx.x * blockDim.x) + threadIdx.x) >> 5; i < n_items; i += warps) {
         const unsigned long long it = __ldg(&items[i]);
@@ -750,8 +760,8 @@ struct XScratch {
     int32_t *light, *heavy;
     const int32_t* huge;
     int32_t* front[2];
-    unsigned long long* huge_items;  // of the huge rows
-    int64_t n_huge_items;
+    unsigned long long* huge_items;  // of the huge rows, n_huge + *n_more
+    unsigned long long* n_more;
     unsigned long long* items;       // of a top-down level
     size_t n_items;
     void* state;
@@ -810,8 +820,8 @@ int run_sweep(fl_graph* g, const XScratch& x, int mode, int64_t nb, const int32_
             if (x.n_huge > 0) {
                 FL_LAUNCH(cls, k_x_huge_clear<W><<<blocks_for(x.n_huge, 256 / W), 256, 0, st>>>(x.huge, x.n_huge,
                                                                                               buf[c ^ 1]));
-                FL_LAUNCH(cls, k_x_huge<W><<<blocks_for(x.n_huge_items, 8), 256, 0, st>>>(
-                                   x.huge_items, x.n_huge_items, rowp, cols, buf[c], buf[c ^ 1], vis, xs));
+                FL_LAUNCH(cls, k_x_huge<W><<<blocks_for(x.n_huge + nnz / kXSeg, 8), 256, 0, st>>>(
+                                   x.huge_items, x.n_huge, x.n_more, rowp, cols, buf[c], buf[c ^ 1], vis, xs));
                 FL_LAUNCH(cls, k_x_huge_done<W><<<blocks_for(x.n_huge, 256 / W, kXLevelBlocks), 256, 0, st>>>(
                                    x.huge, x.n_huge, rowp, buf[c ^ 1], vis, pred, front[fc ^ 1], xs));
             }
@@ -866,13 +876,13 @@ int run_sweeps(fl_graph* g, int mode, int64_t n_src, const int32_t* src, int64_t
     // the back (n), two frontiers (n + kMost each: the first frontier lists the
     // sweep's sources, repeats included); then the top-down work items (uint64,
     // one per kXSeg entries of a frontier row: at most n + kMost + nnz / kXSeg),
-    // those of the huge rows (at most 2 nnz / kXSeg) and the sweep state
+    // those of the huge rows (at most 2 nnz / kXSeg), their number and the sweep state
     const size_t lists = ((size_t)(4 * n + 2 * kMost) * 4 + 255) & ~(size_t)255;
     XScratch x;
     x.n_items = (size_t)(n + kMost + nnz / kXSeg + 1);
     const size_t items_b = (x.n_items * 8 + 255) & ~(size_t)255;
     const size_t huge_b = ((size_t)(2 * (nnz / kXSeg) + 1) * 8 + 255) & ~(size_t)255;
-    FL_TRY(dalloc(g->xaux, lists + items_b + huge_b + sizeof(XState<kXMaxW>)));
+    FL_TRY(dalloc(g->xaux, lists + items_b + huge_b + 256 + sizeof(XState<kXMaxW>)));
     x.vis = g->xbits.as<unsigned long long>();
     x.light = g->xaux.as<int32_t>();
     x.heavy = x.light + n;
@@ -880,7 +890,8 @@ int run_sweeps(fl_graph* g, int mode, int64_t n_src, const int32_t* src, int64_t
     x.front[1] = x.light + 3 * n + kMost;
     x.items = reinterpret_cast<unsigned long long*>(g->xaux.as<char>() + lists);
     x.huge_items = reinterpret_cast<unsigned long long*>(g->xaux.as<char>() + lists + items_b);
-    x.state = g->xaux.as<char>() + lists + items_b + huge_b;
+    x.state = g->xaux.as<char>() + lists + items_b + huge_b + 256;
+    x.n_more = reinterpret_cast<unsigned long long*>(g->xaux.as<char>() + lists + items_b + huge_b);
     Counters* ctr = g->ctr.as<Counters>();
     FL_CUDA(cudaMemsetAsync(g->ctr.p, 0, sizeof(Counters), st));
     FL_LAUNCH(kProfExact, k_x_lists<<<blocks_for(n, 256), 256, 0, st>>>(g->rowp.as<int64_t>(), n, x.light, x.heavy,
@@ -891,14 +902,11 @@ int run_sweeps(fl_graph* g, int mode, int64_t n_src, const int32_t* src, int64_t
     x.n_heavy = (int64_t)g->h_ctr->aux3;
     x.n_huge = (int64_t)g->h_ctr->frontier;
     x.huge = x.heavy + n - x.n_huge;
-    x.n_huge_items = 0;
     if (x.n_huge > 0) {
-        FL_CUDA(cudaMemsetAsync(g->ctr.p, 0, sizeof(Counters), st));
+        FL_CUDA(cudaMemsetAsync(x.n_more, 0, 8, st));
         FL_LAUNCH(kProfExact, k_x_huge_items<<<blocks_for(x.n_huge, 8), 256, 0, st>>>(
-                                  x.huge, x.n_huge, g->rowp.as<int64_t>(), x.huge_items, &ctr->aux0));
+                                  x.huge, x.n_huge, g->rowp.as<int64_t>(), x.huge_items, x.n_more));
         FL_CUDA(cudaGetLastError());
-        FL_TRY(read_counters(g));
-        x.n_huge_items = (int64_t)g->h_ctr->aux0;
     }
     for (int64_t b0 = 0; b0 < n_src;) {
         const int w = width(n_src - b0);
