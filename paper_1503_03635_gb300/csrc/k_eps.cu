@@ -94,8 +94,8 @@ __global__ void k_eps_counts(const double* __restrict__ cost, const uint8_t* __r
 // gamma_c = min over d of fl(M + d), which equals min over facilities of
 // fl(c(f) + d(c, f)) because rounded addition is monotone in each operand.
 //
-// Mn starts as M.  A warp per row, and per segment of a row above `seg` entries:
-// the largest hub's warp was the whole round.  R-MAT, 65 k vertices: 62 us a round
+// Mn starts as M where there are segments.  A warp per row, and per segment of a row
+// above `seg` entries: the largest hub's warp was the whole round.  R-MAT, 65 k vertices: 62 us a round
 // with a warp per row, 16 now; the solve on R-MAT scale 20, eps = 1, 16.4 -> 13.3 ms.
 __global__ void __launch_bounds__(256) k_eps_min_pull(const int64_t* __restrict__ rowp,
                                                       const int32_t* __restrict__ cols, int64_t n,
@@ -123,12 +123,10 @@ __global__ void __launch_bounds__(256) k_eps_min_pull(const int64_t* __restrict_
         for (int64_t e = e0 + lane; e < e1; e += 32) m = min(m, __ldg(&M[cols[e]]));
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) m = min(m, __shfl_xor_sync(kFull, m, o));
-        if (m < own) {
-            ch = true;
-            if (lane == 0) {
-                if (i < n_seg) atomicMin(&Mn[v], m);
-                else Mn[v] = m;
-            }
+        ch |= m < own;
+        if (lane == 0) {
+            if (i >= n_seg) Mn[v] = m;
+            else if (m < own) atomicMin(&Mn[v], m);
         }
     }
     if (__syncthreads_or(ch) && threadIdx.x == 0) *changed = 1;
@@ -546,7 +544,8 @@ int open_facilities_eps(fl_solve* s, double eps) {
     for (int64_t d = 1;; ++d) {
         if (d > n + 1) FL_FAIL(FL_ETIMEOUT, "epsilon phase: cost propagation did not settle");
         FL_CUDA(cudaMemsetAsync(&ctr[3], 0, 8, st));
-        FL_CUDA(cudaMemcpyAsync(M[cur ^ 1], M[cur], (size_t)n * 8, cudaMemcpyDeviceToDevice, st));
+        if (g->n_seg > 0)
+            FL_CUDA(cudaMemcpyAsync(M[cur ^ 1], M[cur], (size_t)n * 8, cudaMemcpyDeviceToDevice, st));
         FL_LAUNCH(kProfMis, k_eps_min_pull<<<std::min(grid_for(n + g->n_seg, 8), 152 * 8), 256, 0, st>>>(
                                 g->rowp.as<int64_t>(), g->cols.as<int32_t>(), n, g->seg_hub.as<int32_t>(), g->n_seg,
                                 g->hub_seg.as<int64_t>(), g->hub_list.as<int32_t>(), g->seg, M[cur], M[cur ^ 1],
