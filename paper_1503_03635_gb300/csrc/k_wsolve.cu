@@ -23,7 +23,7 @@
 // arrivals; times without are passed over.  With three launches per time step
 // a sweep was bound by them and by the largest hub, pushed by one warp: the 24
 // sweeps (2819 times) of an R-MAT graph with 65 k vertices and lengths up to
-// 100 took 45 ms, 12.7 ms now; bound by the barriers (4.5 us per time) and dependent
+// 100 took 45 ms, 12.3 ms now; bound by the barriers (4.5 us per time) and dependent
 // loads.
 //   cover:  facility f enters at time H - B_f with its key ordinal (H = the
 //           largest B_f), so every wave ends at H and the label of v at H is
