@@ -111,23 +111,20 @@ constexpr int kSmallDeg = 8;
 // 1.05 / 1.40, 15.5 M 2.65 / 1.90.
 //
 // A round costs a step per item, and a vertex is an item however short its row:
-// graphs of short rows are bounded by their items too (resident against
-// host-driven in ms, by million items).
-//   MIS, balls of up to 64 hops (kResidentMisItems): Erdos-Renyi 1.2 2.77 / 4.73,
+// graphs of short rows are bounded by their items too (kResidentItems; resident
+// against host-driven in ms, by million items).
+//   MIS, balls of up to 64 hops: Erdos-Renyi 1.2 2.77 / 4.73,
 //   1.5 12.9 / 14.1, 2.0 6.47 / 5.71; R-MAT 1.2 1.80 / 1.63, 2.0 3.34 / 2.30; square
 //   grid, 40 to 48 hops, 1.3 16.8 / 19.9 and 19.4 / 20.9, 1.6 22.1 / 22.2.
 //   MIS, larger balls, whose sweeps are mostly thin (kWideBallItems): grid, 70 to
 //   120 hops, 0.7 20.8 / 28.4, 1.0 31.4 / 37.1, 1.1 21.9 / 19.9, 1.3 21.3 / 18.2, 1.6
 //   32.4 / 23.4, 2.2 79.8 / 53.9.
-//   BFS (kResidentBfsItems): R-MAT 1.0 0.46 / 0.51, 1.2 0.41 / 0.40; Erdos-Renyi 0.8
-//   0.52 / 0.45, 1.0 0.63 / 0.47, 2.0 1.48 / 0.79; grid, 50 levels, 0.7 1.82 / 2.24, 1.0
-//   2.30 / 2.38, 2.2 4.85 / 3.38.  Host-driven rounds of a graph made of parts flag
-//   its parts as well: whole batches, replicas of R-MAT 0.96 2.97 / 3.22, 1.3 4.01 /
-//   4.12, union of Erdos-Renyi graphs 1.2 16.8 / 16.4 (kResidentBfsPartItems).
+//   BFS: R-MAT 1.0 0.30 / 0.53, 1.2 0.36 / 0.39, 2.0 0.58 / 0.64; Erdos-Renyi 1.0 0.38 /
+//   0.47, 1.5 1.05 / 1.12, 2.0 0.86 / 0.82, 4.0 3.18 / 1.80; grid, 55 levels, 1.0 1.86 /
+//   2.44, 1.4 2.51 / 2.78, 2.2 3.74 / 3.42; 6 levels 1.4 0.62 / 0.46.  Whole batches,
+//   replicas of R-MAT 1.3 3.90 / 5.09, union of Erdos-Renyi graphs 1.3 16.7 / 21.4.
 constexpr int64_t kResidentEdges = 10 << 20;
-constexpr int64_t kResidentBfsItems = 1 << 20;
-constexpr int64_t kResidentBfsPartItems = 5 << 18;
-constexpr int64_t kResidentMisItems = 3 << 19;
+constexpr int64_t kResidentItems = 3 << 19;
 constexpr int64_t kWideBallItems = 1 << 20;  // above: only balls of at most kNarrowBall hops
 constexpr int kNarrowBall = 64;
 constexpr int kItemEdges = 64;
@@ -566,7 +563,7 @@ struct fl_graph {
     fl::DBuf seg_hub;              // int32[n_seg]: hub of each segment
     int64_t n_low = 0, n_hubs = 0, n_seg = 0;
     fl::DBuf items;                // int4[n_items]: work items of the resident kernels
-    int64_t n_items = 0;           // 0: the graph is too large for them (kResidentEdges, kResidentMisItems)
+    int64_t n_items = 0;           // 0: the graph is too large for them (kResidentEdges, kResidentItems)
     fl::DBuf part;                 // uint32[n_seg*k]: partial bottom-k of each hub segment (scratch)
     // A graph that is a disjoint union of parts (batched instances): vertex v
     // of the part starting at vbase[v] has local id v - vbase[v], and ranks
@@ -728,10 +725,7 @@ int msbfs_graph(fl_graph* g, const int32_t* src_list, int64_t n_src, int32_t* la
 void graph_bfs_release(GraphBfs* c);
 // resident kernels of small graphs (k_resident.cu): graphs with work items whose
 // schedule leaves the round switches alone (a pull has no push to switch to)
-inline bool resident_mis(const fl_graph* g) { return g->n_items > 0 && !g->sched.switches_rounds(); }
-inline bool resident_bfs(const fl_graph* g) {
-    return resident_mis(g) && g->n_items <= (g->n_parts > 0 ? kResidentBfsPartItems : kResidentBfsItems);
-}
+inline bool runs_resident(const fl_graph* g) { return g->n_items > 0 && !g->sched.switches_rounds(); }
 int build_items(fl_graph* g);
 int mis_resident(fl_solve* s, int64_t m, bool* done);
 int mis_resident_queue(fl_solve* s, int64_t m, uint8_t* acc, int* outcome);

@@ -696,7 +696,7 @@ int build_items(fl_graph* g) {
         if (e == cudaSuccess) e = cudaMemcpyAsync(&c, cnt.as<int32_t>() + n - 1, 4, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) { rc = status_of(e, "work items", __FILE__, __LINE__); break; }
-        if (p + c <= kResidentMisItems) g->n_items = p + c;
+        if (p + c <= kResidentItems) g->n_items = p + c;
     } while (0);
     if (g->n_items == 0) dfree_after(st, {&g->items});
     dfree_after(st, {&cnt, &pos});

@@ -73,7 +73,7 @@ int msbfs(fl_graph* g, const int32_t* src_list, int64_t n_src, int32_t* label, i
         FL_TRY(build_work_lists(g));
         g->lists_ready = 1;
     }
-    if (resident_bfs(g)) return msbfs_resident(g, src_list, n_src, label, dist, frval, X, cls);
+    if (runs_resident(g)) return msbfs_resident(g, src_list, n_src, label, dist, frval, X, cls);
     FL_TRY(dalloc(X, (size_t)n * 16));
     FL_TRY(dalloc(stampb, (size_t)n * 4));
     FL_TRY(dalloc(fr[0], (size_t)n * 4));
@@ -1092,7 +1092,7 @@ static int candidate_keys(fl_solve* s, int64_t known, int64_t* m, unsigned long 
 // *queued = false: not for this path.
 int open_facilities_queued(fl_solve* s, int64_t known, uint8_t* acc, int* outcome, bool* queued) {
     *queued = false;
-    if (!s->g->lists_ready || !resident_mis(s->g) || known > kRankMax) return FL_OK;
+    if (!s->g->lists_ready || !runs_resident(s->g) || known > kRankMax) return FL_OK;
     int64_t m = 0;
     unsigned long long* cnt = nullptr;
     FL_TRY(candidate_keys(s, known, &m, &cnt));
@@ -1113,7 +1113,7 @@ int open_facilities(fl_solve* s) {
         FL_TRY(build_work_lists(g));
         g->lists_ready = 1;
     }
-    if (resident_mis(g)) {
+    if (runs_resident(g)) {
         bool done = false;
         FL_TRY(mis_resident(s, m, &done));
         if (done) return FL_OK;

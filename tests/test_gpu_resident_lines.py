@@ -48,14 +48,14 @@ def _check(g, cost, client, mis, bfs):
     return top
 
 
-# items = vertices: below the BFS line, between it and the MIS line, above both
-@pytest.mark.parametrize("n,mis,bfs", [(1_000_000, True, True), (1_200_000, True, False), (1_700_000, False, False)])
-def test_lines_on_items(n, mis, bfs):
+# items = vertices, below and above the line
+@pytest.mark.parametrize("n,resident", [(1_550_000, True), (1_600_000, False)])
+def test_line_on_items(n, resident):
     rowp, cols = flsynth.er(n, n, 8)
     g = fl.Graph(rowp, cols)
     g.build_sketches(4, 3)
     for cost in (20.0, 1.0e4):
-        assert _check(g, np.full(n, cost), flsynth.bernoulli(n, 2, 0.7), mis, bfs) <= 64
+        assert _check(g, np.full(n, cost), flsynth.bernoulli(n, 2, 0.7), resident, resident) <= 64
     g.close()
 
 
@@ -66,14 +66,13 @@ def test_line_of_large_balls(side, mis):
     n = len(rowp) - 1
     g = fl.Graph(rowp, cols)
     g.build_sketches(4, 3)
-    assert _check(g, np.full(n, 3.0e4), np.ones(n, np.uint8), mis, n < 1 << 20) > 64
-    assert _check(g, np.full(n, 20.0), np.ones(n, np.uint8), True, n < 1 << 20) <= 64
+    assert _check(g, np.full(n, 3.0e4), np.ones(n, np.uint8), mis, True) > 64
+    assert _check(g, np.full(n, 20.0), np.ones(n, np.uint8), True, True) <= 64
     g.close()
 
 
-# parts: the BFS line lies higher
-@pytest.mark.parametrize("n", [1_250_000, 1_350_000])
-def test_line_of_parts(n):
+@pytest.mark.parametrize("n", [1_550_000, 1_600_000])
+def test_batches_on_both_sides(n):
     per = n // 10
     rowp, cols = flsynth.er(per, per, 8)
     g = fl.Graph(rowp, cols)
