@@ -488,7 +488,7 @@ struct BfsArgs {
 constexpr int kBfsPushDiv = 128;
 constexpr int kBfsPushSteps = 4;   // items per group of lanes above which the kernel with pushes runs
 constexpr int kBfsListSteps = 16;
-constexpr int kBfsLong = 512;      // longer rows are pushed by the whole block
+constexpr int kBfsLong = 64;       // longer rows are pushed by the block's warps in parts
 constexpr int kBfsQueue = 256;     // of them, queued per block and level
 
 // Level-synchronous BFS: level L gives every vertex without a distance the
@@ -560,24 +560,26 @@ __global__ void __launch_bounds__(kResThreads, 1) k_bfs_resident(BfsArgs a) {
         }
         reached = 0;
         if (kPush && listed) {
-            // label lab to the vertex of entry e (e >= end: none), all 32 lanes
-            auto offer = [&](int64_t e, int64_t end, uint32_t lab) {
-                bool fresh = false;
-                int32_t u = 0;
-                if (e < end) {
-                    u = __ldg(&a.g.cols[e]);
-                    int32_t d = __ldcg(&a.dist[u]);
-                    if (d < 0) {
-                        d = atomicCAS(&a.dist[u], -1, (int32_t)L);
-                        fresh = d < 0;
-                        if (fresh) d = (int32_t)L;
+            // label lab to the vertices of the entries e, e + step, ... below end, four at a time (all 32 lanes)
+            auto offer = [&](int64_t e, int64_t end, int step, uint32_t lab) {
+                int32_t u[4], d[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) u[j] = e + j * step < end ? __ldg(&a.g.cols[e + j * step]) : -1;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) d[j] = u[j] >= 0 ? __ldcg(&a.dist[u[j]]) : 0;
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (d[j] < 0) d[j] = atomicCAS(&a.dist[u[j]], -1, (int32_t)L);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const bool fresh = d[j] < 0;
+                    if (u[j] >= 0 && (fresh || d[j] == (int32_t)L) && lab < __ldcg(&a.label[u[j]]))
+                        atomicMin(&a.label[u[j]], lab);
+                    const long long at = warp_append(fresh, n_next);
+                    if (at >= 0) {
+                        next[at] = u[j];
+                        reached += weight(u[j]);
                     }
-                    if (d == (int32_t)L && lab < __ldcg(&a.label[u])) atomicMin(&a.label[u], lab);
-                }
-                const long long at = warp_append(fresh, n_next);
-                if (at >= 0) {
-                    next[at] = u;
-                    reached += weight(u);
                 }
             };
             for (int64_t b = group0; b < n_front; b += groups) {
@@ -595,16 +597,18 @@ __global__ void __launch_bounds__(kResThreads, 1) k_bfs_resident(BfsArgs a) {
                     }
                 }
                 const uint32_t lab = v >= 0 ? __ldcg(&a.label[v]) : kNone;
-                for (; __any_sync(kFull, e < end); e += 8) offer(e + sub, end, lab);
+                for (; __any_sync(kFull, e < end); e += 32) offer(e + sub, end, 8, lab);
             }
             __syncthreads();
             const int queued = (int)min(s_queued, (unsigned)kBfsQueue);
+            int dealt = 0;  // 128 entries at a time, dealt to the warps in turn
             for (int q = 0; q < queued; ++q) {
                 const int32_t v = s_queue[q];
-                const int64_t end = __ldg(&a.rowp[v + 1]);
+                const int64_t beg = __ldg(&a.rowp[v]), end = __ldg(&a.rowp[v + 1]);
+                const int turn = ((int)(threadIdx.x >> 5) - dealt) & (kResWarps - 1);
                 const uint32_t lab = __ldcg(&a.label[v]);
-                for (int64_t e = __ldg(&a.rowp[v]) + (threadIdx.x & ~31); e < end; e += kResThreads)
-                    offer(e + lane, end, lab);
+                for (int64_t e = beg + 128 * turn; e < end; e += 128 * kResWarps) offer(e + lane, end, 32, lab);
+                dealt += (int)((end - beg + 127) >> 7);
             }
             __syncthreads();
             if (threadIdx.x == 0) s_queued = 0;

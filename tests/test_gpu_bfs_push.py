@@ -1,5 +1,5 @@
 """The resident BFS of the assignment on graphs whose levels push and pull in turn:
-rows at the length that a whole block takes, thin frontiers after wide ones (which
+rows at the length that a block's warps share, thin frontiers after wide ones (which
 are listed first) and wide ones after thin ones, several labels at one vertex,
 sources without edges and unreached parts."""
 import numpy as np
@@ -67,18 +67,23 @@ def _case(name):
     if name == "hubs":                      # two thin levels, then hubs of 100,000 entries (pulled)
         rowp, cols = _csr(100_050, np.repeat(np.arange(50), 100_000), np.tile(50 + np.arange(100_000), 50))
         return rowp, cols, [77, 50_123]
-    if name.startswith("row"):              # pushed rows around 512 entries, overlapping by half
+    if name.startswith("row"):              # pushed rows, overlapping by half
         deg, hubs = int(name[3:]), 3
         n0 = 1 << 17
         leaf = (np.arange(hubs)[:, None] * (deg // 2) + np.arange(deg)).ravel()
         rowp, cols, n0 = _bulk_and(hubs, np.repeat(n0 + np.arange(hubs), deg), leaf)
         return rowp, cols, [n0, n0 + 1, n0 + 2]
+    if name == "many":                      # 40 rows of 100 entries in one block's share, some vertices with 20 offers
+        n0, hubs = 1 << 17, 40
+        leaf = (np.arange(hubs)[:, None] * 5 + np.arange(100)).ravel()
+        rowp, cols, n0 = _bulk_and(hubs, np.repeat(n0 + np.arange(hubs), 100), leaf)
+        return rowp, cols, list(range(n0, n0 + hubs))
     rowp, cols, n0 = _bulk_and(100, np.zeros(0, np.int64), np.zeros(0, np.int64))
     return rowp, cols, [3, n0 + 7, n0 + 50]  # "isolated": sources without edges, unreached vertices
 
 
-@pytest.mark.parametrize("name", ["grid", "large grid", "wide then thin", "hubs", "row511", "row512", "row513",
-                                  "row3000", "isolated"])
+@pytest.mark.parametrize("name", ["grid", "large grid", "wide then thin", "hubs", "row63", "row64", "row65",
+                                  "row128", "row129", "row4097", "many", "isolated"])
 def test_assignment_matches_plain_bfs(name):
     rowp, cols, opened = _case(name)
     n = len(rowp) - 1
