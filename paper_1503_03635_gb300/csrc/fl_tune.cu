@@ -4,9 +4,10 @@
 // A schedule (fl_schedule) sets how the sketch hop lays out lanes (16 or 32
 // per vertex for k <= 16), when a hop runs sparse (frontier-driven) instead
 // of over every vertex, when a relaxation round (MIS sweeps, BFS) pulls
-// instead of pushing, and whether the assignment BFS runs as one CUDA graph
-// with its level loop on the device.  None of them changes a result.  The tuner times the
-// whole path (sketches, radii, keys and MIS, assignment) on the graph itself
+// instead of pushing (and, on graphs small enough for resident kernels, that
+// these rounds are driven by the host at all), and whether the assignment BFS
+// runs as one CUDA graph with its level loop on the device.  None of them
+// changes a result.  The tuner times the whole path (sketches, radii, keys and MIS, assignment) on the graph itself
 // under candidate schedules, by coordinate descent from the default (each
 // parameter in turn over its candidates, keeping the fastest), and keeps the
 // best; the choice is cached per graph signature (vertices, CSR entries, the
