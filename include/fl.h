@@ -395,7 +395,7 @@ int fl_hop_stats(const fl_graph* g, int64_t cap, int64_t* n_hops, int64_t* scann
  *               conditional WHILE node repeats one pull level on the device
  *               (no host round trip per level; capped at n + 2 levels,
  *               FL_ETIMEOUT beyond); 0 (default): push/pull levels driven by
- *               the host.
+ *               the host, or by one kernel on small graphs.
  *   level_cap   BFS levels at most (both forms; 0 = n + 2, never reached by
  *               a BFS); a BFS that would need more returns FL_ETIMEOUT.
  * Divisors lie in [1, 1024], graph_bfs in {0, 1}, level_cap >= 0 (FL_EINVAL

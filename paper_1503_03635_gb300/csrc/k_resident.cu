@@ -8,7 +8,7 @@
 //
 // Work items: every row is cut into items of at most kItemEdges entries (at
 // least one item per vertex), eight lanes each, so that no warp carries a
-// hub.  A round is a pull over the items: X'[v] = min(X[v], min over the row
+// hub.  A round is a pull over the items (the BFS also pushes thin frontiers): X'[v] = min(X[v], min over the row
 // of X[u]) with two value buffers.  A row of several items lowers X'[v] with
 // atomicMin; X'[v] then still holds the value of two rounds ago, which is at
 // least X[v] (values only fall within a sweep), so it needs no reset.
